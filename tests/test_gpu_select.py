@@ -213,3 +213,27 @@ def test_select_counts_eq7_eq8_on_the_device():
     m.metrics_reset()
     assert m.metrics_read() == (0, 0, 0)
     m.close()
+
+
+@pytest.mark.parametrize("n_frames,n_labels,n_ctx", [(1, 1025, 3), (2049, 40, 65), (4096, 33, 130)])
+def test_select_at_the_edges_of_its_passes(n_frames, n_labels, n_ctx):
+    """More than 32 label words (a second pass over a frame's scores), more frames than one pass of the emission
+    takes (2048), one to three mask words per frame: sets against the oracle, exactly."""
+    import torch
+    ctxs, accs = wl.random_cover_table(21, n_ctx, n_labels, 4, True)
+    m = small_model(ctxs, accs, n_labels, n_frames)
+    m.set_cover(0.6)
+    g = wl.rng_for("select_edges", n_frames)
+    scores = np.full((n_frames, n_labels), 0.1, np.float32)
+    for f in range(n_frames):
+        scores[f, g.choice(n_labels, size=int(g.integers(0, 4)), replace=False)] = 0.9
+    scores[-1, -1] = 0.9                                     # the last label of the last frame
+    off = torch.zeros(n_frames + 1, dtype=torch.int32, device="cuda")
+    ids = torch.full((n_frames * n_ctx,), -1, dtype=torch.int32, device="cuda")
+    m.select(torch.from_numpy(scores).cuda(), 0.5, False, False, None, None, None, off, ids)
+    assert m.status() == 0
+    o, i = off.cpu().numpy(), ids.cpu().numpy()
+    for f in range(n_frames):
+        want = po.detect_contexts(po.labels_from_scores(scores[f], 0.5), None, ctxs, accs, 0.6, None, False)
+        assert sorted(want) == list(i[o[f]:o[f + 1]])
+    m.close()
