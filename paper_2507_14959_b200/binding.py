@@ -86,7 +86,7 @@ def load():
     lib.pm_last_error.restype = C.c_char_p
     lib.pm_launch_count.argtypes = [vp]
     lib.pm_cooccurrence.argtypes = [vp, ip, ip, vp, vp, vp]
-    lib.pm_build_contexts.argtypes = [_FP, ip, ip, ip, ip, C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.POINTER(C.c_int)]
+    lib.pm_build_contexts.argtypes = [vp, ip, ip, ip, ip, vp, vp, C.POINTER(C.c_int)]
     lib.pm_intra_coherence.argtypes = [_FP, ip, C.POINTER(C.c_int32), C.POINTER(C.c_int32), ip, C.POINTER(C.c_double)]
     lib.pm_set_graphs.argtypes = [vp, ip]
     lib.pm_set_small_batch_kernel.argtypes = [vp, ip]
@@ -374,15 +374,16 @@ def build_contexts(co, max_size, max_contexts, allow_overlap):
     """pm_build_contexts (Algorithm 1) on a host matrix; returns the contexts as lists of label ids."""
     co = np.ascontiguousarray(co, dtype=np.float32)
     K = co.shape[0]
-    off = np.zeros(max_contexts + 1, dtype=np.int32)
-    ids = np.zeros(max_contexts * max_size, dtype=np.int32)
+    off = np.zeros(max(0, max_contexts) + 1, dtype=np.int32)
+    ids = np.zeros(max(0, max_contexts * max_size), dtype=np.int32)
     n = C.c_int(0)
-    i32 = C.POINTER(C.c_int32)
-    rc = load().pm_build_contexts(co.ctypes.data_as(_FP), K, int(max_size), int(max_contexts), int(bool(allow_overlap)),
-                                  off.ctypes.data_as(i32), ids.ctypes.data_as(i32), C.byref(n))
+    rc = load().pm_build_contexts(_ptr(co), K, int(max_size), int(max_contexts), int(bool(allow_overlap)), _ptr(off), _ptr(ids),
+                                  C.byref(n))
     if rc != PM_OK:
         raise PolymorphError(rc, "pm_build_contexts")
-    return [ids[off[c]:off[c + 1]].tolist() for c in range(n.value)]
+    bounds = off[:n.value + 1].tolist()
+    flat = ids[:bounds[-1]].tolist()
+    return [flat[b:e] for b, e in zip(bounds, bounds[1:])]
 
 
 def intra_coherence(contexts, co_norm):

@@ -85,3 +85,23 @@ def test_cooccurrence_counts_match_oracle_and_feed_algorithm_1():
     # the counted matrix drives Algorithm 1 the same way on both sides
     assert binding.build_contexts(got, 8, 40, False) == po.build_contexts(want, 8, 40, False)
     assert binding.build_contexts(got, 8, 40, True) == po.build_contexts(want, 8, 40, True)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("K,T", [(1, 40), (33, 1500), (320, 3001), (321, 3001), (1100, 300)])
+def test_cooccurrence_on_both_sides_of_the_histogram_limit(K, T):
+    """Label counts at the edges: one label, the largest label space whose histogram stays in shared memory
+    (320), the first beyond it, ragged last words and ragged last tiles of frames.  Counts are integers."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    g = np.random.default_rng(K)
+    sets = [set(int(k) for k in g.choice(K, size=int(g.integers(0, min(K, 6) + 1)), replace=False)) for _ in range(T)]
+    sets[-1] = set(range(max(0, K - 64), K))
+    bits = np.zeros((T, (K + 31) // 32), dtype=np.uint32)
+    for f, Y in enumerate(sets):
+        for k in Y:
+            bits[f, k // 32] |= np.uint32(1) << np.uint32(k % 32)
+    co = torch.full((K, K), -1.0, device="cuda")
+    binding.cooccurrence(torch.from_numpy(bits.view(np.int32)).cuda(), K, co)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(co.cpu().numpy().astype(np.float64), po.cooccurrence(sets, K))
