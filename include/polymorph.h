@@ -265,7 +265,10 @@ int pm_set_graphs(pm_handle h, int on);
  * rows from the first layer to the last.  pm_forward and pm_forward_device_sets use it for such batches
  * (same results within rounding as the layer-by-layer kernels; about 330 against 545 us per DeiT-tiny
  * frame and step on a B200); pm_set_small_batch_kernel(h, 0) sends them through the layer-by-layer kernels
- * instead.  Default on. */
+ * instead.  Larger models and batches use a second small-batch form while the switch is on: a linear whose rows
+ * are few enough for its output tiles to fit the SMs in one wave runs as one kernel (shrink, LayerNorm
+ * statistics, GEMM and LoRA terms together); switched off, every linear takes the kernels of the large batches.
+ * Default on. */
 int pm_set_small_batch_kernel(pm_handle h, int on);
 
 /* Number of kernels the library has launched on this handle since creation (kernels of a replayed graph included). */

@@ -133,6 +133,7 @@ struct LinearObj {
                 if (!ok) { err = "cuTensorMapEncodeTiled failed (half-tile operands)"; return PM_ERR_CUDA; }
                 dev.has_tm_half = true;
             }
+            if (!small_linear_encode(dev, max_adapters, slabs_max)) { err = "cuTensorMapEncodeTiled failed (few-row operands)"; return PM_ERR_CUDA; }
         }
         return PM_OK;
     }
@@ -222,6 +223,7 @@ struct Router {
         slabs_max = slabs_max_; tokens = tokens_;
         const int frames_per_pair = (2 * PM_TILE_M - 1) / tokens + 2;      // frames a 256-row pair can touch
         slab_cap = std::min(frames_per_pair * max_set, max_adapters) * slabs_max;
+        dev.tile_slab_cap = std::min(((PM_TILE_M - 1) / tokens + 2) * max_set, max_adapters) * slabs_max;
         max_tiles = (int)(((size_t)max_frames * tokens + 2 * PM_TILE_M - 1) / (2 * PM_TILE_M)) * 2;   // even
         auto take = [&](size_t& off, size_t bytes) { off = blob_bytes; blob_bytes += (bytes + 255) & ~(size_t)255; };
         take(off_perm, sizeof(int) * max_frames);
@@ -448,6 +450,7 @@ struct pm_handle_s {
     CUtensorMap tm_patch, tm_att, tm_h, tm_t, tm_x_in;
     CUtensorMap tm_y_qkv, tm_y_x, tm_y_h;      // outputs, for the TMA-store epilogue
     CUtensorMap tm_att_q, tm_att_kv;           // attention operands over QKV
+    SmallActMaps sm_patch, sm_att, sm_h, sm_x;  // x operands of the few-row linear kernel
     int tm_rows = -1;
     Router router;
     // adapters
@@ -607,7 +610,9 @@ int encode_activation_maps(pm_handle_s* h, int rows) {
            && tm_encode_2d(&h->tm_y_x, h->X.p, d, rows, (uint64_t)d * 2, 32, 32, 64)
            && tm_encode_2d(&h->tm_y_h, h->H.p, h->cfg.mlp, rows, (uint64_t)h->cfg.mlp * 2, 32, 32, 64)
            && attention_encode_maps(h->QKV.as<bf16>(), rows / h->tokens, h->tokens, h->cfg.heads, &h->tm_att_q,
-                                    &h->tm_att_kv);
+                                    &h->tm_att_kv)
+           && small_act_encode(&h->sm_patch, h->PATCH.p, h->patch_dim, prow) && small_act_encode(&h->sm_x, h->X.p, d, rows)
+           && small_act_encode(&h->sm_att, h->ATT.p, d, rows) && small_act_encode(&h->sm_h, h->H.p, h->cfg.mlp, rows);
     if (!ok) { h->err = "cuTensorMapEncodeTiled failed (activations)"; return PM_ERR_CUDA; }
     h->tm_rows = rows;
     return PM_OK;
@@ -638,6 +643,12 @@ int forward_t(pm_handle_s* h, const void* frames, int n_frames, int n_slots, int
                       int epi, const T* residual, const PatchEpi& pep, T* y, const float2* st = nullptr) -> cudaError_t {
         if constexpr (TC) {
             const bool use_lora = lora && R.max_set > 0 && lo.n_adapted > 0;
+            // few rows: the whole linear in one kernel, with tiles for one wave of the SMs
+            if (h->lat_on && small_linear_fits(lo.dev, use_lora ? &R : nullptr, nrows, epi, h->n_sms)) {
+                const SmallActMaps& sx = tmx == &h->tm_patch ? h->sm_patch : tmx == &h->tm_att ? h->sm_att : tmx == &h->tm_h ? h->sm_h : h->sm_x;
+                return launch_small_linear(L, lo.dev, use_lora ? &R : nullptr, sx, nrows, epi, (const bf16*)residual, pep, (bf16*)y,
+                                           h->n_sms, c.ln_eps);
+            }
             if (use_lora) {
                 // with LayerNorm folded in, the shrink computes the row statistics on its way through x
                 cudaError_t e = launch_shrink(L, lo.dev, R, tmx, (const bf16*)x, nrows, h->tbuf.as<bf16>(), h->n_sms,
@@ -1279,7 +1290,13 @@ int pm_linear_forward(pm_linear l, const void* x, int n_frames, const int32_t* s
     const RouteDev& R = l->router.dev;
     const int rows = n_frames * l->tokens;
     PatchEpi none;
-    if (l->dtype == 0) {
+    if (l->dtype == 0 && small_linear_fits(l->lin.dev, &R, rows, l->epilogue, l->n_sms)) {
+        SmallActMaps sx;
+        if (((uintptr_t)x | (uintptr_t)y | (uintptr_t)residual) & 15 || !small_act_encode(&sx, x, l->k_in, rows)) {
+            err = "x, y and residual must be 16-byte aligned"; return PM_ERR_CUDA;
+        }
+        CK(launch_small_linear(L, l->lin.dev, &R, sx, rows, l->epilogue, (const bf16*)residual, none, (bf16*)y, l->n_sms, 0.f));
+    } else if (l->dtype == 0) {
         CUtensorMap tm_x;
         if (!tm_encode_2d(&tm_x, x, l->k_in, rows, (uint64_t)l->k_in * 2, 64, PM_TILE_M, 128)) {
             err = "cuTensorMapEncodeTiled failed (x); x must be 16-byte aligned"; return PM_ERR_CUDA;

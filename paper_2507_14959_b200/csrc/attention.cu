@@ -637,11 +637,13 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    dep_release();
 
     if (warp == 0) {
         if (lane == 0) {
             // ---------------------------------------------------------------- TMA producer
             bool ok = true;
+            dep_wait();                            // everything else follows from what these loads bring
             for (int j = 0; j < my_items && ok; ++j) {
                 const int buf = j & 1;
                 // the buffer's previous item (j - 2) must be through its last P V product
@@ -776,6 +778,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
 
     // ---------------------------------------------------------------------- teardown
     __syncwarp();
+    dep_wait();               // never finish before the kernel this one was allowed to overtake
     if (*abort_flag) {
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);    // let copies / MMAs in flight land
     }
@@ -822,9 +825,9 @@ cudaError_t launch_attention_tc(const Launch& L, const CUtensorMap& tm_q, const 
         static SmemGrant grant;
         if (cudaError_t e = grant.ensure(attention_pipe_kernel, (int)psmem); e != cudaSuccess) return e;
         ProfScope ps(L, KC_ATTENTION);
-        attention_pipe_kernel<<<std::min(pa.n_items, n_sms), APIPE_THREADS, psmem, L.st>>>(tm_q, tm_kv, pa);
+        cudaError_t e = launch_overlapped(attention_pipe_kernel, std::min(pa.n_items, n_sms), APIPE_THREADS, psmem, L.st, 1, tm_q, tm_kv, pa);
         BUMP(L);
-        return cudaGetLastError();
+        return e;
     }
     // all of tensor memory and most of the shared memory: one CTA per SM
     size_t smem = (size_t)AQ_BYTES + (size_t)a.n_blocks * 2 * AKB_BYTES + 160 + 2 * ATT_MAX_SHARES * AQ * sizeof(float);

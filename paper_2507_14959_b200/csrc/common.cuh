@@ -15,6 +15,7 @@
 typedef __nv_bfloat16 bf16;
 
 #define PM_TILE_M 128          // rows of one GEMM tile
+#define PM_SMALL_WIDTHS 4      // tile widths of the few-row linear kernel: 64, 128, 192, 256
 #define PM_SLAB 16             // LoRA ranks are handled in slabs of 16 (one UMMA K step)
 
 // ---------------------------------------------------------------------------------------
@@ -39,6 +40,8 @@ struct LinearDev {
     // n_out a multiple of 256: boxes of 128 output columns for the CTA-pair GEMM
     CUtensorMap tm_w_half, tm_bt_half;
     bool has_tm_half = false;
+    // the few-row kernel's (small_linear.cu), by index of its tile width
+    CUtensorMap tm_sw[PM_SMALL_WIDTHS], tm_sbt[PM_SMALL_WIDTHS], tm_sat[2];      // tm_sat: one, two K blocks per copy
     // LayerNorm folded into this linear (its input is the raw residual stream x, not LN(x)):
     //   LN(x) W + b = rstd (x W' - mu g) + b',  W' = gamma o W,  g[n] = sum_k W'[k,n],  b' = b + beta W
     // Wt / bias above then hold W' / b'; the LoRA arena holds A' = gamma o A and, per arena rank j,
@@ -52,6 +55,7 @@ struct LinearDev {
 // frames by adapter set).  All arrays live on the device.
 struct RouteDev {
     int n_frames = 0, tokens = 0, n_tiles = 0, slab_cap = 0, max_set = 0;
+    int tile_slab_cap = 0;      // slabs the rows of one 128-row tile can use
     int* perm = nullptr;        // [F] slot -> caller's frame index
     int* slot_off = nullptr;    // [F+1] CSR over slots
     int* slot_ids = nullptr;    // [nnz] ascending adapter ids per slot
@@ -161,6 +165,16 @@ cudaError_t launch_lora_gemm(const Launch& L, const LinearDev& lin, const RouteD
                              const CUtensorMap& tm_x, const CUtensorMap* tm_t, const CUtensorMap* tm_y,
                              int rows, int epi, const bf16* residual, const PatchEpi& pe, bf16* y,
                              int n_sms, const float2* ln_stats, bool after_shrink = false);
+// ---- one kernel per linear for few rows (small_linear.cu)
+// Tensor maps of an activation as its x operand: one, two K blocks per copy (tm_encode_kblocks, 128 rows).
+struct SmallActMaps { CUtensorMap k[2]; };
+bool small_linear_encode(LinearDev& lin, int max_adapters, int slabs_max);
+bool small_act_encode(SmallActMaps* m, const void* x, int k_in, uint64_t rows);
+// whether launch_small_linear serves this call (R: null = no adapters)
+bool small_linear_fits(const LinearDev& lin, const RouteDev* R, int rows, int epi, int n_sms);
+// The whole linear -- shrink, LayerNorm statistics where the LayerNorm is folded in, GEMM, expand, epilogue -- in one launch.
+cudaError_t launch_small_linear(const Launch& L, const LinearDev& lin, const RouteDev* R, const SmallActMaps& x, int rows,
+                                int epi, const bf16* residual, const PatchEpi& pe, bf16* y, int n_sms, float ln_eps);
 // x rows of slots [first_slot, n_slots) <- x rows of slot src_slot[slot] (a slot below first_slot)
 template <typename T>
 cudaError_t launch_fanout_rows(const Launch& L, T* x, const int* src_slot, int first_slot, int n_slots,
@@ -252,9 +266,40 @@ size_t latency_smem_bytes(int d, int mlp, int patch_dim, int tokens, int layers)
 // with an error instead of starting if it cannot be.
 cudaError_t launch_latency_forward(const Launch& L, const LatArgs& a);
 
+// Launch with programmatic stream serialization (the kernel may start once every CTA of the one before it on the
+// stream has released its dependents; it awaits that kernel's results itself with dep_wait()), with or
+// without thread-block clusters along x.
+template <typename... P, typename... A>
+cudaError_t launch_overlapped(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t st, int cluster, const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 // tensor-map helpers (gemm_tcgen05.cu); return false if the driver entry point is unavailable
 bool tm_encode_2d(CUtensorMap* tm, const void* base, uint64_t inner, uint64_t outer,
                   uint64_t row_stride_bytes, uint32_t box_inner, uint32_t box_outer, int swizzle);
 bool tm_encode_3d(CUtensorMap* tm, const void* base, uint64_t d0, uint64_t d1, uint64_t d2,
                   uint64_t stride1_bytes, uint64_t stride2_bytes, uint32_t b0, uint32_t b1,
                   uint32_t b2, int swizzle);
+bool tm_encode_4d(CUtensorMap* tm, const void* base, const uint64_t* dims4, const uint64_t* strides3, const uint32_t* box4,
+                  int swizzle);
+// K-major [rows, k_in] operand in blocks of 64 columns: one copy (coordinates 0, row, block) brings rows_box rows of
+// kps blocks, each block 128B-swizzled by itself.  The thread that issues the copies spends about 170 clocks on
+// a pipeline stage's barriers and 44 on each copy whatever its size, so narrow stages take two blocks at once.
+bool tm_encode_kblocks(CUtensorMap* tm, const void* base, int k_in, uint64_t rows, int rows_box, int kps);
+// The same for one LoRA slab (16 arena rows): one copy (coordinates 0, 0, block, row / 8) brings its rows of kps
+// blocks as [2 groups of 8 rows][kps blocks][8 rows][128 bytes], so that slabs stack with a constant distance of
+// kps * 1024 bytes between 8-row groups.
+bool tm_encode_slab(CUtensorMap* tm, const void* base, int k_in, uint64_t rows, int kps);

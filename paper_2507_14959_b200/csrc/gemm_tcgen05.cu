@@ -16,6 +16,7 @@
 // When n_out is a multiple of 256 the CTA-pair variant (lora_gemm_pair_kernel, cta_group::2, 256 x 256
 // tiles) is used; the single-CTA kernel serves the narrower shapes.
 #include "common.cuh"
+#include "f32x2.cuh"
 #include "tcgen05_ptx.cuh"
 
 #define BUMP(L) do { if ((L).launches) ++*(L).launches; } while (0)
@@ -27,60 +28,6 @@ constexpr int BK = 64;
 constexpr int STAGES = 4;
 constexpr int SHRINK_THREADS = 192;
 constexpr int SLABS_PER_STAGE = 4;
-
-// Exact-erf GELU x * Phi(x), evaluated in logistic form: Phi(x) = 1 / (1 + exp(-2 x p(x^2))) holds
-// exactly for p = atanh(erf(x / sqrt 2)) / x, which a quadratic in x^2 fits well enough that
-//   | x (1/2 + 1/2 tanh(x q(x^2))) - gelu(x) | < 2.6e-5   for all x     (q = p: 1 / (1 + e^-2u) = 1/2 + 1/2 tanh u),
-// far below the bf16 rounding of the stored result except where the result itself is below 1e-2; the
-// hardware tanh (tanh.approx.f32, relative error about 2^-11) adds less than a quarter of a bf16 step.
-// The epilogue warps share their issue slots with the thread that issues the MMAs, so every
-// instruction saved here counts: the arithmetic runs on pairs (packed fp32) and costs one special-function
-// instruction per element (the form x / (1 + 2^(x q)) it replaces needed an exponential and a
-// reciprocal: fused GEMMs 2.3 % slower in the bench step).
-
-// Two fp32 values in one 64-bit register, for the packed fp32 arithmetic of sm_100 (one issue slot
-// for two results; each half is the ordinary IEEE operation).
-__device__ __forceinline__ uint64_t pk2(float a, float b) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void upk2(uint64_t r, float& a, float& b) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-    uint64_t d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-// the GELU described above, on a pair
-__device__ __forceinline__ uint64_t gelu_erf2(uint64_t v) {
-    // v^2 is capped where Phi has long saturated (the fitted q turns over beyond |v| = 7.2)
-    float t0, t1;
-    upk2(mul2(v, v), t0, t1);
-    const uint64_t t = pk2(fminf(t0, 50.f), fminf(t1, 50.f));
-    uint64_t q = fma2(t, pk2(-3.5151945e-04f, -3.5151945e-04f), pk2(3.7005664e-02f, 3.7005664e-02f));
-    q = fma2(q, t, pk2(0.79750784f, 0.79750784f));
-    float w0, w1, h0, h1;
-    upk2(mul2(v, q), w0, w1);
-    asm("tanh.approx.f32 %0, %1;" : "=f"(h0) : "f"(w0));
-    asm("tanh.approx.f32 %0, %1;" : "=f"(h1) : "f"(w1));
-    return mul2(v, fma2(pk2(h0, h1), pk2(0.5f, 0.5f), pk2(0.5f, 0.5f)));
-}
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-    __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<uint32_t*>(&h);
-}
 
 struct GemmArgs {
     int rows, k_in, n_out, m_tiles, n_tiles, epi;
@@ -1108,6 +1055,30 @@ bool tm_encode_3d(CUtensorMap* tm, const void* base, uint64_t d0, uint64_t d1, u
     return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, swz(swizzle), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool tm_encode_4d(CUtensorMap* tm, const void* base, const uint64_t* dims4, const uint64_t* strides3, const uint32_t* box4,
+                  int swizzle) {
+    EncodeTiledFn fn = get_encode();
+    if (!fn) return false;
+    const cuuint64_t dims[4] = {dims4[0], dims4[1], dims4[2], dims4[3]};
+    const cuuint64_t strides[3] = {strides3[0], strides3[1], strides3[2]};
+    const cuuint32_t box[4] = {box4[0], box4[1], box4[2], box4[3]};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, swz(swizzle), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool tm_encode_kblocks(CUtensorMap* tm, const void* base, int k_in, uint64_t rows, int rows_box, int kps) {
+    return tm_encode_3d(tm, base, 64, rows, (uint64_t)(k_in / 64), (uint64_t)k_in * 2, 128, 64, rows_box, kps, 128);
+}
+
+bool tm_encode_slab(CUtensorMap* tm, const void* base, int k_in, uint64_t rows, int kps) {
+    const uint64_t dims[4] = {64, 8, (uint64_t)(k_in / 64), rows / 8};
+    const uint64_t strides[3] = {(uint64_t)k_in * 2, 128, (uint64_t)k_in * 16};
+    const uint32_t box[4] = {64, 8, (uint32_t)kps, 2};
+    return tm_encode_4d(tm, base, dims, strides, box, 128);
 }
 
 cudaError_t launch_shrink(const Launch& L, const LinearDev& lin, const RouteDev& R,

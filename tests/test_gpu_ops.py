@@ -282,3 +282,48 @@ def test_bounded_wait_gives_up_and_reports():
                                atol=2e-4)
     with pytest.raises(binding.PolymorphError):
         binding.selftest_wait_timeout(10 ** 12, status, trace)       # limits beyond 1e8 cycles are refused
+
+
+@pytest.mark.parametrize("k_in,n_out,frames,tokens,rank,epi,what", [
+    (768, 768, 1, 197, 16, 2, "64-wide tiles"), (320, 576, 2, 130, 24, 0, "64-wide tiles, odd K blocks"),
+    (768, 2304, 3, 197, 64, 0, "128-wide tiles, several slab groups"), (192, 1152, 16, 128, 16, 1, "192-wide tiles, whole row tiles"),
+    (768, 3072, 6, 197, 16, 1, "256-wide tiles"), (3072, 768, 1, 197, 16, 2, "64-wide, K in four"),
+    (1600, 768, 3, 200, 16, 2, "128-wide, K in four, odd K blocks"), (3072, 768, 6, 197, 8, 2, "128-wide, K in two"),
+    (3072, 768, 8, 197, 48, 2, "192-wide, K in two, several slab groups"), (3072, 768, 12, 197, 16, 2, "256-wide, K in two"),
+    (3072, 768, 17, 197, 16, 2, "unsplit"), (768, 768, 33, 197, 16, 2, "beyond one wave: shrink and pair GEMM"),
+    (384, 1152, 30, 197, 16, 0, "beyond one wave, narrow"), (64, 64, 1, 1, 4, 0, "one row")])
+def test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, what):
+    """One case on each side of every line of the few-row kernel's tile rule (on 148 SMs), sets of 0 to 6 of 7
+    adapters, against float64 sums of the same bf16 inputs.  Tolerance: as for the other linears (one bf16 rounding of
+    the output, one of t)."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    gen = torch.Generator(device="cuda").manual_seed(k_in + n_out + frames)
+
+    def draw(shape, std):
+        return (torch.randn(shape, generator=gen, device="cuda") * std).bfloat16()
+    rows, n_ad = frames * tokens, 7
+    x, res, w, b = draw((rows, k_in), 1.0), draw((rows, n_out), 1.0), draw((k_in, n_out), 0.02), draw((n_out,), 0.02)
+    A = [draw((k_in, rank), 0.02) for _ in range(n_ad)]
+    B = [draw((rank, n_out), 0.02) for _ in range(n_ad)]
+    g = np.random.default_rng(rows)
+    sets = [sorted(int(a) for a in g.choice(n_ad, size=int(g.integers(0, 7)), replace=False)) for _ in range(frames)]
+    off, ids = wl.sets_to_csr(sets)
+    host = lambda t: t.float().cpu().numpy()  # noqa: E731
+    lin = binding.Linear(host(w), host(b), max_adapters=n_ad, max_rank=rank, max_set=6, max_frames=frames, tokens=tokens, epilogue=epi)
+    for a in range(n_ad):
+        lin.register(a, rank, 2.0, host(A[a]), host(B[a]))
+    y = torch.full((rows, n_out), float("nan"), device="cuda", dtype=torch.bfloat16)
+    lin.forward(x, frames, off, ids, y, residual=res if epi == 2 else None)
+    assert lin.status() == 0
+    want = x.double() @ w.double() + b.double()
+    for f, s in enumerate(sets):
+        r = slice(f * tokens, (f + 1) * tokens)
+        for a in s:
+            want[r] += 2.0 * (x[r].double() @ A[a].double()) @ B[a].double()
+    if epi == 1:
+        want = torch.nn.functional.gelu(want)
+    elif epi == 2:
+        want = want + res.double()
+    np.testing.assert_allclose(to_np(y), want.cpu().numpy(), **TOL[0])
+    lin.close()
