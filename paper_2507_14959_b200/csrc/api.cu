@@ -450,7 +450,7 @@ struct pm_handle_s {
     CUtensorMap tm_patch, tm_att, tm_h, tm_t, tm_x_in;
     CUtensorMap tm_y_qkv, tm_y_x, tm_y_h;      // outputs, for the TMA-store epilogue
     CUtensorMap tm_att_q, tm_att_kv;           // attention operands over QKV
-    SmallActMaps sm_patch, sm_att, sm_h, sm_x;  // x operands of the few-row linear kernel
+    ActMaps sm_patch, sm_att, sm_h, sm_x;  // x operands of the few-row linear kernel and the shrink
     int tm_rows = -1;
     Router router;
     // adapters
@@ -611,8 +611,8 @@ int encode_activation_maps(pm_handle_s* h, int rows) {
            && tm_encode_2d(&h->tm_y_h, h->H.p, h->cfg.mlp, rows, (uint64_t)h->cfg.mlp * 2, 32, 32, 64)
            && attention_encode_maps(h->QKV.as<bf16>(), rows / h->tokens, h->tokens, h->cfg.heads, &h->tm_att_q,
                                     &h->tm_att_kv)
-           && small_act_encode(&h->sm_patch, h->PATCH.p, h->patch_dim, prow) && small_act_encode(&h->sm_x, h->X.p, d, rows)
-           && small_act_encode(&h->sm_att, h->ATT.p, d, rows) && small_act_encode(&h->sm_h, h->H.p, h->cfg.mlp, rows);
+           && act_encode(&h->sm_patch, h->PATCH.p, h->patch_dim, prow) && act_encode(&h->sm_x, h->X.p, d, rows)
+           && act_encode(&h->sm_att, h->ATT.p, d, rows) && act_encode(&h->sm_h, h->H.p, h->cfg.mlp, rows);
     if (!ok) { h->err = "cuTensorMapEncodeTiled failed (activations)"; return PM_ERR_CUDA; }
     h->tm_rows = rows;
     return PM_OK;
@@ -644,15 +644,13 @@ int forward_t(pm_handle_s* h, const void* frames, int n_frames, int n_slots, int
         if constexpr (TC) {
             const bool use_lora = lora && R.max_set > 0 && lo.n_adapted > 0;
             // few rows: the whole linear in one kernel, with tiles for one wave of the SMs
-            if (h->lat_on && small_linear_fits(lo.dev, use_lora ? &R : nullptr, nrows, epi, h->n_sms)) {
-                const SmallActMaps& sx = tmx == &h->tm_patch ? h->sm_patch : tmx == &h->tm_att ? h->sm_att : tmx == &h->tm_h ? h->sm_h : h->sm_x;
+            const ActMaps& sx = tmx == &h->tm_patch ? h->sm_patch : tmx == &h->tm_att ? h->sm_att : tmx == &h->tm_h ? h->sm_h : h->sm_x;
+            if (h->lat_on && small_linear_fits(lo.dev, use_lora ? &R : nullptr, nrows, epi, h->n_sms))
                 return launch_small_linear(L, lo.dev, use_lora ? &R : nullptr, sx, nrows, epi, (const bf16*)residual, pep, (bf16*)y,
                                            h->n_sms, c.ln_eps);
-            }
             if (use_lora) {
                 // with LayerNorm folded in, the shrink computes the row statistics on its way through x
-                cudaError_t e = launch_shrink(L, lo.dev, R, tmx, (const bf16*)x, nrows, h->tbuf.as<bf16>(), h->n_sms,
-                                              nullptr, const_cast<float2*>(st), c.ln_eps);
+                cudaError_t e = launch_shrink(L, lo.dev, R, sx, nrows, h->tbuf.as<bf16>(), h->n_sms, const_cast<float2*>(st), c.ln_eps);
                 if (e != cudaSuccess) return e;
             } else if (st) {
                 cudaError_t e = launch_row_stats(L, (const bf16*)x, const_cast<float2*>(st), nrows, lo.dev.k_in, c.ln_eps);
@@ -1291,8 +1289,8 @@ int pm_linear_forward(pm_linear l, const void* x, int n_frames, const int32_t* s
     const int rows = n_frames * l->tokens;
     PatchEpi none;
     if (l->dtype == 0 && small_linear_fits(l->lin.dev, &R, rows, l->epilogue, l->n_sms)) {
-        SmallActMaps sx;
-        if (((uintptr_t)x | (uintptr_t)y | (uintptr_t)residual) & 15 || !small_act_encode(&sx, x, l->k_in, rows)) {
+        ActMaps sx;
+        if (((uintptr_t)x | (uintptr_t)y | (uintptr_t)residual) & 15 || !act_encode(&sx, x, l->k_in, rows)) {
             err = "x, y and residual must be 16-byte aligned"; return PM_ERR_CUDA;
         }
         CK(launch_small_linear(L, l->lin.dev, &R, sx, rows, l->epilogue, (const bf16*)residual, none, (bf16*)y, l->n_sms, 0.f));
@@ -1306,7 +1304,11 @@ int pm_linear_forward(pm_linear l, const void* x, int n_frames, const int32_t* s
             err = "cuTensorMapEncodeTiled failed (y); y must be 16-byte aligned"; return PM_ERR_CUDA;
         }
         const bool lora = R.max_set > 0 && l->lin.dev.lora.At != nullptr;
-        if (lora) CK(launch_shrink(L, l->lin.dev, R, &tm_x, (const bf16*)x, rows, l->tbuf.as<bf16>(), l->n_sms, nullptr, nullptr, 0.f));
+        if (lora) {
+            ActMaps sx;
+            if (!act_encode(&sx, x, l->k_in, rows)) { err = "cuTensorMapEncodeTiled failed (x)"; return PM_ERR_CUDA; }
+            CK(launch_shrink(L, l->lin.dev, R, sx, rows, l->tbuf.as<bf16>(), l->n_sms, nullptr, 0.f));
+        }
         CK(launch_lora_gemm(L, l->lin.dev, lora ? &R : nullptr, tm_x, &l->tm_t, &tm_y, rows, l->epilogue,
                             (const bf16*)residual, none, (bf16*)y, l->n_sms, nullptr, lora));
     } else {

@@ -41,7 +41,8 @@ struct LinearDev {
     CUtensorMap tm_w_half, tm_bt_half;
     bool has_tm_half = false;
     // the few-row kernel's (small_linear.cu), by index of its tile width
-    CUtensorMap tm_sw[PM_SMALL_WIDTHS], tm_sbt[PM_SMALL_WIDTHS], tm_sat[2];      // tm_sat: one, two K blocks per copy
+    CUtensorMap tm_sw[PM_SMALL_WIDTHS], tm_sbt[PM_SMALL_WIDTHS];
+    CUtensorMap tm_sat[2];             // one adapter slab, one / two K blocks per copy (few-row kernel and shrink)
     // LayerNorm folded into this linear (its input is the raw residual stream x, not LN(x)):
     //   LN(x) W + b = rstd (x W' - mu g) + b',  W' = gamma o W,  g[n] = sum_k W'[k,n],  b' = b + beta W
     // Wt / bias above then hold W' / b'; the LoRA arena holds A' = gamma o A and, per arena rank j,
@@ -149,13 +150,16 @@ cudaError_t launch_naive_linear(const Launch& L, const LinearDev& lin, const Rou
                                 const AdapterMeta& meta, int slabs_max, const T* x, int rows,
                                 int tokens_per_frame, float* t32, int epi, const T* residual,
                                 const PatchEpi& pe, T* y);
-// tensor-core path (bf16): shrink into the slab buffer, then the fused GEMM
-// A linear with LayerNorm folded in (lin.ln_g != null) needs per-row (mean, 1/sqrt(var + eps)) of x:
-// either ln_stats (already computed) or stats_out (the shrink computes them from the x tiles it
-// streams anyway, uses them and leaves them there for the GEMM), never both.
-cudaError_t launch_shrink(const Launch& L, const LinearDev& lin, const RouteDev& R,
-                          const CUtensorMap* tm_x, const bf16* x, int rows, bf16* tbuf, int n_sms,
-                          const float2* ln_stats, float2* stats_out, float ln_eps);
+// Tensor maps of an activation as the x operand of the shrink and of the few-row linear kernel: one, two K blocks per
+// copy (tm_encode_kblocks, 128 rows).
+struct ActMaps { CUtensorMap k[2]; };
+bool act_encode(ActMaps* m, const void* x, int k_in, uint64_t rows);
+// tensor-core path (bf16): shrink into the slab buffer (shrink.cu), then the fused GEMM
+// A linear with LayerNorm folded in (lin.ln_g != null) needs per-row (mean, 1/sqrt(var + eps)) of x: the shrink
+// computes them from the x tiles it streams anyway, uses them and leaves them in stats_out for the GEMM; null for a
+// linear without.
+cudaError_t launch_shrink(const Launch& L, const LinearDev& lin, const RouteDev& R, const ActMaps& x, int rows,
+                          bf16* tbuf, int n_sms, float2* stats_out, float ln_eps);
 cudaError_t launch_row_stats(const Launch& L, const bf16* x, float2* stats, int rows, int d, float eps);
 // after_shrink: the kernel enqueued just before on the stream is this linear's launch_shrink; the GEMM
 // may then start before it has finished (programmatic dependent launch) and awaits its results itself.
@@ -166,14 +170,11 @@ cudaError_t launch_lora_gemm(const Launch& L, const LinearDev& lin, const RouteD
                              int rows, int epi, const bf16* residual, const PatchEpi& pe, bf16* y,
                              int n_sms, const float2* ln_stats, bool after_shrink = false);
 // ---- one kernel per linear for few rows (small_linear.cu)
-// Tensor maps of an activation as its x operand: one, two K blocks per copy (tm_encode_kblocks, 128 rows).
-struct SmallActMaps { CUtensorMap k[2]; };
 bool small_linear_encode(LinearDev& lin, int max_adapters, int slabs_max);
-bool small_act_encode(SmallActMaps* m, const void* x, int k_in, uint64_t rows);
 // whether launch_small_linear serves this call (R: null = no adapters)
 bool small_linear_fits(const LinearDev& lin, const RouteDev* R, int rows, int epi, int n_sms);
 // The whole linear -- shrink, LayerNorm statistics where the LayerNorm is folded in, GEMM, expand, epilogue -- in one launch.
-cudaError_t launch_small_linear(const Launch& L, const LinearDev& lin, const RouteDev* R, const SmallActMaps& x, int rows,
+cudaError_t launch_small_linear(const Launch& L, const LinearDev& lin, const RouteDev* R, const ActMaps& x, int rows,
                                 int epi, const bf16* residual, const PatchEpi& pe, bf16* y, int n_sms, float ln_eps);
 // x rows of slots [first_slot, n_slots) <- x rows of slot src_slot[slot] (a slot below first_slot)
 template <typename T>

@@ -632,7 +632,7 @@ bool small_linear_encode(LinearDev& lin, int max_adapters, int slabs_max) {
     return true;
 }
 
-bool small_act_encode(SmallActMaps* m, const void* x, int k_in, uint64_t rows) {
+bool act_encode(ActMaps* m, const void* x, int k_in, uint64_t rows) {
     return tm_encode_kblocks(&m->k[0], x, k_in, rows, BM, 1) && tm_encode_kblocks(&m->k[1], x, k_in, rows, BM, 2);
 }
 
@@ -645,7 +645,7 @@ bool small_linear_fits(const LinearDev& lin, const RouteDev* R, int rows, int ep
     return pick_shape(lin, lora, rows, epi, n_sms).width >= 0 && (!lora || R->tile_slab_cap <= LIST);
 }
 
-cudaError_t launch_small_linear(const Launch& L, const LinearDev& lin, const RouteDev* R, const SmallActMaps& x, int rows,
+cudaError_t launch_small_linear(const Launch& L, const LinearDev& lin, const RouteDev* R, const ActMaps& x, int rows,
                                 int epi, const bf16* residual, const PatchEpi& pe, bf16* y, int n_sms, float ln_eps) {
     if (rows <= 0) return cudaSuccess;
     const bool lora = has_lora(lin, R);

@@ -291,7 +291,10 @@ def test_bounded_wait_gives_up_and_reports():
     (1600, 768, 3, 200, 16, 2, "128-wide, K in four, odd K blocks"), (3072, 768, 6, 197, 8, 2, "128-wide, K in two"),
     (3072, 768, 8, 197, 48, 2, "192-wide, K in two, several slab groups"), (3072, 768, 12, 197, 16, 2, "256-wide, K in two"),
     (3072, 768, 17, 197, 16, 2, "unsplit"), (768, 768, 33, 197, 16, 2, "beyond one wave: shrink and pair GEMM"),
-    (384, 1152, 30, 197, 16, 0, "beyond one wave, narrow"), (64, 64, 1, 1, 4, 0, "one row")])
+    (384, 1152, 30, 197, 16, 0, "beyond one wave, narrow"),
+    (1600, 1536, 20, 197, 16, 2, "shrink with K in four, odd K blocks"), (1536, 1536, 40, 197, 48, 2, "shrink with K in two, several slab groups"),
+    (320, 768, 70, 130, 64, 1, "shrink of one tile per SM, odd K blocks, slabs beyond the list"),
+    (192, 768, 300, 100, 24, 0, "shrink of two tiles per SM"), (192, 256, 300, 197, 40, 1, "shrink of three tiles per SM"), (64, 64, 1, 1, 4, 0, "one row")])
 def test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, what):
     """One case on each side of every line of the few-row kernel's tile rule (on 148 SMs), sets of 0 to 6 of 7
     adapters, against float64 sums of the same bf16 inputs.  Tolerance: as for the other linears (one bf16 rounding of
