@@ -125,14 +125,7 @@ struct LinearObj {
             }
             if (!ok) { err = "cuTensorMapEncodeTiled failed (static operands)"; return PM_ERR_CUDA; }
             dev.has_tm = true;
-            if (n_out % 256 == 0) {
-                ok = tm_encode_2d(&dev.tm_w_half, wt.p, k_in, n_out, (uint64_t)k_in * 2, 64, 128, 128);
-                if (ok && dev.lora.At)
-                    ok = tm_encode_2d(&dev.tm_bt_half, bt.p, PM_SLAB, (uint64_t)max_adapters * slabs_max * n_out,
-                                      PM_SLAB * 2, PM_SLAB, 128, 32);
-                if (!ok) { err = "cuTensorMapEncodeTiled failed (half-tile operands)"; return PM_ERR_CUDA; }
-                dev.has_tm_half = true;
-            }
+            if (!gemm_encode_pair_maps(dev, max_adapters, slabs_max)) { err = "cuTensorMapEncodeTiled failed (half-tile operands)"; return PM_ERR_CUDA; }
             if (!small_linear_encode(dev, max_adapters, slabs_max)) { err = "cuTensorMapEncodeTiled failed (few-row operands)"; return PM_ERR_CUDA; }
         }
         return PM_OK;

@@ -339,6 +339,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        dep_wait();                            // everything else follows from what these loads bring
         // all operand loads of the head go out before tensor memory is requested, in the order of their
         // first use and each block on a barrier of its own: the first scores need the query tile and the
         // first key block only
@@ -363,6 +364,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     const uint32_t o_tmem = tmem_base + args.o_col;
+    dep_release();
 
     if (warp == 0) {
         if (lane == 0) {
@@ -546,6 +548,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 
     // ---------------------------------------------------------------------- teardown
     __syncwarp();
+    dep_wait();               // never finish before the kernel this one was allowed to overtake
     if (*abort_flag) {
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);    // let copies / MMAs in flight land
     }
@@ -834,9 +837,10 @@ cudaError_t launch_attention_tc(const Launch& L, const CUtensorMap& tm_q, const 
     static SmemGrant grant;
     if (cudaError_t e = grant.ensure(attention_tc_kernel<ATT_SHARES>, (int)smem); e != cudaSuccess) return e;
     ProfScope ps(L, KC_ATTENTION);
-    attention_tc_kernel<ATT_SHARES><<<n_frames * heads * a.q_split, 32 + 128 * ATT_SHARES, smem, L.st>>>(tm_q, tm_kv, a);
+    cudaError_t e = launch_overlapped(attention_tc_kernel<ATT_SHARES>, n_frames * heads * a.q_split, 32 + 128 * ATT_SHARES, smem, L.st, 1,
+                                      tm_q, tm_kv, a);
     BUMP(L);
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_attention_mma(const Launch& L, const bf16* qkv, bf16* out, int n_frames, int tokens,

@@ -15,6 +15,7 @@
 typedef __nv_bfloat16 bf16;
 
 #define PM_TILE_M 128          // rows of one GEMM tile
+#define PM_PAIR_WIDTHS 2       // tile widths of the CTA-pair GEMM: 192, 256
 #define PM_SMALL_WIDTHS 4      // tile widths of the few-row linear kernel: 64, 128, 192, 256
 #define PM_SLAB 16             // LoRA ranks are handled in slabs of 16 (one UMMA K step)
 
@@ -37,9 +38,8 @@ struct LinearDev {
     // tensor maps of the static operands (bf16 build only)
     CUtensorMap tm_w, tm_at, tm_bt;
     bool has_tm = false;
-    // n_out a multiple of 256: boxes of 128 output columns for the CTA-pair GEMM
-    CUtensorMap tm_w_half, tm_bt_half;
-    bool has_tm_half = false;
+    // the CTA-pair GEMM's, by index of its tile width: boxes of half a tile's output columns
+    CUtensorMap tm_pw[PM_PAIR_WIDTHS], tm_pbt[PM_PAIR_WIDTHS];
     // the few-row kernel's (small_linear.cu), by index of its tile width
     CUtensorMap tm_sw[PM_SMALL_WIDTHS], tm_sbt[PM_SMALL_WIDTHS];
     CUtensorMap tm_sat[2];             // one adapter slab, one / two K blocks per copy (few-row kernel and shrink)
@@ -161,8 +161,8 @@ bool act_encode(ActMaps* m, const void* x, int k_in, uint64_t rows);
 cudaError_t launch_shrink(const Launch& L, const LinearDev& lin, const RouteDev& R, const ActMaps& x, int rows,
                           bf16* tbuf, int n_sms, float2* stats_out, float ln_eps);
 cudaError_t launch_row_stats(const Launch& L, const bf16* x, float2* stats, int rows, int d, float eps);
-// after_shrink: the kernel enqueued just before on the stream is this linear's launch_shrink; the GEMM
-// may then start before it has finished (programmatic dependent launch) and awaits its results itself.
+// The GEMM may start before the kernel ahead of it on the stream has finished (programmatic dependent launch) and
+// awaits its results itself.  after_shrink: that kernel is this linear's launch_shrink, so x is complete already.
 // tm_y: [rows, n_out] output map with a (32 x 32) box and 64B swizzle for the TMA-store epilogue, or
 // null to store straight from registers (always the case for EPI_PATCH, whose rows are remapped)
 cudaError_t launch_lora_gemm(const Launch& L, const LinearDev& lin, const RouteDev* R,
@@ -170,6 +170,7 @@ cudaError_t launch_lora_gemm(const Launch& L, const LinearDev& lin, const RouteD
                              int rows, int epi, const bf16* residual, const PatchEpi& pe, bf16* y,
                              int n_sms, const float2* ln_stats, bool after_shrink = false);
 // ---- one kernel per linear for few rows (small_linear.cu)
+bool gemm_encode_pair_maps(LinearDev& lin, int max_adapters, int slabs_max);      // gemm_tcgen05.cu
 bool small_linear_encode(LinearDev& lin, int max_adapters, int slabs_max);
 // whether launch_small_linear serves this call (R: null = no adapters)
 bool small_linear_fits(const LinearDev& lin, const RouteDev* R, int rows, int epi, int n_sms);

@@ -13,8 +13,9 @@
 // warps per TMEM lane quarter, each taking half of the tile's columns).
 // Every mbarrier wait is bounded: on expiry the CTA raises an abort flag, records
 // PM_ERR_TIMEOUT in the status word, drains and returns.
-// When n_out is a multiple of 256 the CTA-pair variant (lora_gemm_pair_kernel, cta_group::2, 256 x 256
-// tiles) is used; the single-CTA kernel serves the narrower shapes.
+// The CTA-pair variant (lora_gemm_pair_kernel, cta_group::2, 256 x 256 or 256 x 192 tiles) serves most shapes, the single-CTA
+// kernel short K and other widths (pick_pair_width).  Both start while the kernel before them on the stream still runs
+// (programmatic dependent launch): 768 -> 768 with shrink on 197 x 256 rows 83.1 -> 79.5 us, on 197 x 37 rows 20.8 -> 19.6 us.
 #include "common.cuh"
 #include "f32x2.cuh"
 #include "tcgen05_ptx.cuh"
@@ -39,8 +40,7 @@ struct GemmArgs {
     const int* tile_slab;
     int slab_cap;
     int tma_store;             // 1: the epilogue stores through shared memory + TMA (tm_y valid)
-    int overlap_prev;          // host side only: launch with programmatic serialization (the kernel before it on
-                               // the stream is this linear's shrink, whose results are awaited with dep_wait())
+    int wait_x;                // 0: the kernel before on the stream is this linear's shrink, x is complete; 1: await it first
     int* status;
     // LayerNorm folded into the linear (LNF kernels): y = rstd (acc - mean g) + bias, per row / column
     const float* ln_g;
@@ -49,6 +49,7 @@ struct GemmArgs {
 
 constexpr int STAGING_BYTES_PER_WARP = 2 * 32 * 64;     // two [32 rows x 32 bf16] buffers
 constexpr int PLAN_BYTES = 2048;
+constexpr int P_ACC_COLS = 256;                        // pair kernel: tensor-memory columns of one of the two accumulators
 
 // EW = number of epilogue warps (4 or 8); the CTA has 2 + EW warps.
 template <int BN, int EW>
@@ -123,7 +124,7 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs& args, const CUtens
         orow = (size_t)(row / args.pe.g2) * args.pe.tokens + 1 + p;
         pos_row = args.pe.pos + (size_t)(1 + p) * args.n_out;
     }
-    const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN);
+    const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * (PAIR ? P_ACC_COLS : BN));
     float2 st = make_float2(0.f, 1.f);                 // (mean, rstd) of this thread's row
     if (LNF && row_ok) st = args.ln_stats[row];
 #pragma unroll
@@ -294,6 +295,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    dep_release();
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
@@ -302,6 +304,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
             uint32_t phase = 0;
             bool ok = true, dep_done = false;
             int it = 0;
+            if (args.wait_x) { dep_wait(); dep_done = true; }
             for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++it) {
                 const int m = tile / args.n_tiles, n = tile % args.n_tiles;
                 for (int kb = 0; kb < num_kb && ok; ++kb) {
@@ -391,7 +394,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
         const int quarter = warp & 3;                 // TMEM lanes 32*quarter .. +31
         const int half = (warp - 2) >> 2;             // which share of the tile's 32-column chunks
         const uint32_t staging = base + S::STAGING_OFFSET + (uint32_t)(warp - 2) * STAGING_BYTES_PER_WARP;
-        dep_wait();                                   // the row statistics come from the shrink kernel
+        dep_wait();                                   // row statistics, residual; rows that the kernel before still reads
         int acc = 0;
         uint32_t acc_phase = 0;
         uint32_t chunk_no = 0;                        // running chunk counter: picks the staging buffer
@@ -423,8 +426,8 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
 }
 
 // ---------------------------------------------------------------------------------------
-// The same GEMM on CTA pairs (n_out a multiple of 256).  Two CTAs of a cluster share one
-// 256 x 256 output tile: each stages its own 128 rows of x (and of the t slabs) and HALF of the
+// The same GEMM on CTA pairs (BN = 192 or 256).  Two CTAs of a cluster share one
+// 256 x BN output tile: each stages its own 128 rows of x (and of the t slabs) and HALF of the
 // W^T tile (and of the B slabs), so every byte of W^T crosses the L2 -> SM fabric once per 256
 // rows instead of once per 128, and one tcgen05.mma.cta_group::2 (M = 256) issued by the even
 // CTA drives the tensor cores of both SMs, each accumulating its own 128 rows in its own TMEM.
@@ -432,41 +435,44 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
 //   empty[s]   (both CTAs)  the pair MMAs that read stage s are done (multicast commit)
 //   tfull[a]   (both CTAs)  accumulator a is complete (multicast commit)
 //   tempty[a]  (even CTA)   both CTAs' epilogue warps have drained accumulator a
-// Six 32 KB stages per CTA.  No TMA multicast is used.
+// Up to six stages per CTA.  No TMA multicast is used.
 // ---------------------------------------------------------------------------------------
-constexpr int P_BN = 256;
 constexpr int P_EW = 8;
-// Ring depth and residual landing area by epilogue: the residual epilogue trades two of the six 32 KB
-// stages for a 64 KB area into which TMA fetches the tile's residual rows ahead of the accumulator.
-template <int EPI, bool RESS>
-struct PairCfg {
-    static constexpr bool RES = EPI == EPI_RESIDUAL && RESS;
-    static constexpr int STAGES = RES ? 4 : 6;
-    static constexpr int RES_BYTES_PER_WARP = RES ? 4 * 32 * 64 : 0;       // four [32 rows x 32 bf16] chunks
-};
+constexpr int P_THREADS = 64 + 32 * P_EW;
 constexpr int P_A_BYTES = BM * BK * 2;                 // 16 KB: this CTA's 128 rows of x
-constexpr int P_B_BYTES = (P_BN / 2) * BK * 2;         // 16 KB: this CTA's half of the W^T tile
-constexpr int P_STAGE_BYTES = P_A_BYTES + P_B_BYTES;
 constexpr int P_T_SLAB_BYTES = BM * PM_SLAB * 2;       // 4 KB
-constexpr int P_B_SLAB_BYTES = (P_BN / 2) * PM_SLAB * 2;   // 4 KB
 constexpr int P_MAX_STAGES = 6;
-constexpr int P_STAGING_OFFSET = P_MAX_STAGES * P_STAGE_BYTES;      // stages, then (residual kernels) the
-constexpr int P_PLAN_OFFSET = P_STAGING_OFFSET + P_EW * STAGING_BYTES_PER_WARP;   // residual area inside them
+constexpr int P_RING_BYTES = 192 * 1024;               // stages, then (residual kernels) the residual landing area
+constexpr int P_STAGING_OFFSET = P_RING_BYTES;
+constexpr int P_PLAN_OFFSET = P_STAGING_OFFSET + P_EW * STAGING_BYTES_PER_WARP;
 constexpr int P_BAR_OFFSET = P_PLAN_OFFSET + PLAN_BYTES;
 constexpr int P_SMEM_TOTAL = P_BAR_OFFSET + 256;
-constexpr int P_THREADS = 64 + 32 * P_EW;
+// By tile width and epilogue: a residual epilogue that takes the residual rows through shared memory (RESS) gives part
+// of the ring to an area into which TMA fetches the tile's rows ahead of the accumulator.
+template <int BN, int EPI, bool RESS>
+struct PairCfg {
+    static constexpr bool RES = EPI == EPI_RESIDUAL && RESS;
+    static constexpr int B_BYTES = (BN / 2) * BK * 2;                      // this CTA's half of the W^T tile
+    static constexpr int STAGE_BYTES = P_A_BYTES + B_BYTES;
+    static constexpr int B_SLAB_BYTES = (BN / 2) * PM_SLAB * 2;
+    static constexpr int RES_BYTES_PER_WARP = RES ? (BN / 64) * 32 * 64 : 0;       // [32 rows x 32 bf16] chunks
+    static constexpr int FIT = (P_RING_BYTES - P_EW * RES_BYTES_PER_WARP) / STAGE_BYTES;
+    static constexpr int STAGES = FIT < P_MAX_STAGES ? FIT : P_MAX_STAGES;
+    static constexpr int RES_OFFSET = STAGES * STAGE_BYTES;
+    static_assert(SLABS_PER_STAGE * B_SLAB_BYTES <= B_BYTES, "LoRA stage");
+};
 
 // RESS (residual epilogue only): residual through shared memory with a four-stage ring (short K, where
 // the epilogue is exposed) instead of per-thread loads with the full six stages (long K).
-template <int EPI, bool LNF, bool RESS>
+template <int BN, int EPI, bool LNF, bool RESS>
 __global__ void __launch_bounds__(P_THREADS, 1)
 lora_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                       const __grid_constant__ CUtensorMap tm_t, const __grid_constant__ CUtensorMap tm_bt,
                       const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_res,
                       const GemmArgs args) {
-    constexpr int BN = P_BN;
+    using C = PairCfg<BN, EPI, RESS>;
     constexpr int HALVES = P_EW / 4;
-    constexpr int P_STAGES = PairCfg<EPI, RESS>::STAGES;
+    constexpr int P_STAGES = C::STAGES;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = smem_u32(smem_raw);
     const uint32_t rank = cluster_ctarank();          // 0: issues the MMAs, 1: its peer
@@ -530,6 +536,7 @@ lora_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     // both CTAs must hold the same TMEM columns (the pair MMA uses one address for both); tell the peer
     if (threadIdx.x == 0) st_cluster_u32(mapa_cluster(smem_u32((const void*)peer_slot), rank ^ 1u), tmem_base);
     cluster_sync_all();          // barriers initialised and TMEM bases exchanged in both CTAs
+    dep_release();
     const bool usable = ((base & 1023u) == 0) && (*peer_slot == tmem_base);
     if (!usable && threadIdx.x == 0) atomicCAS(args.status, 0, (int)PM_ERR_CUDA);
 
@@ -542,15 +549,31 @@ lora_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             uint32_t phase = 0;
             bool ok = true, dep_done = false;
             int it = 0;
+            // x comes from the kernel before (unless that one is this linear's shrink, which releases this kernel
+            // only when x is complete): until it has finished, the first stages' weights are fetched alone
+            int pre = 0;
+            if (args.wait_x) {
+                pre = min(P_STAGES, num_kb);
+                const int m = 2 * (pair_id / args.n_tiles) + (int)rank, n = pair_id % args.n_tiles;
+                for (int kb = 0; kb < pre; ++kb) {
+                    if (rank == 0) mbar_expect_tx(full_bar(kb), 2 * C::STAGE_BYTES);
+                    tma_load_2d_pair(base + kb * C::STAGE_BYTES + P_A_BYTES, &tm_w, kb * BK, n * BN + (int)rank * (BN / 2), mapa_cluster(full_bar(kb), 0));
+                }
+                dep_wait();
+                dep_done = true;
+                for (int kb = 0; kb < pre; ++kb)
+                    tma_load_2d_pair(base + kb * C::STAGE_BYTES, &tm_x, kb * BK, m * BM, mapa_cluster(full_bar(kb), 0));
+                if (pre == P_STAGES) phase = 1u; else stage = pre;
+            }
             for (int tile = pair_id; tile < total_tiles && ok; tile += n_pairs, ++it) {
                 const int m2 = tile / args.n_tiles, n = tile % args.n_tiles;
                 const int m = 2 * m2 + (int)rank;                   // this CTA's 128-row tile
-                for (int kb = 0; kb < num_kb && ok; ++kb) {
+                for (int kb = it == 0 ? pre : 0; kb < num_kb && ok; ++kb) {
                     ok = mbar_wait_cluster(empty_bar(stage), phase ^ 1u, abort_flag, args.status);
                     if (!ok) break;
                     const uint32_t fb = mapa_cluster(full_bar(stage), 0);
-                    if (rank == 0) mbar_expect_tx(full_bar(stage), 2 * P_STAGE_BYTES);
-                    const uint32_t sa = base + stage * P_STAGE_BYTES;
+                    if (rank == 0) mbar_expect_tx(full_bar(stage), 2 * C::STAGE_BYTES);
+                    const uint32_t sa = base + stage * C::STAGE_BYTES;
                     tma_load_2d_pair(sa, &tm_x, kb * BK, m * BM, fb);
                     tma_load_2d_pair(sa + P_A_BYTES, &tm_w, kb * BK, n * BN + (int)rank * (BN / 2), fb);
                     if (++stage == P_STAGES) { stage = 0; phase ^= 1u; }
@@ -562,13 +585,13 @@ lora_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                     ok = mbar_wait_cluster(empty_bar(stage), phase ^ 1u, abort_flag, args.status);
                     if (!ok) break;
                     const uint32_t fb = mapa_cluster(full_bar(stage), 0);
-                    if (rank == 0) mbar_expect_tx(full_bar(stage), 2 * cnt * (P_T_SLAB_BYTES + P_B_SLAB_BYTES));
-                    const uint32_t sa = base + stage * P_STAGE_BYTES;
+                    if (rank == 0) mbar_expect_tx(full_bar(stage), 2 * cnt * (P_T_SLAB_BYTES + C::B_SLAB_BYTES));
+                    const uint32_t sa = base + stage * C::STAGE_BYTES;
                     for (int i = 0; i < cnt; ++i) {
                         const int slot = m * args.slab_cap + g0 + i;
                         const int slab = tile_slab_id(it, m, g0 + i);
                         tma_load_2d_pair(sa + i * P_T_SLAB_BYTES, &tm_t, 0, slot * BM, fb);
-                        tma_load_2d_pair(sa + P_A_BYTES + i * P_B_SLAB_BYTES, &tm_bt, 0,
+                        tma_load_2d_pair(sa + P_A_BYTES + i * C::B_SLAB_BYTES, &tm_bt, 0,
                                          slab * args.n_out + n * BN + (int)rank * (BN / 2), fb);
                     }
                     if (++stage == P_STAGES) { stage = 0; phase ^= 1u; }
@@ -592,13 +615,13 @@ lora_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                 ok = mbar_wait_cluster(tempty_bar(acc), acc_phase ^ 1u, abort_flag, args.status);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
+                const uint32_t d_tmem = tmem_base + (uint32_t)(acc * P_ACC_COLS);
                 uint32_t accumulate = 0;
                 for (int kb = 0; kb < num_kb && ok; ++kb) {
                     ok = mbar_wait_cluster(full_bar(stage), phase, abort_flag, args.status);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint64_t so = (uint64_t)(stage * (P_STAGE_BYTES >> 4));
+                    const uint64_t so = (uint64_t)(stage * (C::STAGE_BYTES >> 4));
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k) {
                         umma_bf16_pair(d_tmem, da0 + so + 2 * k, db0 + so + 2 * k, idesc, accumulate);
@@ -612,11 +635,11 @@ lora_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                     ok = mbar_wait_cluster(full_bar(stage), phase, abort_flag, args.status);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t sa = base + stage * P_STAGE_BYTES;
+                    const uint32_t sa = base + stage * C::STAGE_BYTES;
                     const uint32_t sb = sa + P_A_BYTES;
                     for (int i = 0; i < cnt; ++i) {
                         umma_bf16_pair(d_tmem, smem_desc(sa + i * P_T_SLAB_BYTES, 32),
-                                       smem_desc(sb + i * P_B_SLAB_BYTES, 32), idesc, accumulate);
+                                       smem_desc(sb + i * C::B_SLAB_BYTES, 32), idesc, accumulate);
                         accumulate = 1;
                     }
                     umma_commit_pair(empty_bar(stage));
@@ -631,17 +654,17 @@ lora_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         const int quarter = warp & 3;
         const int half = (warp - 2) >> 2;
         const uint32_t staging = base + P_STAGING_OFFSET + (uint32_t)(warp - 2) * STAGING_BYTES_PER_WARP;
-        dep_wait();                                   // the row statistics come from the shrink kernel
+        dep_wait();                                   // row statistics, residual; rows that the kernel before still reads
         int acc = 0;
         uint32_t acc_phase = 0, res_phase = 0;
         uint32_t chunk_no = 0;
         bool ok = true;
         for (int tile = pair_id; tile < total_tiles && ok; tile += n_pairs) {
             const int m = 2 * (tile / args.n_tiles) + (int)rank, n = tile % args.n_tiles;
-            ok = epilogue_tile<BN, EPI, HALVES, true, LNF, PairCfg<EPI, RESS>::RES>(
+            ok = epilogue_tile<BN, EPI, HALVES, true, LNF, C::RES>(
                 args, tm_y, staging, chunk_no, tmem_base, acc, acc_phase, tfull_bar(acc),
                 mapa_cluster(tempty_bar(acc), 0), abort_flag, m, n, quarter, half, lane, &tm_res,
-                base + PairCfg<EPI, RESS>::STAGES * P_STAGE_BYTES + (uint32_t)(warp - 2) * PairCfg<EPI, RESS>::RES_BYTES_PER_WARP,
+                base + C::RES_OFFSET + (uint32_t)(warp - 2) * C::RES_BYTES_PER_WARP,
                 res_bar(warp - 2), res_phase);
             res_phase ^= 1u;
             if (!ok) break;
@@ -812,21 +835,11 @@ static cudaError_t launch_gemm_bn(const Launch& L, const CUtensorMap& tm_x, cons
     static SmemGrant grant;
     if (cudaError_t e = grant.ensure(lora_gemm_kernel<BN, EPI, EW, LNF>, Smem<BN, EW>::TOTAL); e != cudaSuccess) return e;
     const int total = a.m_tiles * a.n_tiles;
-    const int grid = total < n_sms ? total : n_sms;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(64 + 32 * EW);
-    cfg.dynamicSmemBytes = Smem<BN, EW>::TOTAL;
-    cfg.stream = L.st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = a.overlap_prev ? 1 : 0;
     ProfScope ps(L, KC_GEMM);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, lora_gemm_kernel<BN, EPI, EW, LNF>, tm_x, tm_w, tm_t, tm_bt, tm_y, a);
+    cudaError_t e = launch_overlapped(lora_gemm_kernel<BN, EPI, EW, LNF>, total < n_sms ? total : n_sms, 64 + 32 * EW, Smem<BN, EW>::TOTAL,
+                                      L.st, 1, tm_x, tm_w, tm_t, tm_bt, tm_y, a);
     BUMP(L);
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return e;
 }
 
 template <int BN>
@@ -846,7 +859,7 @@ static cudaError_t launch_gemm_epi(const Launch& L, const CUtensorMap& tm_x, con
     }
 }
 
-template <int EPI, bool LNF = false, bool RESS = false>
+template <int BN, int EPI, bool LNF = false, bool RESS = false>
 static cudaError_t launch_gemm_pair(const Launch& L, const CUtensorMap& tm_x, const CUtensorMap& tm_w,
                                     const CUtensorMap& tm_t, const CUtensorMap& tm_bt, const CUtensorMap& tm_y,
                                     const GemmArgs& a, int n_sms) {
@@ -857,47 +870,63 @@ static cudaError_t launch_gemm_pair(const Launch& L, const CUtensorMap& tm_x, co
             return cudaErrorInvalidValue;
     }
     static SmemGrant grant;
-    if (cudaError_t e = grant.ensure(lora_gemm_pair_kernel<EPI, LNF, RESS>, P_SMEM_TOTAL); e != cudaSuccess) return e;
+    if (cudaError_t e = grant.ensure(lora_gemm_pair_kernel<BN, EPI, LNF, RESS>, P_SMEM_TOTAL); e != cudaSuccess) return e;
     const int total = a.m_tiles * a.n_tiles;
     const int pairs = total < n_sms / 2 ? total : n_sms / 2;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * pairs);
-    cfg.blockDim = dim3(P_THREADS);
-    cfg.dynamicSmemBytes = P_SMEM_TOTAL;
-    cfg.stream = L.st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = a.overlap_prev ? 2 : 1;
     ProfScope ps(L, KC_GEMM);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, lora_gemm_pair_kernel<EPI, LNF, RESS>, tm_x, tm_w, tm_t, tm_bt, tm_y, tm_res, a);
+    cudaError_t e = launch_overlapped(lora_gemm_pair_kernel<BN, EPI, LNF, RESS>, 2 * pairs, P_THREADS, P_SMEM_TOTAL, L.st, 2,
+                                      tm_x, tm_w, tm_t, tm_bt, tm_y, tm_res, a);
     BUMP(L);
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return e;
 }
 
+template <int BN>
 static cudaError_t launch_gemm_pair_epi(const Launch& L, const CUtensorMap& tm_x, const CUtensorMap& tm_w,
                                         const CUtensorMap& tm_t, const CUtensorMap& tm_bt, const CUtensorMap& tm_y,
                                         const GemmArgs& a, int n_sms) {
     if (a.ln_stats) {
-        if (a.epi == EPI_GELU) return launch_gemm_pair<EPI_GELU, true>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
-        if (a.epi == EPI_NONE) return launch_gemm_pair<EPI_NONE, true>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
+        if (a.epi == EPI_GELU) return launch_gemm_pair<BN, EPI_GELU, true>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
+        if (a.epi == EPI_NONE) return launch_gemm_pair<BN, EPI_NONE, true>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
         return cudaErrorInvalidValue;
     }
     switch (a.epi) {
-        case EPI_GELU: return launch_gemm_pair<EPI_GELU>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
+        case EPI_GELU: return launch_gemm_pair<BN, EPI_GELU>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
         case EPI_RESIDUAL:
-            if (a.k_in <= 1024) return launch_gemm_pair<EPI_RESIDUAL, false, true>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
-            return launch_gemm_pair<EPI_RESIDUAL>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
-        case EPI_PATCH: return launch_gemm_pair<EPI_PATCH>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
-        default: return launch_gemm_pair<EPI_NONE>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
+            if (a.k_in <= 1024) return launch_gemm_pair<BN, EPI_RESIDUAL, false, true>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
+            return launch_gemm_pair<BN, EPI_RESIDUAL>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
+        case EPI_PATCH: return launch_gemm_pair<BN, EPI_PATCH>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
+        default: return launch_gemm_pair<BN, EPI_NONE>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
     }
 }
 
-// lin.tm_w / lin.tm_bt are encoded for the BN chosen by gemm_tile_n(lin.n_out); lin.tm_w_half /
-// lin.tm_bt_half (n_out a multiple of 256) fetch 128 of a tile's 256 columns for the pair kernel.
+constexpr int PAIR_WIDTHS[PM_PAIR_WIDTHS] = {192, 256};
+
+bool gemm_encode_pair_maps(LinearDev& lin, int max_adapters, int slabs_max) {
+    for (int i = 0; i < PM_PAIR_WIDTHS; ++i) {
+        const int half = PAIR_WIDTHS[i] / 2;
+        if (!tm_encode_2d(&lin.tm_pw[i], lin.Wt, lin.k_in, lin.n_out, (uint64_t)lin.k_in * 2, BK, half, 128)) return false;
+        if (lin.lora.At && !tm_encode_2d(&lin.tm_pbt[i], lin.lora.Bt, PM_SLAB, (uint64_t)max_adapters * slabs_max * lin.n_out,
+                                         PM_SLAB * 2, PM_SLAB, half, 32)) return false;
+    }
+    return true;
+}
+
+// The tile width of the pair kernel (index into PAIR_WIDTHS), or -1 for the single-CTA kernel.  Measured on 64 and 256
+// frames of 197 tokens, rank-16 adapters, us per linear (pair against single-CTA):
+//   K = 768 and more, 256-wide: 768 -> 768 23.8 / 26.5 and 80.0 / 90.7, 768 -> 3072 58.4 / 62.5 and 223 / 251;
+//   K up to 384, 256-wide: 384 -> 1536 28.0 / 24.1 and 86.8 / 85.6, 192 -> 768 18.3 / 15.9 and 44.8 / 36.8 -- a tile's K loop
+//   is too short to hide what the two CTAs of a pair wait for each other;
+//   192-wide (multiples of 192, not of 256): 384 -> 1152 21.6 / 23.7 and 69.7 / 83.2, 1536 -> 384 28.8 / 29.3 and 93.6 / 110,
+//   384 -> 384 15.2 / 15.0 and 40.2 / 46.1, but without adapters 10.3 / 10.2 and 31.4 / 28.5.
+// For multiples of both, 192-wide tiles lose: 768 -> 3072 64.1 and 246.
+static int pick_pair_width(int n_out, int k_in, bool lora) {
+    if (n_out % 256 == 0) return k_in <= 384 ? -1 : 1;
+    if (n_out % 192 == 0) return n_out <= 384 && k_in <= 384 && !lora ? -1 : 0;
+    return -1;
+}
+
+// lin.tm_w / lin.tm_bt are encoded for the BN chosen by gemm_tile_n(lin.n_out) (single-CTA kernel); lin.tm_pw /
+// lin.tm_pbt fetch half of a tile's columns for the pair kernel.
 int gemm_tile_n(int n_out) { return (n_out % 256 == 0) ? 256 : 128; }
 
 cudaError_t launch_lora_gemm(const Launch& L, const LinearDev& lin, const RouteDev* R,
@@ -917,15 +946,18 @@ cudaError_t launch_lora_gemm(const Launch& L, const LinearDev& lin, const RouteD
     a.tile_slab = lora ? R->tile_slab : nullptr;
     a.slab_cap = lora ? R->slab_cap : 0;
     a.status = L.status;
-    a.overlap_prev = (after_shrink && lora) ? 1 : 0;
+    a.wait_x = (after_shrink && lora) ? 0 : 1;
     a.ln_g = lin.ln_g; a.ln_stats = ln_stats;
     a.tma_store = (tm_y != nullptr && epi != EPI_PATCH) ? 1 : 0;
     const CUtensorMap& tt = lora ? *tm_t : tm_x;      // placeholders are never dereferenced
     const CUtensorMap& ty = a.tma_store ? *tm_y : tm_x;
-    if (lin.has_tm_half && n_sms >= 2 && (epi != EPI_RESIDUAL || a.tma_store)) {
+    const int pw = n_sms >= 2 && (epi != EPI_RESIDUAL || a.tma_store) ? pick_pair_width(lin.n_out, lin.k_in, lora) : -1;
+    if (pw >= 0) {
         a.m_tiles = (rows + 2 * BM - 1) / (2 * BM);       // 256-row tiles
-        a.n_tiles = lin.n_out / P_BN;
-        return launch_gemm_pair_epi(L, tm_x, lin.tm_w_half, tt, lora ? lin.tm_bt_half : lin.tm_w_half, ty, a, n_sms);
+        a.n_tiles = lin.n_out / PAIR_WIDTHS[pw];
+        const CUtensorMap& tpb = lora ? lin.tm_pbt[pw] : lin.tm_pw[pw];
+        return PAIR_WIDTHS[pw] == 192 ? launch_gemm_pair_epi<192>(L, tm_x, lin.tm_pw[pw], tt, tpb, ty, a, n_sms)
+                                      : launch_gemm_pair_epi<256>(L, tm_x, lin.tm_pw[pw], tt, tpb, ty, a, n_sms);
     }
     const CUtensorMap& tb = lora ? lin.tm_bt : lin.tm_w;
     if (bn == 256) return launch_gemm_epi<256>(L, tm_x, lin.tm_w, tt, tb, ty, a, n_sms);
