@@ -660,9 +660,8 @@ int forward_t(pm_handle_s* h, const void* frames, int n_frames, int n_slots, int
         }
     };
 
-    CK(launch_im2col<T>(L, (const T*)frames, R.perm, P, n_frames, c.img, c.patch));
+    CK(launch_im2col<T>(L, (const T*)frames, R.perm, P, n_frames, c.img, c.patch, h->cls.as<float>(), h->pos.as<float>(), X, d));
     CK(linear(h->patch, P, &h->tm_patch, n_frames * h->g2, h->g2, false, EPI_PATCH, nullptr, pe, X));
-    CK(launch_cls_rows<T>(L, h->cls.as<float>(), h->pos.as<float>(), X, n_frames, T_, d));
     int n_cur = n_frames;                     // slots the blocks currently run on
     for (int l = 0; l <= c.layers; ++l) {
         if (l == trunk_layers && n_slots != n_cur) {

@@ -138,12 +138,10 @@ bool attention_encode_maps(const bf16* qkv, int n_frames, int tokens, int heads,
 // n_sms > 0 selects the pipelined persistent kernel where it applies (one key block); 0 = never
 cudaError_t launch_attention_tc(const Launch& L, const CUtensorMap& tm_q, const CUtensorMap& tm_kv,
                                 bf16* out, int n_frames, int tokens, int heads, int n_sms);
+// patch gather, and the CLS rows of x
 template <typename T>
 cudaError_t launch_im2col(const Launch& L, const T* frames, const int* perm, T* out, int n_frames,
-                          int img, int patch);
-template <typename T>
-cudaError_t launch_cls_rows(const Launch& L, const float* cls, const float* pos, T* x, int n_frames,
-                            int tokens, int d);
+                          int img, int patch, const float* cls, const float* pos, T* x, int d);
 // fp32 debug / reference-quality linear: t32 = scaled shrink per (row, set position, rank)
 template <typename T>
 cudaError_t launch_naive_linear(const Launch& L, const LinearDev& lin, const RouteDev& R,

@@ -5,6 +5,7 @@
 #include <atomic>
 
 #include "common.cuh"
+#include "tcgen05_ptx.cuh"
 
 #define BUMP(L) do { if ((L).launches) ++*(L).launches; } while (0)
 
@@ -189,19 +190,22 @@ template cudaError_t launch_layernorm<bf16>(const Launch&, const bf16*, const fl
 // ---------------------------------------------------------------------------------------
 // patch gather (im2col) and CLS rows
 // ---------------------------------------------------------------------------------------
-// out[slot*g*g + (gy*g+gx)][c*P*P + py*P + px] = frames[perm[slot]][c][gy*P+py][gx*P+px]
+// out[slot*g*g + (gy*g+gx)][c*P*P + py*P + px] = frames[perm[slot]][c][gy*P+py][gx*P+px], and the CLS row of every
+// slot (cls + pos[0]) to x: one launch for all the projection does not write.
 template <typename T>
 __global__ void __launch_bounds__(256) im2col_kernel(const T* __restrict__ frames,
                                                      const int* __restrict__ perm,
                                                      T* __restrict__ out, int n_frames, int img,
-                                                     int patch) {
+                                                     int patch, const float* __restrict__ cls,
+                                                     const float* __restrict__ pos, T* __restrict__ x, int d) {
+    dep_release();                                  // the projection's weights need not wait for these rows
     constexpr int VEC = Vec16<T>::N;
     const int g = img / patch;
     const int pd = 3 * patch * patch;
     const int chunks_per_row = pd / VEC;
     const size_t total = (size_t)n_frames * g * g * chunks_per_row;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (size_t)gridDim.x * blockDim.x) {
+    const size_t first = (size_t)blockIdx.x * blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+    for (size_t i = first; i < total; i += step) {
         const int ch = (int)(i % chunks_per_row);
         const size_t r = i / chunks_per_row;
         const int p = (int)(r % (g * g));
@@ -215,42 +219,27 @@ __global__ void __launch_bounds__(256) im2col_kernel(const T* __restrict__ frame
                        gx * patch + px;
         *reinterpret_cast<uint4*>(out + r * pd + col) = *reinterpret_cast<const uint4*>(src);
     }
+    const size_t slot_elems = (size_t)(g * g + 1) * d;
+    for (size_t i = first; i < (size_t)n_frames * d; i += step) {
+        const int c = (int)(i % d);
+        x[i / d * slot_elems + c] = from_f<T>(cls[c] + pos[c]);
+    }
 }
 
 template <typename T>
 cudaError_t launch_im2col(const Launch& L, const T* frames, const int* perm, T* out, int n_frames,
-                          int img, int patch) {
+                          int img, int patch, const float* cls, const float* pos, T* x, int d) {
     const int g = img / patch;
     const size_t total = (size_t)n_frames * g * g * (3 * patch * patch / Vec16<T>::N);
     const int blocks = (int)((total + 255) / 256 < 148 * 16 ? (total + 255) / 256 : 148 * 16);
     if (blocks == 0) return cudaSuccess;
     ProfScope ps(L, KC_OTHER);
-    im2col_kernel<T><<<blocks, 256, 0, L.st>>>(frames, perm, out, n_frames, img, patch);
+    im2col_kernel<T><<<blocks, 256, 0, L.st>>>(frames, perm, out, n_frames, img, patch, cls, pos, x, d);
     BUMP(L);
     return cudaGetLastError();
 }
-template cudaError_t launch_im2col<float>(const Launch&, const float*, const int*, float*, int, int, int);
-template cudaError_t launch_im2col<bf16>(const Launch&, const bf16*, const int*, bf16*, int, int, int);
-
-template <typename T>
-__global__ void cls_rows_kernel(const float* __restrict__ cls, const float* __restrict__ pos,
-                                T* __restrict__ x, int n_frames, int tokens, int d) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_frames * d) return;
-    const int f = i / d, c = i % d;
-    x[(size_t)f * tokens * d + c] = from_f<T>(cls[c] + pos[c]);
-}
-
-template <typename T>
-cudaError_t launch_cls_rows(const Launch& L, const float* cls, const float* pos, T* x, int n_frames,
-                            int tokens, int d) {
-    ProfScope ps(L, KC_OTHER);
-    cls_rows_kernel<T><<<(n_frames * d + 255) / 256, 256, 0, L.st>>>(cls, pos, x, n_frames, tokens, d);
-    BUMP(L);
-    return cudaGetLastError();
-}
-template cudaError_t launch_cls_rows<float>(const Launch&, const float*, const float*, float*, int, int, int);
-template cudaError_t launch_cls_rows<bf16>(const Launch&, const float*, const float*, bf16*, int, int, int);
+template cudaError_t launch_im2col<float>(const Launch&, const float*, const int*, float*, int, int, int, const float*, const float*, float*, int);
+template cudaError_t launch_im2col<bf16>(const Launch&, const bf16*, const int*, bf16*, int, int, int, const float*, const float*, bf16*, int);
 
 // ---------------------------------------------------------------------------------------
 // fp32 debug build: linear with unmerged LoRA terms on CUDA cores
@@ -469,12 +458,223 @@ __device__ __forceinline__ float dot_row(const float* __restrict__ z, const T* _
 
 __device__ __forceinline__ float sigmoidf_acc(float v) { return 1.f / (1.f + expf(-v)); }
 
+// The heads of the bf16 build, one launch: blocks [0, base_blocks) make 16 slots x 16 NT classes of the base head, the
+// others the adapter heads of one slot each.  Every block normalises the CLS rows it needs itself (a row is d values;
+// a kernel of its own for that was a launch in the chain), and all weights are requested before the kernel waits for
+// the last block's output (programmatic dependent launch).
+//   Base head: a [slots x d] x [d x classes] product on mma.sync; the fp32 features enter as three bf16 parts each,
+// whose sum is the fp32 value, so nothing is rounded (weights are bf16 as stored).  Two groups of four warps share
+// the classes, the warps of a group share d; a thread takes 8 consecutive values of every 32 (16-byte loads), which
+// permutes the summation index the same way on both sides.
+//   Adapter heads: a warp normalises the slot's row into registers and walks the class rows of the active adapters,
+// four at a time.  Scores are positive, so the maximum over adapters is an integer atomicMax on the float bit pattern
+// of a zeroed row (order-free, hence deterministic).
+// 256 slots, 800 classes, d = 768: 73 us in three launches and a clearing before, 21.6 us now; one slot: 33 and 9.5 us.
+constexpr int HB_SLOTS = 16;
+
+// z = LayerNorm(row) of one row by one warp; v[i * 8 + j] = element (lane + 32 i) * 8 + j
+__device__ __forceinline__ void ln_regs(const bf16* __restrict__ xr, const float* __restrict__ g, const float* __restrict__ b,
+                                        int d, float eps, int lane, float (&v)[32]) {
+    const int nch = d >> 3;
+    float sum = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (lane + 32 * i < nch) load16<bf16>(xr + (lane + 32 * i) * 8, v + i * 8);
+        else
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[i * 8 + j] = 0.f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) sum += v[i * 8 + j];
+    }
+    const float mean = warp_sum(sum) / (float)d;
+    float sq = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (lane + 32 * i < nch)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) { const float t = v[i * 8 + j] - mean; sq += t * t; }
+    const float rstd = rsqrtf(warp_sum(sq) / (float)d + eps);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int c = (lane + 32 * i) * 8;
+        if (lane + 32 * i < nch)
+#pragma unroll
+            for (int j = 0; j < 8; j += 4) {
+                const float4 gg = __ldg(reinterpret_cast<const float4*>(g + c + j)), bb = __ldg(reinterpret_cast<const float4*>(b + c + j));
+                v[i * 8 + j + 0] = (v[i * 8 + j + 0] - mean) * rstd * gg.x + bb.x;
+                v[i * 8 + j + 1] = (v[i * 8 + j + 1] - mean) * rstd * gg.y + bb.y;
+                v[i * 8 + j + 2] = (v[i * 8 + j + 2] - mean) * rstd * gg.z + bb.z;
+                v[i * 8 + j + 3] = (v[i * 8 + j + 3] - mean) * rstd * gg.w + bb.w;
+            }
+    }
+}
+
+struct HeadArgs {
+    const bf16* x;
+    int n_slots, n_base_slots, tokens, d, n_classes, base_blocks, base_cols;     // base_cols: blocks along the classes
+    float eps;
+    const float *lnf_g, *lnf_b;
+    const bf16* base_wt;
+    const float* base_b;
+    float* base_out;
+    const bf16* hcat;
+    const float* hbias;
+    const int *hcls, *hoff, *slot_off, *slot_ids, *perm;
+    float* scores;
+    int zero_rows;             // 1: a slot's block owns its row of scores and zeroes it; 0: rows are zero already
+};
+
+__device__ __forceinline__ void mma_16x8x16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+template <int NT>
+__global__ void __launch_bounds__(256, 2) heads_kernel(const HeadArgs args) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int d = args.d;
+    if ((int)blockIdx.x < args.base_blocks) {
+        // ------------------------------------------------------------------ base head
+        constexpr int MAX_CHUNKS = 8;                          // d <= 1024: 32 chunks of 32 values over four warps
+        const int stride = d * 2 + 64;                         // bytes of a row of one part: 64 mod 128, no bank conflicts
+        const int n0 = ((int)blockIdx.x % args.base_cols) * 16 * NT + (warp >> 2) * 8 * NT;     // this warp's first class
+        const int s0 = (int)blockIdx.x / args.base_cols * HB_SLOTS;
+        const int kg = warp & 3, g = lane >> 2, t = lane & 3;
+        const int chunks = d / 32, c0 = chunks * kg / 4, c1 = chunks * (kg + 1) / 4;
+        uint4 w[MAX_CHUNKS][NT];
+#pragma unroll
+        for (int i = 0; i < MAX_CHUNKS; ++i)
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                const int k = n0 + j * 8 + g;
+                w[i][j] = c0 + i < c1 && k < args.n_classes ? __ldg(reinterpret_cast<const uint4*>(args.base_wt + (size_t)k * d + (c0 + i) * 32 + t * 8))
+                                                            : make_uint4(0, 0, 0, 0);
+            }
+        dep_wait();
+        for (int r = warp; r < HB_SLOTS; r += 8) {
+            uint8_t* row = smem + r * stride;
+            float v[32];
+            if (s0 + r < args.n_base_slots) {
+                ln_regs(args.x + (size_t)(s0 + r) * args.tokens * d, args.lnf_g, args.lnf_b, d, args.eps, lane, v);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 32; ++i) v[i] = 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if ((lane + 32 * i) * 8 >= d) break;
+                uint32_t part[3][4];
+#pragma unroll
+                for (int j = 0; j < 8; j += 2) {
+                    float lo = v[i * 8 + j], hi = v[i * 8 + j + 1];
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+                        part[q][j >> 1] = *reinterpret_cast<const uint32_t*>(&h);
+                        lo -= __low2float(h);
+                        hi -= __high2float(h);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    *reinterpret_cast<uint4*>(row + q * HB_SLOTS * stride + (lane + 32 * i) * 16) = make_uint4(part[q][0], part[q][1], part[q][2], part[q][3]);
+            }
+        }
+        __syncthreads();
+        float acc[NT][4];
+#pragma unroll
+        for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+#pragma unroll
+        for (int i = 0; i < MAX_CHUNKS; ++i) {
+            if (c0 + i >= c1) break;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const uint8_t* at = smem + (q * HB_SLOTS + g) * stride + (c0 + i) * 64 + t * 16;
+                const uint4 lo = *reinterpret_cast<const uint4*>(at), hi = *reinterpret_cast<const uint4*>(at + 8 * stride);
+#pragma unroll
+                for (int j = 0; j < NT; ++j) {
+                    mma_16x8x16(acc[j], lo.x, hi.x, lo.y, hi.y, w[i][j].x, w[i][j].y);
+                    mma_16x8x16(acc[j], lo.z, hi.z, lo.w, hi.w, w[i][j].z, w[i][j].w);
+                }
+            }
+        }
+        __syncthreads();                                       // the features are no longer needed: partial sums go there
+        float* red = reinterpret_cast<float*>(smem);           // [warp][NT * 4][lane]
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) red[((warp * NT + j) * 4 + e) * 32 + lane] = acc[j][e];
+        __syncthreads();
+        for (int i = threadIdx.x; i < 2 * NT * 128; i += 256) {
+            const int half = i / (NT * 128), o = i % (NT * 128);           // o = (j * 4 + e) * 32 + lane
+            float v = 0.f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v += red[(half * 4 + q) * NT * 128 + o];
+            const int l = o & 31, e = (o >> 5) & 3, j = o >> 7;
+            const int slot = s0 + (l >> 2) + (e >> 1) * 8;
+            const int k = n0 - (warp >> 2) * 8 * NT + half * 8 * NT + j * 8 + (l & 3) * 2 + (e & 1);
+            if (slot < args.n_base_slots && k < args.n_classes)
+                args.base_out[(size_t)args.perm[slot] * args.n_classes + k] = sigmoidf_acc(v + args.base_b[k]);
+        }
+        return;
+    }
+    // ---------------------------------------------------------------------- adapter heads of one slot
+    const int slot = (int)blockIdx.x - args.base_blocks;
+    float* out = args.scores + (size_t)args.perm[slot] * args.n_classes;
+    const int p0 = args.slot_off[slot], p1 = args.slot_off[slot + 1];
+    dep_wait();
+    if (args.zero_rows) {
+        for (int k = threadIdx.x; k < args.n_classes; k += 256) out[k] = 0.f;
+        __syncthreads();
+    }
+    if (p0 == p1) return;
+    float z[32];
+    ln_regs(args.x + (size_t)slot * args.tokens * d, args.lnf_g, args.lnf_b, d, args.eps, lane, z);
+    const int nch = d >> 3;
+    for (int p = p0; p < p1; ++p) {
+        const int a = args.slot_ids[p];
+        const int r0 = args.hoff[a], r1 = args.hoff[a + 1];
+        for (int rb = r0 + warp * 4; rb < r1; rb += 32) {
+            float acc[4];
+            uint4 w[4][4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    w[q][i] = rb + q < r1 && lane + 32 * i < nch ? __ldg(reinterpret_cast<const uint4*>(args.hcat + (size_t)(rb + q) * d) + lane + 32 * i)
+                                                                 : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint32_t ww[4] = {w[q][i].x, w[q][i].y, w[q][i].z, w[q][i].w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        c[e] = fmaf(z[i * 8 + 2 * e], __uint_as_float(ww[e] << 16), c[e]);
+                        c[e] = fmaf(z[i * 8 + 2 * e + 1], __uint_as_float(ww[e] & 0xFFFF0000u), c[e]);
+                    }
+                }
+                acc[q] = (c[0] + c[1]) + (c[2] + c[3]);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[q] += __shfl_xor_sync(0xFFFFFFFFu, acc[q], o);
+            if (lane < 4 && rb + lane < r1) {
+                const float v = lane == 0 ? acc[0] : lane == 1 ? acc[1] : lane == 2 ? acc[2] : acc[3];
+                atomicMax(reinterpret_cast<int*>(out + args.hcls[rb + lane]), __float_as_int(sigmoidf_acc(v + args.hbias[rb + lane])));
+            }
+        }
+    }
+}
+
+// fp32 debug build.
 // grid (ceil(K/32), ceil(F/8)): a block owns 32 classes x 8 slots.  The 8 CLS features are staged once in
-// shared memory and shared by the block's 8 warps (read straight from global memory, every class of a
-// block would fetch them again: F x K x d x 4 bytes of cache traffic in all); each warp takes four of the
-// classes in turn, keeps the weight row of the class in registers and walks the slots (the next class's
-// row is fetched while this one is multiplied).  base_out rows are in the caller's order.
-// NV = ceil(d / 32) values per lane; the dot product runs in four chains.
+// shared memory and shared by the block's 8 warps; each warp takes four of the classes in turn, keeps the weight row of
+// the class in registers and walks the slots (the next class's row is fetched while this one is multiplied).
+// base_out rows are in the caller's order.  NV = ceil(d / 32) values per lane; the dot product runs in four chains.
 constexpr int BASE_HEAD_FRAMES = 8;
 constexpr int BASE_HEAD_CLASSES = 32;
 template <typename T, int NV>
@@ -548,25 +748,51 @@ cudaError_t launch_heads(const Launch& L, const T* x, int n_slots, int n_out_fra
                          const RouteDev& R, float* scores_out, float* base_out) {
     if (n_slots <= 0) return cudaSuccess;
     ProfScope ps(L, KC_HEADS);
-    final_ln_kernel<T><<<(n_slots + 7) / 8, 256, 0, L.st>>>(x, lnf_g, lnf_b, z, n_slots, tokens, d, eps);
-    BUMP(L);
-    if (base_out && n_base_slots > 0) {
-        dim3 grid((n_classes + BASE_HEAD_CLASSES - 1) / BASE_HEAD_CLASSES, (n_base_slots + BASE_HEAD_FRAMES - 1) / BASE_HEAD_FRAMES);
-        const int nv = (d + 31) / 32;                  // d <= 1024
-        auto kern = nv <= 6 ? base_head_kernel<T, 6> : nv <= 12 ? base_head_kernel<T, 12>
-                  : nv <= 24 ? base_head_kernel<T, 24> : base_head_kernel<T, 32>;
-        kern<<<grid, 256, 0, L.st>>>(z, base_wt, base_b, R.perm, d, n_classes, n_base_slots, base_out);
-        BUMP(L);
+    // one row of scores per slot: its block zeroes it; several slots per row (branches): zeroed beforehand
+    const bool zero_rows = sizeof(T) == 2 && n_slots == n_out_frames;
+    if (!zero_rows) {
+        cudaError_t e = cudaMemsetAsync(scores_out, 0, (size_t)n_out_frames * n_classes * sizeof(float), L.st);
+        if (e != cudaSuccess) return e;
     }
-    cudaError_t e = cudaMemsetAsync(scores_out, 0, (size_t)n_out_frames * n_classes * sizeof(float), L.st);
-    if (e != cudaSuccess) return e;
-    if (R.max_set > 0) {
-        dim3 grid(R.max_set, n_slots);
-        adapter_heads_kernel<T><<<grid, 256, 0, L.st>>>(z, hcat, hbias, hcls, hoff, R.slot_off, R.slot_ids,
-                                                       R.perm, d, n_classes, scores_out);
+    if constexpr (sizeof(T) == 2) {
+        HeadArgs a;
+        a.x = x; a.n_slots = n_slots; a.n_base_slots = n_base_slots; a.tokens = tokens; a.d = d; a.n_classes = n_classes; a.eps = eps;
+        a.lnf_g = lnf_g; a.lnf_b = lnf_b; a.base_wt = base_wt; a.base_b = base_b; a.base_out = base_out;
+        a.hcat = hcat; a.hbias = hbias; a.hcls = hcls; a.hoff = hoff;
+        a.slot_off = R.slot_off; a.slot_ids = R.slot_ids; a.perm = R.perm; a.scores = scores_out; a.zero_rows = zero_rows;
+        const int rows = base_out ? (n_base_slots + HB_SLOTS - 1) / HB_SLOTS : 0;
+        // few slots: narrow blocks, so that the classes spread over the SMs; many: wide ones, which normalise their rows less often
+        const bool narrow = rows * ((n_classes + 31) / 32) < 148;
+        a.base_cols = narrow ? (n_classes + 15) / 16 : (n_classes + 31) / 32;
+        a.base_blocks = rows * a.base_cols;
+        const int adapter_blocks = zero_rows || R.max_set > 0 ? n_slots : 0;
+        const int smem = 3 * HB_SLOTS * (d * 2 + 64);
+        static SmemGrant grant1, grant2;
+        cudaError_t e = narrow ? grant1.ensure(heads_kernel<1>, smem) : grant2.ensure(heads_kernel<2>, smem);
+        if (e != cudaSuccess) return e;
+        if (a.base_blocks + adapter_blocks == 0) return cudaSuccess;
+        e = launch_overlapped(narrow ? heads_kernel<1> : heads_kernel<2>, a.base_blocks + adapter_blocks, 256, smem, L.st, 1, a);
         BUMP(L);
+        return e;
+    } else {
+        final_ln_kernel<T><<<(n_slots + 7) / 8, 256, 0, L.st>>>(x, lnf_g, lnf_b, z, n_slots, tokens, d, eps);
+        BUMP(L);
+        if (base_out && n_base_slots > 0) {
+            dim3 grid((n_classes + BASE_HEAD_CLASSES - 1) / BASE_HEAD_CLASSES, (n_base_slots + BASE_HEAD_FRAMES - 1) / BASE_HEAD_FRAMES);
+            const int nv = (d + 31) / 32;                  // d <= 1024
+            auto kern = nv <= 6 ? base_head_kernel<T, 6> : nv <= 12 ? base_head_kernel<T, 12>
+                      : nv <= 24 ? base_head_kernel<T, 24> : base_head_kernel<T, 32>;
+            kern<<<grid, 256, 0, L.st>>>(z, base_wt, base_b, R.perm, d, n_classes, n_base_slots, base_out);
+            BUMP(L);
+        }
+        if (R.max_set > 0) {
+            dim3 grid(R.max_set, n_slots);
+            adapter_heads_kernel<T><<<grid, 256, 0, L.st>>>(z, hcat, hbias, hcls, hoff, R.slot_off, R.slot_ids,
+                                                           R.perm, d, n_classes, scores_out);
+            BUMP(L);
+        }
+        return cudaGetLastError();
     }
-    return cudaGetLastError();
 }
 template cudaError_t launch_heads<float>(const Launch&, const float*, int, int, int, int, int, float, const float*, const float*, float*, const float*, const float*, int, const float*, const float*, const int*, const int*, const RouteDev&, float*, float*);
 template cudaError_t launch_heads<bf16>(const Launch&, const bf16*, int, int, int, int, int, float, const float*, const float*, float*, const bf16*, const float*, int, const bf16*, const float*, const int*, const int*, const RouteDev&, float*, float*);
@@ -623,6 +849,7 @@ __global__ void __launch_bounds__(SELECT_THREADS) select_kernel(const float* __r
 
     const int f = blockIdx.x * nwarps + warp;
     bool changed = false;
+    dep_wait();
     if (f < n_frames) {
         const float* row = scores + (size_t)f * n_classes;
         uint32_t* lab = prev_labels ? prev_labels + (size_t)f * NW : nullptr;
@@ -771,11 +998,11 @@ cudaError_t launch_select(const Launch& L, const float* scores, int n_frames, in
     const int blocks = n_frames > 0 ? (n_frames + SELECT_THREADS / 32 - 1) / (SELECT_THREADS / 32) : 1;
     const int aw = (n_adapters + 63) / 64;     // at most 256 adapters
     auto kern = aw <= 1 ? select_kernel<1> : aw == 2 ? select_kernel<2> : aw == 3 ? select_kernel<3> : select_kernel<4>;
-    kern<<<blocks, SELECT_THREADS, 0, L.st>>>(scores, n_frames, n_classes, n_adapters, thr, context_copy,
-                                        has_prev, prev_labels, prev_off, prev_ids, first, provider,
-                                        mask_scratch, next_off, next_ids, ids_capacity, L.status, metrics);
+    const cudaError_t e = launch_overlapped(kern, blocks, SELECT_THREADS, 0, L.st, 1, scores, n_frames, n_classes, n_adapters, thr, context_copy,
+                                            has_prev, prev_labels, prev_off, prev_ids, first, provider,
+                                            mask_scratch, next_off, next_ids, ids_capacity, L.status, metrics);
     BUMP(L);
-    return cudaGetLastError();
+    return e;
 }
 
 // ---------------------------------------------------------------------------------------
