@@ -137,7 +137,7 @@ bool attention_encode_maps(const bf16* qkv, int n_frames, int tokens, int heads,
                            CUtensorMap* tm_kv);
 // n_sms > 0 selects the pipelined persistent kernel where it applies (one key block); 0 = never
 cudaError_t launch_attention_tc(const Launch& L, const CUtensorMap& tm_q, const CUtensorMap& tm_kv,
-                                bf16* out, int n_frames, int tokens, int heads, int n_sms);
+                                const bf16* qkv, bf16* out, int n_frames, int tokens, int heads, int n_sms);
 // patch gather, and the CLS rows of x
 template <typename T>
 cudaError_t launch_im2col(const Launch& L, const T* frames, const int* perm, T* out, int n_frames,
@@ -270,9 +270,9 @@ cudaError_t launch_latency_forward(const Launch& L, const LatArgs& a);
 // stream has released its dependents; it awaits that kernel's results itself with dep_wait()), with or
 // without thread-block clusters along x.
 template <typename... P, typename... A>
-cudaError_t launch_overlapped(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t st, int cluster, const A&... args) {
+cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, int cluster, const A&... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;

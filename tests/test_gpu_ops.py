@@ -330,3 +330,21 @@ def test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, 
         want = want + res.double()
     np.testing.assert_allclose(to_np(y), want.cpu().numpy(), **TOL[0])
     lin.close()
+
+
+@pytest.mark.parametrize("frames,tokens,heads", [(1, 1, 1), (2, 16, 3), (1, 17, 2), (3, 49, 1), (1, 208, 12), (49, 33, 1),     # a few pairs
+                                                 (50, 33, 1), (60, 1, 1), (20, 197, 3), (17, 208, 4), (13, 129, 12)])           # the pipelined kernel
+def test_attention_of_one_key_block_on_both_sides_of_the_pair_limit(frames, tokens, heads):
+    """Up to 208 tokens: few (frame, head) pairs run as one CTA per 16 query rows, more as the pipelined kernel (limit:
+    49 pairs on 148 SMs); token counts at the edges of 16-key groups and query tiles.  Against the oracle."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    d = heads * 64
+    qkv = wl.normal((frames * tokens, 3 * d), 1.0, "attn_gpu_few", frames, tokens, heads)
+    od = torch.full((frames * tokens, d), float("nan"), device="cuda", dtype=torch.bfloat16)
+    binding.attention(to_dev(qkv, 0), od, frames, tokens, heads, 0)
+    torch.cuda.synchronize()
+    got = to_np(od)
+    for f in sorted({0, frames // 2, frames - 1}):
+        want = po.attention(qkv[f * tokens:(f + 1) * tokens].astype(np.float64), heads)
+        np.testing.assert_allclose(got[f * tokens:(f + 1) * tokens], want, **TOL[0])
