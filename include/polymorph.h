@@ -271,7 +271,8 @@ int pm_set_graphs(pm_handle h, int on);
  * Default on. */
 int pm_set_small_batch_kernel(pm_handle h, int on);
 
-/* Number of kernels the library has launched on this handle since creation (kernels of a replayed graph included). */
+/* Number of kernels the library has launched on this handle since creation (kernels of a replayed graph included;
+ * uploads of a routing plan built on the host not). */
 long long pm_launch_count(pm_handle h);
 
 /* Device timing of the library's own kernels, by class, with CUDA events recorded on the launching

@@ -122,14 +122,37 @@ def _ptr(t):
     if t is None:
         return None
     if isinstance(t, np.ndarray):
-        return t.ctypes.data
+        try:
+            return C.addressof(_Start.from_buffer(t))      # a third of the time of the array's own attributes
+        except (TypeError, ValueError, BufferError):       # read-only
+            return t.ctypes.data
     return t.data_ptr()
+
+
+_Start = C.c_byte * 0
+
+
+def _i32(a):
+    """The array itself if it is contiguous int32 already (the usual case, and cheaper to see than to convert)."""
+    if a.dtype == _INT32 and a.flags.c_contiguous:
+        return a
+    return np.ascontiguousarray(a, dtype=np.int32)
+
+
+_INT32 = np.dtype(np.int32)
+_raw_stream = None             # () -> cudaStream_t of the current device's current stream
 
 
 def _stream_ptr(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        global _raw_stream
+        if _raw_stream is None:
+            import torch
+            torch.cuda.current_stream()                    # initialises CUDA
+            get, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+            # the Stream object that torch.cuda.current_stream() builds costs more than a kernel launch
+            _raw_stream = (lambda: get(device())) if get and device else (lambda: torch.cuda.current_stream().cuda_stream)
+        return _raw_stream()
     return getattr(stream, "cuda_stream", stream)
 
 
@@ -175,37 +198,37 @@ class Model:
     def forward(self, frames, set_offsets, set_ids, scores_out, base_out=None, stream=None):
         """frames/scores_out/base_out: torch CUDA tensors; set lists: numpy int32 (host) or torch
         CUDA int32 tensors."""
-        n = int(frames.shape[0])
+        n = frames.size(0)
         if isinstance(set_offsets, np.ndarray):
-            set_offsets = np.ascontiguousarray(set_offsets, dtype=np.int32)
+            set_offsets = _i32(set_offsets)
         if isinstance(set_ids, np.ndarray):
-            set_ids = np.ascontiguousarray(set_ids, dtype=np.int32)
+            set_ids = _i32(set_ids)
         self._check(self.lib.pm_forward(self.handle, _ptr(frames), n, _ptr(set_offsets), _ptr(set_ids),
                                         _ptr(scores_out), _ptr(base_out), _stream_ptr(stream)), "pm_forward")
 
     def forward_device_sets(self, frames, set_offsets, set_ids, scores_out, base_out=None, stream=None):
         """pm_forward_device_sets: the set lists are torch CUDA int32 tensors (e.g. written by
         select()); the plan is built on the device, nothing synchronises."""
-        self._check(self.lib.pm_forward_device_sets(self.handle, _ptr(frames), int(frames.shape[0]),
+        self._check(self.lib.pm_forward_device_sets(self.handle, _ptr(frames), frames.size(0),
                                                     _ptr(set_offsets), _ptr(set_ids), _ptr(scores_out),
                                                     _ptr(base_out), _stream_ptr(stream)), "pm_forward_device_sets")
 
     def forward_branched(self, frames, set_offsets, set_ids, trunk_layers, scores_out, base_out=None, stream=None):
         """pm_forward_branched: shared trunk of `trunk_layers` blocks, then one branch per active
         adapter (and the base branch if base_out is given).  Arguments as for forward()."""
-        n = int(frames.shape[0])
+        n = frames.size(0)
         if isinstance(set_offsets, np.ndarray):
-            set_offsets = np.ascontiguousarray(set_offsets, dtype=np.int32)
+            set_offsets = _i32(set_offsets)
         if isinstance(set_ids, np.ndarray):
-            set_ids = np.ascontiguousarray(set_ids, dtype=np.int32)
+            set_ids = _i32(set_ids)
         self._check(self.lib.pm_forward_branched(self.handle, _ptr(frames), n, _ptr(set_offsets), _ptr(set_ids),
                                                  int(trunk_layers), _ptr(scores_out), _ptr(base_out),
                                                  _stream_ptr(stream)), "pm_forward_branched")
 
     def select(self, scores, score_thr, context_copy, has_prev, prev_labels, prev_offsets, prev_ids,
                next_offsets, next_ids, stream=None):
-        n = int(scores.shape[0])
-        cap = 0 if next_ids is None else int(next_ids.numel())
+        n = scores.size(0)
+        cap = 0 if next_ids is None else next_ids.numel()
         self._check(self.lib.pm_select(self.handle, _ptr(scores), n, score_thr, int(context_copy),
                                        int(has_prev), _ptr(prev_labels), _ptr(prev_offsets), _ptr(prev_ids),
                                        _ptr(next_offsets), _ptr(next_ids), cap, _stream_ptr(stream)), "pm_select")
@@ -290,8 +313,8 @@ class Linear:
                     "pm_linear_register")
 
     def forward(self, x, n_frames, set_offsets, set_ids, y, residual=None, stream=None):
-        so = np.ascontiguousarray(set_offsets, dtype=np.int32)
-        si = np.ascontiguousarray(set_ids, dtype=np.int32)
+        so = _i32(set_offsets) if isinstance(set_offsets, np.ndarray) else np.ascontiguousarray(set_offsets, dtype=np.int32)
+        si = _i32(set_ids) if isinstance(set_ids, np.ndarray) else np.ascontiguousarray(set_ids, dtype=np.int32)
         self._check(self.lib.pm_linear_forward(self.handle, _ptr(x), n_frames, _ptr(so), _ptr(si),
                                                _ptr(residual), _ptr(y), _stream_ptr(stream)), "pm_linear_forward")
 

@@ -199,8 +199,7 @@ struct Router {
     int last_frames = -1;
     bool last_sorted = false;
     std::vector<int> perm_host, sorted_ids;
-    struct SlabRows { int slab; uint32_t mask[8]; };     // arena slab -> 256-bit mask of the pair's rows using it
-    std::vector<SlabRows> pair_slabs;                    // scratch of build(): the slabs of the pair at hand
+    uint64_t row_mask[256][4];       // scratch of build(): the rows of the pair at hand that use an adapter
     long long plans_built = 0;       // host plans built (cache misses) and the host time they took
     double plan_host_ms = 0.0;
 
@@ -248,7 +247,7 @@ struct Router {
     // already in slot order; slot i reports to output row frame_of_slot[i] and starts from the trunk
     // rows of slot src_of_slot[i] (the branched forward's plan).
     int build(int n_frames, const int32_t* offsets, const int32_t* ids, const std::vector<int>& ranks,
-              const std::vector<float>& scales, bool sort_frames, cudaStream_t st, std::string& err,
+              const std::vector<float>& scales, bool sort_frames, const Launch& L, std::string& err,
               const int* frame_of_slot = nullptr, const int* src_of_slot = nullptr) {
         if (n_frames < 0 || (n_frames > 0 && (!offsets))) { err = "bad frame count or NULL set_offsets"; return PM_ERR_ARG; }
         if (n_frames > max_frames) { err = "n_frames exceeds max_frames"; return PM_ERR_CAPACITY; }
@@ -313,52 +312,66 @@ struct Router {
         const long long rows = (long long)n_frames * tokens;
         const int n_pairs = (int)((rows + 2 * PM_TILE_M - 1) / (2 * PM_TILE_M));
         const int n_tiles = 2 * n_pairs;
-        pair_slabs.resize(std::max(slab_cap, 1));
-        SlabRows* ps = pair_slabs.data();
         for (int p = 0; p < n_pairs; ++p) {
             const long long r0 = (long long)p * 2 * PM_TILE_M, r1 = std::min(rows, r0 + 2 * PM_TILE_M);
-            int n_ps = 0;                                   // kept in ascending slab order
+            uint64_t used[4] = {0, 0, 0, 0};                // adapters of the pair's frames, and how many slabs they have
+            int n_ps = 0;
             for (int slot = (int)(r0 / tokens); slot <= (int)((r1 - 1) / tokens); ++slot) {
                 const int b0 = (int)(std::max(r0, (long long)slot * tokens) - r0);
                 const int b1 = (int)(std::min(r1, (long long)(slot + 1) * tokens) - r0);     // bits [b0, b1)
-                uint32_t m[8];
-                for (int q = 0; q < 8; ++q) {
-                    const int lo = std::max(b0, 32 * q) - 32 * q, hi = std::min(b1, 32 * q + 32) - 32 * q;
-                    m[q] = hi <= lo ? 0u : (hi - lo == 32 ? 0xFFFFFFFFu : ((1u << (hi - lo)) - 1u) << lo);
+                uint64_t m[4];
+                for (int q = 0; q < 4; ++q) {
+                    const int lo = std::max(b0, 64 * q) - 64 * q, hi = std::min(b1, 64 * q + 64) - 64 * q;
+                    m[q] = hi <= lo ? 0ull : (hi - lo == 64 ? ~0ull : ((1ull << (hi - lo)) - 1ull) << lo);
                 }
                 const auto st_ = set_of(perm_host[slot]);
                 for (const int* ap = st_.first; ap != st_.second; ++ap) {
-                    const int ns = (ranks[*ap] + PM_SLAB - 1) / PM_SLAB;
-                    for (int j = 0; j < ns; ++j) {
-                        const int slab = *ap * slabs_max + j;
-                        int at = 0;
-                        while (at < n_ps && ps[at].slab < slab) ++at;
-                        if (at == n_ps || ps[at].slab != slab) {
-                            if (n_ps >= slab_cap) { err = "tile needs more LoRA slabs than the plan capacity"; return PM_ERR_CAPACITY; }
-                            for (int i = n_ps; i > at; --i) ps[i] = ps[i - 1];
-                            ps[at].slab = slab;
-                            for (int q = 0; q < 8; ++q) ps[at].mask[q] = 0u;
-                            ++n_ps;
-                        }
-                        for (int q = 0; q < 8; ++q) ps[at].mask[q] |= m[q];
+                    uint64_t* rm = row_mask[*ap];
+                    const uint64_t bit = 1ull << (*ap & 63);
+                    if (!(used[*ap >> 6] & bit)) {
+                        used[*ap >> 6] |= bit;
+                        n_ps += (ranks[*ap] + PM_SLAB - 1) / PM_SLAB;
+                        for (int q = 0; q < 4; ++q) rm[q] = m[q];
+                    } else {
+                        for (int q = 0; q < 4; ++q) rm[q] |= m[q];
                     }
                 }
             }
-            for (int half = 0; half < 2; ++half) {
-                const int t = 2 * p + half;
-                h_tn[t] = n_ps;
-                for (int i = 0; i < n_ps; ++i) {
-                    const size_t at = (size_t)t * slab_cap + i;
-                    h_ts[at] = ps[i].slab;
-                    h_tsc[at] = scales[ps[i].slab / slabs_max];
-                    for (int q = 0; q < 4; ++q) h_tm[at * 4 + q] = ps[i].mask[half * 4 + q];
+            if (n_ps > slab_cap) { err = "tile needs more LoRA slabs than the plan capacity"; return PM_ERR_CAPACITY; }
+            h_tn[2 * p] = h_tn[2 * p + 1] = n_ps;
+            size_t at0 = (size_t)(2 * p) * slab_cap, at1 = at0 + slab_cap;
+            for (int w = 0; w < 4; ++w)
+                for (uint64_t bits = used[w]; bits; bits &= bits - 1) {
+                    const int a = w * 64 + __builtin_ctzll(bits);
+                    const int nsl = (ranks[a] + PM_SLAB - 1) / PM_SLAB;
+                    for (int j = 0; j < nsl; ++j, ++at0, ++at1) {
+                        h_ts[at0] = h_ts[at1] = a * slabs_max + j;
+                        h_tsc[at0] = h_tsc[at1] = scales[a];
+                        std::memcpy(h_tm + at0 * 4, row_mask[a], 16);          // rows 0..127 (little-endian words)
+                        std::memcpy(h_tm + at1 * 4, row_mask[a] + 2, 16);      // rows 128..255
+                    }
                 }
-            }
         }
         plan_host_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_start).count();
         ++plans_built;
-        CK(cudaMemcpyAsync(blob.p, stage[si], blob_bytes, cudaMemcpyHostToDevice, st));
-        CK(cudaEventRecord(uploaded[si], st));
+        PlanSegments seg;
+        seg.n = 0;
+        auto used_part = [&](size_t off, size_t bytes) {
+            if (bytes == 0) return;
+            seg.at[seg.n] = (uint32_t)(off / 16);
+            seg.units[seg.n++] = (uint32_t)((bytes + 15) / 16);
+        };
+        const size_t entries = (size_t)n_tiles * slab_cap;
+        used_part(off_perm, sizeof(int) * n_frames);
+        used_part(off_soff, sizeof(int) * (n_frames + 1));
+        used_part(off_sids, sizeof(int) * nnz);
+        used_part(off_src, sizeof(int) * n_frames);
+        used_part(off_tn, sizeof(int) * n_tiles);
+        used_part(off_ts, sizeof(int) * entries);
+        used_part(off_tsc, sizeof(float) * entries);
+        used_part(off_tm, sizeof(uint32_t) * 4 * entries);
+        CK(launch_plan_upload(L, stage[si], blob.p, seg));
+        CK(cudaEventRecord(uploaded[si], L.st));
         upload_pending[si] = true;
         ++version; device_plan_frames = -1;
         dev.n_frames = n_frames; dev.n_tiles = n_tiles; dev.max_set = widest;
@@ -972,7 +985,8 @@ int pm_forward(pm_handle h, const void* frames, int n_frames, const int32_t* set
     const int32_t *o, *i;
     int rc = fetch_csr(set_offsets, set_ids, n_frames, st, hoff, hids, &o, &i, err);
     if (rc) return rc;
-    rc = h->router.build(n_frames, o, i, h->ranks, h->scales, true, st, err);
+    Launch up; up.st = st;
+    rc = h->router.build(n_frames, o, i, h->ranks, h->scales, true, up, err);
     if (rc) return rc;
     if (h->heads_dirty) {
         rc = h->cfg.dtype == 0 ? rebuild_heads<bf16>(h) : rebuild_heads<float>(h);
@@ -1085,7 +1099,8 @@ int pm_forward_branched(pm_handle h, const void* frames, int n_frames, const int
         fos.push_back(e.second); src.push_back(e.second);
     }
     if (bids.empty()) bids.push_back(0);
-    rc = h->router.build((int)n_slots, boff.data(), bids.data(), h->ranks, h->scales, false, st, err,
+    Launch up; up.st = st;
+    rc = h->router.build((int)n_slots, boff.data(), bids.data(), h->ranks, h->scales, false, up, err,
                          fos.data(), src.data());
     if (rc) return rc;
     if (h->heads_dirty) {
@@ -1274,9 +1289,9 @@ int pm_linear_forward(pm_linear l, const void* x, int n_frames, const int32_t* s
     if (n_frames < 0 || (n_frames > 0 && (!x || !y || !set_offsets))) { err = "NULL argument"; return PM_ERR_ARG; }
     if (l->epilogue == EPI_RESIDUAL && n_frames > 0 && !residual) { err = "epilogue 2 needs a residual"; return PM_ERR_ARG; }
     if (n_frames == 0) return PM_OK;
-    int rc = l->router.build(n_frames, set_offsets, set_ids, l->ranks, l->scales, false, st, err);
-    if (rc) return rc;
     Launch L; L.st = st; L.launches = &l->launches; L.status = l->status.as<int>();
+    int rc = l->router.build(n_frames, set_offsets, set_ids, l->ranks, l->scales, false, L, err);
+    if (rc) return rc;
     const RouteDev& R = l->router.dev;
     const int rows = n_frames * l->tokens;
     PatchEpi none;

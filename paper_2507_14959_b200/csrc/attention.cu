@@ -996,7 +996,7 @@ cudaError_t launch_attention_tc(const Launch& L, const CUtensorMap& tm_q, const 
         static SmemGrant grant;
         if (cudaError_t e = grant.ensure(attention_few_kernel, (int)sizeof(AttnFewSmem)); e != cudaSuccess) return e;
         ProfScope ps(L, KC_ATTENTION);
-        cudaError_t e = launch_overlapped(attention_few_kernel, dim3(row_tiles, n_frames * heads), 32 * AFEW_WARPS, sizeof(AttnFewSmem), L.st, 1,
+        cudaError_t e = launch_overlapped(L, attention_few_kernel, dim3(row_tiles, n_frames * heads), 32 * AFEW_WARPS, sizeof(AttnFewSmem), 1,
                                           tm_kv, qkv, out, tokens, heads, L.status);
         BUMP(L);
         return e;
@@ -1010,7 +1010,7 @@ cudaError_t launch_attention_tc(const Launch& L, const CUtensorMap& tm_q, const 
         static SmemGrant grant;
         if (cudaError_t e = grant.ensure(attention_pipe_kernel, (int)psmem); e != cudaSuccess) return e;
         ProfScope ps(L, KC_ATTENTION);
-        cudaError_t e = launch_overlapped(attention_pipe_kernel, std::min(pa.n_items, n_sms), APIPE_THREADS, psmem, L.st, 1, tm_q, tm_kv, pa);
+        cudaError_t e = launch_overlapped(L, attention_pipe_kernel, std::min(pa.n_items, n_sms), APIPE_THREADS, psmem, 1, tm_q, tm_kv, pa);
         BUMP(L);
         return e;
     }
@@ -1019,7 +1019,7 @@ cudaError_t launch_attention_tc(const Launch& L, const CUtensorMap& tm_q, const 
     static SmemGrant grant;
     if (cudaError_t e = grant.ensure(attention_tc_kernel<ATT_SHARES>, (int)smem); e != cudaSuccess) return e;
     ProfScope ps(L, KC_ATTENTION);
-    cudaError_t e = launch_overlapped(attention_tc_kernel<ATT_SHARES>, n_frames * heads * a.q_split, 32 + 128 * ATT_SHARES, smem, L.st, 1,
+    cudaError_t e = launch_overlapped(L, attention_tc_kernel<ATT_SHARES>, n_frames * heads * a.q_split, 32 + 128 * ATT_SHARES, smem, 1,
                                       tm_q, tm_kv, a);
     BUMP(L);
     return e;

@@ -102,6 +102,7 @@ struct Launch {
     long long* launches = nullptr;
     int* status = nullptr;      // device status word
     Profiler* prof = nullptr;
+    mutable bool ordered = false;   // a plan upload was enqueued just before: kernels read the plan before they wait
 };
 
 struct ProfScope {              // brackets the launches made while it is alive
@@ -188,6 +189,10 @@ cudaError_t launch_heads(const Launch& L, const T* x, int n_slots, int n_out_fra
                          const T* base_wt, const float* base_b, int n_classes,
                          const T* hcat, const float* hbias, const int* hcls, const int* hoff,
                          const RouteDev& R, float* scores_out, float* base_out);
+// Copies the used parts of a host-built plan (pinned memory) to the device tables: segments of 16-byte units at
+// the same offset in both.
+struct PlanSegments { int n; uint32_t at[8], units[8]; };
+cudaError_t launch_plan_upload(const Launch& L, const void* host, void* dev, const PlanSegments& seg);
 // Builds the routing tables of R (perm, slot CSR, tile plan) on the device from a device CSR
 // (plan_device.cu).  Problems found in the lists go to the status word.
 cudaError_t launch_device_plan(const Launch& L, const RouteDev& R, int n_frames, int max_set, int max_adapters,
@@ -268,17 +273,18 @@ cudaError_t launch_latency_forward(const Launch& L, const LatArgs& a);
 
 // Launch with programmatic stream serialization (the kernel may start once every CTA of the one before it on the
 // stream has released its dependents; it awaits that kernel's results itself with dep_wait()), with or
-// without thread-block clusters along x.
+// without thread-block clusters along x.  The first one after L.ordered was set starts behind its predecessor's end.
 template <typename... P, typename... A>
-cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, int cluster, const A&... args) {
+cudaError_t launch_overlapped(const Launch& L, void (*kernel)(P...), dim3 grid, int block, size_t smem, int cluster, const A&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
+    cfg.stream = L.st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = L.ordered ? 0 : 1;
+    L.ordered = false;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;

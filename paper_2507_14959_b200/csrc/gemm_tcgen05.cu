@@ -836,8 +836,7 @@ static cudaError_t launch_gemm_bn(const Launch& L, const CUtensorMap& tm_x, cons
     if (cudaError_t e = grant.ensure(lora_gemm_kernel<BN, EPI, EW, LNF>, Smem<BN, EW>::TOTAL); e != cudaSuccess) return e;
     const int total = a.m_tiles * a.n_tiles;
     ProfScope ps(L, KC_GEMM);
-    cudaError_t e = launch_overlapped(lora_gemm_kernel<BN, EPI, EW, LNF>, total < n_sms ? total : n_sms, 64 + 32 * EW, Smem<BN, EW>::TOTAL,
-                                      L.st, 1, tm_x, tm_w, tm_t, tm_bt, tm_y, a);
+    cudaError_t e = launch_overlapped(L, lora_gemm_kernel<BN, EPI, EW, LNF>, total < n_sms ? total : n_sms, 64 + 32 * EW, Smem<BN, EW>::TOTAL, 1, tm_x, tm_w, tm_t, tm_bt, tm_y, a);
     BUMP(L);
     return e;
 }
@@ -874,7 +873,7 @@ static cudaError_t launch_gemm_pair(const Launch& L, const CUtensorMap& tm_x, co
     const int total = a.m_tiles * a.n_tiles;
     const int pairs = total < n_sms / 2 ? total : n_sms / 2;
     ProfScope ps(L, KC_GEMM);
-    cudaError_t e = launch_overlapped(lora_gemm_pair_kernel<BN, EPI, LNF, RESS>, 2 * pairs, P_THREADS, P_SMEM_TOTAL, L.st, 2,
+    cudaError_t e = launch_overlapped(L, lora_gemm_pair_kernel<BN, EPI, LNF, RESS>, 2 * pairs, P_THREADS, P_SMEM_TOTAL, 2,
                                       tm_x, tm_w, tm_t, tm_bt, tm_y, tm_res, a);
     BUMP(L);
     return e;

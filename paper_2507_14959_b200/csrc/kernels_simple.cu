@@ -771,7 +771,7 @@ cudaError_t launch_heads(const Launch& L, const T* x, int n_slots, int n_out_fra
         cudaError_t e = narrow ? grant1.ensure(heads_kernel<1>, smem) : grant2.ensure(heads_kernel<2>, smem);
         if (e != cudaSuccess) return e;
         if (a.base_blocks + adapter_blocks == 0) return cudaSuccess;
-        e = launch_overlapped(narrow ? heads_kernel<1> : heads_kernel<2>, a.base_blocks + adapter_blocks, 256, smem, L.st, 1, a);
+        e = launch_overlapped(L, narrow ? heads_kernel<1> : heads_kernel<2>, a.base_blocks + adapter_blocks, 256, smem, 1, a);
         BUMP(L);
         return e;
     } else {
@@ -998,7 +998,7 @@ cudaError_t launch_select(const Launch& L, const float* scores, int n_frames, in
     const int blocks = n_frames > 0 ? (n_frames + SELECT_THREADS / 32 - 1) / (SELECT_THREADS / 32) : 1;
     const int aw = (n_adapters + 63) / 64;     // at most 256 adapters
     auto kern = aw <= 1 ? select_kernel<1> : aw == 2 ? select_kernel<2> : aw == 3 ? select_kernel<3> : select_kernel<4>;
-    const cudaError_t e = launch_overlapped(kern, blocks, SELECT_THREADS, 0, L.st, 1, scores, n_frames, n_classes, n_adapters, thr, context_copy,
+    const cudaError_t e = launch_overlapped(L, kern, blocks, SELECT_THREADS, 0, 1, scores, n_frames, n_classes, n_adapters, thr, context_copy,
                                             has_prev, prev_labels, prev_off, prev_ids, first, provider,
                                             mask_scratch, next_off, next_ids, ids_capacity, L.status, metrics);
     BUMP(L);

@@ -467,8 +467,7 @@ cudaError_t launch(const Launch& L, const CUtensorMap& tm_x, const CUtensorMap& 
     static SmemGrant grant;
     if (cudaError_t e = grant.ensure(shrink_kernel<F, STATS, S>, a.ring_bytes + OTHER); e != cudaSuccess) return e;
     ProfScope ps(L, KC_SHRINK);
-    const cudaError_t e = launch_overlapped(shrink_kernel<F, STATS, S>, a.n_tiles * S, 32 * (FIRST_EW + F::EW), a.ring_bytes + OTHER,
-                                            L.st, S, tm_x, tm_at, a);
+    const cudaError_t e = launch_overlapped(L, shrink_kernel<F, STATS, S>, a.n_tiles * S, 32 * (FIRST_EW + F::EW), a.ring_bytes + OTHER, S, tm_x, tm_at, a);
     BUMP(L);
     return e;
 }

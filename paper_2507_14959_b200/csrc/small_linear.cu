@@ -571,7 +571,7 @@ cudaError_t launch(const Launch& L, const Maps& t, SmallArgs a, int tiles) {
     if (cudaError_t e = grant.ensure(small_linear_kernel<BN, EPI, LNF, S>, WORK + OTHER); e != cudaSuccess) return e;
     a.work_bytes = WORK;
     ProfScope ps(L, KC_GEMM);
-    const cudaError_t e = launch_overlapped(small_linear_kernel<BN, EPI, LNF, S>, tiles * S, THREADS, WORK + OTHER, L.st, S,
+    const cudaError_t e = launch_overlapped(L, small_linear_kernel<BN, EPI, LNF, S>, tiles * S, THREADS, WORK + OTHER, S,
                                             t.x, t.w, t.bt, t.at, a);
     BUMP(L);
     return e;
