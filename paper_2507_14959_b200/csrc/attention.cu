@@ -15,6 +15,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "f32x2.cuh"
 #include "tcgen05_ptx.cuh"
 
 #define BUMP(L) do { if ((L).launches) ++*(L).launches; } while (0)
@@ -178,23 +179,23 @@ __global__ void __launch_bounds__(512) attention_mma_kernel(const bf16* __restri
     }
 }
 // ---------------------------------------------------------------------------------------
-// tcgen05 attention.  One CTA per (frame, head); K and V of the head are brought in once by TMA
-// (128B swizzle), the query rows are taken 128 at a time:
+// tcgen05 attention.  K and V of a (frame, head) pair are brought in by TMA (128B swizzle), the query rows are taken
+// 128 at a time:
 //     S = Q K^T            UMMA 128 x nb x 16, four K steps, fp32 scores in tensor memory
-//     P = exp2(c (S - m))  four warps, one score row per thread (tcgen05.ld), written back over S
-//                          as packed bf16 (tcgen05.st), row sums kept in registers
+//     P = exp2(c (S - m))  one score row per thread (tcgen05.ld), written back over S as packed bf16 (tcgen05.st),
+//                          row sums kept in registers; m: see score_reference
 //     O = P V              UMMA 128 x 64 x 16 with the A operand read from tensor memory and V as
 //                          an MN-major shared-memory operand, one K step per 16 keys
 //     out = O / rowsum     tcgen05.ld, bf16, straight to global memory
-// Keys come in blocks of up to 208 (13 x 16).  With one block (up to 208 tokens) the row maximum
-// comes from the same scores.  With several blocks the scores are formed twice: a first sweep
-// yields each row's maximum over all keys, the second forms P against that final maximum and
-// accumulates O over the blocks, so no rescaling of O is ever needed.
-// Tensor memory holds two regions of scores (208 columns each) and O behind them; the issuing thread
-// forms the scores of the next step in the other region while the softmax warps sweep this one
-// (per region: one mbarrier "scores formed", one "scores consumed"), and issues a block's P V
-// product as soon as its probabilities are written.  ATT_SHARES softmax warps per lane quarter
-// split the key columns of a block; they exchange row maxima and row sums through shared memory.
+// Keys come in blocks of up to 208 (13 x 16).  attention_tc_kernel serves several key blocks: every block's scores are
+// formed once and taken relative to the row's first 16 scores, so O is never rescaled and no pass for the maxima is
+// needed.  One CTA per SM walks a contiguous range of (pair, query tile) units, keeping the pair's keys and values and
+// fetching the next query tile ahead.  Tensor memory holds two regions of scores (208 columns each) and O behind
+// them; the issuing thread forms the scores of the next step in the other region while the softmax warps sweep this
+// one (per region: one mbarrier "scores formed", one "probabilities written"), and issues a block's P V product as
+// soon as its probabilities are written.  ATT_SHARES softmax warps per lane quarter split the key columns of a
+// block; they exchange row sums through shared memory.
+// 16 frames of 577 tokens, 12 heads: 77.3 us with a pass for the maxima and a CTA per tile, 47.9 us now.
 // (One key block goes to the pipelined kernel further down.)
 // ---------------------------------------------------------------------------------------
 constexpr int AQ = 128;                    // query rows per tile
@@ -208,10 +209,11 @@ constexpr int AQ_BYTES = AQ * 128;
 constexpr int AKB_BYTES = AKB * 128;
 constexpr int ATT_MAX_BLOCKS = 3;
 
+constexpr uint32_t ATT_O_COL = 2 * AKB;    // tensor-memory columns: two regions of scores, O behind them
+
 struct AttnArgs {
-    int tokens, heads, tpad, n_blocks, n_qtiles;
-    int q_split;               // CTAs per (frame, head); each takes a contiguous share of the query tiles
-    uint32_t tmem_cols, o_col;
+    int tokens, heads, tpad, n_blocks, n_qtiles, n_units;
+    const bf16* qkv;
     bf16* out;
     int* status;
 };
@@ -232,38 +234,50 @@ __device__ __forceinline__ float ex2_approx(float x) {     // one MUFU instructi
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-// p_j = exp2(c s_j - mc) (0 beyond lim), packed to bf16 pairs; returns the sum of the p_j
+// p_j = exp2(c s_j - mc) (0 beyond lim), packed to bf16 pairs; adds the p_j to the two halves of sum
 template <int N, bool MASK>
-__device__ __forceinline__ float chunk_probs(const uint32_t* v, int lim, float c, float mc, uint32_t* packed) {
-    float sum[4] = {0.f, 0.f, 0.f, 0.f};                     // four independent chains
+__device__ __forceinline__ void chunk_probs(const uint32_t* v, int lim, uint64_t c2, uint64_t nmc2, uint32_t* packed, uint64_t& sum) {
+    uint64_t t[2] = {sum, pk2(0.f, 0.f)};                    // independent chains
 #pragma unroll
     for (int j = 0; j < N; j += 2) {
-        float p0 = ex2_approx(fmaf(__uint_as_float(v[j]), c, -mc));
-        float p1 = ex2_approx(fmaf(__uint_as_float(v[j + 1]), c, -mc));
+        float x0, x1;
+        upk2(fma2(pk2(__uint_as_float(v[j]), __uint_as_float(v[j + 1])), c2, nmc2), x0, x1);
+        float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
         if (MASK) { p0 = j < lim ? p0 : 0.f; p1 = j + 1 < lim ? p1 : 0.f; }
-        sum[(j >> 1) & 3] += p0 + p1;
+        t[(j >> 1) & 1] = add2(t[(j >> 1) & 1], pk2(p0, p1));
         packed[j >> 1] = pack2(p0, p1);
     }
-    return (sum[0] + sum[1]) + (sum[2] + sum[3]);
+    sum = add2(t[0], t[1]);
 }
 
-// Sweep over the score columns [0, ncols) that start at tensor-memory address t_s (ncols a multiple
-// of 16, `valid` of them real), 16 at a time with the next load in flight.  PROBS = false: running
-// row maximum.  PROBS = true: P (packed bf16, 8 columns per 16 scores) goes to t_p onwards and the
-// row sum of this range is added to acc.
-template <bool PROBS>
-__device__ __forceinline__ float score_range_sweep(uint32_t t_s, uint32_t t_p, int ncols, int valid, float c, float mc,
-                                                   float acc) {
+// What a row's exponentials are taken relative to: not the row's maximum but the maximum of its first 16 scores.
+// Softmax does not depend on the reference as long as nothing overflows (the reference is one of the scores, so the
+// largest term is at least 1), and this one needs 16 scores instead of a pass over all of them -- nor an exchange
+// between the warps that share a row: each reads those 16.  A row whose sum says that a score lies more than
+// about 100 / c = 550 above the reference (or is not a number) is computed again by attention_row_exact.
+__device__ __forceinline__ float score_reference(uint32_t t_s, int valid) {
+    uint32_t v[16];
+    tmem_ld16(t_s, v);
+    tmem_ld_wait();
+    return valid >= 16 ? chunk_max<16, false>(v, 16, -INFINITY) : chunk_max<16, true>(v, valid, -INFINITY);
+}
+constexpr float ROW_SUM_LIMIT = 1.2676506e30f;               // 2^100
+
+// Sweep over the score columns [0, ncols) that start at tensor-memory address t_s (ncols a multiple of 16, `valid` of
+// them real), 16 at a time with the next load in flight: P (packed bf16, 8 columns per 16 scores) goes to t_p onwards
+// and the row sum of this range is returned.  P of a piece is stored when the next piece has been loaded, so t_p may
+// lie up to 16 columns behind t_s.
+__device__ __forceinline__ float score_probs_sweep(uint32_t t_s, uint32_t t_p, int ncols, int valid, float c, float mc) {
     uint32_t va[16], vb[16];
+    const uint64_t c2 = pk2(c, c), nmc2 = pk2(-mc, -mc);
+    uint64_t sum = pk2(0.f, 0.f);
     auto piece = [&](const uint32_t* v, int c0) {
         const int lim = valid - c0;
-        if (PROBS) {
-            uint32_t pk[8];
-            acc += lim >= 16 ? chunk_probs<16, false>(v, 16, c, mc, pk) : chunk_probs<16, true>(v, lim, c, mc, pk);
-            tmem_st8(t_p + (uint32_t)(c0 >> 1), pk);
-        } else {
-            acc = lim >= 16 ? chunk_max<16, false>(v, 16, acc) : chunk_max<16, true>(v, lim, acc);
-        }
+        uint32_t pk[8];
+        if (lim >= 16) chunk_probs<16, false>(v, 16, c2, nmc2, pk, sum);
+        else chunk_probs<16, true>(v, lim, c2, nmc2, pk, sum);
+        tmem_ld_wait();
+        tmem_st8(t_p + (uint32_t)(c0 >> 1), pk);
     };
     tmem_ld16(t_s, va);
     tmem_ld_wait();
@@ -271,14 +285,40 @@ __device__ __forceinline__ float score_range_sweep(uint32_t t_s, uint32_t t_p, i
     for (int c0 = 0; c0 < ncols; c0 += 32) {
         if (c0 + 16 < ncols) tmem_ld16(t_s + (uint32_t)(c0 + 16), vb);
         piece(va, c0);
-        tmem_ld_wait();
         if (c0 + 16 < ncols) {
             if (c0 + 32 < ncols) tmem_ld16(t_s + (uint32_t)(c0 + 32), va);
             piece(vb, c0 + 16);
-            tmem_ld_wait();
         }
     }
-    return acc;
+    float lo, hi;
+    upk2(sum, lo, hi);
+    return lo + hi;
+}
+
+// One output row by one warp with the row's true maximum, straight from global memory: for the rows described above.
+// Two dimensions per lane, every score is formed twice.
+__device__ __noinline__ void attention_row_exact(const bf16* qkv, bf16* out, int tokens, int d, int f, int h, int q_row) {
+    const int lane = threadIdx.x & 31;
+    const float c = 0.125f * 1.4426950408889634f;
+    const bf16* row0 = qkv + (size_t)f * tokens * 3 * d + h * HD + 2 * lane;
+    const float2 q = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(row0 + (size_t)q_row * 3 * d));
+    auto score = [&](int j) {
+        const float2 k = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(row0 + (size_t)j * 3 * d + d));
+        float t = q.x * k.x + q.y * k.y;
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+        return t * c;
+    };
+    float m = -INFINITY;
+    for (int j = 0; j < tokens; ++j) m = fmaxf(m, score(j));
+    float l = 0.f, o0 = 0.f, o1 = 0.f;
+    for (int j = 0; j < tokens; ++j) {
+        const float p = ex2_approx(score(j) - m);
+        const float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(row0 + (size_t)j * 3 * d + 2 * d));
+        l += p;
+        o0 = fmaf(p, v.x, o0);
+        o1 = fmaf(p, v.y, o1);
+    }
+    *reinterpret_cast<uint32_t*>(out + ((size_t)f * tokens + q_row) * d + h * HD + 2 * lane) = pack2(o0 / l, o1 / l);
 }
 
 // Share k of `shares` takes the 16-key pieces [att_first(shares, k), att_first(shares, k + 1)) of a key
@@ -298,141 +338,135 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         if (threadIdx.x == 0) atomicCAS(args.status, 0, (int)PM_ERR_CUDA);
         return;
     }
-    const int fh = blockIdx.x / args.q_split, part = blockIdx.x % args.q_split;
-    const int f = fh / args.heads, h = fh % args.heads;
-    const int per = (args.n_qtiles + args.q_split - 1) / args.q_split;
-    const int qt0 = part * per, qt1 = min(args.n_qtiles, qt0 + per);          // this CTA's query tiles
+    // this CTA's query tiles: a contiguous range of all (pair, query tile) units, pair by pair
+    const int u0 = (int)((long long)args.n_units * blockIdx.x / gridDim.x), u1 = (int)((long long)args.n_units * (blockIdx.x + 1) / gridDim.x);
     const int d = args.heads * HD;
     const int T = args.tokens;
     const int n_blocks = args.n_blocks;
-    const uint32_t q_s = base;
-    const uint32_t k_s = q_s + AQ_BYTES;
+    auto q_s = [&](int u) { return base + (uint32_t)((u - u0) & 1) * AQ_BYTES; };       // two query tiles in turn
+    const uint32_t k_s = base + 2 * AQ_BYTES;
     const uint32_t v_s = k_s + n_blocks * AKB_BYTES;
     const uint32_t bars = v_s + n_blocks * AKB_BYTES;
-    // barriers: operands landed (kv, q); scores of a step formed, per score region (s_bar[2]); a step's scores
-    // consumed by all softmax warps -- maxima taken, or probabilities written (c_bar[2]); O complete (o_bar);
-    // O read out (ofree_bar); the shares' row maxima / row sums exchanged (max_bar, sum_bar)
-    const uint32_t q_bar = bars + 8, o_bar = bars + 48, ofree_bar = bars + 56;
-    auto k_bar = [&](int b) { return bars + 96u + 8u * (uint32_t)b; };       // key block b landed
-    auto v_bar = [&](int b) { return bars + 120u + 8u * (uint32_t)b; };      // value block b landed
-    const uint32_t max_bar = bars + 64, sum_bar = bars + 72;
-    auto s_bar = [&](uint32_t r) { return bars + 16u + 8u * r; };
-    auto c_bar = [&](uint32_t r) { return bars + 32u + 8u * r; };
+    // barriers: scores of a step formed, per score region (s_bar[2]); a step's probabilities written by all softmax
+    // warps (c_bar[2]); O complete (o_bar); O read out (ofree_bar); the shares' row sums exchanged (sum_bar);
+    // operands landed (q_bar[2], k_bar, v_bar)
+    auto s_bar = [&](uint32_t r) { return bars + 8u * r; };
+    auto c_bar = [&](uint32_t r) { return bars + 16u + 8u * r; };
+    const uint32_t o_bar = bars + 32, ofree_bar = bars + 40, sum_bar = bars + 48;
+    auto q_bar = [&](int u) { return bars + 56u + 8u * (uint32_t)((u - u0) & 1); };
+    auto k_bar = [&](int b) { return bars + 72u + 8u * (uint32_t)b; };       // key block b landed
+    auto v_bar = [&](int b) { return bars + 96u + 8u * (uint32_t)b; };       // value block b landed
     uint8_t* bar_ptr = smem_raw + (bars - base);
-    float* xchg = reinterpret_cast<float*>(bar_ptr + 160);       // [max | sum][share][row]
+    float* sums_base = reinterpret_cast<float*>(bar_ptr + 160);  // two tiles in turn: [share][row]
     constexpr int shares = SHARES;
-    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(bar_ptr + 80);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_ptr + 88);
+    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(bar_ptr + 128);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_ptr + 136);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // score steps of one query tile: with several key blocks the scores are formed twice (all of a row's
-    // maxima must be known before its first exponential, and tensor memory holds two blocks of scores
-    // beside O, not three): steps 0 .. n_blocks-1 for the maxima, n_blocks .. 2 n_blocks-1 for the
-    // probabilities.  Step s of the CTA (all tiles) uses score region s % 2.
-    const int n_steps = n_blocks > 1 ? 2 * n_blocks : 1;
 
     if (threadIdx.x == 0) {
-        mbar_init(q_bar, 1);
         for (int b = 0; b < ATT_MAX_BLOCKS; ++b) { mbar_init(k_bar(b), 1); mbar_init(v_bar(b), 1); }
-        for (uint32_t r = 0; r < 2; ++r) { mbar_init(s_bar(r), 1); mbar_init(c_bar(r), 4 * shares); }
+        for (uint32_t r = 0; r < 2; ++r) { mbar_init(s_bar(r), 1); mbar_init(c_bar(r), 4 * shares); mbar_init(q_bar(u0 + (int)r), 1); }
         mbar_init(o_bar, 1); mbar_init(ofree_bar, 4 * shares);
-        mbar_init(max_bar, 4 * shares); mbar_init(sum_bar, 4 * shares);
+        mbar_init(sum_bar, 4 * shares);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        dep_wait();                            // everything else follows from what these loads bring
-        // all operand loads of the head go out before tensor memory is requested, in the order of their
-        // first use and each block on a barrier of its own: the first scores need the query tile and the
-        // first key block only
-        mbar_expect_tx(q_bar, AQ_BYTES);
-        tma_load_2d(q_s, &tm_q, h * HD, f * T + qt0 * AQ, q_bar);
-        for (int b = 0; b < n_blocks; ++b) {
-            mbar_expect_tx(k_bar(b), (uint32_t)AKB_BYTES);
-            tma_load_2d(k_s + b * AKB_BYTES, &tm_kv, d + h * HD, f * T + b * AKB, k_bar(b));
-        }
-        for (int b = 0; b < n_blocks; ++b) {
-            mbar_expect_tx(v_bar(b), (uint32_t)AKB_BYTES);
-            tma_load_2d(v_s + b * AKB_BYTES, &tm_kv, 2 * d + h * HD, f * T + b * AKB, v_bar(b));
-        }
     }
     __syncwarp();
     if (warp == 0) {
-        tmem_alloc(smem_u32((const void*)tmem_slot), args.tmem_cols);
+        tmem_alloc(smem_u32((const void*)tmem_slot), 512);
         tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    const uint32_t o_tmem = tmem_base + args.o_col;
+    const uint32_t o_tmem = tmem_base + ATT_O_COL;
     dep_release();
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (lane == 0 && u0 < u1) {
             // ------------------------------------------------------ TMA + MMA issue
-            // The scores of step s + 1 are formed in the other region while the softmax warps are at step s;
-            // products issued by this thread run in issue order, so a region's P V product is through
-            // before the scores that are issued after it overwrite the region.
+            // Steps run over all tiles: key block g % n_blocks of tile u0 + g / n_blocks.  The scores of step g + 1 are formed
+            // in the other region while the softmax warps are at step g; products issued by this thread run in issue
+            // order, so a region's P V product is through before the scores issued after it overwrite the region.
             const uint32_t idesc_pv = instr_desc_b_mn(HD);
             // descriptors built once; a K step adds 2 (32 B) for Q / K and 128 (2048 B) for V
-            const uint64_t dq0 = smem_desc(q_s, 128), dk0 = smem_desc(k_s, 128), dv0 = smem_desc(v_s, 128);
-            uint32_t s = 0;                                      // score steps issued so far
+            const uint64_t dk0 = smem_desc(k_s, 128), dv0 = smem_desc(v_s, 128);
             bool ok = true;
-            auto issue_scores = [&](int i) {                     // step i of the tile: key block i % n_blocks
-                const int b = i % n_blocks;
-                const uint32_t r = s & 1u;
-                // the region's previous scores (step s - 2) must have been consumed
-                ok = mbar_wait(c_bar(r), ((s >> 1) & 1u) ^ 1u, abort_flag, args.status);
-                if (ok && s < (uint32_t)n_blocks) ok = mbar_wait(k_bar(b), 0, abort_flag, args.status);   // a block's first use
+            int pair = u0 / args.n_qtiles, loads = 0;            // the pair whose keys and values are here; how often they were brought
+            auto load_q = [&](int u) {
+                const int fh = u / args.n_qtiles, f = fh / args.heads, h = fh % args.heads;
+                mbar_expect_tx(q_bar(u), AQ_BYTES);
+                tma_load_2d(q_s(u), &tm_q, h * HD, f * T + (u % args.n_qtiles) * AQ, q_bar(u));
+            };
+            auto load_kv = [&](int which, uint32_t to, auto bar) {             // which: 1 keys, 2 values
+                const int f = pair / args.heads, h = pair % args.heads;
+                for (int b = 0; b < n_blocks; ++b) {
+                    mbar_expect_tx(bar(b), (uint32_t)AKB_BYTES);
+                    tma_load_2d(to + b * AKB_BYTES, &tm_kv, which * d + h * HD, f * T + b * AKB, bar(b));
+                }
+            };
+            dep_wait();                                          // everything else follows from what these loads bring
+            load_q(u0);
+            load_kv(1, k_s, k_bar);
+            load_kv(2, v_s, v_bar);
+            if (u0 + 1 < u1) load_q(u0 + 1);
+            const uint32_t n_steps = (uint32_t)((u1 - u0) * n_blocks);
+            auto issue_scores = [&](uint32_t g) {
+                const int b = (int)g % n_blocks, u = u0 + (int)g / n_blocks;
+                const uint32_t r = g & 1u;
+                // the region's previous scores (step g - 2) must have been consumed
+                ok = mbar_wait(c_bar(r), ((g >> 1) & 1u) ^ 1u, abort_flag, args.status);
+                if (ok && b == 0) ok = mbar_wait(q_bar(u), (uint32_t)((u - u0) >> 1) & 1u, abort_flag, args.status);
+                if (ok) ok = mbar_wait(k_bar(b), (uint32_t)loads & 1u, abort_flag, args.status);
                 if (!ok) return;
                 tc_fence_after();
-                const int nb = min(AKB, args.tpad - b * AKB);
-                const uint32_t idesc_s = instr_desc(nb);
-                const uint64_t bo = (uint64_t)((b * AKB_BYTES) >> 4);
+                const uint32_t idesc_s = instr_desc(min(AKB, args.tpad - b * AKB));
+                const uint64_t dq = smem_desc(q_s(u), 128), bo = (uint64_t)((b * AKB_BYTES) >> 4);
 #pragma unroll
                 for (int k = 0; k < HD / 16; ++k)
-                    umma_bf16(tmem_base + r * (uint32_t)AKB, dq0 + 2 * k, dk0 + bo + 2 * k, idesc_s, k > 0);
+                    umma_bf16(tmem_base + r * (uint32_t)AKB, dq + 2 * k, dk0 + bo + 2 * k, idesc_s, k > 0);
                 umma_commit(s_bar(r));
-                ++s;
             };
-            for (int qt = qt0; qt < qt1 && ok; ++qt) {
-                ok = mbar_wait(q_bar, (qt - qt0) & 1, abort_flag, args.status);
+            issue_scores(0);
+            for (uint32_t g = 0; g < n_steps && ok; ++g) {
+                const int b = (int)g % n_blocks, u = u0 + (int)g / n_blocks;
+                const uint32_t r = g & 1u;
+                const bool last = b == n_blocks - 1;
+                const bool new_pair = last && g + 1 < n_steps && (u + 1) / args.n_qtiles != pair;
+                if (!new_pair && g + 1 < n_steps) issue_scores(g + 1);
+                // the step's probabilities are written (so its scores, the tile's last ones included, exist)
+                ok = ok && mbar_wait(c_bar(r), (g >> 1) & 1u, abort_flag, args.status);
+                if (ok) ok = mbar_wait(v_bar(b), (uint32_t)loads & 1u, abort_flag, args.status);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t s0 = s;                           // the tile's first step
-                issue_scores(0);
-                for (int i = 0; i < n_steps && ok; ++i) {
-                    if (i + 1 < n_steps) issue_scores(i + 1);
-                    if (!ok) break;
-                    if (n_blocks > 1 && i < n_blocks) continue;  // a step for the maxima: nothing to multiply
-                    const int b = i % n_blocks;
-                    const uint32_t si = s0 + (uint32_t)i, r = si & 1u;
-                    // the step's probabilities are written (so its scores, the tile's last ones included, exist)
-                    ok = mbar_wait(c_bar(r), (si >> 1) & 1u, abort_flag, args.status);
-                    if (ok && qt == qt0) ok = mbar_wait(v_bar(b), 0, abort_flag, args.status);          // a block's first use
+                if (last && u + 2 < u1) load_q(u + 2);           // this tile's query rows are no longer needed
+                if (new_pair) { ++pair; load_kv(1, k_s, k_bar); }            // nor the pair's keys
+                if (b == 0 && u > u0) {
+                    // the first product of a tile overwrites O: the previous tile's must have been read out
+                    ok = mbar_wait(ofree_bar, (uint32_t)(u - u0 - 1) & 1u, abort_flag, args.status);
                     if (!ok) break;
                     tc_fence_after();
-                    if (b == n_blocks - 1 && qt + 1 < qt1) {
-                        // the query rows are no longer needed: fetch the next tile's behind the P V products
-                        mbar_expect_tx(q_bar, AQ_BYTES);
-                        tma_load_2d(q_s, &tm_q, h * HD, f * T + (qt + 1) * AQ, q_bar);
-                    }
-                    if (b == 0 && qt > qt0) {
-                        // the first product of a tile overwrites O: the previous tile's must have been read out
-                        ok = mbar_wait(ofree_bar, (uint32_t)(qt - qt0 - 1) & 1u, abort_flag, args.status);
-                        if (!ok) break;
-                        tc_fence_after();
-                    }
-                    const int nb = min(AKB, args.tpad - b * AKB);
-                    const uint64_t bo = (uint64_t)((b * AKB_BYTES) >> 4);
-                    // P of piece kk sits where its share left it: at the start of that share's columns
-                    uint32_t p_col = 0;
-                    for (int kk = 0; kk < nb / 16; ++kk) {
-                        if (kk == att_first(shares, 1) || kk == att_first(shares, 2)) p_col = (uint32_t)(kk * 16);
-                        umma_bf16_ts(o_tmem, tmem_base + r * (uint32_t)AKB + p_col, dv0 + bo + 128 * kk, idesc_pv,
-                                     (b > 0 || kk > 0) ? 1u : 0u);
-                        p_col += 8;
-                    }
-                    if (b == n_blocks - 1) umma_commit(o_bar);
+                }
+                const int pieces = min(AKB, args.tpad - b * AKB) / 16;
+                const uint64_t bo = (uint64_t)((b * AKB_BYTES) >> 4);
+                // P of piece kk sits where its share left it: the first share's from column 16 on (columns 0..15 of a tile's
+                // first block are everybody's reference), the others' at the start of their own columns
+                uint32_t p_col = 16;
+                for (int kk = 0; kk < pieces; ++kk) {
+                    if (kk > 0 && (kk == att_first(shares, 1) || kk == att_first(shares, 2))) p_col = (uint32_t)(kk * 16);
+                    umma_bf16_ts(o_tmem, tmem_base + r * (uint32_t)AKB + p_col, dv0 + bo + 128 * kk, idesc_pv, (b > 0 || kk > 0) ? 1u : 0u);
+                    p_col += 8;
+                }
+                if (last) umma_commit(o_bar);
+                if (new_pair) {
+                    ++loads;
+                    // the values are free once the tile's O is complete
+                    ok = mbar_wait(o_bar, (uint32_t)(u - u0) & 1u, abort_flag, args.status);
+                    if (!ok) break;
+                    load_kv(2, v_s, v_bar);
+                    issue_scores(g + 1);
                 }
             }
         }
@@ -443,56 +477,37 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         const int row = quarter * 32 + lane;
         const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16);
         const float c = 0.125f * 1.4426950408889634f;            // 1/sqrt(64) * log2(e)
-        float* maxes = xchg;                                     // [share][row]
-        float* sums = xchg + ATT_MAX_SHARES * AQ;
-        uint32_t s = 0, tile_no = 0;
+        uint32_t g = 0;
         bool ok = true;
-        // this warp's columns of key block b: [col0, col0 + ncols), `valid` of them real
-        auto my_cols = [&](int b, int& col0, int& ncols, int& valid) {
-            const int np = min(AKB, args.tpad - b * AKB) / 16;
-            const int p0 = min(att_first(shares, share), np), p1 = min(att_first(shares, share + 1), np);
-            col0 = p0 * 16; ncols = (p1 - p0) * 16; valid = T - b * AKB - col0;
-        };
-        for (int qt = qt0; qt < qt1 && ok; ++qt, ++tile_no) {
+        for (int u = u0; u < u1 && ok; ++u) {
+            const uint32_t par = (uint32_t)(u - u0) & 1u;
+            float* sums = sums_base + par * ATT_MAX_SHARES * AQ;
+            const int fh = u / args.n_qtiles, qt = u % args.n_qtiles, f = fh / args.heads, h = fh % args.heads;
             const int q_row = qt * AQ + row;
             const bool warp_active = qt * AQ + quarter * 32 < T;      // else: no row of this warp exists
-            float m = -INFINITY, l = 0.f;
-            int col0, ncols, valid;
-            for (int i = 0; i < n_steps; ++i, ++s) {
-                const int b = i % n_blocks;
-                const bool probs = n_blocks == 1 || i >= n_blocks;
-                const uint32_t r = s & 1u;
-                ok = mbar_wait(s_bar(r), (s >> 1) & 1u, abort_flag, args.status);
+            float mc = 0.f, l = 0.f;
+            for (int b = 0; b < n_blocks; ++b, ++g) {
+                const uint32_t r = g & 1u;
+                ok = mbar_wait(s_bar(r), (g >> 1) & 1u, abort_flag, args.status);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t t_s = t_lane + r * (uint32_t)AKB;
-                my_cols(b, col0, ncols, valid);
-                if (!probs || n_blocks == 1) {
-                    if (warp_active && ncols > 0)
-                        m = score_range_sweep<false>(t_s + (uint32_t)col0, 0u, ncols, valid, 0.f, 0.f, m);
-                }
-                if (probs) {
-                    if (b == 0 && shares > 1) {
-                        // the row maximum over all keys: every share's part, through shared memory
-                        maxes[share * AQ + row] = m;
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(max_bar);
-                        ok = mbar_wait(max_bar, tile_no & 1u, abort_flag, args.status);
-                        ok = __all_sync(0xFFFFFFFFu, ok);
-                        if (!ok) break;
-#pragma unroll
-                        for (int k = 0; k < shares; ++k) m = fmaxf(m, maxes[k * AQ + row]);
-                    }
-                    if (warp_active && ncols > 0) {
-                        l = score_range_sweep<true>(t_s + (uint32_t)col0, t_s + (uint32_t)col0, ncols, valid, c, m * c, l);
+                // this warp's columns of key block b
+                const int np = min(AKB, args.tpad - b * AKB) / 16;
+                const int p0 = min(att_first(shares, share), np), p1 = min(att_first(shares, share + 1), np);
+                if (warp_active) {
+                    if (b == 0) mc = score_reference(t_s, T) * c;
+                    if (p1 > p0) {
+                        const uint32_t at = t_s + (uint32_t)(p0 * 16);
+                        l += score_probs_sweep(at, share == 0 ? at + 16u : at, (p1 - p0) * 16, T - b * AKB - p0 * 16, c, mc);
                         tmem_st_wait();
                     }
-                    if (shares > 1 && b == n_blocks - 1) {
-                        sums[share * AQ + row] = l;
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(sum_bar);
-                    }
+                }
+                if (b == n_blocks - 1 && shares > 1) {
+                    sums[share * AQ + row] = l;
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(sum_bar);
                 }
                 tc_fence_before();
                 __syncwarp();
@@ -500,7 +515,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             }
             if (!ok) break;
             if (shares > 1) {
-                ok = mbar_wait(sum_bar, tile_no & 1u, abort_flag, args.status);
+                ok = mbar_wait(sum_bar, par, abort_flag, args.status);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
                 l = 0.f;
@@ -508,41 +523,43 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 for (int k = 0; k < shares; ++k) l += sums[k * AQ + row];
             }
             // O = sum over the key blocks of P V is complete: the finished rows are written out
-            ok = mbar_wait(o_bar, tile_no & 1u, abort_flag, args.status);
+            ok = mbar_wait(o_bar, par, abort_flag, args.status);
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
             tc_fence_after();
-            {
-                // the output columns are split between the first two shares (all 64 to the only one)
-                const int ocols = shares == 1 ? 64 : 32;
-                if (warp_active && share * ocols < 64) {
-                    const float inv = 1.f / l;
-                    bf16* orow = args.out + ((size_t)f * T + q_row) * d + h * HD + share * ocols;
-                    for (int part = 0; part < ocols / 32; ++part) {
-                        uint32_t v[32];
-                        tmem_ld32((t_lane + args.o_col) + (uint32_t)(share * ocols + part * 32), v);
-                        tmem_ld_wait();
-                        if (q_row < T) {
-                            // 32-byte stores: one full sector per row per instruction
+            // the output columns are split between the first two shares (all 64 to the only one)
+            constexpr int OCOLS = shares == 1 ? 64 : 32;
+            uint32_t v[OCOLS];
+            const bool writes = warp_active && share * OCOLS < 64;
+            if (writes) {
 #pragma unroll
-                            for (int q = 0; q < 2; ++q) {
-                                uint32_t o[8];
-#pragma unroll
-                                for (int e = 0; e < 8; ++e)
-                                    o[e] = pack2(__uint_as_float(v[q * 16 + 2 * e]) * inv,
-                                                 __uint_as_float(v[q * 16 + 2 * e + 1]) * inv);
-                                asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                                             ::"l"(orow + part * 32 + q * 16), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]),
-                                               "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7])
-                                             : "memory");
-                            }
-                        }
-                    }
-                }
+                for (int part = 0; part < OCOLS / 32; ++part) tmem_ld32(t_lane + ATT_O_COL + (uint32_t)(share * OCOLS + part * 32), v + part * 32);
+                tmem_ld_wait();
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(ofree_bar);
+            if (lane == 0) mbar_arrive(ofree_bar);               // O is in registers: the next tile's products may start
+            if (writes) {
+                const float inv = 1.f / l;
+                bf16* orow = args.out + ((size_t)f * T + q_row) * d + h * HD + share * OCOLS;
+                if (q_row < T && l < ROW_SUM_LIMIT) {
+                    // 32-byte stores: one full sector per row per instruction
+#pragma unroll
+                    for (int q = 0; q < OCOLS / 16; ++q) {
+                        uint32_t o[8];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            o[e] = pack2(__uint_as_float(v[q * 16 + 2 * e]) * inv, __uint_as_float(v[q * 16 + 2 * e + 1]) * inv);
+                        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                                     ::"l"(orow + q * 16), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]),
+                                       "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7])
+                                     : "memory");
+                    }
+                }
+                if (share == 0)
+                    for (uint32_t redo = __ballot_sync(0xFFFFFFFFu, q_row < T && !(l < ROW_SUM_LIMIT)); redo; redo &= redo - 1)
+                        attention_row_exact(args.qkv, args.out, T, d, f, h, qt * AQ + quarter * 32 + __ffs((int)redo) - 1);
+            }
         }
     }
 
@@ -556,7 +573,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, args.tmem_cols);
+        tmem_dealloc(tmem_base, 512);
     }
 }
 
@@ -571,21 +588,23 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 // so the tensor pipe, the two softmax groups and the loads of the following items overlap inside one
 // CTA.  Two warps share each quarter of the 128 rows (a warp reaches the tensor-memory lanes
 // 32 (w mod 4) .. +31 only) and split the key columns: the first seven 16-key pieces and the rest.
-// The sweeps are chains of dependent operations, so what bounds them is how many warps a scheduler
-// can switch between: four per scheduler here against two with one warp per quarter.  The halves
-// exchange their row maxima and row sums through shared memory (mbarriers, bounded waits).
-// Column map of a tile's 256-column slot: scores 0..207; P of the first half over 0..55, P of the
-// second half in 208..255 (so that it never lands on scores the first half still reads); O in
-// 128..191 once both halves are done.  Tile c of a CTA is query tile c % nq of its item c / nq.
+// The sweeps are chains of dependent operations, so what bounds them is how many warps a scheduler can switch between
+// -- four per scheduler here against two with one warp per quarter -- and how many sweeps a tile needs: one (see
+// score_reference; with a sweep for the row maxima and their exchange in front of it, 256 frames of 197 tokens, 12 heads: 99.6 us, now 86.6).
+// The halves exchange their row sums through shared memory (mbarriers, bounded waits).
+// Column map of a tile's 256-column slot: scores 0..207; P of the first half over 16..71 (the first 16 columns stay:
+// both halves read their reference there), P of the second half in 208..255 (so that it never lands on scores the
+// first half still reads); O in 128..191 once both halves are done.  Tile c of a CTA is query tile c % nq of its item c / nq.
 // ---------------------------------------------------------------------------------------
 constexpr int APIPE_GROUP_WARPS = 8;
 constexpr int APIPE_THREADS = 64 + 2 * 32 * APIPE_GROUP_WARPS;      // 576
 constexpr int APIPE_ITEM_BYTES = 2 * AKB_BYTES + 2 * AQ_BYTES;      // K, V, two query tiles
 constexpr int APIPE_SPLIT = 7;                                       // 16-key pieces of the first half
-constexpr int APIPE_XCHG_BYTES = 2 * 2 * 2 * AQ * 4;                 // [max | sum][group][half][row]
+constexpr int APIPE_XCHG_BYTES = 2 * 2 * AQ * 4;                     // row sums [group][half][row]
 
 struct AttnPipeArgs {
     int tokens, heads, tpad, nq, n_items;
+    const bf16* qkv;
     bf16* out;
     int* status;
 };
@@ -614,7 +633,6 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     auto p_ready = [&](int sl) { return bars + 48u + 8u * sl; };
     auto o_ready = [&](int sl) { return bars + 64u + 8u * sl; };
     auto slot_free = [&](int sl) { return bars + 80u + 8u * sl; };
-    auto max_bar = [&](int sl) { return bars + 96u + 8u * sl; };
     auto sum_bar = [&](int sl) { return bars + 112u + 8u * sl; };
     uint8_t* bar_ptr = smem_raw + (bars - base);
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(bar_ptr + 128);
@@ -626,7 +644,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             mbar_init(kv_full(i), 1); mbar_init(buf_free(i), 1);
             mbar_init(s_ready(i), 1); mbar_init(p_ready(i), APIPE_GROUP_WARPS);
             mbar_init(o_ready(i), 1); mbar_init(slot_free(i), APIPE_GROUP_WARPS);
-            mbar_init(max_bar(i), APIPE_GROUP_WARPS); mbar_init(sum_bar(i), APIPE_GROUP_WARPS);
+            mbar_init(sum_bar(i), APIPE_GROUP_WARPS);
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -674,7 +692,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 const uint32_t s_tmem = tmem_base + (uint32_t)(slot * 256);
                 const uint64_t dv0 = smem_desc(v_s(buf), 128);
                 for (int kk = 0; kk < n_pieces; ++kk) {
-                    const uint32_t p_col = kk < split ? (uint32_t)(kk * 8) : (uint32_t)(208 + (kk - split) * 8);
+                    const uint32_t p_col = kk < split ? (uint32_t)(16 + kk * 8) : (uint32_t)(208 + (kk - split) * 8);
                     umma_bf16_ts(s_tmem + 128u, s_tmem + p_col, dv0 + 128 * kk, idesc_pv, kk > 0 ? 1u : 0u);
                 }
                 umma_commit(o_ready(slot));
@@ -705,11 +723,9 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(group * 256);
         const int col0 = half == 0 ? 0 : split * 16;             // first key column of this warp
         const int ncols = half == 0 ? split * 16 : (n_pieces - split) * 16;
-        const uint32_t t_p = t_lane + (half == 0 ? 0u : 208u);   // where this warp's P goes
-        float* my_max = xchg + ((0 * 2 + group) * 2 + half) * AQ;
-        float* other_max = xchg + ((0 * 2 + group) * 2 + (half ^ 1)) * AQ;
-        float* my_sum = xchg + ((1 * 2 + group) * 2 + half) * AQ;
-        float* other_sum = xchg + ((1 * 2 + group) * 2 + (half ^ 1)) * AQ;
+        const uint32_t t_p = t_lane + (half == 0 ? 16u : 208u);  // where this warp's P goes
+        float* my_sum = xchg + (group * 2 + half) * AQ;
+        float* other_sum = xchg + (group * 2 + (half ^ 1)) * AQ;
         const float c_ = 0.125f * 1.4426950408889634f;           // 1/sqrt(64) * log2(e)
         bool ok = true;
         for (int c = group; c < my_tiles && ok; c += 2) {
@@ -723,20 +739,10 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
             tc_fence_after();
-            // row maximum: own columns, then the other half's through shared memory
-            float m = -INFINITY;
-            if (warp_active && ncols > 0)
-                m = score_range_sweep<false>(t_lane + (uint32_t)col0, 0u, ncols, T - col0, 0.f, 0.f, m);
-            my_max[row] = m;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(max_bar(group));
-            ok = mbar_wait(max_bar(group), par, abort_flag, args.status);
-            ok = __all_sync(0xFFFFFFFFu, ok);
-            if (!ok) break;
-            m = fmaxf(m, other_max[row]);
             float l = 0.f;
-            if (warp_active && ncols > 0) {
-                l = score_range_sweep<true>(t_lane + (uint32_t)col0, t_p, ncols, T - col0, c_, m * c_, 0.f);
+            if (warp_active) {
+                const float mc = score_reference(t_lane, T) * c_;    // columns 0..15: no P is written there
+                if (ncols > 0) l = score_probs_sweep(t_lane + (uint32_t)col0, t_p, ncols, T - col0, c_, mc);
                 tmem_st_wait();
             }
             my_sum[row] = l;
@@ -758,7 +764,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 uint32_t v[32];
                 tmem_ld32((t_lane + 128u) + (uint32_t)(half * 32), v);
                 tmem_ld_wait();
-                if (q_row < T) {
+                if (q_row < T && l < ROW_SUM_LIMIT) {
 #pragma unroll
                     for (int q = 0; q < 2; ++q) {
                         uint32_t o[8];
@@ -772,6 +778,9 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                                      : "memory");
                     }
                 }
+                if (half == 0)
+                    for (uint32_t redo = __ballot_sync(0xFFFFFFFFu, q_row < T && !(l < ROW_SUM_LIMIT)); redo; redo &= redo - 1)
+                        attention_row_exact(args.qkv, args.out, T, d, f, h, qt * AQ + quarter * 32 + __ffs((int)redo) - 1);
             }
             tc_fence_before();
             __syncwarp();
@@ -982,13 +991,8 @@ cudaError_t launch_attention_tc(const Launch& L, const CUtensorMap& tm_q, const 
     a.tpad = (tokens + 15) / 16 * 16;
     a.n_blocks = (a.tpad + AKB - 1) / AKB;
     a.n_qtiles = (tokens + AQ - 1) / AQ;
-    // one key block: a CTA per head (three fit an SM).  Several key blocks: one CTA per SM, so each
-    // head's query tiles are spread over several CTAs when there are too few heads to fill the GPU.
-    a.q_split = (a.n_blocks > 1 && n_frames * heads < 4 * 148) ? a.n_qtiles : 1;
-    // two regions of scores (208 columns each), O behind them
-    a.tmem_cols = 512u;
-    a.o_col = 2u * AKB;
-    a.out = out; a.status = L.status;
+    a.n_units = n_frames * heads * a.n_qtiles;
+    a.qkv = qkv; a.out = out; a.status = L.status;
     // up to a third as many (frame, head) pairs as SMs: 12 pairs of 197 tokens 4.4 against 7.6 us, 48 pairs 7.6 against 7.7, 72
     // pairs 9.8 against 7.8; 65 tokens: 48 pairs 3.9 against 4.6, 96 pairs 5.7 against 4.8
     const int row_tiles = (tokens + AFEW_ROWS - 1) / AFEW_ROWS;
@@ -1005,7 +1009,7 @@ cudaError_t launch_attention_tc(const Launch& L, const CUtensorMap& tm_q, const 
         // one key block: the pipelined persistent kernel
         AttnPipeArgs pa;
         pa.tokens = tokens; pa.heads = heads; pa.tpad = a.tpad; pa.nq = a.n_qtiles;
-        pa.n_items = n_frames * heads; pa.out = out; pa.status = L.status;
+        pa.n_items = n_frames * heads; pa.qkv = qkv; pa.out = out; pa.status = L.status;
         const size_t psmem = 2 * (size_t)APIPE_ITEM_BYTES + APIPE_XCHG_BYTES + 192;
         static SmemGrant grant;
         if (cudaError_t e = grant.ensure(attention_pipe_kernel, (int)psmem); e != cudaSuccess) return e;
@@ -1015,12 +1019,12 @@ cudaError_t launch_attention_tc(const Launch& L, const CUtensorMap& tm_q, const 
         return e;
     }
     // all of tensor memory and most of the shared memory: one CTA per SM
-    size_t smem = (size_t)AQ_BYTES + (size_t)a.n_blocks * 2 * AKB_BYTES + 160 + 2 * ATT_MAX_SHARES * AQ * sizeof(float);
+    const size_t smem = 2 * (size_t)AQ_BYTES + (size_t)a.n_blocks * 2 * AKB_BYTES + 160 + 2 * ATT_MAX_SHARES * AQ * sizeof(float);
     static SmemGrant grant;
     if (cudaError_t e = grant.ensure(attention_tc_kernel<ATT_SHARES>, (int)smem); e != cudaSuccess) return e;
     ProfScope ps(L, KC_ATTENTION);
-    cudaError_t e = launch_overlapped(L, attention_tc_kernel<ATT_SHARES>, n_frames * heads * a.q_split, 32 + 128 * ATT_SHARES, smem, 1,
-                                      tm_q, tm_kv, a);
+    cudaError_t e = launch_overlapped(L, attention_tc_kernel<ATT_SHARES>, n_sms > 0 ? std::min(a.n_units, n_sms) : a.n_units, 32 + 128 * ATT_SHARES,
+                                      smem, 1, tm_q, tm_kv, a);
     BUMP(L);
     return e;
 }

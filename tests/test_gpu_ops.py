@@ -348,3 +348,25 @@ def test_attention_of_one_key_block_on_both_sides_of_the_pair_limit(frames, toke
     for f in sorted({0, frames // 2, frames - 1}):
         want = po.attention(qkv[f * tokens:(f + 1) * tokens].astype(np.float64), heads)
         np.testing.assert_allclose(got[f * tokens:(f + 1) * tokens], want, **TOL[0])
+
+
+@pytest.mark.parametrize("frames,tokens,heads", [(18, 197, 3), (1, 300, 2), (2, 577, 1)])
+def test_attention_rows_whose_first_scores_are_far_below_the_largest(frames, tokens, heads):
+    """The tensor-memory kernels take a row's exponentials relative to the maximum of its first 16 scores; a row with a
+    score far above it is computed again with its true maximum.  Here keys 0..15 are zero and a later key of every row
+    in the first frame's first head scores about 2000, in the last frame's last head moderate scores stay as they are: both
+    kinds of rows against the oracle, in one launch."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    d = heads * 64
+    qkv = wl.normal((frames * tokens, 3 * d), 1.0, "attn_gpu_far", frames, tokens, heads)
+    qkv[:tokens, :64] = 16.0                                   # queries of frame 0, head 0
+    qkv[:16, d:d + 64] = 0.0                                   # its keys 0..15
+    qkv[tokens - 40, d:d + 64] = 16.0                          # score 16 * 16 * 64 / 8 = 2048
+    od = torch.full((frames * tokens, d), float("nan"), device="cuda", dtype=torch.bfloat16)
+    binding.attention(to_dev(qkv, 0), od, frames, tokens, heads, 0)
+    torch.cuda.synchronize()
+    got = to_np(od)
+    for f in sorted({0, frames - 1}):
+        want = po.attention(qkv[f * tokens:(f + 1) * tokens].astype(np.float64), heads)
+        np.testing.assert_allclose(got[f * tokens:(f + 1) * tokens], want, **TOL[0])
