@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(512) attention_mma_kernel(const bf16* __restri
 // one (per region: one mbarrier "scores formed", one "probabilities written"), and issues a block's P V product as
 // soon as its probabilities are written.  ATT_SHARES softmax warps per lane quarter split the key columns of a
 // block; they exchange row sums through shared memory.
-// 16 frames of 577 tokens, 12 heads: 77.3 us with a pass for the maxima and a CTA per tile, 47.9 us now.
+// 16 frames of 577 tokens, 12 heads: 77.3 us with a pass for the maxima and a CTA per tile, 44.7 us now.
 // (One key block goes to the pipelined kernel further down.)
 // ---------------------------------------------------------------------------------------
 constexpr int AQ = 128;                    // query rows per tile
@@ -293,6 +293,87 @@ __device__ __forceinline__ float score_probs_sweep(uint32_t t_s, uint32_t t_p, i
     float lo, hi;
     upk2(sum, lo, hi);
     return lo + hi;
+}
+
+// The same sweep over `np` pieces of 16 columns, `valid` of the columns real (only
+// the last piece may have others): P (packed bf16, 8 columns per piece) goes to t_p onwards and the row sum of this
+// range is returned.  Software pipeline: while the exponentials of a piece go through the special-function unit, the
+// next piece is loaded and the one before is summed, packed and stored -- with one piece after the other the warps of
+// a scheduler queued for that unit together and idled together.  P of a piece is stored after the next piece has been
+// loaded.  For the kernel with two softmax warps per scheduler (47.9 -> 44.7 us, see there); with four, whose threads
+// have 96 registers, it spills (86.6 -> 96.9 us).
+__device__ __forceinline__ float score_probs_sweep_ahead(uint32_t t_s, uint32_t t_p, int np, int valid, float c, float mc) {
+    uint32_t va[16], vb[16];
+    float pa[16], pb[16];
+    const uint64_t c2 = pk2(c, c), nmc2 = pk2(-mc, -mc);
+    uint64_t sum0 = pk2(0.f, 0.f), sum1 = sum0;
+    auto load = [&](uint32_t* v, int i) { tmem_ld16(t_s + (uint32_t)(16 * i), v); };
+    auto exps = [&](const uint32_t* v, float* p) {
+#pragma unroll
+        for (int j = 0; j < 16; j += 2) {
+            float x0, x1;
+            upk2(fma2(pk2(__uint_as_float(v[j]), __uint_as_float(v[j + 1])), c2, nmc2), x0, x1);
+            p[j] = ex2_approx(x0);
+            p[j + 1] = ex2_approx(x1);
+        }
+    };
+    auto finish = [&](const float* p, int i) {
+        uint32_t pk[8];
+#pragma unroll
+        for (int j = 0; j < 16; j += 4) {
+            sum0 = add2(sum0, pk2(p[j], p[j + 1]));
+            sum1 = add2(sum1, pk2(p[j + 2], p[j + 3]));
+            pk[j >> 1] = pack2(p[j], p[j + 1]);
+            pk[(j >> 1) + 1] = pack2(p[j + 2], p[j + 3]);
+        }
+        tmem_st8(t_p + (uint32_t)(8 * i), pk);
+    };
+    auto mask = [&](float* p, int i) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) p[j] = 16 * i + j < valid ? p[j] : 0.f;
+    };
+    auto result = [&]() {
+        float a0, a1;
+        upk2(add2(sum0, sum1), a0, a1);
+        return a0 + a1;
+    };
+    load(va, 0);
+    tmem_ld_wait();
+    if (np == 1) {
+        exps(va, pa);
+        mask(pa, 0);
+        finish(pa, 0);
+        return result();
+    }
+    load(vb, 1);
+    exps(va, pa);
+    tmem_ld_wait();
+    int i = 1;
+#pragma unroll 1
+    while (i + 1 < np) {                     // vb: piece i; pa: piece i - 1, not finished
+        load(va, i + 1);
+        exps(vb, pb);
+        finish(pa, i - 1);
+        tmem_ld_wait();
+        ++i;
+        if (i + 1 >= np) {
+            exps(va, pa);
+            finish(pb, i - 1);
+            mask(pa, i);
+            finish(pa, i);
+            return result();
+        }
+        load(vb, i + 1);
+        exps(va, pa);
+        finish(pb, i - 1);
+        tmem_ld_wait();
+        ++i;
+    }
+    exps(vb, pb);
+    finish(pa, i - 1);
+    mask(pb, i);
+    finish(pb, i);
+    return result();
 }
 
 // One output row by one warp with the row's true maximum, straight from global memory: for the rows described above.
@@ -500,7 +581,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                     if (b == 0) mc = score_reference(t_s, T) * c;
                     if (p1 > p0) {
                         const uint32_t at = t_s + (uint32_t)(p0 * 16);
-                        l += score_probs_sweep(at, share == 0 ? at + 16u : at, (p1 - p0) * 16, T - b * AKB - p0 * 16, c, mc);
+                        l += score_probs_sweep_ahead(at, share == 0 ? at + 16u : at, p1 - p0, T - b * AKB - p0 * 16, c, mc);
                         tmem_st_wait();
                     }
                 }
