@@ -5,6 +5,7 @@
 #include <atomic>
 
 #include "common.cuh"
+#include "f32x2.cuh"
 #include "tcgen05_ptx.cuh"
 
 #define BUMP(L) do { if ((L).launches) ++*(L).launches; } while (0)
@@ -133,46 +134,71 @@ __global__ void __launch_bounds__(256) layernorm_kernel(const T* __restrict__ x,
     ln_row<T, T>(x + (size_t)row * d, g, b, y + (size_t)row * d, d, eps, threadIdx.x & 31);
 }
 
-// Row statistics only (mean and 1/sqrt(var + eps), biased variance, two passes over the registers):
-// for the linears that have LayerNorm folded into their weights the normalised rows are never
-// written out; the GEMM and shrink epilogues apply the statistics instead.
+// Row statistics only (mean and 1/sqrt(var + eps), biased variance): for the linears that have LayerNorm folded into
+// their weights the normalised rows are never written out; the GEMM and shrink epilogues apply the statistics instead.
+// Bound by the latency of its loads: a warp takes four rows at once (twelve 16-byte loads per lane in flight at width
+// 768), in one pass relative to each row's first element, which keeps the sum of squares well conditioned.
+// 18912 rows of 768: 9.3 us with a row per warp, 8.3 now; 46492 rows: 17.9 and 14.1.
+constexpr int STATS_ROWS = 4;
 __global__ void __launch_bounds__(256) row_stats_kernel(const bf16* __restrict__ x, float2* __restrict__ stats,
                                                         int rows, int d, float eps) {
-    const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (row >= rows) return;
+    const int row0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * STATS_ROWS;
     const int lane = threadIdx.x & 31;
     const int nch = d >> 3;
-    const bf16* xr = x + (size_t)row * d;
-    float v[32];
-    float sum = 0.f;
+    dep_release();
+    dep_wait();
+    uint4 q[STATS_ROWS][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int c = lane + 32 * i;
-        if (c < nch) {
-            load16<bf16>(xr + c * 8, v + i * 8);
+    for (int r = 0; r < STATS_ROWS; ++r) {
+        const uint4* src = reinterpret_cast<const uint4*>(x + (size_t)min(row0 + r, rows - 1) * d);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) sum += v[i * 8 + j];
-        }
+        for (int i = 0; i < 4; ++i) q[r][i] = lane + 32 * i < nch ? src[lane + 32 * i] : make_uint4(0, 0, 0, 0);
     }
-    const float mean = warp_sum(sum) / (float)d;
-    float sq = 0.f;
+    float s1[STATS_ROWS], s2[STATS_ROWS], pivot[STATS_ROWS];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        if (lane + 32 * i < nch) {
+    for (int r = 0; r < STATS_ROWS; ++r) {
+        pivot[r] = __uint_as_float(__shfl_sync(0xFFFFFFFFu, q[r][0].x, 0) << 16);
+        const uint64_t np = pk2(-pivot[r], -pivot[r]);
+        uint64_t a1 = pk2(0.f, 0.f), a2 = a1;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) { const float t = v[i * 8 + j] - mean; sq += t * t; }
+        for (int i = 0; i < 4; ++i) {
+            if (lane + 32 * i < nch) {
+                const uint32_t w[4] = {q[r][i].x, q[r][i].y, q[r][i].z, q[r][i].w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const uint64_t a = add2(pk2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xFFFF0000u)), np);
+                    a1 = add2(a1, a);
+                    a2 = fma2(a, a, a2);
+                }
+            }
         }
+        float lo, hi;
+        upk2(a1, lo, hi); s1[r] = lo + hi;
+        upk2(a2, lo, hi); s2[r] = lo + hi;
     }
-    const float rstd = rsqrtf(warp_sum(sq) / (float)d + eps);
-    if (lane == 0) stats[row] = make_float2(mean, rstd);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int r = 0; r < STATS_ROWS; ++r) {
+            s1[r] += __shfl_xor_sync(0xFFFFFFFFu, s1[r], o);
+            s2[r] += __shfl_xor_sync(0xFFFFFFFFu, s2[r], o);
+        }
+    if (lane < STATS_ROWS && row0 + lane < rows) {
+        const float a = lane == 0 ? s1[0] : lane == 1 ? s1[1] : lane == 2 ? s1[2] : s1[3];
+        const float b = lane == 0 ? s2[0] : lane == 1 ? s2[1] : lane == 2 ? s2[2] : s2[3];
+        const float p = lane == 0 ? pivot[0] : lane == 1 ? pivot[1] : lane == 2 ? pivot[2] : pivot[3];
+        const float m1 = a / (float)d;
+        stats[row0 + lane] = make_float2(p + m1, rsqrtf(fmaxf(b / (float)d - m1 * m1, 0.f) + eps));
+    }
 }
 
 cudaError_t launch_row_stats(const Launch& L, const bf16* x, float2* stats, int rows, int d, float eps) {
     if (rows <= 0) return cudaSuccess;
     ProfScope ps(L, KC_LAYERNORM);
-    row_stats_kernel<<<(rows + 7) / 8, 256, 0, L.st>>>(x, stats, rows, d, eps);
+    const int per_block = 8 * STATS_ROWS;
+    const cudaError_t e = launch_overlapped(L, row_stats_kernel, (rows + per_block - 1) / per_block, 256, 0, 1, x, stats, rows, d, eps);
     BUMP(L);
-    return cudaGetLastError();
+    return e;
 }
 
 template <typename T>
