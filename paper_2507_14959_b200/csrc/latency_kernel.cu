@@ -15,6 +15,12 @@
 // (bounded) and fetches the heads' keys and values, the next head's while this one is computed.  Each CTA
 // attends from its 16 query rows to all keys of its frame: four warp pairs split the keys, the two warps
 // of a pair split the head dimension, partial softmax results are merged through shared memory.
+// What bounds a whole tile per CTA is the instruction chain of eight warps, not the weights (a third of what an SM can draw
+// from L2), so while the batch leaves SMs idle a cluster with one CTA per head shares each tile: a CTA computes its
+// head's queries, keys and values, attends for that head, and computes its part of the outputs of every other linear;
+// rows it finishes go to the same place in every CTA of the cluster (distributed shared memory), four exchanges per block
+// on an mbarrier (bounded waits).  DeiT-tiny, one CTA per tile -> one per head: one frame 299 -> 239 us (no
+// adapter), 314 -> 249 (three), three frames 316 -> 248; from the fourth frame on the clusters do not fit 148 SMs.
 // Contractions run on mma.sync m16n8k16 (bf16 in, fp32 accumulate): with 16 rows per CTA there is no
 // 128-row tile to give to tcgen05.
 // LayerNorm uses the folded form the other kernels use: y = rstd (x W' - mean g) + b'.
@@ -34,6 +40,7 @@ constexpr int LT_MAX_SLOTS = 8;
 constexpr int LT_MAX_SET = 8;
 constexpr int LT_MAX_SLABS = 8;              // active LoRA slabs of one linear
 constexpr int LT_HD = 64;
+constexpr int LT_MAX_SHARE = 6;              // CTAs that share a row tile, one per head (rows of up to 384)
 constexpr int LT_KSPLIT = 4;                 // key ranges of the attention warps
 constexpr int LT_ST = 8;                     // key tiles (8 keys) of one range, at most (256 tokens)
 constexpr long long LT_WAIT_CYCLES = 4000000000ll;
@@ -140,6 +147,8 @@ struct Ctx {
     int warp, lane, g, t, ns;
     uint32_t slot, phase;      // ring position: the same in every consumer thread (and in the producer)
     uint32_t li;               // linears done so far (their vector packs alternate between two buffers)
+    int share, rank;           // CTAs on this row tile (a cluster) and this one's place among them
+    uint32_t xphase;           // exchanges of rows between them so far (parity)
     int* status;
     volatile int* abort_flag;
 };
@@ -154,6 +163,51 @@ __device__ __forceinline__ uint32_t vempty_bar(const Ctx& cx) { return bars(cx) 
 __device__ __forceinline__ uint32_t cfull_bar(const Ctx& cx, uint32_t b) { return bars(cx) + 160u + 8u * b; }
 __device__ __forceinline__ uint32_t cempty_bar(const Ctx& cx, uint32_t b) { return bars(cx) + 176u + 8u * b; }
 __device__ __forceinline__ uint32_t kvdone_bar(const Ctx& cx, uint32_t part) { return bars(cx) + 192u + 8u * part; }
+
+__device__ __forceinline__ uint32_t xchg_bar(const Ctx& cx) { return bars(cx) + 208u; }
+
+// Shared tiles: the columns of chunk i of this CTA's part of a linear, as two halves of 64 (b < 0: only one).
+// qkv: its head's keys and values, then its head's queries; other linears: the rank'th part of the outputs.
+struct Halves { int a, b; };
+__device__ __forceinline__ int share_chunks(const Ctx& cx, int N, bool qkv) { return qkv ? 2 : (N / cx.share + 127) >> 7; }
+__device__ __forceinline__ Halves share_chunk(const Ctx& cx, int N, int d, bool qkv, int i) {
+    Halves hv;
+    if (qkv) {
+        hv.a = (i == 0 ? d : 0) + cx.rank * LT_HD;
+        hv.b = i == 0 ? 2 * d + cx.rank * LT_HD : -1;
+        return hv;
+    }
+    const int cols = N / cx.share;
+    hv.a = cx.rank * cols + i * 128;
+    hv.b = i * 128 + 64 < cols ? hv.a + 64 : -1;
+    return hv;
+}
+// the same shared-memory address in CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t peer_addr(uint32_t addr, int rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+// a value of a row goes to this CTA's buffer, or to the same place in every CTA of the tile
+template <bool CL>
+__device__ __forceinline__ void put(const Ctx& cx, uint32_t* p, uint32_t v) {
+    if (!CL) { *p = v; return; }
+    for (int r = 0; r < cx.share; ++r)
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_addr(s_u32(p), r)), "r"(v) : "memory");
+}
+template <bool CL>
+__device__ __forceinline__ void put(const Ctx& cx, uint2* p, uint2 v) {
+    if (!CL) { *p = v; return; }
+    for (int r = 0; r < cx.share; ++r)
+        asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(peer_addr(s_u32(p), r)), "r"(v.x), "r"(v.y) : "memory");
+}
+template <bool CL>
+__device__ __forceinline__ void put(const Ctx& cx, float2* p, float2 v) {
+    put<CL>(cx, reinterpret_cast<uint2*>(p), make_uint2(__float_as_uint(v.x), __float_as_uint(v.y)));
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
 
 // The order in which a linear's chunks of 128 outputs are taken (producer and consumers alike).  qkv (width d):
 // the chunk with the first head's keys, the chunk with its values, the other chunks with key or value
@@ -197,6 +251,31 @@ __device__ __forceinline__ void bar_wait(const Ctx& cx, uint32_t bar, uint32_t p
         }
     }
 }
+// Every consumer warp of the tile's CTAs has written its part of the rows (put) and sees the others'.  One such
+// point lies between any two uses of a buffer that the peers write, so a peer never overwrites rows still read here:
+// rows written after exchange e were last read before their reader took part in e.
+template <bool CL>
+__device__ __forceinline__ void rows_sync(Ctx& cx) {
+    if (!CL) { consumer_sync(); return; }
+    __syncwarp();
+    if (cx.lane < cx.share) {
+        asm volatile("fence.acq_rel.cluster;" ::: "memory");
+        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(peer_addr(xchg_bar(cx), cx.lane)) : "memory");
+    }
+    const long long t0 = clock64();
+    for (;;) {
+        uint32_t ok;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(xchg_bar(cx)), "r"(cx.xphase) : "memory");
+        if (ok || *cx.abort_flag) break;
+        if (clock64() - t0 > LT_WAIT_CYCLES) {
+            *cx.abort_flag = 1;
+            atomicCAS(cx.status, 0, (int)PM_ERR_TIMEOUT);
+            break;
+        }
+    }
+    cx.xphase ^= 1u;
+}
 __device__ __forceinline__ void ring_advance(Ctx& cx) {
     if (++cx.slot == (uint32_t)cx.ns) { cx.slot = 0; cx.phase ^= 1u; }
 }
@@ -224,6 +303,9 @@ __device__ __forceinline__ uint32_t step_claim(Ctx& cx, uint32_t bytes) {
 //   for each chunk of 128 outputs, in the order of chunk_at(): K/128 steps of W^T, each two
 //   K boxes of the chunk ([64 rows][64] boxes, two per K box of a full chunk), then the chunk's rows of
 //   the active slabs' B^T ([128 rows][16] boxes, four per step).
+// Shared tiles: this CTA's chunks only, each as its halves; the B^T rows come as one [128 rows][16] box per half
+// (its second 64 rows unused), the halves 4 KB apart.
+template <bool CL>
 __device__ void produce_linear(Ctx& cx, const LatLinear* lin, const SlabTab& st, const ActiveSet& as, int rs, int slabs_max,
                                int d, bool qkv) {
     const int N = lin->n_out, K = lin->k_in, k_boxes = K >> 6, n_chunks = (N + 127) >> 7, n_sl = st.n;
@@ -257,6 +339,33 @@ __device__ void produce_linear(Ctx& cx, const LatLinear* lin, const SlabTab& st,
             ring_advance(cx);
         }
     }
+    if (CL) {
+        const int mine = share_chunks(cx, N, qkv);
+        for (int ci = 0; ci < mine; ++ci) {
+            const Halves hv = share_chunk(cx, N, d, qkv, ci);
+            const int halves = hv.b < 0 ? 1 : 2;
+            for (int kb0 = 0; kb0 < k_boxes && !*cx.abort_flag; kb0 += 2) {
+                const int nb = min(2, k_boxes - kb0);
+                const uint32_t dst = step_claim(cx, (uint32_t)(nb * halves) * 8192u);
+                for (int b = 0; b < nb; ++b) {
+                    tma_box(dst + b * LT_BOX_BYTES, &lin->tm_w, (kb0 + b) * 64, hv.a, full_bar(cx, cx.slot));
+                    if (halves == 2) tma_box(dst + b * LT_BOX_BYTES + 8192u, &lin->tm_w, (kb0 + b) * 64, hv.b, full_bar(cx, cx.slot));
+                }
+                ring_advance(cx);
+            }
+            for (int s0 = 0; s0 < n_sl && !*cx.abort_flag; s0 += 4) {
+                const int cnt = min(4, n_sl - s0);
+                const uint32_t dst = step_claim(cx, (uint32_t)(cnt * halves) * 4096u);
+                for (int j = 0; j < cnt; ++j) {
+                    const int row = (as.id[st.who[s0 + j]] * slabs_max + st.sl[s0 + j]) * N;
+                    tma_box(dst + j * 8192u, &lin->tm_bt, 0, row + hv.a, full_bar(cx, cx.slot));
+                    if (halves == 2) tma_box(dst + j * 8192u + 4096u, &lin->tm_bt, 0, row + hv.b, full_bar(cx, cx.slot));
+                }
+                ring_advance(cx);
+            }
+        }
+        return;
+    }
     const ChunkOrder order = chunk_order(N, d, qkv);
     for (int ci = 0; ci < n_chunks; ++ci) {
         const int nc = chunk_at(order, ci);
@@ -281,28 +390,30 @@ __device__ void produce_linear(Ctx& cx, const LatLinear* lin, const SlabTab& st,
     }
 }
 
+// one K box of weights (row r of it per lane) against 64 columns of A
+__device__ __forceinline__ void mma_box(const Ctx& cx, uint32_t a_row, uint32_t box, int r, float (&acc)[2][2][4]) {
+    const int mi = cx.lane >> 3;
+    // all eight fetches first, then the eight multiplications (four independent accumulators in turn)
+    uint32_t a[4][4], b[4][4];
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+        ldsm4(a_row + ks * 32, a[ks][0], a[ks][1], a[ks][2], a[ks][3]);
+        const int c = ks * 2 + (mi & 1);
+        ldsm4(box + r * 128 + ((c ^ (r & 7)) << 4), b[ks][0], b[ks][1], b[ks][2], b[ks][3]);
+    }
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+        mma16816(acc[0][ks & 1], a[ks], b[ks][0], b[ks][1]);
+        mma16816(acc[1][ks & 1], a[ks], b[ks][2], b[ks][3]);
+    }
+}
 // one ring step of weights ([rows][64 inputs], this warp's 16 rows) against 64 columns of A (bf16, shared memory)
 __device__ __forceinline__ void mma_step(Ctx& cx, uint32_t a_row0, int nb, bool active, float (&acc)[2][2][4]) {
     const uint32_t box0 = step_acquire(cx);
     if (active) {
         const int mi = cx.lane >> 3;
         const int r = cx.warp * 16 + (mi >> 1) * 8 + (cx.lane & 7);
-        for (int bx = 0; bx < nb; ++bx) {
-        const uint32_t box = box0 + bx * LT_BOX_BYTES, a_row = a_row0 + bx * 128;
-        // all eight fetches first, then the eight multiplications (four independent accumulators in turn)
-        uint32_t a[4][4], b[4][4];
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks) {
-            ldsm4(a_row + ks * 32, a[ks][0], a[ks][1], a[ks][2], a[ks][3]);
-            const int c = ks * 2 + (mi & 1);
-            ldsm4(box + r * 128 + ((c ^ (r & 7)) << 4), b[ks][0], b[ks][1], b[ks][2], b[ks][3]);
-        }
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks) {
-            mma16816(acc[0][ks & 1], a[ks], b[ks][0], b[ks][1]);
-            mma16816(acc[1][ks & 1], a[ks], b[ks][2], b[ks][3]);
-        }
-        }
+        for (int bx = 0; bx < nb; ++bx) mma_box(cx, a_row0 + bx * 128, box0 + bx * LT_BOX_BYTES, r, acc);
     }
     step_release(cx);
 }
@@ -366,6 +477,76 @@ __device__ void linear16(Ctx& cx, const bf16* A, int lda, int K, int N, int n_sl
             }
         }
     }
+}
+
+// The same for the chunks of a shared tile.  A chunk of 128 columns: a warp per 16 of them, as above.  A chunk of 64:
+// four warps per K box of a step, the second four's sums added through `red` (4 KB that nothing else uses
+// meanwhile), so a K of 768 costs six box times instead of twelve.
+template <typename Epi>
+__device__ void linear16_shared(Ctx& cx, const bf16* A, int lda, int K, int N, int n_sl, int d, bool qkv, void* red, Epi epi) {
+    const int k_boxes = K >> 6, mine = share_chunks(cx, N, qkv), half = cx.warp >> 2, wq = cx.warp & 3, mi = cx.lane >> 3;
+    const uint32_t a_base = s_u32(A) + ((cx.lane & 15) * lda + (cx.lane >> 4) * 8) * 2;
+    const uint32_t t_row = s_u32(cx.sm + cx.L.tbuf) + ((cx.lane & 15) * cx.L.ldt + (cx.lane >> 4) * 8) * 2;
+    for (int ci = 0; ci < mine; ++ci) {
+        const Halves hv = share_chunk(cx, N, d, qkv, ci);
+        const bool two = hv.b >= 0;
+        float acc[2][2][4];
+        acc_zero(acc);
+        const int r = (two ? cx.warp : wq) * 16 + (mi >> 1) * 8 + (cx.lane & 7);
+        for (int kb0 = 0; kb0 < k_boxes; kb0 += 2) {
+            const int nb = min(2, k_boxes - kb0);
+            const uint32_t box0 = step_acquire(cx);
+            for (int bx = two ? 0 : half; bx < (two ? nb : min(nb, half + 1)); ++bx)
+                mma_box(cx, a_base + (kb0 + bx) * 128, box0 + bx * LT_BOX_BYTES, r, acc);
+            step_release(cx);
+        }
+        for (int s0 = 0; s0 < n_sl; s0 += 4) {
+            const uint32_t box = step_acquire(cx);
+            if (two || half == 0) {
+                const int n = wq * 16 + ((cx.lane >> 4) & 1) * 8 + (cx.lane & 7), c = (cx.lane >> 3) & 1;
+                const uint32_t b_row = box + half * 4096 + n * 32 + ((c ^ ((n >> 2) & 1)) << 4);
+                const int cnt = min(4, n_sl - s0);
+                for (int j = 0; j < cnt; ++j) {
+                    uint32_t a[4], b0, b1, b2, b3;
+                    ldsm4(t_row + (s0 + j) * 32, a[0], a[1], a[2], a[3]);
+                    ldsm4(b_row + j * 8192, b0, b1, b2, b3);
+                    mma16816(acc[0][j & 1], a, b0, b1);
+                    mma16816(acc[1][j & 1], a, b2, b3);
+                }
+            }
+            step_release(cx);
+        }
+        float y[2][4];
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) y[q][e] = acc[q][0][e] + acc[q][1][e];
+        if (!two) {
+            float4* rd = reinterpret_cast<float4*>(red) + wq * 64 + cx.lane;
+            if (half) {
+                rd[0] = make_float4(y[0][0], y[0][1], y[0][2], y[0][3]);
+                rd[32] = make_float4(y[1][0], y[1][1], y[1][2], y[1][3]);
+            }
+            asm volatile("bar.sync %0, 64;" ::"r"(2 + wq) : "memory");
+            if (!half) {
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const float4 v = rd[q * 32];
+                    y[q][0] += v.x; y[q][1] += v.y; y[q][2] += v.z; y[q][3] += v.w;
+                }
+            }
+        }
+        if (two || half == 0) epi((half ? hv.b : hv.a) + wq * 16 + 2 * cx.t, y);
+        if (qkv && ci == 0) {                       // this warp's keys and values of the block are stored
+            __syncwarp();
+            if (cx.lane == 0) bar_arrive(kvdone_bar(cx, 0));
+        }
+    }
+}
+template <bool CL, typename Epi>
+__device__ __forceinline__ void linear_rows(Ctx& cx, const bf16* A, int lda, int K, int N, int n_sl, int d, bool qkv, void* red, Epi epi) {
+    if constexpr (CL) linear16_shared(cx, A, lda, K, N, n_sl, d, qkv, red, epi);
+    else linear16(cx, A, lda, K, N, n_sl, d, qkv, epi);
 }
 
 // The consumers' side of a linear's shrink steps: warp i < n_sl multiplies the rows by slab i of A^T and
@@ -448,6 +629,8 @@ __device__ void round_rows_and_stats(Ctx& cx, int d, float eps) {
     }
 }
 
+// CL: the cluster's CTAs (as many as heads) share one tile of 16 rows.
+template <bool CL>
 __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __grid_constant__ LatArgs args) {
     extern __shared__ __align__(1024) uint8_t smem[];
     if (s_u32(smem) & 1023u) {                 // swizzled boxes need a 1024-byte aligned window
@@ -459,7 +642,11 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
     cx.L = lat_layout(args.d, args.mlp, args.patch_dim, args.tokens, args.layers, args.ring_slots);
     cx.ns = args.ring_slots;
     cx.warp = threadIdx.x >> 5; cx.lane = threadIdx.x & 31; cx.g = cx.lane >> 2; cx.t = cx.lane & 3;
-    const int f = blockIdx.x / args.tiles_pf, rt = blockIdx.x % args.tiles_pf;     // slot, row tile
+    cx.share = CL ? args.heads : 1;
+    cx.rank = CL ? (int)(blockIdx.x % (unsigned)cx.share) : 0;
+    cx.xphase = 0;
+    const int tile = CL ? (int)(blockIdx.x / (unsigned)cx.share) : (int)blockIdx.x;
+    const int f = tile / args.tiles_pf, rt = tile % args.tiles_pf;     // slot, row tile
     const int frame = args.perm ? args.perm[f] : f;                                  // input / output row
     const int T = args.tokens, d = args.d, r0 = rt * LT_ROWS;
     const int tpad = (T + 15) / 16 * 16;
@@ -480,6 +667,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
         bar_init(vfull_bar(cx), 1); bar_init(vempty_bar(cx), LT_CWARPS);
         for (int b = 0; b < 2; ++b) { bar_init(cfull_bar(cx, b), 1); bar_init(cempty_bar(cx, b), LT_CWARPS); }
         bar_init(kvdone_bar(cx, 0), LT_CWARPS); bar_init(kvdone_bar(cx, 1), LT_CWARPS);
+        if (CL) bar_init(xchg_bar(cx), LT_CWARPS * cx.share);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -529,40 +717,43 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
         slabtab[threadIdx.x] = st;
     }
     __syncthreads();
+    if (CL) cluster_barrier();                    // every peer runs and has set its barriers up
     // ---- the weight producer: one thread, the whole network's static operands in consumption order
     if (cx.warp == LT_CWARPS) {
-        if (cx.lane != 0) return;
-        SlabTab none;
-        none.n = 0;
-        produce_linear(cx, args.lin + (size_t)args.layers * 4, none, *as, rs, args.slabs_max, d, false);
-        for (int l = 0; l < args.layers && !*abort_flag; ++l)
-            for (int j = 0; j < 4; ++j)
-                produce_linear(cx, args.lin + (size_t)l * 4 + j, slabtab[l * 4 + j], *as, rs, args.slabs_max, d, j == 0);
+        if (cx.lane == 0) {
+            SlabTab none;
+            none.n = 0;
+            produce_linear<CL>(cx, args.lin + (size_t)args.layers * 4, none, *as, rs, args.slabs_max, d, false);
+            for (int l = 0; l < args.layers && !*abort_flag; ++l)
+                for (int j = 0; j < 4; ++j)
+                    produce_linear<CL>(cx, args.lin + (size_t)l * 4 + j, slabtab[l * 4 + j], *as, rs, args.slabs_max, d, j == 0);
+        }
+        if (CL) { __syncwarp(); cluster_barrier(); }
         return;
     }
     // ---- the key/value producer: per block, wait for the frame's CTAs, then one head after the other
     if (cx.warp == LT_CWARPS + 1) {
-        if (cx.lane != 0) return;
+        unsigned int* counter = args.bar + (CL ? f * cx.share + cx.rank : f);       // shared tiles: one per frame and head
         uint32_t idx = 0;
-        for (int l = 0; l < args.layers && !*abort_flag; ++l) {
+        for (int l = 0; cx.lane == 0 && l < args.layers && !*abort_flag; ++l) {
             // Twice per block -- for the first head, then for the others -- : the consumer warps have stored this
             // CTA's keys and values (ordinary stores, fetched by TMA on the other side: order the two proxies as
             // well as the scopes), so the CTA counts itself in: everything its threads stored up to there is
             // visible to whoever sees the count.  Then the heads' keys and values, one after the other.
             const int kv_row0 = ((l & 1) * args.n_frames + f) * T;
-            const bool two = chunk_order(3 * d, d, true).reorder;   // else: one count-in per block
+            const bool two = !CL && chunk_order(3 * d, d, true).reorder;   // else: one count-in per block
             for (int part = 0; part < (two ? 2 : 1) && !*abort_flag; ++part) {
-                bar_wait(cx, kvdone_bar(cx, two ? part : 1), (uint32_t)l & 1u);
+                bar_wait(cx, kvdone_bar(cx, CL ? 0 : two ? part : 1), (uint32_t)l & 1u);
                 if (*abort_flag) break;
                 asm volatile("fence.proxy.async.global;" ::: "memory");
                 __threadfence();
-                atomicAdd(args.bar + f, 1u);
+                atomicAdd(counter, 1u);
                 const unsigned int per = two ? 2u : 1u;
                 const unsigned int want = (unsigned int)args.tiles_pf * (per * (unsigned int)l + (unsigned int)part + 1u);
                 const long long t0 = clock64();
                 unsigned int seen;
                 do {
-                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(args.bar + f) : "memory");
+                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(counter) : "memory");
                     if (seen < want && (*abort_flag || clock64() - t0 > LT_WAIT_CYCLES)) {
                         if (!*abort_flag) { *abort_flag = 1; atomicCAS(args.status, 0, (int)PM_ERR_TIMEOUT); }
                         break;
@@ -570,7 +761,8 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                 } while (seen < want);
                 if (*abort_flag) break;
                 asm volatile("fence.proxy.async.global;" ::: "memory");
-                const int h0 = !two ? 0 : part == 0 ? 0 : 1, h1 = !two ? args.heads : part == 0 ? 1 : args.heads;
+                const int h0 = CL ? cx.rank : !two ? 0 : part == 0 ? 0 : 1;
+                const int h1 = CL ? cx.rank + 1 : !two ? args.heads : part == 0 ? 1 : args.heads;
                 for (int h = h0; h < h1; ++h, ++idx) {
                     bar_wait(cx, kempty_bar(cx), (idx & 1u) ^ 1u);
                     bar_expect(kfull_bar(cx), (uint32_t)tpad * 128u);
@@ -581,6 +773,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                 }
             }
         }
+        if (CL) { __syncwarp(); cluster_barrier(); }
         return;
     }
 
@@ -618,7 +811,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
     // ---- patch projection + positions; the CLS row
     {
         const float* cv = pack_acquire();
-        linear16(cx, hbuf, cx.L.ldh, args.patch_dim, d, 0, d, false, [&](int n0, float (&y)[2][4]) {
+        linear_rows<CL>(cx, hbuf, cx.L.ldh, args.patch_dim, d, 0, d, false, abuf, [&](int n0, float (&y)[2][4]) {
 #pragma unroll
             for (int hi = 0; hi < 2; ++hi) {
                 const int r = cx.g + 8 * hi, tok = r0 + r;
@@ -633,13 +826,13 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                     float2 out = make_float2(0.f, 0.f);             // rows past the frame stay zero
                     if (tok == 0) out = make_float2(args.cls[n] + p[q].x, args.cls[n + 1] + p[q].y);
                     else if (tok < T) out = make_float2(y[q][2 * hi] + cv[n] + p[q].x, y[q][2 * hi + 1] + cv[n + 1] + p[q].y);
-                    *reinterpret_cast<float2*>(xres + r * d + n) = out;
+                    put<CL>(cx, reinterpret_cast<float2*>(xres + r * d + n), out);
                 }
             }
         });
         pack_release();
     }
-    consumer_sync();
+    rows_sync<CL>(cx);
 
     // LoRA shrink of a linear with slab table `st` on the rows A: t[r][16 i + j] (bf16) = s_a (x A_a)
     // (folded linears: s_a ((x A' - mean c1) + c2 / rstd), the fused accumulator being scaled by rstd afterwards)
@@ -658,7 +851,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
         consumer_sync();
     };
     auto residual = [&](const float* cv) {
-        return [=](int n0, float (&y)[2][4]) {
+        return [=, &cx](int n0, float (&y)[2][4]) {
             float2 x[2][2], b[2];
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
@@ -671,13 +864,16 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
 #pragma unroll
                 for (int hi = 0; hi < 2; ++hi)
                     if (r0 + cx.g + 8 * hi < T)
-                        *reinterpret_cast<float2*>(xres + (cx.g + 8 * hi) * d + n0 + 8 * q) =
-                            make_float2(x[q][hi].x + y[q][2 * hi] + b[q].x, x[q][hi].y + y[q][2 * hi + 1] + b[q].y);
+                        put<CL>(cx, reinterpret_cast<float2*>(xres + (cx.g + 8 * hi) * d + n0 + 8 * q),
+                                make_float2(x[q][hi].x + y[q][2 * hi] + b[q].x, x[q][hi].y + y[q][2 * hi + 1] + b[q].y));
         };
     };
 
     const float att_scale = 0.125f * 1.4426950408889634f;  // 1/sqrt(64) * log2(e)
     uint32_t head_no = 0;                                    // heads attended so far (all blocks)
+    // the attended rows; shared tiles: beside this head's queries, since a peer may be done while qkv still reads abuf here
+    bf16* att = CL ? qbuf : abuf;
+    const int ldatt = CL ? cx.L.ldq : cx.L.lda;
     for (int l = 0; l < args.layers; ++l) {
         const SlabTab* st = slabtab + l * 4;
         bf16* kvb = args.kv + (size_t)(l & 1) * args.n_frames * T * 2 * d + (size_t)f * T * 2 * d;
@@ -688,7 +884,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
             const float* cv = pack_acquire();
             shrink(st[0], abuf, cx.L.lda, d, 3 * d, true, cv);
             const float4 s_lo = stats[cx.g], s_hi = stats[cx.g + 8];
-            linear16(cx, abuf, cx.L.lda, d, 3 * d, st[0].n, d, true, [&](int n0, float (&y)[2][4]) {
+            linear_rows<CL>(cx, abuf, cx.L.lda, d, 3 * d, st[0].n, d, true, hbuf, [&](int n0, float (&y)[2][4]) {
                 float2 b[2], gs[2];
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
@@ -730,7 +926,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
             for (int n = 0; n < 2; ++n)
                 v_addr[n] = s_u32(smem + cx.L.vbuf) + (t8_lo * 8 + (mi & 1) * 8 + l7) * 128 + (((dh * 4 + n * 2 + (mi >> 1)) ^ l7) << 4);
             float* part = reinterpret_cast<float*>(smem + cx.L.hbuf);
-            for (int h = 0; h < args.heads; ++h, ++head_no) {
+            for (int h = cx.rank; h < (CL ? cx.rank + 1 : args.heads); ++h, ++head_no) {
                 uint32_t qa[4][4];
 #pragma unroll
                 for (int ks = 0; ks < 4; ++ks)
@@ -842,19 +1038,19 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                     uint2 pkd;
                     pkd.x = pk_bf16(num[0] * inv, num[1] * inv);
                     pkd.y = pk_bf16(num[2] * inv, num[3] * inv);
-                    *reinterpret_cast<uint2*>(abuf + r * cx.L.lda + h * LT_HD + c4) = pkd;
+                    put<CL>(cx, reinterpret_cast<uint2*>(att + r * ldatt + h * LT_HD + c4), pkd);
                 }
-                consumer_sync();
+                rows_sync<CL>(cx);
             }
         }
         // ---- proj (+ residual)
         {
             const float* cv = pack_acquire();
-            shrink(st[1], abuf, cx.L.lda, d, d, false, cv);
-            linear16(cx, abuf, cx.L.lda, d, d, st[1].n, d, false, residual(cv));
+            shrink(st[1], att, ldatt, d, d, false, cv);
+            linear_rows<CL>(cx, att, ldatt, d, d, st[1].n, d, false, abuf, residual(cv));
             pack_release();
         }
-        consumer_sync();
+        rows_sync<CL>(cx);
         // ---- fc1 (LayerNorm 2 folded, GELU) and fc2 (+ residual)
         round_rows_and_stats(cx, d, args.eps);
         consumer_sync();
@@ -863,7 +1059,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
             const int N = args.mlp;
             shrink(st[2], abuf, cx.L.lda, d, N, true, cv);
             const float4 s_lo = stats[cx.g], s_hi = stats[cx.g + 8];
-            linear16(cx, abuf, cx.L.lda, d, N, st[2].n, d, false, [&](int n0, float (&y)[2][4]) {
+            linear_rows<CL>(cx, abuf, cx.L.lda, d, N, st[2].n, d, false, nullptr, [&](int n0, float (&y)[2][4]) {
                 float2 b[2], gs[2];
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
@@ -873,29 +1069,28 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
                     const int n = n0 + 8 * q;
-                    *reinterpret_cast<uint32_t*>(hbuf + cx.g * cx.L.ldh + n) =
-                        pk_bf16(gelu_fit(s_lo.y * (y[q][0] - s_lo.x * gs[q].x) + b[q].x), gelu_fit(s_lo.y * (y[q][1] - s_lo.x * gs[q].y) + b[q].y));
-                    *reinterpret_cast<uint32_t*>(hbuf + (cx.g + 8) * cx.L.ldh + n) =
-                        pk_bf16(gelu_fit(s_hi.y * (y[q][2] - s_hi.x * gs[q].x) + b[q].x), gelu_fit(s_hi.y * (y[q][3] - s_hi.x * gs[q].y) + b[q].y));
+                    put<CL>(cx, reinterpret_cast<uint32_t*>(hbuf + cx.g * cx.L.ldh + n),
+                            pk_bf16(gelu_fit(s_lo.y * (y[q][0] - s_lo.x * gs[q].x) + b[q].x), gelu_fit(s_lo.y * (y[q][1] - s_lo.x * gs[q].y) + b[q].y)));
+                    put<CL>(cx, reinterpret_cast<uint32_t*>(hbuf + (cx.g + 8) * cx.L.ldh + n),
+                            pk_bf16(gelu_fit(s_hi.y * (y[q][2] - s_hi.x * gs[q].x) + b[q].x), gelu_fit(s_hi.y * (y[q][3] - s_hi.x * gs[q].y) + b[q].y)));
                 }
             });
             pack_release();
         }
-        consumer_sync();
+        rows_sync<CL>(cx);
         {
             const float* cv = pack_acquire();
             shrink(st[3], hbuf, cx.L.ldh, args.mlp, d, false, cv);
-            linear16(cx, hbuf, cx.L.ldh, args.mlp, d, st[3].n, d, false, residual(cv));
+            linear_rows<CL>(cx, hbuf, cx.L.ldh, args.mlp, d, st[3].n, d, false, abuf, residual(cv));
             pack_release();
         }
-        consumer_sync();
+        rows_sync<CL>(cx);
     }
 
-    if (*abort_flag) {
+    if (*abort_flag)
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);     // copies still in flight land before shared memory goes away
-        return;
-    }
-    if (rt != 0) return;
+    if (CL) cluster_barrier();                                // no peer writes here any more, aborted or not
+    if (*abort_flag || rt != 0 || cx.rank != 0) return;
 
     // ---- heads on the CLS row (row 0 of the frame's first CTA): final LayerNorm, base head, adapter heads
     float* z = reinterpret_cast<float*>(smem + cx.L.hbuf);
@@ -959,6 +1154,37 @@ int lat_ring_slots(int d, int mlp, int patch_dim, int tokens, int layers) {
     return room / LT_SLOT_BYTES < LT_MAX_SLOTS ? room / LT_SLOT_BYTES : LT_MAX_SLOTS;
 }
 
+// CTAs per tile of 16 rows.  One per head (each takes its head and its part of every linear's outputs, and the rows are
+// exchanged through distributed shared memory) while clusters for all tiles of the batch are resident at once, and where
+// the hidden layer splits into parts of whole 128-column chunks; else one CTA does the whole tile.
+int lat_share(const LatArgs& a, size_t smem) {
+    const int c = a.heads;
+    if (c < 2 || c > LT_MAX_SHARE || a.mlp % (128 * c) != 0) return 1;
+    // clusters of c CTAs the device holds at once; the shared memory is that of one CTA per SM whatever the geometry
+    static std::atomic<int> resident[64][LT_MAX_SHARE + 1];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    std::atomic<int>& known = resident[dev & 63][c];
+    if (const int n = known.load(std::memory_order_relaxed); n > 0) return a.n_frames * a.tiles_pf <= n ? c : 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(a.n_frames * a.tiles_pf * c);
+    cfg.blockDim = dim3(LT_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)c;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, latency_forward_kernel<true>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 1;
+    }
+    known.store(clusters, std::memory_order_relaxed);
+    return a.n_frames * a.tiles_pf <= clusters ? c : 1;
+}
+
 }  // namespace
 
 size_t latency_smem_bytes(int d, int mlp, int patch_dim, int tokens, int layers) {
@@ -971,27 +1197,32 @@ cudaError_t launch_latency_forward(const Launch& L, const LatArgs& a) {
     const int slots = lat_ring_slots(a.d, a.mlp, a.patch_dim, a.tokens, a.layers);
     if (!slots || a.layers * 4 > LT_THREADS) return cudaErrorInvalidValue;
     const size_t smem = (size_t)lat_layout(a.d, a.mlp, a.patch_dim, a.tokens, a.layers, slots).total;
-    static SmemGrant grant;
-    if (cudaError_t e = grant.ensure(latency_forward_kernel, (int)smem); e != cudaSuccess) return e;
+    static SmemGrant grant[2];
+    if (cudaError_t e = grant[0].ensure(latency_forward_kernel<false>, (int)smem); e != cudaSuccess) return e;
+    if (cudaError_t e = grant[1].ensure(latency_forward_kernel<true>, (int)smem); e != cudaSuccess) return e;
+    const int share = lat_share(a, smem), ctas = a.n_frames * a.tiles_pf * share;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.n_frames * a.tiles_pf);
+    cfg.gridDim = dim3(ctas);
     cfg.blockDim = dim3(LT_THREADS);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = L.st;
     // the CTAs of a frame wait for one another: all of them must be resident at once
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)share;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = share > 1 ? 2 : 1;
     ProfScope ps(L, KC_GEMM);
     LatArgs copy = a;
     copy.status = L.status;
     copy.ring_slots = slots;
     // the frames' arrival counters start at zero (an aborted launch may have left them anywhere)
-    cudaError_t e = cudaMemsetAsync(a.bar, 0, sizeof(unsigned int) * a.n_frames, L.st);
+    cudaError_t e = cudaMemsetAsync(a.bar, 0, sizeof(unsigned int) * a.n_frames * share, L.st);
     if (e != cudaSuccess) return e;
-    e = cudaLaunchKernelEx(&cfg, latency_forward_kernel, copy);
+    e = share > 1 ? cudaLaunchKernelEx(&cfg, latency_forward_kernel<true>, copy) : cudaLaunchKernelEx(&cfg, latency_forward_kernel<false>, copy);
     BUMP(L);
     return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -97,6 +97,38 @@ def test_small_batch_kernel_odd_geometry():
     m.close()
 
 
+@pytest.mark.parametrize("d,heads,mlp,img,n_frames", [(128, 2, 512, 80, 4), (192, 3, 384, 48, 1), (256, 4, 1024, 112, 2),
+                                                       (320, 5, 640, 64, 3), (192, 3, 768, 224, 4)])
+def test_small_batch_kernel_tiles_shared_by_a_cluster(d, heads, mlp, img, n_frames):
+    """Row tiles shared by one CTA per head: hidden layers of one, two and four 128-column chunks per CTA, clusters of two
+    to five, last row tiles with a few rows, K splits with an odd number of boxes, up to five LoRA slabs; the last
+    geometry has one frame more than the clusters of three that fit 148 SMs, so its CTAs take whole tiles.  Against the
+    oracle and the layer-by-layer kernels, and the same bits on a second call."""
+    from paper_2507_14959_b200 import binding
+    name = f"shared_tiles_{d}_{mlp}_{img}"
+    spec = wl.ModelSpec(img=img, d=d, heads=heads, mlp=mlp, n_classes=24, layers=3)
+    bb = wl.make_backbone(name, spec)
+    ads = [wl.make_adapter(name, spec, a, r, np.arange(6 * a, 6 * a + 6)) for a, r in enumerate((8, 24, 16, 4))]
+    sets = [[0, 1, 2, 3], [1], [], [3, 0]][:n_frames]
+    off, ids = wl.sets_to_csr(sets)
+    w = wl.Workload(name, spec, bb, ads, wl.make_frames(name, spec, len(sets)), off, ids)
+    so, bo = po.forward(w.backbone, w.adapters, w.frames, off, ids, spec.heads, spec.patch, spec.ln_eps, spec.n_classes)
+    m = binding.model_from_workload(w, dtype=0, max_frames=len(sets), max_set=4)
+    got = {}
+    for on in (True, False):
+        m.set_small_batch_kernel(on)
+        n0 = m.launch_count()
+        got[on] = run_forward(m, w, 0)
+        launches = m.launch_count() - n0
+        assert (launches == 1) if on else (launches > 10)
+        assert np.abs(got[on][0] - so).max() < 1e-2 and np.abs(got[on][1] - bo).max() < 1e-2
+        again = run_forward(m, w, 0)
+        np.testing.assert_array_equal(again[0], got[on][0])
+        np.testing.assert_array_equal(again[1], got[on][1])
+    assert np.abs(got[True][0] - got[False][0]).max() < 5e-3
+    m.close()
+
+
 def test_small_batch_kernel_largest_batch_and_first_batch_beyond_it():
     """The whole-network kernel takes as many frames as there are SMs for their 16-row tiles (13 tiles per
     197-token frame: 11 frames on 148 SMs), frames with different sets (empty, one, three adapters) side
