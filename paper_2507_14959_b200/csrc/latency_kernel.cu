@@ -18,9 +18,10 @@
 // What bounds a whole tile per CTA is the instruction chain of eight warps, not the weights (a third of what an SM can draw
 // from L2), so while the batch leaves SMs idle a cluster with one CTA per head shares each tile: a CTA computes its
 // head's queries, keys and values, attends for that head, and computes its part of the outputs of every other linear;
-// rows it finishes go to the same place in every CTA of the cluster (distributed shared memory), four exchanges per block
-// on an mbarrier (bounded waits).  DeiT-tiny, one CTA per tile -> one per head: one frame 299 -> 239 us (no
-// adapter), 314 -> 249 (three), three frames 316 -> 248; from the fourth frame on the clusters do not fit 148 SMs.
+// rows it finishes go, rounded, to the same place in every CTA of the cluster (distributed shared memory), four
+// exchanges per block on mbarriers that count the bytes (bounded waits).  DeiT-tiny, one CTA per tile -> one per
+// head: one frame 299 -> 182 us (no adapter), 314 -> 196 (three), three frames 316 -> 195; from the fourth frame on
+// the clusters do not fit 148 SMs.
 // Contractions run on mma.sync m16n8k16 (bf16 in, fp32 accumulate): with 16 rows per CTA there is no
 // 128-row tile to give to tcgen05.
 // LayerNorm uses the folded form the other kernels use: y = rstd (x W' - mean g) + b'.
@@ -148,7 +149,7 @@ struct Ctx {
     uint32_t slot, phase;      // ring position: the same in every consumer thread (and in the producer)
     uint32_t li;               // linears done so far (their vector packs alternate between two buffers)
     int share, rank;           // CTAs on this row tile (a cluster) and this one's place among them
-    uint32_t xphase;           // exchanges of rows between them so far (parity)
+    uint32_t xno;              // exchanges of rows between them so far (two barriers used in turn)
     int* status;
     volatile int* abort_flag;
 };
@@ -164,7 +165,7 @@ __device__ __forceinline__ uint32_t cfull_bar(const Ctx& cx, uint32_t b) { retur
 __device__ __forceinline__ uint32_t cempty_bar(const Ctx& cx, uint32_t b) { return bars(cx) + 176u + 8u * b; }
 __device__ __forceinline__ uint32_t kvdone_bar(const Ctx& cx, uint32_t part) { return bars(cx) + 192u + 8u * part; }
 
-__device__ __forceinline__ uint32_t xchg_bar(const Ctx& cx) { return bars(cx) + 208u; }
+__device__ __forceinline__ uint32_t xchg_bar(const Ctx& cx) { return bars(cx) + 208u + 8u * (cx.xno & 1u); }
 
 // Shared tiles: the columns of chunk i of this CTA's part of a linear, as two halves of 64 (b < 0: only one).
 // qkv: its head's keys and values, then its head's queries; other linears: the rank'th part of the outputs.
@@ -188,22 +189,35 @@ __device__ __forceinline__ uint32_t peer_addr(uint32_t addr, int rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-// a value of a row goes to this CTA's buffer, or to the same place in every CTA of the tile
-template <bool CL>
-__device__ __forceinline__ void put(const Ctx& cx, uint32_t* p, uint32_t v) {
-    if (!CL) { *p = v; return; }
-    for (int r = 0; r < cx.share; ++r)
-        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_addr(s_u32(p), r)), "r"(v) : "memory");
+// A warp's 16 x 16 part of the rows (the accumulator layout of mma: lo[q] / hi[q] = columns n0 + 8 q, + 1 of rows g and
+// g + 8, n0 = 16-aligned column + 2 t) goes to the same place in every CTA of the tile: a 4 x 4 transpose in each
+// quad makes it one 16-byte store per lane and CTA, and the stores to peers count their bytes on the peers' exchange barrier
+// themselves, so nobody waits for stores to be performed before saying so.  (4-byte stores of fp32 rows and a release: 239
+// against 182 us per frame.)
+__device__ __forceinline__ void put_rows(const Ctx& cx, bf16* buf, int ld, int n0, const uint32_t (&lo)[2], const uint32_t (&hi)[2]) {
+    const int t = cx.t;
+    const uint32_t r0 = __shfl_xor_sync(0xFFFFFFFFu, t & 1 ? lo[0] : hi[0], 1), r1 = __shfl_xor_sync(0xFFFFFFFFu, t & 1 ? lo[1] : hi[1], 1);
+    const uint32_t p0 = t & 1 ? r0 : lo[0], p1 = t & 1 ? hi[0] : r0, q0 = t & 1 ? r1 : lo[1], q1 = t & 1 ? hi[1] : r1;
+    const uint32_t e0 = __shfl_xor_sync(0xFFFFFFFFu, t & 2 ? p0 : q0, 2), e1 = __shfl_xor_sync(0xFFFFFFFFu, t & 2 ? p1 : q1, 2);
+    const uint4 v = t & 2 ? make_uint4(e0, e1, q0, q1) : make_uint4(p0, p1, e0, e1);
+    bf16* dst = buf + (cx.g + 8 * (t & 1)) * ld + (n0 - 2 * t) + 8 * (t >> 1);
+    *reinterpret_cast<uint4*>(dst) = v;
+    const uint32_t addr = s_u32(dst), bar = xchg_bar(cx);
+    for (int i = 1, r = cx.rank + 1; i < cx.share; ++i, ++r) {
+        if (r == cx.share) r = 0;
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                     ::"r"(peer_addr(addr, r)), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(peer_addr(bar, r)) : "memory");
+    }
 }
-template <bool CL>
-__device__ __forceinline__ void put(const Ctx& cx, uint2* p, uint2 v) {
-    if (!CL) { *p = v; return; }
-    for (int r = 0; r < cx.share; ++r)
-        asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(peer_addr(s_u32(p), r)), "r"(v.x), "r"(v.y) : "memory");
-}
-template <bool CL>
-__device__ __forceinline__ void put(const Ctx& cx, float2* p, float2 v) {
-    put<CL>(cx, reinterpret_cast<uint2*>(p), make_uint2(__float_as_uint(v.x), __float_as_uint(v.y)));
+// eight bytes of a row
+__device__ __forceinline__ void put_piece(const Ctx& cx, bf16* dst, uint2 v) {
+    *reinterpret_cast<uint2*>(dst) = v;
+    const uint32_t addr = s_u32(dst), bar = xchg_bar(cx);
+    for (int i = 1, r = cx.rank + 1; i < cx.share; ++i, ++r) {
+        if (r == cx.share) r = 0;
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
+                     ::"r"(peer_addr(addr, r)), "r"(v.x), "r"(v.y), "r"(peer_addr(bar, r)) : "memory");
+    }
 }
 __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
@@ -251,22 +265,25 @@ __device__ __forceinline__ void bar_wait(const Ctx& cx, uint32_t bar, uint32_t p
         }
     }
 }
-// Every consumer warp of the tile's CTAs has written its part of the rows (put) and sees the others'.  One such
-// point lies between any two uses of a buffer that the peers write, so a peer never overwrites rows still read here:
-// rows written after exchange e were last read before their reader took part in e.
+// The end of a linear (or of attention) whose `cols` columns per CTA went to all CTAs of the tile: this CTA's warps have
+// written theirs and the peers' bytes are here.  One such point lies between any two uses of a buffer that the peers
+// write, so a peer never overwrites rows still read here: rows written after exchange e were last read before their
+// reader sent its own part of e.  Bytes of exchange e + 1 may land before this CTA's last warp is through with e, hence two
+// barriers; those of e + 2 cannot.
 template <bool CL>
-__device__ __forceinline__ void rows_sync(Ctx& cx) {
-    if (!CL) { consumer_sync(); return; }
+__device__ __forceinline__ void rows_sync(Ctx& cx, int cols) {
+    if constexpr (!CL) { consumer_sync(); return; }
+    const uint32_t bar = xchg_bar(cx), parity = (cx.xno >> 1) & 1u;
     __syncwarp();
-    if (cx.lane < cx.share) {
-        asm volatile("fence.acq_rel.cluster;" ::: "memory");
-        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(peer_addr(xchg_bar(cx), cx.lane)) : "memory");
+    if (cx.lane == 0) {
+        if (cx.warp == 0) bar_expect(bar, (uint32_t)((cx.share - 1) * cols * LT_ROWS * 2));
+        else bar_arrive(bar);
     }
     const long long t0 = clock64();
     for (;;) {
         uint32_t ok;
         asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(ok) : "r"(xchg_bar(cx)), "r"(cx.xphase) : "memory");
+                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
         if (ok || *cx.abort_flag) break;
         if (clock64() - t0 > LT_WAIT_CYCLES) {
             *cx.abort_flag = 1;
@@ -274,7 +291,7 @@ __device__ __forceinline__ void rows_sync(Ctx& cx) {
             break;
         }
     }
-    cx.xphase ^= 1u;
+    ++cx.xno;
 }
 __device__ __forceinline__ void ring_advance(Ctx& cx) {
     if (++cx.slot == (uint32_t)cx.ns) { cx.slot = 0; cx.phase ^= 1u; }
@@ -629,6 +646,38 @@ __device__ void round_rows_and_stats(Ctx& cx, int d, float eps) {
     }
 }
 
+// stats[r] of the rounded rows in abuf (shared tiles: they arrive there rounded).  Half a warp per row.
+__device__ void stats_of_rows(Ctx& cx, int d, float eps) {
+    const bf16* a = reinterpret_cast<const bf16*>(cx.sm + cx.L.abuf);
+    float4* st = reinterpret_cast<float4*>(cx.sm + cx.L.stats);
+    const int n2 = d >> 6, r = 2 * cx.warp + (cx.lane >> 4), l = cx.lane & 15;
+    float2 v[12];
+    float sum = 0.f;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        v[2 * i] = v[2 * i + 1] = make_float2(0.f, 0.f);
+        if (i < n2) {
+            const uint2 u = *reinterpret_cast<const uint2*>(a + r * cx.L.lda + 4 * l + 64 * i);
+            v[2 * i] = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
+            v[2 * i + 1] = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+            sum += (v[2 * i].x + v[2 * i].y) + (v[2 * i + 1].x + v[2 * i + 1].y);
+        }
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+    const float inv_d = 1.f / (float)d, mean = sum * inv_d;
+    float sq = 0.f;
+#pragma unroll
+    for (int i = 0; i < 12; ++i)
+        if (i < 2 * n2) { const float t0 = v[i].x - mean, t1 = v[i].y - mean; sq += t0 * t0 + t1 * t1; }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) sq += __shfl_xor_sync(0xFFFFFFFFu, sq, o);
+    if (l == 0) {
+        const float rstd = rsqrtf(sq * inv_d + eps);
+        st[r] = make_float4(mean, rstd, 1.f / rstd, 0.f);
+    }
+}
+
 // CL: the cluster's CTAs (as many as heads) share one tile of 16 rows.
 template <bool CL>
 __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __grid_constant__ LatArgs args) {
@@ -644,7 +693,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
     cx.warp = threadIdx.x >> 5; cx.lane = threadIdx.x & 31; cx.g = cx.lane >> 2; cx.t = cx.lane & 3;
     cx.share = CL ? args.heads : 1;
     cx.rank = CL ? (int)(blockIdx.x % (unsigned)cx.share) : 0;
-    cx.xphase = 0;
+    cx.xno = 0;
     const int tile = CL ? (int)(blockIdx.x / (unsigned)cx.share) : (int)blockIdx.x;
     const int f = tile / args.tiles_pf, rt = tile % args.tiles_pf;     // slot, row tile
     const int frame = args.perm ? args.perm[f] : f;                                  // input / output row
@@ -667,7 +716,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
         bar_init(vfull_bar(cx), 1); bar_init(vempty_bar(cx), LT_CWARPS);
         for (int b = 0; b < 2; ++b) { bar_init(cfull_bar(cx, b), 1); bar_init(cempty_bar(cx, b), LT_CWARPS); }
         bar_init(kvdone_bar(cx, 0), LT_CWARPS); bar_init(kvdone_bar(cx, 1), LT_CWARPS);
-        if (CL) bar_init(xchg_bar(cx), LT_CWARPS * cx.share);
+        if (CL) { bar_init(xchg_bar(cx), LT_CWARPS); ++cx.xno; bar_init(xchg_bar(cx), LT_CWARPS); cx.xno = 0; }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -811,7 +860,8 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
     // ---- patch projection + positions; the CLS row
     {
         const float* cv = pack_acquire();
-        linear_rows<CL>(cx, hbuf, cx.L.ldh, args.patch_dim, d, 0, d, false, abuf, [&](int n0, float (&y)[2][4]) {
+        linear_rows<CL>(cx, hbuf, cx.L.ldh, args.patch_dim, d, 0, d, false, qbuf, [&](int n0, float (&y)[2][4]) {
+            uint32_t row[2][2];                             // [hi][q], rounded
 #pragma unroll
             for (int hi = 0; hi < 2; ++hi) {
                 const int r = cx.g + 8 * hi, tok = r0 + r;
@@ -826,13 +876,15 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                     float2 out = make_float2(0.f, 0.f);             // rows past the frame stay zero
                     if (tok == 0) out = make_float2(args.cls[n] + p[q].x, args.cls[n + 1] + p[q].y);
                     else if (tok < T) out = make_float2(y[q][2 * hi] + cv[n] + p[q].x, y[q][2 * hi + 1] + cv[n + 1] + p[q].y);
-                    put<CL>(cx, reinterpret_cast<float2*>(xres + r * d + n), out);
+                    *reinterpret_cast<float2*>(xres + r * d + n) = out;
+                    row[hi][q] = pk_bf16(out.x, out.y);
                 }
             }
+            if constexpr (CL) put_rows(cx, abuf, cx.L.lda, n0, row[0], row[1]);
         });
         pack_release();
     }
-    rows_sync<CL>(cx);
+    rows_sync<CL>(cx, LT_HD);
 
     // LoRA shrink of a linear with slab table `st` on the rows A: t[r][16 i + j] (bf16) = s_a (x A_a)
     // (folded linears: s_a ((x A' - mean c1) + c2 / rstd), the fused accumulator being scaled by rstd afterwards)
@@ -850,7 +902,9 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
         });
         consumer_sync();
     };
-    auto residual = [&](const float* cv) {
+    // x += y + b.  Shared tiles: the fp32 rows stay with the CTA that owns their columns, the others get them rounded; the
+    // first CTA of the frame's first tile also gets the CLS row behind the last block, for the heads.
+    auto residual = [&](const float* cv, bool last) {
         return [=, &cx](int n0, float (&y)[2][4]) {
             float2 x[2][2], b[2];
 #pragma unroll
@@ -859,13 +913,22 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                 x[q][0] = *reinterpret_cast<const float2*>(xres + cx.g * d + n0 + 8 * q);
                 x[q][1] = *reinterpret_cast<const float2*>(xres + (cx.g + 8) * d + n0 + 8 * q);
             }
+            uint32_t row[2][2];
 #pragma unroll
             for (int q = 0; q < 2; ++q)
 #pragma unroll
-                for (int hi = 0; hi < 2; ++hi)
-                    if (r0 + cx.g + 8 * hi < T)
-                        put<CL>(cx, reinterpret_cast<float2*>(xres + (cx.g + 8 * hi) * d + n0 + 8 * q),
-                                make_float2(x[q][hi].x + y[q][2 * hi] + b[q].x, x[q][hi].y + y[q][2 * hi + 1] + b[q].y));
+                for (int hi = 0; hi < 2; ++hi) {
+                    float2 v = x[q][hi];
+                    if (r0 + cx.g + 8 * hi < T) {
+                        v = make_float2(v.x + y[q][2 * hi] + b[q].x, v.y + y[q][2 * hi + 1] + b[q].y);
+                        *reinterpret_cast<float2*>(xres + (cx.g + 8 * hi) * d + n0 + 8 * q) = v;
+                    }
+                    row[hi][q] = pk_bf16(v.x, v.y);
+                    if (CL && last && hi == 0 && cx.g == 0)
+                        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};"
+                                     ::"r"(peer_addr(s_u32(xres + n0 + 8 * q), 0)), "f"(v.x), "f"(v.y) : "memory");
+                }
+            if constexpr (CL) put_rows(cx, abuf, cx.L.lda, n0, row[0], row[1]);
         };
     };
 
@@ -878,7 +941,8 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
         const SlabTab* st = slabtab + l * 4;
         bf16* kvb = args.kv + (size_t)(l & 1) * args.n_frames * T * 2 * d + (size_t)f * T * 2 * d;
         // ---- qkv (LayerNorm 1 folded): q stays here, k and v go to the frame's exchange buffer
-        round_rows_and_stats(cx, d, args.eps);
+        if constexpr (CL) stats_of_rows(cx, d, args.eps);
+        else round_rows_and_stats(cx, d, args.eps);
         consumer_sync();
         {
             const float* cv = pack_acquire();
@@ -1038,21 +1102,24 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                     uint2 pkd;
                     pkd.x = pk_bf16(num[0] * inv, num[1] * inv);
                     pkd.y = pk_bf16(num[2] * inv, num[3] * inv);
-                    put<CL>(cx, reinterpret_cast<uint2*>(att + r * ldatt + h * LT_HD + c4), pkd);
+                    bf16* dst = att + r * ldatt + h * LT_HD + c4;
+                    if constexpr (CL) put_piece(cx, dst, pkd);
+                    else *reinterpret_cast<uint2*>(dst) = pkd;
                 }
-                rows_sync<CL>(cx);
+                rows_sync<CL>(cx, LT_HD);
             }
         }
         // ---- proj (+ residual)
         {
             const float* cv = pack_acquire();
             shrink(st[1], att, ldatt, d, d, false, cv);
-            linear_rows<CL>(cx, att, ldatt, d, d, st[1].n, d, false, abuf, residual(cv));
+            linear_rows<CL>(cx, att, ldatt, d, d, st[1].n, d, false, hbuf, residual(cv, false));
             pack_release();
         }
-        rows_sync<CL>(cx);
+        rows_sync<CL>(cx, LT_HD);
         // ---- fc1 (LayerNorm 2 folded, GELU) and fc2 (+ residual)
-        round_rows_and_stats(cx, d, args.eps);
+        if constexpr (CL) stats_of_rows(cx, d, args.eps);
+        else round_rows_and_stats(cx, d, args.eps);
         consumer_sync();
         {
             const float* cv = pack_acquire();
@@ -1066,30 +1133,34 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                     b[q] = *reinterpret_cast<const float2*>(cv + n0 + 8 * q);
                     gs[q] = *reinterpret_cast<const float2*>(cv + N + n0 + 8 * q);
                 }
+                uint32_t lo[2], hi[2];
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
                     const int n = n0 + 8 * q;
-                    put<CL>(cx, reinterpret_cast<uint32_t*>(hbuf + cx.g * cx.L.ldh + n),
-                            pk_bf16(gelu_fit(s_lo.y * (y[q][0] - s_lo.x * gs[q].x) + b[q].x), gelu_fit(s_lo.y * (y[q][1] - s_lo.x * gs[q].y) + b[q].y)));
-                    put<CL>(cx, reinterpret_cast<uint32_t*>(hbuf + (cx.g + 8) * cx.L.ldh + n),
-                            pk_bf16(gelu_fit(s_hi.y * (y[q][2] - s_hi.x * gs[q].x) + b[q].x), gelu_fit(s_hi.y * (y[q][3] - s_hi.x * gs[q].y) + b[q].y)));
+                    lo[q] = pk_bf16(gelu_fit(s_lo.y * (y[q][0] - s_lo.x * gs[q].x) + b[q].x), gelu_fit(s_lo.y * (y[q][1] - s_lo.x * gs[q].y) + b[q].y));
+                    hi[q] = pk_bf16(gelu_fit(s_hi.y * (y[q][2] - s_hi.x * gs[q].x) + b[q].x), gelu_fit(s_hi.y * (y[q][3] - s_hi.x * gs[q].y) + b[q].y));
+                    if (!CL) {
+                        *reinterpret_cast<uint32_t*>(hbuf + cx.g * cx.L.ldh + n) = lo[q];
+                        *reinterpret_cast<uint32_t*>(hbuf + (cx.g + 8) * cx.L.ldh + n) = hi[q];
+                    }
                 }
+                if constexpr (CL) put_rows(cx, hbuf, cx.L.ldh, n0, lo, hi);
             });
             pack_release();
         }
-        rows_sync<CL>(cx);
+        rows_sync<CL>(cx, args.mlp / cx.share);
         {
             const float* cv = pack_acquire();
             shrink(st[3], hbuf, cx.L.ldh, args.mlp, d, false, cv);
-            linear_rows<CL>(cx, hbuf, cx.L.ldh, args.mlp, d, st[3].n, d, false, abuf, residual(cv));
+            linear_rows<CL>(cx, hbuf, cx.L.ldh, args.mlp, d, st[3].n, d, false, qbuf, residual(cv, l == args.layers - 1));
             pack_release();
         }
-        rows_sync<CL>(cx);
+        rows_sync<CL>(cx, LT_HD);
     }
 
+    if (CL) cluster_barrier();                                // no peer sends rows any more, aborted or not
     if (*abort_flag)
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);     // copies still in flight land before shared memory goes away
-    if (CL) cluster_barrier();                                // no peer writes here any more, aborted or not
     if (*abort_flag || rt != 0 || cx.rank != 0) return;
 
     // ---- heads on the CLS row (row 0 of the frame's first CTA): final LayerNorm, base head, adapter heads
