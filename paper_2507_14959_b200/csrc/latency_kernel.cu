@@ -20,7 +20,7 @@
 // head's queries, keys and values, attends for that head, and computes its part of the outputs of every other linear;
 // rows it finishes go, rounded, to the same place in every CTA of the cluster (distributed shared memory), four
 // exchanges per block on mbarriers that count the bytes (bounded waits).  DeiT-tiny, one CTA per tile -> one per
-// head: one frame 299 -> 182 us (no adapter), 314 -> 196 (three), three frames 316 -> 195; from the fourth frame on
+// head: one frame 299 -> 179 us (no adapter), 314 -> 193 (three), three frames 316 -> 192; from the fourth frame on
 // the clusters do not fit 148 SMs.
 // Contractions run on mma.sync m16n8k16 (bf16 in, fp32 accumulate): with 16 rows per CTA there is no
 // 128-row tile to give to tcgen05.
@@ -37,6 +37,9 @@ constexpr int LT_CTHREADS = LT_CWARPS * 32;
 constexpr int LT_THREADS = LT_CTHREADS + 64; // + the weight producer's warp + the key/value producer's warp
 constexpr int LT_BOX_BYTES = 128 * 128;      // [128 output rows][64 bf16 inputs], 128B swizzle
 constexpr int LT_SLOT_BYTES = 2 * LT_BOX_BYTES;  // a ring step: two K boxes of a chunk of outputs
+// shared tiles: a ring step is six [64 outputs][64 inputs] boxes, so that a linear is one or two steps: waiting for a slot
+// and handing it back costs a warp about 260 cycles even when the data are long there
+constexpr int LT_SLOT_SHARED = 6 * 8192;
 constexpr int LT_MAX_SLOTS = 8;
 constexpr int LT_MAX_SET = 8;
 constexpr int LT_MAX_SLABS = 8;              // active LoRA slabs of one linear
@@ -44,6 +47,7 @@ constexpr int LT_HD = 64;
 constexpr int LT_MAX_SHARE = 6;              // CTAs that share a row tile, one per head (rows of up to 384)
 constexpr int LT_KSPLIT = 4;                 // key ranges of the attention warps
 constexpr int LT_ST = 8;                     // key tiles (8 keys) of one range, at most (256 tokens)
+constexpr int LT_LDX = LT_HD + 8;            // shared tiles: row stride of a CTA's 64 fp32 columns (conflict-free)
 constexpr long long LT_WAIT_CYCLES = 4000000000ll;
 
 __device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -109,7 +113,7 @@ struct LatSmem {               // offsets (bytes) into dynamic shared memory
     int cv_floats;             // one vector pack: bias[nmax], g[nmax], c1[128], c2[128]
 };
 
-__host__ __device__ inline LatSmem lat_layout(int d, int mlp, int patch_dim, int tokens, int layers, int slots) {
+__host__ __device__ inline LatSmem lat_layout(int d, int mlp, int patch_dim, int tokens, int layers, int ring_bytes, bool shared) {
     LatSmem s;
     auto up = [](int v) { return (v + 127) & ~127; };
     const int wide = mlp > patch_dim ? mlp : patch_dim, nmax = 3 * d > mlp ? 3 * d : mlp;
@@ -118,14 +122,14 @@ __host__ __device__ inline LatSmem lat_layout(int d, int mlp, int patch_dim, int
     s.kv_bytes = ((tpad * 128 + 1023) & ~1023) + 1024;      // + 1 KB that stays zero behind the values (see the P V loop)
     s.cv_floats = 2 * nmax + 2 * LT_MAX_SLABS * PM_SLAB;
     int o = 0;
-    s.ring = o; o += slots * LT_SLOT_BYTES;                      // 1024-byte aligned, as the 128B swizzle wants
+    s.ring = o; o += ring_bytes;                      // 1024-byte aligned, as the 128B swizzle wants
     s.kbuf = o; o += s.kv_bytes;
     s.vbuf = o; o += s.kv_bytes;
-    s.xres = o; o = up(o + LT_ROWS * d * 4);
+    s.xres = o; o = up(o + (shared ? LT_ROWS * LT_LDX + d : LT_ROWS * d) * 4);       // shared: own columns, then a whole CLS row
     s.abuf = o; o = up(o + LT_ROWS * s.lda * 2);
     s.qbuf = o; o = up(o + LT_ROWS * s.ldq * 2);
     // the MLP's hidden rows (and the gathered patches); between blocks' MLPs: the attention warps' partial results
-    const int hb = LT_ROWS * s.ldh * 2, pb = LT_KSPLIT * LT_ROWS * (LT_HD + 2) * 4;
+    const int hb = LT_ROWS * s.ldh * 2, pb = (shared ? LT_CWARPS : LT_KSPLIT) * LT_ROWS * (LT_HD + 2) * 4;
     s.hbuf = o; o = up(o + (hb > pb ? hb : pb));
     s.tbuf = o; o = up(o + LT_ROWS * s.ldt * 2);
     s.stats = o; o = up(o + LT_ROWS * 16);
@@ -149,6 +153,8 @@ struct Ctx {
     uint32_t slot, phase;      // ring position: the same in every consumer thread (and in the producer)
     uint32_t li;               // linears done so far (their vector packs alternate between two buffers)
     int share, rank;           // CTAs on this row tile (a cluster) and this one's place among them
+    uint32_t slot_bytes;
+    bool ready;                // shared tiles: the next step's slot has been waited for already
     uint32_t xno;              // exchanges of rows between them so far (two barriers used in turn)
     int* status;
     volatile int* abort_flag;
@@ -194,13 +200,18 @@ __device__ __forceinline__ uint32_t peer_addr(uint32_t addr, int rank) {
 // quad makes it one 16-byte store per lane and CTA, and the stores to peers count their bytes on the peers' exchange barrier
 // themselves, so nobody waits for stores to be performed before saying so.  (4-byte stores of fp32 rows and a release: 239
 // against 182 us per frame.)
-__device__ __forceinline__ void put_rows(const Ctx& cx, bf16* buf, int ld, int n0, const uint32_t (&lo)[2], const uint32_t (&hi)[2]) {
-    const int t = cx.t;
+__device__ __forceinline__ uint4 quad_transpose(int t, const uint32_t (&lo)[2], const uint32_t (&hi)[2]) {
     const uint32_t r0 = __shfl_xor_sync(0xFFFFFFFFu, t & 1 ? lo[0] : hi[0], 1), r1 = __shfl_xor_sync(0xFFFFFFFFu, t & 1 ? lo[1] : hi[1], 1);
     const uint32_t p0 = t & 1 ? r0 : lo[0], p1 = t & 1 ? hi[0] : r0, q0 = t & 1 ? r1 : lo[1], q1 = t & 1 ? hi[1] : r1;
     const uint32_t e0 = __shfl_xor_sync(0xFFFFFFFFu, t & 2 ? p0 : q0, 2), e1 = __shfl_xor_sync(0xFFFFFFFFu, t & 2 ? p1 : q1, 2);
-    const uint4 v = t & 2 ? make_uint4(e0, e1, q0, q1) : make_uint4(p0, p1, e0, e1);
-    bf16* dst = buf + (cx.g + 8 * (t & 1)) * ld + (n0 - 2 * t) + 8 * (t >> 1);
+    return t & 2 ? make_uint4(e0, e1, q0, q1) : make_uint4(p0, p1, e0, e1);
+}
+// ... for row quad_row(), columns n0 + quad_col() .. + 7
+__device__ __forceinline__ int quad_row(const Ctx& cx) { return cx.g + 8 * (cx.t & 1); }
+__device__ __forceinline__ int quad_col(const Ctx& cx) { return 8 * (cx.t >> 1) - 2 * cx.t; }
+__device__ __forceinline__ void put_rows(const Ctx& cx, bf16* buf, int ld, int n0, const uint32_t (&lo)[2], const uint32_t (&hi)[2]) {
+    const uint4 v = quad_transpose(cx.t, lo, hi);
+    bf16* dst = buf + quad_row(cx) * ld + n0 + quad_col(cx);
     *reinterpret_cast<uint4*>(dst) = v;
     const uint32_t addr = s_u32(dst), bar = xchg_bar(cx);
     for (int i = 1, r = cx.rank + 1; i < cx.share; ++i, ++r) {
@@ -265,13 +276,20 @@ __device__ __forceinline__ void bar_wait(const Ctx& cx, uint32_t bar, uint32_t p
         }
     }
 }
+// the vectors and the first step of the next linear
+__device__ __forceinline__ void linear_ready(Ctx& cx) {
+    bar_wait(cx, cfull_bar(cx, cx.li & 1u), (cx.li >> 1) & 1u);
+    bar_wait(cx, full_bar(cx, cx.slot), cx.phase);
+    cx.ready = true;
+}
 // The end of a linear (or of attention) whose `cols` columns per CTA went to all CTAs of the tile: this CTA's warps have
 // written theirs and the peers' bytes are here.  One such point lies between any two uses of a buffer that the peers
 // write, so a peer never overwrites rows still read here: rows written after exchange e were last read before their
 // reader sent its own part of e.  Bytes of exchange e + 1 may land before this CTA's last warp is through with e, hence two
 // barriers; those of e + 2 cannot.
+// While the bytes are on their way the warps wait for the next linear's vectors and first step (`more`: there is one).
 template <bool CL>
-__device__ __forceinline__ void rows_sync(Ctx& cx, int cols) {
+__device__ __forceinline__ void rows_sync(Ctx& cx, int cols, bool more) {
     if constexpr (!CL) { consumer_sync(); return; }
     const uint32_t bar = xchg_bar(cx), parity = (cx.xno >> 1) & 1u;
     __syncwarp();
@@ -279,6 +297,7 @@ __device__ __forceinline__ void rows_sync(Ctx& cx, int cols) {
         if (cx.warp == 0) bar_expect(bar, (uint32_t)((cx.share - 1) * cols * LT_ROWS * 2));
         else bar_arrive(bar);
     }
+    if (more) linear_ready(cx);
     const long long t0 = clock64();
     for (;;) {
         uint32_t ok;
@@ -298,8 +317,9 @@ __device__ __forceinline__ void ring_advance(Ctx& cx) {
 }
 // consumer side of one ring step: wait until the slot's copies have landed / hand the slot back
 __device__ __forceinline__ uint32_t step_acquire(Ctx& cx) {
-    bar_wait(cx, full_bar(cx, cx.slot), cx.phase);
-    return s_u32(cx.sm + cx.L.ring) + cx.slot * LT_SLOT_BYTES;
+    if (!cx.ready) bar_wait(cx, full_bar(cx, cx.slot), cx.phase);
+    cx.ready = false;
+    return s_u32(cx.sm + cx.L.ring) + cx.slot * cx.slot_bytes;
 }
 __device__ __forceinline__ void step_release(Ctx& cx) {
     __syncwarp();
@@ -310,7 +330,7 @@ __device__ __forceinline__ void step_release(Ctx& cx) {
 __device__ __forceinline__ uint32_t step_claim(Ctx& cx, uint32_t bytes) {
     bar_wait(cx, empty_bar(cx, cx.slot), cx.phase ^ 1u);
     bar_expect(full_bar(cx, cx.slot), bytes);
-    return s_u32(cx.sm + cx.L.ring) + cx.slot * LT_SLOT_BYTES;
+    return s_u32(cx.sm + cx.L.ring) + cx.slot * cx.slot_bytes;
 }
 
 // What the weight producer sends for one linear, in this order (the consumers take it in the same order):
@@ -320,8 +340,9 @@ __device__ __forceinline__ uint32_t step_claim(Ctx& cx, uint32_t bytes) {
 //   for each chunk of 128 outputs, in the order of chunk_at(): K/128 steps of W^T, each two
 //   K boxes of the chunk ([64 rows][64] boxes, two per K box of a full chunk), then the chunk's rows of
 //   the active slabs' B^T ([128 rows][16] boxes, four per step).
-// Shared tiles: this CTA's chunks only, each as its halves; the B^T rows come as one [128 rows][16] box per half
-// (its second 64 rows unused), the halves 4 KB apart.
+// Shared tiles: this CTA's chunks only, in steps of up to six 8 KB boxes (a K box of a chunk = its one or two halves);
+// A^T in steps of up to 24 [16 rows][64] boxes; the B^T rows come as one [128 rows][16] box per slab and half (its second
+// 64 rows unused), up to twelve per step.
 template <bool CL>
 __device__ void produce_linear(Ctx& cx, const LatLinear* lin, const SlabTab& st, const ActiveSet& as, int rs, int slabs_max,
                                int d, bool qkv) {
@@ -345,7 +366,18 @@ __device__ void produce_linear(Ctx& cx, const LatLinear* lin, const SlabTab& st,
         }
         ++cx.li;
     }
-    if (n_sl) {
+    if (CL && n_sl) {
+        const int per = 24 / n_sl;
+        for (int kb0 = 0; kb0 < k_boxes && !*cx.abort_flag; kb0 += per) {
+            const int nb = min(per, k_boxes - kb0);
+            const uint32_t dst = step_claim(cx, (uint32_t)(nb * n_sl) * 2048u);
+            for (int b = 0; b < nb; ++b)
+                for (int i = 0; i < n_sl; ++i)
+                    tma_box(dst + (uint32_t)(b * n_sl + i) * 2048u, &lin->tm_at, (kb0 + b) * 64, as.id[st.who[i]] * rs + st.sl[i] * PM_SLAB,
+                            full_bar(cx, cx.slot));
+            ring_advance(cx);
+        }
+    } else if (n_sl) {
         for (int kb0 = 0; kb0 < k_boxes && !*cx.abort_flag; kb0 += 2) {
             const int nb = min(2, k_boxes - kb0);
             const uint32_t dst = step_claim(cx, (uint32_t)(nb * n_sl) * 2048u);
@@ -360,22 +392,22 @@ __device__ void produce_linear(Ctx& cx, const LatLinear* lin, const SlabTab& st,
         const int mine = share_chunks(cx, N, qkv);
         for (int ci = 0; ci < mine; ++ci) {
             const Halves hv = share_chunk(cx, N, d, qkv, ci);
-            const int halves = hv.b < 0 ? 1 : 2;
-            for (int kb0 = 0; kb0 < k_boxes && !*cx.abort_flag; kb0 += 2) {
-                const int nb = min(2, k_boxes - kb0);
+            const int halves = hv.b < 0 ? 1 : 2, per = 6 / halves, slabs = 12 / halves;
+            for (int kb0 = 0; kb0 < k_boxes && !*cx.abort_flag; kb0 += per) {
+                const int nb = min(per, k_boxes - kb0);
                 const uint32_t dst = step_claim(cx, (uint32_t)(nb * halves) * 8192u);
                 for (int b = 0; b < nb; ++b) {
-                    tma_box(dst + b * LT_BOX_BYTES, &lin->tm_w, (kb0 + b) * 64, hv.a, full_bar(cx, cx.slot));
-                    if (halves == 2) tma_box(dst + b * LT_BOX_BYTES + 8192u, &lin->tm_w, (kb0 + b) * 64, hv.b, full_bar(cx, cx.slot));
+                    tma_box(dst + (uint32_t)(b * halves) * 8192u, &lin->tm_w, (kb0 + b) * 64, hv.a, full_bar(cx, cx.slot));
+                    if (halves == 2) tma_box(dst + b * 16384u + 8192u, &lin->tm_w, (kb0 + b) * 64, hv.b, full_bar(cx, cx.slot));
                 }
                 ring_advance(cx);
             }
-            for (int s0 = 0; s0 < n_sl && !*cx.abort_flag; s0 += 4) {
-                const int cnt = min(4, n_sl - s0);
+            for (int s0 = 0; s0 < n_sl && !*cx.abort_flag; s0 += slabs) {
+                const int cnt = min(slabs, n_sl - s0);
                 const uint32_t dst = step_claim(cx, (uint32_t)(cnt * halves) * 4096u);
                 for (int j = 0; j < cnt; ++j) {
                     const int row = (as.id[st.who[s0 + j]] * slabs_max + st.sl[s0 + j]) * N;
-                    tma_box(dst + j * 8192u, &lin->tm_bt, 0, row + hv.a, full_bar(cx, cx.slot));
+                    tma_box(dst + (uint32_t)(j * halves) * 4096u, &lin->tm_bt, 0, row + hv.a, full_bar(cx, cx.slot));
                     if (halves == 2) tma_box(dst + j * 8192u + 4096u, &lin->tm_bt, 0, row + hv.b, full_bar(cx, cx.slot));
                 }
                 ring_advance(cx);
@@ -496,9 +528,30 @@ __device__ void linear16(Ctx& cx, const bf16* A, int lda, int K, int N, int n_sl
     }
 }
 
+// n K steps of 16 from K step k0 of a ring step: boxes of [64 inputs] `box_bytes` apart, row r of them per lane
+__device__ __forceinline__ void mma_run(const Ctx& cx, uint32_t a_row, uint32_t slot, uint32_t box_bytes, int r, int k0, int n, float (&acc)[2][2][4]) {
+    const int mi = cx.lane >> 3;
+    const uint32_t row = slot + r * 128;
+#pragma unroll 2
+    for (int i = 0; i < n; i += 2) {
+        uint32_t a[2][4], b[2][4];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int k = k0 + i + q, c = (k & 3) * 2 + (mi & 1);
+            ldsm4(a_row + k * 32, a[q][0], a[q][1], a[q][2], a[q][3]);
+            ldsm4(row + (k >> 2) * box_bytes + ((c ^ (r & 7)) << 4), b[q][0], b[q][1], b[q][2], b[q][3]);
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            mma16816(acc[0][q], a[q], b[q][0], b[q][1]);
+            mma16816(acc[1][q], a[q], b[q][2], b[q][3]);
+        }
+    }
+}
+
 // The same for the chunks of a shared tile.  A chunk of 128 columns: a warp per 16 of them, as above.  A chunk of 64:
-// four warps per K box of a step, the second four's sums added through `red` (4 KB that nothing else uses
-// meanwhile), so a K of 768 costs six box times instead of twelve.
+// four warps for each half of a step's K, the second four's sums added through `red` (4 KB that nothing else uses
+// meanwhile).
 template <typename Epi>
 __device__ void linear16_shared(Ctx& cx, const bf16* A, int lda, int K, int N, int n_sl, int d, bool qkv, void* red, Epi epi) {
     const int k_boxes = K >> 6, mine = share_chunks(cx, N, qkv), half = cx.warp >> 2, wq = cx.warp & 3, mi = cx.lane >> 3;
@@ -507,26 +560,26 @@ __device__ void linear16_shared(Ctx& cx, const bf16* A, int lda, int K, int N, i
     for (int ci = 0; ci < mine; ++ci) {
         const Halves hv = share_chunk(cx, N, d, qkv, ci);
         const bool two = hv.b >= 0;
+        const int halves = two ? 2 : 1, per = 6 / halves, slabs = 12 / halves;
         float acc[2][2][4];
         acc_zero(acc);
         const int r = (two ? cx.warp : wq) * 16 + (mi >> 1) * 8 + (cx.lane & 7);
-        for (int kb0 = 0; kb0 < k_boxes; kb0 += 2) {
-            const int nb = min(2, k_boxes - kb0);
-            const uint32_t box0 = step_acquire(cx);
-            for (int bx = two ? 0 : half; bx < (two ? nb : min(nb, half + 1)); ++bx)
-                mma_box(cx, a_base + (kb0 + bx) * 128, box0 + bx * LT_BOX_BYTES, r, acc);
+        for (int kb0 = 0; kb0 < k_boxes; kb0 += per) {
+            const int nb = min(per, k_boxes - kb0);
+            const uint32_t slot = step_acquire(cx);
+            mma_run(cx, a_base + kb0 * 128, slot, (uint32_t)halves * 8192u, r, two ? 0 : half * 2 * nb, two ? 4 * nb : 2 * nb, acc);
             step_release(cx);
         }
-        for (int s0 = 0; s0 < n_sl; s0 += 4) {
+        for (int s0 = 0; s0 < n_sl; s0 += slabs) {
             const uint32_t box = step_acquire(cx);
             if (two || half == 0) {
                 const int n = wq * 16 + ((cx.lane >> 4) & 1) * 8 + (cx.lane & 7), c = (cx.lane >> 3) & 1;
                 const uint32_t b_row = box + half * 4096 + n * 32 + ((c ^ ((n >> 2) & 1)) << 4);
-                const int cnt = min(4, n_sl - s0);
+                const int cnt = min(slabs, n_sl - s0);
                 for (int j = 0; j < cnt; ++j) {
                     uint32_t a[4], b0, b1, b2, b3;
                     ldsm4(t_row + (s0 + j) * 32, a[0], a[1], a[2], a[3]);
-                    ldsm4(b_row + j * 8192, b0, b1, b2, b3);
+                    ldsm4(b_row + j * halves * 4096, b0, b1, b2, b3);
                     mma16816(acc[0][j & 1], a, b0, b1);
                     mma16816(acc[1][j & 1], a, b2, b3);
                 }
@@ -568,14 +621,23 @@ __device__ __forceinline__ void linear_rows(Ctx& cx, const bf16* A, int lda, int
 
 // The consumers' side of a linear's shrink steps: warp i < n_sl multiplies the rows by slab i of A^T and
 // hands epi(row, i, j, v[j], v[j + 1]) its 16 x 16 result (even j).
-template <typename Epi>
+template <bool CL, typename Epi>
 __device__ void shrink16(Ctx& cx, const bf16* A, int lda, int K, int n_sl, Epi epi) {
     const int k_boxes = K >> 6;
     const uint32_t a_base = s_u32(A) + ((cx.lane & 15) * lda + (cx.lane >> 4) * 8) * 2;
     const bool active = cx.warp < n_sl;
     float acc[2][2][4];
     acc_zero(acc);
-    for (int kb0 = 0; kb0 < k_boxes; kb0 += 2) mma_step(cx, a_base + kb0 * 128, min(2, k_boxes - kb0), active, acc);
+    if (CL) {
+        const int per = 24 / n_sl, mi = cx.lane >> 3, r = cx.warp * 16 + (mi >> 1) * 8 + (cx.lane & 7);
+        for (int kb0 = 0; kb0 < k_boxes; kb0 += per) {
+            const uint32_t slot = step_acquire(cx);
+            if (active) mma_run(cx, a_base + kb0 * 128, slot, (uint32_t)n_sl * 2048u, r, 0, 4 * min(per, k_boxes - kb0), acc);
+            step_release(cx);
+        }
+    } else {
+        for (int kb0 = 0; kb0 < k_boxes; kb0 += 2) mma_step(cx, a_base + kb0 * 128, min(2, k_boxes - kb0), active, acc);
+    }
     if (active) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
@@ -688,7 +750,8 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
     }
     Ctx cx;
     cx.sm = smem;
-    cx.L = lat_layout(args.d, args.mlp, args.patch_dim, args.tokens, args.layers, args.ring_slots);
+    cx.slot_bytes = CL ? LT_SLOT_SHARED : LT_SLOT_BYTES; cx.ready = false;
+    cx.L = lat_layout(args.d, args.mlp, args.patch_dim, args.tokens, args.layers, args.ring_slots * (int)cx.slot_bytes, CL);
     cx.ns = args.ring_slots;
     cx.warp = threadIdx.x >> 5; cx.lane = threadIdx.x & 31; cx.g = cx.lane >> 2; cx.t = cx.lane & 3;
     cx.share = CL ? args.heads : 1;
@@ -700,7 +763,8 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
     const int T = args.tokens, d = args.d, r0 = rt * LT_ROWS;
     const int tpad = (T + 15) / 16 * 16;
     const int rs = args.slabs_max * PM_SLAB;
-    float* xres = reinterpret_cast<float*>(smem + cx.L.xres);
+    float* xres = reinterpret_cast<float*>(smem + cx.L.xres);    // element (r, n) at r * ldx + n - x0
+    const int ldx = CL ? LT_LDX : args.d, x0 = CL ? cx.rank * LT_HD : 0;
     bf16* abuf = reinterpret_cast<bf16*>(smem + cx.L.abuf);
     bf16* hbuf = reinterpret_cast<bf16*>(smem + cx.L.hbuf);
     bf16* qbuf = reinterpret_cast<bf16*>(smem + cx.L.qbuf);
@@ -846,10 +910,11 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
     for (int i = threadIdx.x; i < 256; i += LT_CTHREADS)
         reinterpret_cast<uint32_t*>(smem + cx.L.vbuf + cx.L.kv_bytes - 1024)[i] = 0u;
     consumer_sync();
+    if (CL) linear_ready(cx);
 
     // the vector pack of the linear the consumers are at: wait for it / hand its buffer back
     auto pack_acquire = [&]() -> const float* {
-        bar_wait(cx, cfull_bar(cx, cx.li & 1u), (cx.li >> 1) & 1u);
+        if (!CL) bar_wait(cx, cfull_bar(cx, cx.li & 1u), (cx.li >> 1) & 1u);      // shared tiles: linear_ready() has
         return reinterpret_cast<const float*>(smem + cx.L.colv) + (cx.li & 1u) * cx.L.cv_floats;
     };
     auto pack_release = [&]() {
@@ -876,7 +941,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                     float2 out = make_float2(0.f, 0.f);             // rows past the frame stay zero
                     if (tok == 0) out = make_float2(args.cls[n] + p[q].x, args.cls[n + 1] + p[q].y);
                     else if (tok < T) out = make_float2(y[q][2 * hi] + cv[n] + p[q].x, y[q][2 * hi + 1] + cv[n + 1] + p[q].y);
-                    *reinterpret_cast<float2*>(xres + r * d + n) = out;
+                    *reinterpret_cast<float2*>(xres + r * ldx + n - x0) = out;
                     row[hi][q] = pk_bf16(out.x, out.y);
                 }
             }
@@ -884,13 +949,13 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
         });
         pack_release();
     }
-    rows_sync<CL>(cx, LT_HD);
+    rows_sync<CL>(cx, LT_HD, true);
 
     // LoRA shrink of a linear with slab table `st` on the rows A: t[r][16 i + j] (bf16) = s_a (x A_a)
     // (folded linears: s_a ((x A' - mean c1) + c2 / rstd), the fused accumulator being scaled by rstd afterwards)
     auto shrink = [&](const SlabTab& st, const bf16* A, int lda, int K, int N, bool folded, const float* cv) {
         if (!st.n) return;
-        shrink16(cx, A, lda, K, st.n, [&](int r, int i, int j, float v0, float v1) {
+        shrink16<CL>(cx, A, lda, K, st.n, [&](int r, int i, int j, float v0, float v1) {
             if (folded) {
                 const float* c1 = cv + 2 * N + i * PM_SLAB + j;
                 const float* c2 = c1 + LT_MAX_SLABS * PM_SLAB;
@@ -910,8 +975,8 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 b[q] = *reinterpret_cast<const float2*>(cv + n0 + 8 * q);
-                x[q][0] = *reinterpret_cast<const float2*>(xres + cx.g * d + n0 + 8 * q);
-                x[q][1] = *reinterpret_cast<const float2*>(xres + (cx.g + 8) * d + n0 + 8 * q);
+                x[q][0] = *reinterpret_cast<const float2*>(xres + cx.g * ldx + n0 - x0 + 8 * q);
+                x[q][1] = *reinterpret_cast<const float2*>(xres + (cx.g + 8) * ldx + n0 - x0 + 8 * q);
             }
             uint32_t row[2][2];
 #pragma unroll
@@ -921,12 +986,12 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                     float2 v = x[q][hi];
                     if (r0 + cx.g + 8 * hi < T) {
                         v = make_float2(v.x + y[q][2 * hi] + b[q].x, v.y + y[q][2 * hi + 1] + b[q].y);
-                        *reinterpret_cast<float2*>(xres + (cx.g + 8 * hi) * d + n0 + 8 * q) = v;
+                        *reinterpret_cast<float2*>(xres + (cx.g + 8 * hi) * ldx + n0 - x0 + 8 * q) = v;
                     }
                     row[hi][q] = pk_bf16(v.x, v.y);
                     if (CL && last && hi == 0 && cx.g == 0)
                         asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};"
-                                     ::"r"(peer_addr(s_u32(xres + n0 + 8 * q), 0)), "f"(v.x), "f"(v.y) : "memory");
+                                     ::"r"(peer_addr(s_u32(xres + LT_ROWS * LT_LDX + n0 + 8 * q), 0)), "f"(v.x), "f"(v.y) : "memory");
                 }
             if constexpr (CL) put_rows(cx, abuf, cx.L.lda, n0, row[0], row[1]);
         };
@@ -955,18 +1020,26 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                     b[q] = *reinterpret_cast<const float2*>(cv + n0 + 8 * q);
                     gs[q] = *reinterpret_cast<const float2*>(cv + 3 * d + n0 + 8 * q);
                 }
+                uint32_t lo[2], hi[2];
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
                     const int n = n0 + 8 * q;
-                    const uint32_t lo = pk_bf16(s_lo.y * (y[q][0] - s_lo.x * gs[q].x) + b[q].x, s_lo.y * (y[q][1] - s_lo.x * gs[q].y) + b[q].y);
-                    const uint32_t hi = pk_bf16(s_hi.y * (y[q][2] - s_hi.x * gs[q].x) + b[q].x, s_hi.y * (y[q][3] - s_hi.x * gs[q].y) + b[q].y);
+                    lo[q] = pk_bf16(s_lo.y * (y[q][0] - s_lo.x * gs[q].x) + b[q].x, s_lo.y * (y[q][1] - s_lo.x * gs[q].y) + b[q].y);
+                    hi[q] = pk_bf16(s_hi.y * (y[q][2] - s_hi.x * gs[q].x) + b[q].x, s_hi.y * (y[q][3] - s_hi.x * gs[q].y) + b[q].y);
+                    if (CL) continue;
                     if (n < d) {
-                        *reinterpret_cast<uint32_t*>(qbuf + cx.g * cx.L.ldq + n) = lo;
-                        *reinterpret_cast<uint32_t*>(qbuf + (cx.g + 8) * cx.L.ldq + n) = hi;
+                        *reinterpret_cast<uint32_t*>(qbuf + cx.g * cx.L.ldq + n) = lo[q];
+                        *reinterpret_cast<uint32_t*>(qbuf + (cx.g + 8) * cx.L.ldq + n) = hi[q];
                     } else {
-                        if (r0 + cx.g < T) *reinterpret_cast<uint32_t*>(kvb + (size_t)(r0 + cx.g) * 2 * d + (n - d)) = lo;
-                        if (r0 + cx.g + 8 < T) *reinterpret_cast<uint32_t*>(kvb + (size_t)(r0 + cx.g + 8) * 2 * d + (n - d)) = hi;
+                        if (r0 + cx.g < T) *reinterpret_cast<uint32_t*>(kvb + (size_t)(r0 + cx.g) * 2 * d + (n - d)) = lo[q];
+                        if (r0 + cx.g + 8 < T) *reinterpret_cast<uint32_t*>(kvb + (size_t)(r0 + cx.g + 8) * 2 * d + (n - d)) = hi[q];
                     }
+                }
+                if constexpr (CL) {
+                    const uint4 v = quad_transpose(cx.t, lo, hi);
+                    const int r = quad_row(cx), n = n0 + quad_col(cx);
+                    if (n < d) *reinterpret_cast<uint4*>(qbuf + r * cx.L.ldq + n) = v;
+                    else if (r0 + r < T) *reinterpret_cast<uint4*>(kvb + (size_t)(r0 + r) * 2 * d + (n - d)) = v;
                 }
             });
             pack_release();
@@ -1106,7 +1179,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                     if constexpr (CL) put_piece(cx, dst, pkd);
                     else *reinterpret_cast<uint2*>(dst) = pkd;
                 }
-                rows_sync<CL>(cx, LT_HD);
+                rows_sync<CL>(cx, LT_HD, true);
             }
         }
         // ---- proj (+ residual)
@@ -1116,7 +1189,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
             linear_rows<CL>(cx, att, ldatt, d, d, st[1].n, d, false, hbuf, residual(cv, false));
             pack_release();
         }
-        rows_sync<CL>(cx, LT_HD);
+        rows_sync<CL>(cx, LT_HD, true);
         // ---- fc1 (LayerNorm 2 folded, GELU) and fc2 (+ residual)
         if constexpr (CL) stats_of_rows(cx, d, args.eps);
         else round_rows_and_stats(cx, d, args.eps);
@@ -1148,14 +1221,14 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
             });
             pack_release();
         }
-        rows_sync<CL>(cx, args.mlp / cx.share);
+        rows_sync<CL>(cx, args.mlp / cx.share, true);
         {
             const float* cv = pack_acquire();
             shrink(st[3], hbuf, cx.L.ldh, args.mlp, d, false, cv);
             linear_rows<CL>(cx, hbuf, cx.L.ldh, args.mlp, d, st[3].n, d, false, qbuf, residual(cv, l == args.layers - 1));
             pack_release();
         }
-        rows_sync<CL>(cx, LT_HD);
+        rows_sync<CL>(cx, LT_HD, l + 1 < args.layers);
     }
 
     if (CL) cluster_barrier();                                // no peer sends rows any more, aborted or not
@@ -1165,10 +1238,11 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
 
     // ---- heads on the CLS row (row 0 of the frame's first CTA): final LayerNorm, base head, adapter heads
     float* z = reinterpret_cast<float*>(smem + cx.L.hbuf);
+    const float* cls_row = CL ? xres + LT_ROWS * LT_LDX : xres;
     if (cx.warp == 0) {
         float v[12], sum = 0.f;
 #pragma unroll
-        for (int i = 0; i < 12; ++i) { const int c = cx.lane + 32 * i; v[i] = c < d ? xres[c] : 0.f; sum += v[i]; }
+        for (int i = 0; i < 12; ++i) { const int c = cx.lane + 32 * i; v[i] = c < d ? cls_row[c] : 0.f; sum += v[i]; }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
         const float mean = sum / (float)d;
@@ -1218,11 +1292,11 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
 }
 
 // the most ring slots that fit beside everything else (0: the geometry does not fit at all)
-int lat_ring_slots(int d, int mlp, int patch_dim, int tokens, int layers) {
-    const int fixed = lat_layout(d, mlp, patch_dim, tokens, layers, 0).total;
-    const int room = 227 * 1024 - fixed;
-    if (room < 2 * LT_SLOT_BYTES) return 0;
-    return room / LT_SLOT_BYTES < LT_MAX_SLOTS ? room / LT_SLOT_BYTES : LT_MAX_SLOTS;
+int lat_ring_slots(int d, int mlp, int patch_dim, int tokens, int layers, bool shared) {
+    const int room = 227 * 1024 - lat_layout(d, mlp, patch_dim, tokens, layers, 0, shared).total;
+    const int slot = shared ? LT_SLOT_SHARED : LT_SLOT_BYTES;
+    if (room < 2 * slot) return 0;
+    return room / slot < LT_MAX_SLOTS ? room / slot : LT_MAX_SLOTS;
 }
 
 // CTAs per tile of 16 rows.  One per head (each takes its head and its part of every linear's outputs, and the rows are
@@ -1259,23 +1333,30 @@ int lat_share(const LatArgs& a, size_t smem) {
 }  // namespace
 
 size_t latency_smem_bytes(int d, int mlp, int patch_dim, int tokens, int layers) {
-    const int slots = lat_ring_slots(d, mlp, patch_dim, tokens, layers);
+    const int slots = lat_ring_slots(d, mlp, patch_dim, tokens, layers, false);
     if (!slots) return (size_t)1 << 30;
-    return (size_t)lat_layout(d, mlp, patch_dim, tokens, layers, slots).total;
+    return (size_t)lat_layout(d, mlp, patch_dim, tokens, layers, slots * LT_SLOT_BYTES, false).total;
 }
 
 cudaError_t launch_latency_forward(const Launch& L, const LatArgs& a) {
-    const int slots = lat_ring_slots(a.d, a.mlp, a.patch_dim, a.tokens, a.layers);
-    if (!slots || a.layers * 4 > LT_THREADS) return cudaErrorInvalidValue;
-    const size_t smem = (size_t)lat_layout(a.d, a.mlp, a.patch_dim, a.tokens, a.layers, slots).total;
+    if (a.layers * 4 > LT_THREADS) return cudaErrorInvalidValue;
     static SmemGrant grant[2];
-    if (cudaError_t e = grant[0].ensure(latency_forward_kernel<false>, (int)smem); e != cudaSuccess) return e;
-    if (cudaError_t e = grant[1].ensure(latency_forward_kernel<true>, (int)smem); e != cudaSuccess) return e;
-    const int share = lat_share(a, smem), ctas = a.n_frames * a.tiles_pf * share;
+    int share = 1, slots = 0, smem = 0;
+    for (int shared = 1; shared >= 0; --shared) {
+        slots = lat_ring_slots(a.d, a.mlp, a.patch_dim, a.tokens, a.layers, shared != 0);
+        if (!slots) continue;
+        smem = lat_layout(a.d, a.mlp, a.patch_dim, a.tokens, a.layers, slots * (shared ? LT_SLOT_SHARED : LT_SLOT_BYTES), shared != 0).total;
+        if (cudaError_t e = shared ? grant[1].ensure(latency_forward_kernel<true>, smem) : grant[0].ensure(latency_forward_kernel<false>, smem);
+            e != cudaSuccess) return e;
+        share = shared ? lat_share(a, (size_t)smem) : 1;
+        if (!shared || share > 1) break;
+    }
+    if (!slots) return cudaErrorInvalidValue;
+    const int ctas = a.n_frames * a.tiles_pf * share;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas);
     cfg.blockDim = dim3(LT_THREADS);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = L.st;
     // the CTAs of a frame wait for one another: all of them must be resident at once
     cudaLaunchAttribute attr[2];
