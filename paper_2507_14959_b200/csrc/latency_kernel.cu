@@ -20,7 +20,7 @@
 // head's queries, keys and values, attends for that head, and computes its part of the outputs of every other linear;
 // rows it finishes go, rounded, to the same place in every CTA of the cluster (distributed shared memory), four
 // exchanges per block on mbarriers that count the bytes (bounded waits).  DeiT-tiny, one CTA per tile -> one per
-// head: one frame 299 -> 179 us (no adapter), 314 -> 193 (three), three frames 316 -> 192; from the fourth frame on
+// head: one frame 299 -> 176 us (no adapter), 314 -> 189 (three), three frames 316 -> 188; from the fourth frame on
 // the clusters do not fit 148 SMs.
 // Contractions run on mma.sync m16n8k16 (bf16 in, fp32 accumulate): with 16 rows per CTA there is no
 // 128-row tile to give to tcgen05.
@@ -859,8 +859,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                 bar_wait(cx, kvdone_bar(cx, CL ? 0 : two ? part : 1), (uint32_t)l & 1u);
                 if (*abort_flag) break;
                 asm volatile("fence.proxy.async.global;" ::: "memory");
-                __threadfence();
-                atomicAdd(counter, 1u);
+                asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
                 const unsigned int per = two ? 2u : 1u;
                 const unsigned int want = (unsigned int)args.tiles_pf * (per * (unsigned int)l + (unsigned int)part + 1u);
                 const long long t0 = clock64();
@@ -1049,18 +1048,21 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
         // Keys and values of a head are one TMA box each ([tpad rows][64 dims], 128B swizzle; rows past the
         // frame hold a neighbour's rows or zeros and are masked below).
         {
-            const int kr = cx.warp >> 1, dh = cx.warp & 1;
+            // shared tiles: eight key ranges, a warp takes all 64 dims; else four, the two warps of a pair split the dims
+            // (with the count-in above as one release: 179 -> 176 us per frame)
+            constexpr int RANGES = CL ? LT_CWARPS : LT_KSPLIT, ST = CL ? LT_ST / 2 : LT_ST, NP = CL ? 4 : 2;
+            const int kr = CL ? cx.warp : cx.warp >> 1, dh = CL ? 0 : cx.warp & 1;
             const int n_t8 = tpad / 8;
-            const int t8_lo = (n_t8 * kr) / LT_KSPLIT, t8_hi = (n_t8 * (kr + 1)) / LT_KSPLIT, n_t = t8_hi - t8_lo;   // <= LT_ST tiles
+            const int t8_lo = (n_t8 * kr) / RANGES, t8_hi = (n_t8 * (kr + 1)) / RANGES, n_t = t8_hi - t8_lo;   // <= ST tiles
             // a key tile is 8 rows of 128 bytes, so a lane's row keeps its swizzle phase (lane & 7) from tile
             // to tile: one address per k16 step (keys) or pair of dim tiles (values), plus a multiple of 1 KB
             const int l7 = cx.lane & 7, mi = cx.lane >> 3;
-            uint32_t k_addr[2], v_addr[2];
+            uint32_t k_addr[2], v_addr[NP];
 #pragma unroll
             for (int kp = 0; kp < 2; ++kp)                   // one fetch brings a tile's keys for two k16 steps (32 dims)
                 k_addr[kp] = s_u32(smem + cx.L.kbuf) + (t8_lo * 8 + l7) * 128 + (((kp * 4 + mi) ^ l7) << 4);
 #pragma unroll
-            for (int n = 0; n < 2; ++n)
+            for (int n = 0; n < NP; ++n)
                 v_addr[n] = s_u32(smem + cx.L.vbuf) + (t8_lo * 8 + (mi & 1) * 8 + l7) * 128 + (((dh * 4 + n * 2 + (mi >> 1)) ^ l7) << 4);
             float* part = reinterpret_cast<float*>(smem + cx.L.hbuf);
             for (int h = cx.rank; h < (CL ? cx.rank + 1 : args.heads); ++h, ++head_no) {
@@ -1070,28 +1072,28 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                     ldsm4(s_u32(qbuf) + ((cx.lane & 15) * cx.L.ldq + h * LT_HD + ks * 16 + (cx.lane >> 4) * 8) * 2,
                           qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3]);
                 bar_wait(cx, kfull_bar(cx), head_no & 1u);
-                float s[LT_ST][4];
+                float s[ST][4];
 #pragma unroll
-                for (int j = 0; j < LT_ST; ++j) s[j][0] = s[j][1] = s[j][2] = s[j][3] = 0.f;
+                for (int j = 0; j < ST; ++j) s[j][0] = s[j][1] = s[j][2] = s[j][3] = 0.f;
                 // tile by tile inside each k16 step: consecutive multiplications go to different accumulators
 #pragma unroll
                 for (int kp = 0; kp < 2; ++kp) {
-                    uint32_t kf[LT_ST][4];
+                    uint32_t kf[ST][4];
 #pragma unroll
-                    for (int j = 0; j < LT_ST; ++j)
+                    for (int j = 0; j < ST; ++j)
                         if (j < n_t) ldsm4(k_addr[kp] + j * 1024, kf[j][0], kf[j][1], kf[j][2], kf[j][3]);
 #pragma unroll
-                    for (int j = 0; j < LT_ST; ++j)
+                    for (int j = 0; j < ST; ++j)
                         if (j < n_t) mma16816(s[j], qa[2 * kp], kf[j][0], kf[j][1]);
 #pragma unroll
-                    for (int j = 0; j < LT_ST; ++j)
+                    for (int j = 0; j < ST; ++j)
                         if (j < n_t) mma16816(s[j], qa[2 * kp + 1], kf[j][2], kf[j][3]);
                 }
                 __syncwarp();
                 if (cx.lane == 0) bar_arrive(kempty_bar(cx));        // the next head's keys may land
                 float m_lo = -INFINITY, m_hi = -INFINITY;
 #pragma unroll
-                for (int j = 0; j < LT_ST; ++j) {
+                for (int j = 0; j < ST; ++j) {
                     const int key = (t8_lo + j) * 8 + 2 * cx.t;
                     if (j >= n_t || (t8_lo + j) * 8 + 8 > T) {       // only the frame's last tile has keys to mask
 #pragma unroll
@@ -1110,9 +1112,9 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                 m_lo *= att_scale; m_hi *= att_scale;
                 const float ms_lo = m_lo == -INFINITY ? 0.f : m_lo, ms_hi = m_hi == -INFINITY ? 0.f : m_hi;
                 float l_lo = 0.f, l_hi = 0.f;
-                uint32_t pa[LT_ST / 2][4];
+                uint32_t pa[ST / 2][4];
 #pragma unroll
-                for (int j = 0; j < LT_ST; ++j) {
+                for (int j = 0; j < ST; ++j) {
                     const float p0 = ex2(fmaf(s[j][0], att_scale, -ms_lo)), p1 = ex2(fmaf(s[j][1], att_scale, -ms_lo));
                     const float p2 = ex2(fmaf(s[j][2], att_scale, -ms_hi)), p3 = ex2(fmaf(s[j][3], att_scale, -ms_hi));
                     l_lo += p0 + p1;
@@ -1124,17 +1126,17 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                 l_lo += __shfl_xor_sync(0xFFFFFFFFu, l_lo, 2);
                 l_hi += __shfl_xor_sync(0xFFFFFFFFu, l_hi, 1);
                 l_hi += __shfl_xor_sync(0xFFFFFFFFu, l_hi, 2);
-                float o[4][4];
+                float o[2 * NP][4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) { o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f; }
+                for (int i = 0; i < 2 * NP; ++i) { o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f; }
                 bar_wait(cx, vfull_bar(cx), head_no & 1u);
                 // 16-key steps of this warp's keys.  The second tile of the last step may belong to the next
                 // range (its probabilities are 0 here) or lie behind the last key (the kilobyte of zeros)
 #pragma unroll
-                for (int kk = 0; kk < LT_ST / 2; ++kk) {
+                for (int kk = 0; kk < ST / 2; ++kk) {
                     if (2 * kk < n_t) {
 #pragma unroll
-                        for (int n = 0; n < 2; ++n) {            // pairs of 8-dim tiles
+                        for (int n = 0; n < NP; ++n) {           // pairs of 8-dim tiles
                             uint32_t b0, b1, b2, b3;
                             ldsm4t(v_addr[n] + kk * 2048, b0, b1, b2, b3);
                             mma16816(o[2 * n], pa[kk], b0, b1);
@@ -1147,7 +1149,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                 // partial results: part[range][row][0..63] = o, [64] = max, [65] = sum
                 float* pw = part + (size_t)kr * LT_ROWS * (LT_HD + 2);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
+                for (int i = 0; i < 2 * NP; ++i) {
                     const int c = dh * 32 + i * 8 + 2 * cx.t;
                     *reinterpret_cast<float2*>(pw + cx.g * (LT_HD + 2) + c) = make_float2(o[i][0], o[i][1]);
                     *reinterpret_cast<float2*>(pw + (cx.g + 8) * (LT_HD + 2) + c) = make_float2(o[i][2], o[i][3]);
@@ -1161,10 +1163,10 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                     const int r = threadIdx.x >> 4, c4 = (threadIdx.x & 15) * 4;
                     float m = -INFINITY;
 #pragma unroll
-                    for (int w = 0; w < LT_KSPLIT; ++w) m = fmaxf(m, part[(w * LT_ROWS + r) * (LT_HD + 2) + 64]);
+                    for (int w = 0; w < RANGES; ++w) m = fmaxf(m, part[(w * LT_ROWS + r) * (LT_HD + 2) + 64]);
                     float den = 0.f, num[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                    for (int w = 0; w < LT_KSPLIT; ++w) {
+                    for (int w = 0; w < RANGES; ++w) {
                         const float* pr = part + (w * LT_ROWS + r) * (LT_HD + 2);
                         const float e = pr[64] == -INFINITY ? 0.f : ex2(pr[64] - m);
                         den += e * pr[65];
