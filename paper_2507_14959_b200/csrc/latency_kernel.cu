@@ -20,7 +20,7 @@
 // head's queries, keys and values, attends for that head, and computes its part of the outputs of every other linear;
 // rows it finishes go, rounded, to the same place in every CTA of the cluster (distributed shared memory), four
 // exchanges per block on mbarriers that count the bytes (bounded waits).  DeiT-tiny, one CTA per tile -> one per
-// head: one frame 299 -> 176 us (no adapter), 314 -> 189 (three), three frames 316 -> 188; from the fourth frame on
+// head: one frame 299 -> 172 us (no adapter), 314 -> 185 (three), three frames 316 -> 184; from the fourth frame on
 // the clusters do not fit 148 SMs.
 // Contractions run on mma.sync m16n8k16 (bf16 in, fp32 accumulate): with 16 rows per CTA there is no
 // 128-row tile to give to tcgen05.
@@ -142,7 +142,7 @@ __host__ __device__ inline LatSmem lat_layout(int d, int mlp, int patch_dim, int
 
 struct ActiveSet { int n; int id[LT_MAX_SET]; int slabs[LT_MAX_SET]; float scale[LT_MAX_SET]; };
 // the LoRA slabs one linear applies to this frame: slab i belongs to set member who[i] and is its slab sl[i]
-struct SlabTab { int n; uint8_t who[LT_MAX_SLABS]; uint8_t sl[LT_MAX_SLABS]; int pad[3]; };
+struct SlabTab { int n; uint8_t who[LT_MAX_SLABS]; uint8_t sl[LT_MAX_SLABS]; int per; int pad[2]; };   // per: K boxes of A^T in a step of a shared tile
 static_assert(sizeof(SlabTab) == 32, "one table entry is 32 bytes");
 static_assert(sizeof(ActiveSet) <= 128, "the adapter set sits in the first 128 bytes of the last region");
 
@@ -176,17 +176,17 @@ __device__ __forceinline__ uint32_t xchg_bar(const Ctx& cx) { return bars(cx) + 
 // Shared tiles: the columns of chunk i of this CTA's part of a linear, as two halves of 64 (b < 0: only one).
 // qkv: its head's keys and values, then its head's queries; other linears: the rank'th part of the outputs.
 struct Halves { int a, b; };
-__device__ __forceinline__ int share_chunks(const Ctx& cx, int N, bool qkv) { return qkv ? 2 : (N / cx.share + 127) >> 7; }
-__device__ __forceinline__ Halves share_chunk(const Ctx& cx, int N, int d, bool qkv, int i) {
+// (part: outputs of the linear per CTA, passed in: a division in front of every chunk cost 2 % of a frame.)
+__device__ __forceinline__ int share_chunks(int part, bool qkv) { return qkv ? 2 : (part + 127) >> 7; }
+__device__ __forceinline__ Halves share_chunk(const Ctx& cx, int part, int d, bool qkv, int i) {
     Halves hv;
     if (qkv) {
         hv.a = (i == 0 ? d : 0) + cx.rank * LT_HD;
         hv.b = i == 0 ? 2 * d + cx.rank * LT_HD : -1;
         return hv;
     }
-    const int cols = N / cx.share;
-    hv.a = cx.rank * cols + i * 128;
-    hv.b = i * 128 + 64 < cols ? hv.a + 64 : -1;
+    hv.a = cx.rank * part + i * 128;
+    hv.b = i * 128 + 64 < part ? hv.a + 64 : -1;
     return hv;
 }
 // the same shared-memory address in CTA `rank` of the cluster
@@ -367,7 +367,7 @@ __device__ void produce_linear(Ctx& cx, const LatLinear* lin, const SlabTab& st,
         ++cx.li;
     }
     if (CL && n_sl) {
-        const int per = 24 / n_sl;
+        const int per = st.per;
         for (int kb0 = 0; kb0 < k_boxes && !*cx.abort_flag; kb0 += per) {
             const int nb = min(per, k_boxes - kb0);
             const uint32_t dst = step_claim(cx, (uint32_t)(nb * n_sl) * 2048u);
@@ -389,10 +389,10 @@ __device__ void produce_linear(Ctx& cx, const LatLinear* lin, const SlabTab& st,
         }
     }
     if (CL) {
-        const int mine = share_chunks(cx, N, qkv);
+        const int part = N / cx.share, mine = share_chunks(part, qkv);
         for (int ci = 0; ci < mine; ++ci) {
-            const Halves hv = share_chunk(cx, N, d, qkv, ci);
-            const int halves = hv.b < 0 ? 1 : 2, per = 6 / halves, slabs = 12 / halves;
+            const Halves hv = share_chunk(cx, part, d, qkv, ci);
+            const int halves = hv.b < 0 ? 1 : 2, per = halves == 2 ? 3 : 6, slabs = halves == 2 ? 6 : 12;
             for (int kb0 = 0; kb0 < k_boxes && !*cx.abort_flag; kb0 += per) {
                 const int nb = min(per, k_boxes - kb0);
                 const uint32_t dst = step_claim(cx, (uint32_t)(nb * halves) * 8192u);
@@ -553,14 +553,15 @@ __device__ __forceinline__ void mma_run(const Ctx& cx, uint32_t a_row, uint32_t 
 // four warps for each half of a step's K, the second four's sums added through `red` (4 KB that nothing else uses
 // meanwhile).
 template <typename Epi>
-__device__ void linear16_shared(Ctx& cx, const bf16* A, int lda, int K, int N, int n_sl, int d, bool qkv, void* red, Epi epi) {
-    const int k_boxes = K >> 6, mine = share_chunks(cx, N, qkv), half = cx.warp >> 2, wq = cx.warp & 3, mi = cx.lane >> 3;
+__device__ void linear16_shared(Ctx& cx, const bf16* A, int lda, int K, int part, int n_sl, int d, bool qkv, void* red, Epi epi) {
+    const int k_boxes = K >> 6, mine = share_chunks(part, qkv), half = cx.warp >> 2, wq = cx.warp & 3, mi = cx.lane >> 3;
     const uint32_t a_base = s_u32(A) + ((cx.lane & 15) * lda + (cx.lane >> 4) * 8) * 2;
     const uint32_t t_row = s_u32(cx.sm + cx.L.tbuf) + ((cx.lane & 15) * cx.L.ldt + (cx.lane >> 4) * 8) * 2;
+#pragma unroll 1
     for (int ci = 0; ci < mine; ++ci) {
-        const Halves hv = share_chunk(cx, N, d, qkv, ci);
+        const Halves hv = share_chunk(cx, part, d, qkv, ci);
         const bool two = hv.b >= 0;
-        const int halves = two ? 2 : 1, per = 6 / halves, slabs = 12 / halves;
+        const int halves = two ? 2 : 1, per = two ? 3 : 6, slabs = two ? 6 : 12;
         float acc[2][2][4];
         acc_zero(acc);
         const int r = (two ? cx.warp : wq) * 16 + (mi >> 1) * 8 + (cx.lane & 7);
@@ -614,22 +615,22 @@ __device__ void linear16_shared(Ctx& cx, const bf16* A, int lda, int K, int N, i
     }
 }
 template <bool CL, typename Epi>
-__device__ __forceinline__ void linear_rows(Ctx& cx, const bf16* A, int lda, int K, int N, int n_sl, int d, bool qkv, void* red, Epi epi) {
-    if constexpr (CL) linear16_shared(cx, A, lda, K, N, n_sl, d, qkv, red, epi);
+__device__ __forceinline__ void linear_rows(Ctx& cx, const bf16* A, int lda, int K, int N, int part, int n_sl, int d, bool qkv, void* red, Epi epi) {
+    if constexpr (CL) linear16_shared(cx, A, lda, K, part, n_sl, d, qkv, red, epi);
     else linear16(cx, A, lda, K, N, n_sl, d, qkv, epi);
 }
 
 // The consumers' side of a linear's shrink steps: warp i < n_sl multiplies the rows by slab i of A^T and
 // hands epi(row, i, j, v[j], v[j + 1]) its 16 x 16 result (even j).
 template <bool CL, typename Epi>
-__device__ void shrink16(Ctx& cx, const bf16* A, int lda, int K, int n_sl, Epi epi) {
+__device__ void shrink16(Ctx& cx, const bf16* A, int lda, int K, int n_sl, int per, Epi epi) {
     const int k_boxes = K >> 6;
     const uint32_t a_base = s_u32(A) + ((cx.lane & 15) * lda + (cx.lane >> 4) * 8) * 2;
     const bool active = cx.warp < n_sl;
     float acc[2][2][4];
     acc_zero(acc);
     if (CL) {
-        const int per = 24 / n_sl, mi = cx.lane >> 3, r = cx.warp * 16 + (mi >> 1) * 8 + (cx.lane & 7);
+        const int mi = cx.lane >> 3, r = cx.warp * 16 + (mi >> 1) * 8 + (cx.lane & 7);
         for (int kb0 = 0; kb0 < k_boxes; kb0 += per) {
             const uint32_t slot = step_acquire(cx);
             if (active) mma_run(cx, a_base + kb0 * 128, slot, (uint32_t)n_sl * 2048u, r, 0, 4 * min(per, k_boxes - kb0), acc);
@@ -827,6 +828,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
                 for (int s = 0; s < as->slabs[i] && st.n < LT_MAX_SLABS; ++s) { st.who[st.n] = (uint8_t)i; st.sl[st.n] = (uint8_t)s; ++st.n; }
             }
         }
+        st.per = st.n ? 24 / st.n : 24;
         slabtab[threadIdx.x] = st;
     }
     __syncthreads();
@@ -924,7 +926,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
     // ---- patch projection + positions; the CLS row
     {
         const float* cv = pack_acquire();
-        linear_rows<CL>(cx, hbuf, cx.L.ldh, args.patch_dim, d, 0, d, false, qbuf, [&](int n0, float (&y)[2][4]) {
+        linear_rows<CL>(cx, hbuf, cx.L.ldh, args.patch_dim, d, LT_HD, 0, d, false, qbuf, [&](int n0, float (&y)[2][4]) {
             uint32_t row[2][2];                             // [hi][q], rounded
 #pragma unroll
             for (int hi = 0; hi < 2; ++hi) {
@@ -954,7 +956,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
     // (folded linears: s_a ((x A' - mean c1) + c2 / rstd), the fused accumulator being scaled by rstd afterwards)
     auto shrink = [&](const SlabTab& st, const bf16* A, int lda, int K, int N, bool folded, const float* cv) {
         if (!st.n) return;
-        shrink16<CL>(cx, A, lda, K, st.n, [&](int r, int i, int j, float v0, float v1) {
+        shrink16<CL>(cx, A, lda, K, st.n, st.per, [&](int r, int i, int j, float v0, float v1) {
             if (folded) {
                 const float* c1 = cv + 2 * N + i * PM_SLAB + j;
                 const float* c2 = c1 + LT_MAX_SLABS * PM_SLAB;
@@ -997,6 +999,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
     };
 
     const float att_scale = 0.125f * 1.4426950408889634f;  // 1/sqrt(64) * log2(e)
+    const int mlp_part = CL ? args.mlp / cx.share : args.mlp;    // a CTA's columns of the hidden layer
     uint32_t head_no = 0;                                    // heads attended so far (all blocks)
     // the attended rows; shared tiles: beside this head's queries, since a peer may be done while qkv still reads abuf here
     bf16* att = CL ? qbuf : abuf;
@@ -1012,7 +1015,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
             const float* cv = pack_acquire();
             shrink(st[0], abuf, cx.L.lda, d, 3 * d, true, cv);
             const float4 s_lo = stats[cx.g], s_hi = stats[cx.g + 8];
-            linear_rows<CL>(cx, abuf, cx.L.lda, d, 3 * d, st[0].n, d, true, hbuf, [&](int n0, float (&y)[2][4]) {
+            linear_rows<CL>(cx, abuf, cx.L.lda, d, 3 * d, LT_HD, st[0].n, d, true, hbuf, [&](int n0, float (&y)[2][4]) {
                 float2 b[2], gs[2];
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
@@ -1188,7 +1191,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
         {
             const float* cv = pack_acquire();
             shrink(st[1], att, ldatt, d, d, false, cv);
-            linear_rows<CL>(cx, att, ldatt, d, d, st[1].n, d, false, hbuf, residual(cv, false));
+            linear_rows<CL>(cx, att, ldatt, d, d, LT_HD, st[1].n, d, false, hbuf, residual(cv, false));
             pack_release();
         }
         rows_sync<CL>(cx, LT_HD, true);
@@ -1201,7 +1204,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
             const int N = args.mlp;
             shrink(st[2], abuf, cx.L.lda, d, N, true, cv);
             const float4 s_lo = stats[cx.g], s_hi = stats[cx.g + 8];
-            linear_rows<CL>(cx, abuf, cx.L.lda, d, N, st[2].n, d, false, nullptr, [&](int n0, float (&y)[2][4]) {
+            linear_rows<CL>(cx, abuf, cx.L.lda, d, N, mlp_part, st[2].n, d, false, nullptr, [&](int n0, float (&y)[2][4]) {
                 float2 b[2], gs[2];
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
@@ -1223,11 +1226,11 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
             });
             pack_release();
         }
-        rows_sync<CL>(cx, args.mlp / cx.share, true);
+        rows_sync<CL>(cx, mlp_part, true);
         {
             const float* cv = pack_acquire();
             shrink(st[3], hbuf, cx.L.ldh, args.mlp, d, false, cv);
-            linear_rows<CL>(cx, hbuf, cx.L.ldh, args.mlp, d, st[3].n, d, false, qbuf, residual(cv, l == args.layers - 1));
+            linear_rows<CL>(cx, hbuf, cx.L.ldh, args.mlp, d, LT_HD, st[3].n, d, false, qbuf, residual(cv, l == args.layers - 1));
             pack_release();
         }
         rows_sync<CL>(cx, LT_HD, l + 1 < args.layers);
