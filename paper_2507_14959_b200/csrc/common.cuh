@@ -259,7 +259,7 @@ struct LatArgs {
     const int* rank;
     const float* scale;
     bf16* kv;                  // [2][F * tokens][2 d]: keys and values of the blocks, two buffers used in turn
-    unsigned int* bar;         // [F] arrival counters of the frames' CTAs (cleared before every launch)
+    unsigned int* bar;         // arrival counters: [F] of the frames' CTAs, or [F, heads] (cleared before every launch)
     float *scores_out, *base_out;          // [F, n_classes]
     int* status;
 };
@@ -267,8 +267,8 @@ struct LatArgs {
 // bytes of dynamic shared memory the kernel takes for this geometry (more than any device has if it cannot run)
 size_t latency_smem_bytes(int d, int mlp, int patch_dim, int tokens, int layers);
 // One launch for the whole forward of a.n_frames frames; a.status is taken from L.  The grid
-// (n_frames * tiles_pf CTAs, one per SM) must be resident at once: a cooperative launch, which fails
-// with an error instead of starting if it cannot be.
+// (n_frames * tiles_pf CTAs or clusters of one CTA per head, one CTA per SM) must be resident at once: a
+// cooperative launch, which fails with an error instead of starting if it cannot be.
 cudaError_t launch_latency_forward(const Launch& L, const LatArgs& a);
 
 // Launch with programmatic stream serialization (the kernel may start once every CTA of the one before it on the
