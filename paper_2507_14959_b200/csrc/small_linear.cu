@@ -270,7 +270,11 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                     }
                     if (++stage == STG) { stage = 0; phase ^= 1u; }
                 }
-                if (++stage == STG) { stage = 0; phase ^= 1u; }           // the group's B slabs (the other thread's)
+                // The group's B slabs are the other thread's, but this one waits for their stage too: a parity wait tells
+                // only neighbouring uses apart, and in a ring of one stage the next group's wait would be satisfied by
+                // the use before the B slabs.
+                if (ok && g + 1 < n_groups) ok = mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, args.status);
+                if (++stage == STG) { stage = 0; phase ^= 1u; }
             }
         }
     } else if (warp == 2) {

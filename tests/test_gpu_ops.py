@@ -332,6 +332,41 @@ def test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, 
     lin.close()
 
 
+@pytest.mark.parametrize("frames,rank,what", [(1, 16, "64-wide, K in four"), (1, 64, "64-wide, K in four"), (12, 64, "256-wide, K in two")])
+def test_lora_linear_ring_of_one_stage(frames, rank, what):
+    """The few-row kernel's ring holds a single stage where a group of eight slabs and the exchange of partial sums take
+    the rest of the shared memory; further groups of slabs then follow through that one stage.  Eight adapters on every
+    frame: one to eight groups per tile.  Several calls in a row, against float64 sums of the same bf16 inputs; tolerance as
+    for the other linears."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    k_in, n_out, tokens, n_ad, rows = 3072, 768, 197, 16, frames * 197
+    gen = torch.Generator(device="cuda").manual_seed(frames + rank)
+
+    def draw(shape, std):
+        return (torch.randn(shape, generator=gen, device="cuda") * std).bfloat16()
+    x, res, w, b = draw((rows, k_in), 1.0), draw((rows, n_out), 1.0), draw((k_in, n_out), 0.02), draw((n_out,), 0.02)
+    A = [draw((k_in, rank), 0.02) for _ in range(n_ad)]
+    B = [draw((rank, n_out), 0.02) for _ in range(n_ad)]
+    sets = [list(range(f % 2, n_ad, 2)) for f in range(frames)]
+    off, ids = wl.sets_to_csr(sets)
+    host = lambda t: t.float().cpu().numpy()  # noqa: E731
+    lin = binding.Linear(host(w), host(b), max_adapters=n_ad, max_rank=rank, max_set=8, max_frames=frames, tokens=tokens, epilogue=2)
+    for a in range(n_ad):
+        lin.register(a, rank, 1.0, host(A[a]), host(B[a]))
+    y = torch.full((rows, n_out), float("nan"), device="cuda", dtype=torch.bfloat16)
+    for _ in range(4):
+        lin.forward(x, frames, off, ids, y, residual=res)
+    assert lin.status() == 0
+    want = x.double() @ w.double() + b.double() + res.double()
+    for f, s in enumerate(sets):
+        r = slice(f * tokens, (f + 1) * tokens)
+        for a in s:
+            want[r] += (x[r].double() @ A[a].double()) @ B[a].double()
+    np.testing.assert_allclose(to_np(y), want.cpu().numpy(), **TOL[0])
+    lin.close()
+
+
 @pytest.mark.parametrize("frames,tokens,heads", [(1, 1, 1), (2, 16, 3), (1, 17, 2), (3, 49, 1), (1, 208, 12), (49, 33, 1),     # a few pairs
                                                  (50, 33, 1), (60, 1, 1), (20, 197, 3), (17, 208, 4), (13, 129, 12)])           # the pipelined kernel
 def test_attention_of_one_key_block_on_both_sides_of_the_pair_limit(frames, tokens, heads):
