@@ -12,7 +12,8 @@
 //     requested before the kernel waits for it (programmatic dependent launch);
 //   - split K (long K, narrow output): each CTA of the cluster makes a partial tile, its own partial t and
 //     expand included (the expand is linear in t); the partials are exchanged through distributed shared memory
-//     and every CTA sums and stores BN / S columns.
+//     and every CTA sums and stores BN / S columns.  A partial t enters the expand as two bf16 parts (16 significant
+//     bits, two MMAs per slab): rounded to one, shares that cancel would leave their rounding in the sum.
 // One 197-token frame of width 768, rank-16 adapters, back to back, against shrink + pair GEMM: qkv 7.3 (13.4) us,
 // proj 7.3 (14.5), fc1 7.9 (14.6), fc2 10.1 (26.9); eight frames: 13.6 (15.6), 10.9 (16.0), 20.3 (20.9), 18.6 (31.1).
 // Warp roles: 0 = x / W copies, 1 = tensor memory + MMA, 2 = adapter copies, 3 = slab list, 4..11 = statistics, t, epilogue.
@@ -67,6 +68,10 @@ struct SmallArgs {
     int* status;
     int work_bytes;                                    // ring + t
 };
+
+// bytes of a slab's t in shared memory (its second part, if any, follows those of the whole group)
+template <int S>
+__host__ __device__ constexpr int t_bytes() { return S > 1 ? 2 * T_SLAB : T_SLAB; }
 
 template <int BN, int S>
 __host__ __device__ constexpr int recv_bytes() { return S > 1 ? (S - 1) * BM * (BN / S) * 4 : 0; }
@@ -229,8 +234,8 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     const int n_groups = na == 0 ? 1 : (na + GROUP - 1) / GROUP;
     const int per_group = min(na, GROUP);
     const int stage_bytes = X_BYTES + W_BYTES + per_group * A_SLAB;
-    const uint32_t t_s = base + (uint32_t)(args.work_bytes - per_group * T_SLAB);
-    const int STG = min(MAX_STAGES, (args.work_bytes - per_group * T_SLAB) / stage_bytes);
+    const uint32_t t_s = base + (uint32_t)(args.work_bytes - per_group * t_bytes<S>());
+    const int STG = min(MAX_STAGES, (args.work_bytes - per_group * t_bytes<S>()) / stage_bytes);
     const bool usable = (base & 1023u) == 0;       // swizzled operands need a 1024-byte aligned window
     if (!usable && threadIdx.x == 0) atomicCAS(args.status, 0, (int)PM_ERR_CUDA);
 
@@ -348,8 +353,11 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t sb = base + stage * stage_bytes;
-                for (int i = 0; i < cnt; ++i)
+                for (int i = 0; i < cnt; ++i) {
                     umma_bf16(tmem_base, smem_desc(t_s + i * T_SLAB, 32), smem_desc(sb + i * B_SLAB, 32), idesc, 1u);
+                    if constexpr (S > 1)
+                        umma_bf16(tmem_base, smem_desc(t_s + (per_group + i) * T_SLAB, 32), smem_desc(sb + i * B_SLAB, 32), idesc, 1u);
+                }
                 umma_commit(empty_bar(stage));
                 if (++stage == STG) { stage = 0; phase ^= 1u; }
             }
@@ -462,16 +470,28 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                     for (int j = 0; j < PM_SLAB; ++j)
                         v[j] = __float_as_uint(fmaf(-st.x, c[j], __uint_as_float(v[j])) + inv_rstd * c[PM_SLAB + j]);
                 }
-                uint4 o[2];
-                uint32_t* ow = reinterpret_cast<uint32_t*>(o);
-#pragma unroll
-                for (int j = 0; j < PM_SLAB; j += 2)
-                    ow[j >> 1] = pack_bf16(__uint_as_float(v[j]) * sc, __uint_as_float(v[j + 1]) * sc);
                 // K-major operand with 32-byte rows, 32B swizzle: 16-byte chunk c of row r sits at c ^ bit 2 of r
                 const uint32_t dst = t_s + (uint32_t)(i * T_SLAB + r * 32);
                 const uint32_t x = (uint32_t)((r >> 2) & 1) << 4;
+                uint4 o[2];
+                uint32_t* ow = reinterpret_cast<uint32_t*>(o);
+#pragma unroll
+                for (int j = 0; j < PM_SLAB; j += 2) {
+                    const float t0 = __uint_as_float(v[j]) * sc, t1 = __uint_as_float(v[j + 1]) * sc;
+                    ow[j >> 1] = pack_bf16(t0, t1);
+                    if constexpr (S > 1) {             // what the rounding leaves
+                        v[j] = __float_as_uint(t0 - __uint_as_float(ow[j >> 1] << 16));
+                        v[j + 1] = __float_as_uint(t1 - __uint_as_float(ow[j >> 1] & 0xFFFF0000u));
+                    }
+                }
                 st_shared_v4(dst + x, o[0]);
                 st_shared_v4(dst + (x ^ 16u), o[1]);
+                if constexpr (S > 1) {
+#pragma unroll
+                    for (int j = 0; j < PM_SLAB; j += 2) ow[j >> 1] = pack_bf16(__uint_as_float(v[j]), __uint_as_float(v[j + 1]));
+                    st_shared_v4(dst + (uint32_t)(per_group * T_SLAB) + x, o[0]);
+                    st_shared_v4(dst + (uint32_t)(per_group * T_SLAB) + (x ^ 16u), o[1]);
+                }
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             tc_fence_before();
@@ -569,7 +589,7 @@ cudaError_t launch(const Launch& L, const Maps& t, SmallArgs a, int tiles) {
     constexpr int OTHER = recv_bytes<BN, S>() + (int)sizeof(Tail);
     constexpr int WORK = (227 * 1024 - OTHER) / 1024 * 1024;
     // a full group of slabs leaves at least one stage, and its B slabs fit one
-    static_assert((WORK - GROUP * T_SLAB) / (kps_of(BN) * (A_BLOCK + BN * BK * 2 + GROUP * PM_SLAB * BK * 2)) >= 1, "ring");
+    static_assert((WORK - GROUP * t_bytes<S>()) / (kps_of(BN) * (A_BLOCK + BN * BK * 2 + GROUP * PM_SLAB * BK * 2)) >= 1, "ring");
     static_assert(GROUP * BN * PM_SLAB * 2 <= kps_of(BN) * (A_BLOCK + BN * BK * 2 + GROUP * PM_SLAB * BK * 2), "B slabs");
     static SmemGrant grant;
     if (cudaError_t e = grant.ensure(small_linear_kernel<BN, EPI, LNF, S>, WORK + OTHER); e != cudaSuccess) return e;

@@ -367,6 +367,36 @@ def test_lora_linear_ring_of_one_stage(frames, rank, what):
     lin.close()
 
 
+@pytest.mark.parametrize("frames,what", [(1, "64-wide, K in four"), (2, "128-wide, K in four"), (4, "128-wide, K in two"),
+                                         (8, "192-wide, K in two"), (12, "256-wide, K in two"), (33, "shrink with K in two")])
+def test_lora_intermediate_of_a_split_k_is_not_rounded_share_by_share(frames, what):
+    """t = s x A whose K shares cancel: x is 64 times as large on one part of each half of K and the halves take most of it
+    back.  W = 0, so the output is t B.  Root mean square of the error against float64, relative to that of the
+    output: one rounding of t and one of the output to bf16, 2^-9 each at most, give below 2^-8; shares rounded
+    by themselves would leave about 64 * 2^-9."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    k_in, n_out, tokens, rank, rows = 3072, 768, 197, 16, frames * 197
+    gen = torch.Generator(device="cuda").manual_seed(frames)
+
+    def draw(shape, std):
+        return (torch.randn(shape, generator=gen, device="cuda") * std).bfloat16()
+    x, A, B = draw((rows, k_in), 1.0), draw((k_in, rank), 0.02), draw((rank, n_out), 0.02)
+    big = draw((rows, 768), 64.0)
+    A[1536:2304] = A[:768]
+    x[:, :768], x[:, 1536:2304] = big, (x[:, 1536:2304].float() - big.float()).bfloat16()
+    lin = binding.Linear(np.zeros((k_in, n_out), np.float32), np.zeros(n_out, np.float32), max_adapters=1, max_rank=rank, max_set=1,
+                         max_frames=frames, tokens=tokens, epilogue=2)
+    lin.register(0, rank, 1.0, A.float().cpu().numpy(), B.float().cpu().numpy())
+    y = torch.full((rows, n_out), float("nan"), device="cuda", dtype=torch.bfloat16)
+    off, ids = wl.sets_to_csr([[0]] * frames)
+    lin.forward(x, frames, off, ids, y, residual=torch.zeros_like(y))
+    assert lin.status() == 0
+    want = (x.double() @ A.double()) @ B.double()
+    assert float((y.double() - want).norm() / want.norm()) < 2.0 ** -8
+    lin.close()
+
+
 @pytest.mark.parametrize("frames,tokens,heads", [(1, 1, 1), (2, 16, 3), (1, 17, 2), (3, 49, 1), (1, 208, 12), (49, 33, 1),     # a few pairs
                                                  (50, 33, 1), (60, 1, 1), (20, 197, 3), (17, 208, 4), (13, 129, 12)])           # the pipelined kernel
 def test_attention_of_one_key_block_on_both_sides_of_the_pair_limit(frames, tokens, heads):
