@@ -6,7 +6,8 @@
 //   - the tile is the narrowest that fits the SMs in one wave: many CTAs, each with little to fetch;
 //   - the shrink MMAs ride on the K loop's own x stages (their accumulator sits beside the tile's in tensor
 //     memory) and the epilogue warps take the LayerNorm statistics from the same stages: one pass over x;
-//   - t goes from tensor memory to shared memory and straight into the expand MMAs;
+//   - t stays in tensor memory: rounded in place of its accumulator columns, it is the expand MMAs' A operand there, and
+//     the shared memory is the ring's;
 //   - the copies are issued by two threads (x and W; adapter slabs), since issuing is a serial cost;
 //   - weights, adapter slabs, plan entries, bias and LayerNorm vectors do not depend on the kernel before: they are
 //     requested before the kernel waits for it (programmatic dependent launch);
@@ -34,7 +35,6 @@ constexpr int MAX_STAGES = 8;
 constexpr int GROUP = 8;                               // slabs of one pass over x: 128 accumulator columns
 constexpr int LIST = 64;                               // slabs a tile may use
 constexpr int A_BLOCK = BM * BK * 2;                   // 16 KB: one K block of the tile's rows
-constexpr int T_SLAB = BM * PM_SLAB * 2;               // 4 KB
 
 constexpr int WIDTHS[PM_SMALL_WIDTHS] = {64, 128, 192, 256};
 __host__ __device__ constexpr int kps_of(int bn) { return bn == 64 ? 2 : 1; }       // K blocks per stage: two where the MMAs of one are shorter than its issue
@@ -66,12 +66,8 @@ struct SmallArgs {
     const float *ln_g, *ln_c1, *ln_c2;
     float ln_eps;
     int* status;
-    int work_bytes;                                    // ring + t
+    int ring_bytes;
 };
-
-// bytes of a slab's t in shared memory (its second part, if any, follows those of the whole group)
-template <int S>
-__host__ __device__ constexpr int t_bytes() { return S > 1 ? 2 * T_SLAB : T_SLAB; }
 
 template <int BN, int S>
 __host__ __device__ constexpr int recv_bytes() { return S > 1 ? (S - 1) * BM * (BN / S) * 4 : 0; }
@@ -164,8 +160,8 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     constexpr int EMPTY_COUNT = LNF ? 1 + EW : 1;      // MMA commit, and the statistics' readers
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t base = smem_u32(smem);
-    const uint32_t recv_s = base + (uint32_t)args.work_bytes;
-    Tail& tail = *reinterpret_cast<Tail*>(smem + args.work_bytes + recv_bytes<BN, S>());
+    const uint32_t recv_s = base + (uint32_t)args.ring_bytes;
+    Tail& tail = *reinterpret_cast<Tail*>(smem + args.ring_bytes + recv_bytes<BN, S>());
     const uint32_t bars = smem_u32(tail.bars);
     auto full_bar = [&](int s) { return bars + 8u * s; };              // both copying threads' bytes of a stage
     auto empty_bar = [&](int s) { return bars + 8u * (MAX_STAGES + s); };
@@ -234,8 +230,7 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     const int n_groups = na == 0 ? 1 : (na + GROUP - 1) / GROUP;
     const int per_group = min(na, GROUP);
     const int stage_bytes = X_BYTES + W_BYTES + per_group * A_SLAB;
-    const uint32_t t_s = base + (uint32_t)(args.work_bytes - per_group * t_bytes<S>());
-    const int STG = min(MAX_STAGES, (args.work_bytes - per_group * t_bytes<S>()) / stage_bytes);
+    const int STG = min(MAX_STAGES, args.ring_bytes / stage_bytes);
     const bool usable = (base & 1023u) == 0;       // swizzled operands need a 1024-byte aligned window
     if (!usable && threadIdx.x == 0) atomicCAS(args.status, 0, (int)PM_ERR_CUDA);
 
@@ -276,8 +271,8 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                     if (++stage == STG) { stage = 0; phase ^= 1u; }
                 }
                 // The group's B slabs are the other thread's, but this one waits for their stage too: a parity wait tells
-                // only neighbouring uses apart, and in a ring of one stage the next group's wait would be satisfied by
-                // the use before the B slabs.
+                // only neighbouring uses apart, and in a ring of one stage the next group's wait would be satisfied
+                // by the use before the B slabs.
                 if (ok && g + 1 < n_groups) ok = mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, args.status);
                 if (++stage == STG) { stage = 0; phase ^= 1u; }
             }
@@ -354,9 +349,8 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                 tc_fence_after();
                 const uint32_t sb = base + stage * stage_bytes;
                 for (int i = 0; i < cnt; ++i) {
-                    umma_bf16(tmem_base, smem_desc(t_s + i * T_SLAB, 32), smem_desc(sb + i * B_SLAB, 32), idesc, 1u);
-                    if constexpr (S > 1)
-                        umma_bf16(tmem_base, smem_desc(t_s + (per_group + i) * T_SLAB, 32), smem_desc(sb + i * B_SLAB, 32), idesc, 1u);
+                    umma_bf16_ts(tmem_base, t_tmem + i * PM_SLAB, smem_desc(sb + i * B_SLAB, 32), idesc, 1u);
+                    if constexpr (S > 1) umma_bf16_ts(tmem_base, t_tmem + i * PM_SLAB + PM_SLAB / 2, smem_desc(sb + i * B_SLAB, 32), idesc, 1u);
                 }
                 umma_commit(empty_bar(stage));
                 if (++stage == STG) { stage = 0; phase ^= 1u; }
@@ -470,30 +464,19 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                     for (int j = 0; j < PM_SLAB; ++j)
                         v[j] = __float_as_uint(fmaf(-st.x, c[j], __uint_as_float(v[j])) + inv_rstd * c[PM_SLAB + j]);
                 }
-                // K-major operand with 32-byte rows, 32B swizzle: 16-byte chunk c of row r sits at c ^ bit 2 of r
-                const uint32_t dst = t_s + (uint32_t)(i * T_SLAB + r * 32);
-                const uint32_t x = (uint32_t)((r >> 2) & 1) << 4;
-                uint4 o[2];
-                uint32_t* ow = reinterpret_cast<uint32_t*>(o);
+                // over the slab's own accumulator columns: a row's 16 values as 8 columns of bf16 pairs, then (K split) what the
+                // rounding leaves of them as 8 more
+                uint32_t o[PM_SLAB];
 #pragma unroll
                 for (int j = 0; j < PM_SLAB; j += 2) {
                     const float t0 = __uint_as_float(v[j]) * sc, t1 = __uint_as_float(v[j + 1]) * sc;
-                    ow[j >> 1] = pack_bf16(t0, t1);
-                    if constexpr (S > 1) {             // what the rounding leaves
-                        v[j] = __float_as_uint(t0 - __uint_as_float(ow[j >> 1] << 16));
-                        v[j + 1] = __float_as_uint(t1 - __uint_as_float(ow[j >> 1] & 0xFFFF0000u));
-                    }
+                    const uint32_t hi = o[j >> 1] = pack_bf16(t0, t1);
+                    o[(PM_SLAB + j) >> 1] = pack_bf16(t0 - __uint_as_float(hi << 16), t1 - __uint_as_float(hi & 0xFFFF0000u));
                 }
-                st_shared_v4(dst + x, o[0]);
-                st_shared_v4(dst + (x ^ 16u), o[1]);
-                if constexpr (S > 1) {
-#pragma unroll
-                    for (int j = 0; j < PM_SLAB; j += 2) ow[j >> 1] = pack_bf16(__uint_as_float(v[j]), __uint_as_float(v[j + 1]));
-                    st_shared_v4(dst + (uint32_t)(per_group * T_SLAB) + x, o[0]);
-                    st_shared_v4(dst + (uint32_t)(per_group * T_SLAB) + (x ^ 16u), o[1]);
-                }
+                if constexpr (S > 1) tmem_st16(t_lane + (uint32_t)(i * PM_SLAB), o);
+                else tmem_st8(t_lane + (uint32_t)(i * PM_SLAB), o);
             }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            tmem_st_wait();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(tready_bar);
@@ -587,15 +570,15 @@ struct Maps { CUtensorMap x, w, bt, at; };
 template <int BN, int EPI, bool LNF = false, int S = 1>
 cudaError_t launch(const Launch& L, const Maps& t, SmallArgs a, int tiles) {
     constexpr int OTHER = recv_bytes<BN, S>() + (int)sizeof(Tail);
-    constexpr int WORK = (227 * 1024 - OTHER) / 1024 * 1024;
-    // a full group of slabs leaves at least one stage, and its B slabs fit one
-    static_assert((WORK - GROUP * t_bytes<S>()) / (kps_of(BN) * (A_BLOCK + BN * BK * 2 + GROUP * PM_SLAB * BK * 2)) >= 1, "ring");
+    constexpr int RING = (227 * 1024 - OTHER) / 1024 * 1024;
+    // a full group of slabs leaves two stages, and its B slabs fit one
+    static_assert(RING / (kps_of(BN) * (A_BLOCK + BN * BK * 2 + GROUP * PM_SLAB * BK * 2)) >= 2, "ring");
     static_assert(GROUP * BN * PM_SLAB * 2 <= kps_of(BN) * (A_BLOCK + BN * BK * 2 + GROUP * PM_SLAB * BK * 2), "B slabs");
     static SmemGrant grant;
-    if (cudaError_t e = grant.ensure(small_linear_kernel<BN, EPI, LNF, S>, WORK + OTHER); e != cudaSuccess) return e;
-    a.work_bytes = WORK;
+    if (cudaError_t e = grant.ensure(small_linear_kernel<BN, EPI, LNF, S>, RING + OTHER); e != cudaSuccess) return e;
+    a.ring_bytes = RING;
     ProfScope ps(L, KC_GEMM);
-    const cudaError_t e = launch_overlapped(L, small_linear_kernel<BN, EPI, LNF, S>, tiles * S, THREADS, WORK + OTHER, S,
+    const cudaError_t e = launch_overlapped(L, small_linear_kernel<BN, EPI, LNF, S>, tiles * S, THREADS, RING + OTHER, S,
                                             t.x, t.w, t.bt, t.at, a);
     BUMP(L);
     return e;

@@ -333,11 +333,11 @@ def test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, 
 
 
 @pytest.mark.parametrize("frames,rank,what", [(1, 16, "64-wide, K in four"), (1, 64, "64-wide, K in four"), (12, 64, "256-wide, K in two")])
-def test_lora_linear_ring_of_one_stage(frames, rank, what):
-    """The few-row kernel's ring holds a single stage where a group of eight slabs and the exchange of partial sums take
-    the rest of the shared memory; further groups of slabs then follow through that one stage.  Eight adapters on every
-    frame: one to eight groups per tile.  Several calls in a row, against float64 sums of the same bf16 inputs; tolerance as
-    for the other linears."""
+def test_lora_linear_several_slab_groups_through_the_shortest_ring(frames, rank, what):
+    """The few-row kernel's ring is shortest where a group of eight slabs and the exchange of partial sums take the
+    rest of the shared memory; further groups of slabs then follow through those stages, x from one thread and the slabs
+    from another.  Eight adapters on every frame: one to eight groups per tile.  Several calls in a row, against float64
+    sums of the same bf16 inputs; tolerance as for the other linears."""
     import torch
     from paper_2507_14959_b200 import binding
     k_in, n_out, tokens, n_ad, rows = 3072, 768, 197, 16, frames * 197
