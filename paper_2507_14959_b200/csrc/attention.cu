@@ -212,7 +212,7 @@ constexpr int ATT_MAX_BLOCKS = 3;
 constexpr uint32_t ATT_O_COL = 2 * AKB;    // tensor-memory columns: two regions of scores, O behind them
 
 struct AttnArgs {
-    int tokens, heads, tpad, n_blocks, n_qtiles, n_units;
+    int tokens, heads, tpad, n_blocks, n_qtiles, n_items, n_units;      // items: (frame, head) pairs; units: their query tiles
     const bf16* qkv;
     bf16* out;
     int* status;
@@ -254,7 +254,7 @@ __device__ __forceinline__ void chunk_probs(const uint32_t* v, int lim, uint64_t
 // Softmax does not depend on the reference as long as nothing overflows (the reference is one of the scores, so the
 // largest term is at least 1), and this one needs 16 scores instead of a pass over all of them -- nor an exchange
 // between the warps that share a row: each reads those 16.  A row whose sum says that a score lies more than
-// about 100 / c = 550 above the reference (or is not a number) is computed again by attention_row_exact.
+// about 100 / c = 550 above the reference (or is not a number) is computed again by attention_rows_exact.
 __device__ __forceinline__ float score_reference(uint32_t t_s, int valid) {
     uint32_t v[16];
     tmem_ld16(t_s, v);
@@ -376,30 +376,127 @@ __device__ __forceinline__ float score_probs_sweep_ahead(uint32_t t_s, uint32_t 
     return result();
 }
 
-// One output row by one warp with the row's true maximum, straight from global memory: for the rows described above.
-// Two dimensions per lane, every score is formed twice.
-__device__ __noinline__ void attention_row_exact(const bf16* qkv, bf16* out, int tokens, int d, int f, int h, int q_row) {
-    const int lane = threadIdx.x & 31;
-    const float c = 0.125f * 1.4426950408889634f;
-    const bf16* row0 = qkv + (size_t)f * tokens * 3 * d + h * HD + 2 * lane;
-    const float2 q = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(row0 + (size_t)q_row * 3 * d));
-    auto score = [&](int j) {
-        const float2 k = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(row0 + (size_t)j * 3 * d + d));
-        float t = q.x * k.x + q.y * k.y;
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
-        return t * c;
+// The rows described above are computed again when the CTA's tiles are done and the operands' shared memory is free, in groups
+// of 16 query rows.  (A call in the sweep's loop costs its registers: 256 frames 87 -> 130 us.)  Until then a thread notes them
+// as one bit per tile of its row; the last bit stands for all further tiles.  256 frames of 197 tokens, 12 heads: 86 us
+// without such rows, 153 with one row in a hundred out of range, 401 with all (row by row in the loop: 87, 1700, 35000).
+__device__ __forceinline__ uint32_t redo_bit(int tile) { return 1u << min(tile, 31); }
+
+// One group by one warp, with the rows' true (running) maxima on mma.sync.  `stage`: REDO_STAGE bytes of shared memory of
+// this warp: two buffers in turn, each 16 keys and their values (16-byte chunks XOR-swizzled by row).
+constexpr int REDO_STAGE = 2 * 2 * 16 * 128;
+__device__ __noinline__ void attention_rows_exact(const bf16* qkv, bf16* out, int tokens, int d, int f, int h, int q0, uint32_t stage) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, mi = lane >> 3, l7 = lane & 7;
+    const float c_ = 0.125f * 1.4426950408889634f;
+    const bf16* base = qkv + (size_t)f * tokens * 3 * d + h * HD;
+    auto fetch = [&](int k0) {                                     // 16 keys and values; keys past the end read as zero
+        const uint32_t to = stage + (uint32_t)((k0 >> 4) & 1) * (REDO_STAGE / 2);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int row = mi + 4 * (i & 3), key = k0 + row;
+            const bf16* src = base + (size_t)min(key, tokens - 1) * 3 * d + (1 + (i >> 2)) * d + l7 * 8;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                         ::"r"(to + (uint32_t)((i >> 2) * 2048 + row * 128 + ((l7 ^ (row & 7)) << 4))), "l"(src), "r"(key < tokens ? 16 : 0) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    float m = -INFINITY;
-    for (int j = 0; j < tokens; ++j) m = fmaxf(m, score(j));
-    float l = 0.f, o0 = 0.f, o1 = 0.f;
-    for (int j = 0; j < tokens; ++j) {
-        const float p = ex2_approx(score(j) - m);
-        const float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(row0 + (size_t)j * 3 * d + 2 * d));
-        l += p;
-        o0 = fmaf(p, v.x, o0);
-        o1 = fmaf(p, v.y, o1);
+    fetch(0);
+    uint32_t qa[4][4];
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int row = q0 + g + 8 * (e & 1), c = ks * 16 + 2 * t + 8 * (e >> 1);
+            qa[ks][e] = row < tokens ? *reinterpret_cast<const uint32_t*>(base + (size_t)row * 3 * d + c) : 0u;
+        }
+    float o[8][4], m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
+#pragma unroll 1
+    for (int k0 = 0; k0 < tokens; k0 += 16) {
+        if (k0 + 16 < tokens) {
+            fetch(k0 + 16);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncwarp();
+        const uint32_t k_s = stage + (uint32_t)((k0 >> 4) & 1) * (REDO_STAGE / 2), v_s = k_s + 2048u;
+        float s[2][4] = {};
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {
+            const int r = (mi >> 1) * 8 + l7, c = ks * 2 + (mi & 1);
+            uint32_t b0, b1, b2, b3;
+            ldsm_x4(k_s + r * 128 + ((c ^ (r & 7)) << 4), b0, b1, b2, b3);
+            mma_bf16(s[0], qa[ks], b0, b1);
+            mma_bf16(s[1], qa[ks], b2, b3);
+        }
+        uint32_t pa[4];
+#pragma unroll
+        for (int hi = 0; hi < 2; ++hi) {                           // rows g, g + 8
+            float x[4], nm = m[hi];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                x[e] = k0 + (e >> 1) * 8 + 2 * t + (e & 1) < tokens ? s[e >> 1][2 * hi + (e & 1)] * c_ : -INFINITY;
+                nm = fmaxf(nm, x[e]);
+            }
+            nm = fmaxf(nm, __shfl_xor_sync(0xFFFFFFFFu, nm, 1));
+            nm = fmaxf(nm, __shfl_xor_sync(0xFFFFFFFFu, nm, 2));
+            const float cf = ex2_approx(m[hi] - nm);               // 0 the first time
+            m[hi] = nm;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) x[e] = ex2_approx(x[e] - nm);
+            l[hi] = l[hi] * cf + ((x[0] + x[1]) + (x[2] + x[3]));
+            pa[hi] = pack2(x[0], x[1]);
+            pa[2 + hi] = pack2(x[2], x[3]);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) { o[i][2 * hi] *= cf; o[i][2 * hi + 1] *= cf; }
+        }
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            const int r = (mi & 1) * 8 + l7, c = n * 2 + (mi >> 1);
+            uint32_t b0, b1, b2, b3;
+            ldsm_x4_t(v_s + r * 128 + ((c ^ (r & 7)) << 4), b0, b1, b2, b3);
+            mma_bf16(o[2 * n], pa, b0, b1);
+            mma_bf16(o[2 * n + 1], pa, b2, b3);
+        }
+        __syncwarp();                                              // this buffer is fetched into again two steps on
     }
-    *reinterpret_cast<uint32_t*>(out + ((size_t)f * tokens + q_row) * d + h * HD + 2 * lane) = pack2(o0 / l, o1 / l);
+#pragma unroll
+    for (int hi = 0; hi < 2; ++hi) {
+        float sum = l[hi];
+        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 1);
+        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 2);
+        const float inv = 1.f / sum;
+        const int row = q0 + g + 8 * hi;
+        bf16* orow = out + ((size_t)f * tokens + row) * d + h * HD;
+        if (row < tokens)
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                *reinterpret_cast<uint32_t*>(orow + i * 8 + 2 * t) = pack2(o[i][2 * hi] * inv, o[i][2 * hi + 1] * inv);
+    }
+}
+
+// Warp `me` of `warps`: every warps'th of the groups that are noted in marks[n_sets][parts][AQ rows], tile by tile (warps at work
+// side by side share keys and values).  Tile i of set k is the CTA's tile c = i * n_sets + k of n_tiles, that is query tile
+// c % n_qtiles of unit u0 + c / n_qtiles * step.
+__device__ __noinline__ void redo_groups(const AttnArgs& args, const uint32_t* marks, int n_sets, int parts, int u0, int step, int n_tiles,
+                                         int me, int warps) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    const int lane = threadIdx.x & 31;
+    uint32_t m = 0;                                              // lane e: 16-row group e % 8 of set e / 8
+    if (lane < n_sets * 8)
+        for (int i = 0; i < parts * 16; ++i) m |= marks[((lane >> 3) * parts + (i >> 4)) * AQ + (lane & 7) * 16 + (i & 15)];
+    int turn = 0;
+    for (int i = 0; i * n_sets < n_tiles; ++i)
+        for (uint32_t groups = __ballot_sync(0xFFFFFFFFu, (m & redo_bit(i)) != 0u); groups; groups &= groups - 1) {
+            const int e = __ffs((int)groups) - 1, c = i * n_sets + (e >> 3);
+            if (turn++ % warps != me || c >= n_tiles) continue;
+            const int u = u0 + c / args.n_qtiles * step + c % args.n_qtiles, fh = u / args.n_qtiles, q0 = u % args.n_qtiles * AQ + (e & 7) * 16;
+            if (q0 < args.tokens)
+                attention_rows_exact(args.qkv, args.out, args.tokens, args.heads * HD, fh / args.heads, fh % args.heads, q0,
+                                     smem_u32(smem_raw) + (uint32_t)(me * REDO_STAGE));
+        }
 }
 
 // Share k of `shares` takes the 16-key pieces [att_first(shares, k), att_first(shares, k + 1)) of a key
@@ -412,7 +509,7 @@ __host__ __device__ constexpr int att_first(int shares, int k) {
 template <int SHARES>
 __global__ void __launch_bounds__(32 + 128 * SHARES, 1)
 attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kv,
-                    const AttnArgs args) {
+                    const __grid_constant__ AttnArgs args) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = smem_u32(smem_raw);
     if (base & 1023u) {                       // swizzled operands need a 1024-byte aligned window
@@ -463,6 +560,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     const uint32_t o_tmem = tmem_base + ATT_O_COL;
+    uint32_t redo = 0;                                           // this thread's rows to compute again, see redo_bit
     dep_release();
 
     if (warp == 0) {
@@ -603,6 +701,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 #pragma unroll
                 for (int k = 0; k < shares; ++k) l += sums[k * AQ + row];
             }
+            if (q_row < T && !(l < ROW_SUM_LIMIT)) redo |= redo_bit(u - u0);
             // O = sum over the key blocks of P V is complete: the finished rows are written out
             ok = mbar_wait(o_bar, par, abort_flag, args.status);
             ok = __all_sync(0xFFFFFFFFu, ok);
@@ -637,9 +736,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                                      : "memory");
                     }
                 }
-                if (share == 0)
-                    for (uint32_t redo = __ballot_sync(0xFFFFFFFFu, q_row < T && !(l < ROW_SUM_LIMIT)); redo; redo &= redo - 1)
-                        attention_row_exact(args.qkv, args.out, T, d, f, h, qt * AQ + quarter * 32 + __ffs((int)redo) - 1);
             }
         }
     }
@@ -651,10 +747,16 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);    // let copies / MMAs in flight land
     }
     tc_fence_before();
-    __syncthreads();
+    const int any = __syncthreads_or(redo != 0u);
     if (warp == 0) {
         tc_fence_after();
         tmem_dealloc(tmem_base, 512);
+    }
+    if (any && !*abort_flag) {
+        uint32_t* marks = reinterpret_cast<uint32_t*>(sums_base);
+        if (warp > 0) marks[(warp - 1) / 4 * AQ + (warp & 3) * 32 + lane] = redo;
+        __syncthreads();
+        if (warp > 0) redo_groups(args, marks, 1, shares, u0, args.n_qtiles, u1 - u0, warp - 1, 4 * shares);
     }
 }
 
@@ -683,24 +785,21 @@ constexpr int APIPE_ITEM_BYTES = 2 * AKB_BYTES + 2 * AQ_BYTES;      // K, V, two
 constexpr int APIPE_SPLIT = 7;                                       // 16-key pieces of the first half
 constexpr int APIPE_XCHG_BYTES = 2 * 2 * AQ * 4;                     // row sums [group][half][row]
 
-struct AttnPipeArgs {
-    int tokens, heads, tpad, nq, n_items;
-    const bf16* qkv;
-    bf16* out;
-    int* status;
-};
+__device__ __forceinline__ int pipe_items(const AttnArgs& args) {      // of this CTA: blockIdx.x, + gridDim.x, ...
+    return (args.n_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+}
 
 __global__ void __launch_bounds__(APIPE_THREADS, 1)
 attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kv,
-                      const AttnPipeArgs args) {
+                      const __grid_constant__ AttnArgs args) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = smem_u32(smem_raw);
     if (base & 1023u) {                       // swizzled operands need a 1024-byte aligned window
         if (threadIdx.x == 0) atomicCAS(args.status, 0, (int)PM_ERR_CUDA);
         return;
     }
-    const int T = args.tokens, nq = args.nq, d = args.heads * HD;
-    const int my_items = (args.n_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int T = args.tokens, nq = args.n_qtiles, d = args.heads * HD;
+    const int my_items = pipe_items(args);
     const int my_tiles = my_items * nq;
     const int n_pieces = args.tpad / 16, split = min(APIPE_SPLIT, n_pieces);
     auto k_s = [&](int buf) { return base + buf * APIPE_ITEM_BYTES; };
@@ -739,6 +838,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    uint32_t redo = 0;                                           // this thread's rows to compute again, see redo_bit
     dep_release();
 
     if (warp == 0) {
@@ -834,6 +934,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
             l += other_sum[row];
+            if (q_row < T && !(l < ROW_SUM_LIMIT)) redo |= redo_bit(c >> 1);
             ok = mbar_wait(o_ready(group), par, abort_flag, args.status);
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
@@ -859,9 +960,6 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                                      : "memory");
                     }
                 }
-                if (half == 0)
-                    for (uint32_t redo = __ballot_sync(0xFFFFFFFFu, q_row < T && !(l < ROW_SUM_LIMIT)); redo; redo &= redo - 1)
-                        attention_row_exact(args.qkv, args.out, T, d, f, h, qt * AQ + quarter * 32 + __ffs((int)redo) - 1);
             }
             tc_fence_before();
             __syncwarp();
@@ -876,10 +974,18 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);    // let copies / MMAs in flight land
     }
     tc_fence_before();
-    __syncthreads();
+    const int any = __syncthreads_or(redo != 0u);
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, 512);
+    }
+    if (any && !*abort_flag) {
+        uint32_t* marks = reinterpret_cast<uint32_t*>(xchg);
+        if (warp > 1) marks[(warp - 2) / 4 * AQ + (warp & 3) * 32 + lane] = redo;
+        __syncthreads();
+        if (warp > 1)
+            redo_groups(args, marks, 2, 2, (int)blockIdx.x * args.n_qtiles, (int)gridDim.x * args.n_qtiles, pipe_items(args) * args.n_qtiles,
+                        warp - 2, 2 * APIPE_GROUP_WARPS);
     }
 }
 
@@ -1072,7 +1178,8 @@ cudaError_t launch_attention_tc(const Launch& L, const CUtensorMap& tm_q, const 
     a.tpad = (tokens + 15) / 16 * 16;
     a.n_blocks = (a.tpad + AKB - 1) / AKB;
     a.n_qtiles = (tokens + AQ - 1) / AQ;
-    a.n_units = n_frames * heads * a.n_qtiles;
+    a.n_items = n_frames * heads;
+    a.n_units = a.n_items * a.n_qtiles;
     a.qkv = qkv; a.out = out; a.status = L.status;
     // up to a third as many (frame, head) pairs as SMs: 12 pairs of 197 tokens 4.4 against 7.6 us, 48 pairs 7.6 against 7.7, 72
     // pairs 9.8 against 7.8; 65 tokens: 48 pairs 3.9 against 4.6, 96 pairs 5.7 against 4.8
@@ -1088,14 +1195,11 @@ cudaError_t launch_attention_tc(const Launch& L, const CUtensorMap& tm_q, const 
     }
     if (a.n_blocks == 1 && a.n_qtiles <= 2 && n_sms > 0) {
         // one key block: the pipelined persistent kernel
-        AttnPipeArgs pa;
-        pa.tokens = tokens; pa.heads = heads; pa.tpad = a.tpad; pa.nq = a.n_qtiles;
-        pa.n_items = n_frames * heads; pa.qkv = qkv; pa.out = out; pa.status = L.status;
         const size_t psmem = 2 * (size_t)APIPE_ITEM_BYTES + APIPE_XCHG_BYTES + 192;
         static SmemGrant grant;
         if (cudaError_t e = grant.ensure(attention_pipe_kernel, (int)psmem); e != cudaSuccess) return e;
         ProfScope ps(L, KC_ATTENTION);
-        cudaError_t e = launch_overlapped(L, attention_pipe_kernel, std::min(pa.n_items, n_sms), APIPE_THREADS, psmem, 1, tm_q, tm_kv, pa);
+        cudaError_t e = launch_overlapped(L, attention_pipe_kernel, std::min(a.n_items, n_sms), APIPE_THREADS, psmem, 1, tm_q, tm_kv, a);
         BUMP(L);
         return e;
     }

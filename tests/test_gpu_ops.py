@@ -435,3 +435,55 @@ def test_attention_rows_whose_first_scores_are_far_below_the_largest(frames, tok
     for f in sorted({0, frames - 1}):
         want = po.attention(qkv[f * tokens:(f + 1) * tokens].astype(np.float64), heads)
         np.testing.assert_allclose(got[f * tokens:(f + 1) * tokens], want, **TOL[0])
+
+
+@pytest.mark.parametrize("far", [50, 300, 540, 560, 700])
+@pytest.mark.parametrize("frames,tokens,heads", [(18, 197, 3), (1, 300, 2), (2, 577, 1)])
+def test_attention_rows_over_the_range_of_their_reference(frames, tokens, heads, far):
+    """Rows whose later scores (q k) lie 50 to 700 above those of keys 0..15: exponentials up to 2^100 relative to the
+    reference on one side of 550, computed again on the other.  Six far keys of nearby scores, in both shares of the key columns
+    and in every key block; every other query row of the first frame's first head and all rows of the last frame's
+    last head.  All rows of both frames against the oracle."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    d = heads * 64
+    qkv = wl.normal((frames * tokens, 3 * d), 1.0, "attn_gpu_range", frames, tokens, heads)
+    for f, h, rows in ((0, 0, slice(0, tokens, 2)), (frames - 1, heads - 1, slice(0, tokens))):
+        x = qkv[f * tokens:(f + 1) * tokens]
+        q, k = slice(h * 64, h * 64 + 64), slice(d + h * 64, d + h * 64 + 64)
+        x[rows, q] = 1.0
+        x[:16, k] = 0.0
+        for i, key in enumerate((17, tokens // 3, tokens // 2, tokens // 2 + 30, tokens - 60, tokens - 2)):
+            x[key, k] = far / 64 - i % 3 / 32          # q k = far, far - 2, far - 4 (bf16 steps at most)
+    qkv = wl.round_bf16(qkv)
+    od = torch.full((frames * tokens, d), float("nan"), device="cuda", dtype=torch.bfloat16)
+    binding.attention(to_dev(qkv, 0), od, frames, tokens, heads, 0)
+    torch.cuda.synchronize()
+    got = to_np(od)
+    for f in sorted({0, frames - 1}):
+        want = po.attention(qkv[f * tokens:(f + 1) * tokens].astype(np.float64), heads)
+        np.testing.assert_allclose(got[f * tokens:(f + 1) * tokens], want, **TOL[0])
+
+
+@pytest.mark.parametrize("frames,tokens,heads", [(830, 17, 12), (450, 209, 12)])
+def test_attention_rows_computed_again_in_late_tiles(frames, tokens, heads):
+    """More tiles per CTA than a thread has bits for them: rows out of range in early, middle and last tiles.  Frames with
+    such rows and their neighbours against the oracle."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    d = heads * 64
+    gen = torch.Generator(device="cuda").manual_seed(tokens)
+    qkv = torch.randn((frames, tokens, 3, heads, 64), generator=gen, device="cuda")
+    far = (0, frames // 3, frames // 2, frames - 1)
+    for f in far:
+        qkv[f, 3::5, 0, f % heads] = 1.0
+        qkv[f, :16, 1, f % heads] = 0.0
+        qkv[f, tokens - 1, 1, f % heads] = 12.0
+    qkv = qkv.bfloat16().reshape(frames * tokens, 3 * d)
+    od = torch.full((frames * tokens, d), float("nan"), device="cuda", dtype=torch.bfloat16)
+    binding.attention(qkv, od, frames, tokens, heads, 0)
+    torch.cuda.synchronize()
+    assert torch.isfinite(od.float()).all()
+    for f in sorted({g for f in far for g in (f, min(f + 1, frames - 1))}):
+        rows = slice(f * tokens, (f + 1) * tokens)
+        np.testing.assert_allclose(to_np(od[rows]), po.attention(to_np(qkv[rows]), heads), **TOL[0])
