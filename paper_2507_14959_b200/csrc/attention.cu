@@ -262,6 +262,18 @@ __device__ __forceinline__ float score_reference(uint32_t t_s, int valid) {
     return valid >= 16 ? chunk_max<16, false>(v, 16, -INFINITY) : chunk_max<16, true>(v, valid, -INFINITY);
 }
 constexpr float ROW_SUM_LIMIT = 1.2676506e30f;               // 2^100
+// Large terms times large values may overflow O where the quotient is finite.  A row with a sum beyond this looks at its
+// accumulators and is computed again if one is not finite (below it, only values beyond 2^112 could overflow).
+constexpr float ROW_SUM_CHECK = 65536.f;
+template <int N>
+__device__ __forceinline__ bool all_finite(const uint32_t (&v)[N]) {
+    uint64_t z = pk2(0.f, 0.f);
+#pragma unroll
+    for (int e = 0; e < N; e += 2) z = fma2(pk2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])), pk2(0.f, 0.f), z);
+    float lo, hi;
+    upk2(z, lo, hi);
+    return lo + hi == 0.f;
+}
 
 // Sweep over the score columns [0, ncols) that start at tensor-memory address t_s (ncols a multiple of 16, `valid` of
 // them real), 16 at a time with the next load in flight: P (packed bf16, 8 columns per 16 scores) goes to t_p onwards
@@ -722,6 +734,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             if (writes) {
                 const float inv = 1.f / l;
                 bf16* orow = args.out + ((size_t)f * T + q_row) * d + h * HD + share * OCOLS;
+                if (q_row < T && l > ROW_SUM_CHECK && !all_finite(v)) redo |= redo_bit(u - u0);
                 if (q_row < T && l < ROW_SUM_LIMIT) {
                     // 32-byte stores: one full sector per row per instruction
 #pragma unroll
@@ -946,6 +959,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 uint32_t v[32];
                 tmem_ld32((t_lane + 128u) + (uint32_t)(half * 32), v);
                 tmem_ld_wait();
+                if (q_row < T && l > ROW_SUM_CHECK && !all_finite(v)) redo |= redo_bit(c >> 1);
                 if (q_row < T && l < ROW_SUM_LIMIT) {
 #pragma unroll
                     for (int q = 0; q < 2; ++q) {

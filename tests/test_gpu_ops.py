@@ -487,3 +487,29 @@ def test_attention_rows_computed_again_in_late_tiles(frames, tokens, heads):
     for f in sorted({g for f in far for g in (f, min(f + 1, frames - 1))}):
         rows = slice(f * tokens, (f + 1) * tokens)
         np.testing.assert_allclose(to_np(od[rows]), po.attention(to_np(qkv[rows]), heads), **TOL[0])
+
+
+@pytest.mark.parametrize("exponent", [40, 60, 100])
+@pytest.mark.parametrize("frames,tokens,heads", [(18, 197, 3), (2, 577, 1)])
+def test_attention_of_large_values_under_large_terms(frames, tokens, heads, exponent):
+    """Terms of 2^92 relative to the reference (scores q k = 512 above those of keys 0..15) times values of 2^40 to 2^100:
+    the unnormalised output overflows fp32, the quotient does not.  One value column per half of the head is large.
+    Relative to the oracle, as for the other attention cases."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    d, scale = heads * 64, 2.0 ** exponent
+    qkv = wl.normal((frames * tokens, 3 * d), 1.0, "attn_gpu_large", frames, tokens, heads)
+    qkv[:tokens, :64] = 1.0
+    qkv[:16, d:d + 64] = 0.0
+    qkv[tokens - 40, d:d + 64] = 8.0
+    qkv[tokens - 90, d:d + 64] = 8.0 - 1.0 / 32
+    qkv = wl.round_bf16(qkv)
+    large = (2 * d + 5, 2 * d + 50)
+    sent = qkv.copy()
+    sent[:tokens, large] *= scale
+    od = torch.full((frames * tokens, d), float("nan"), device="cuda", dtype=torch.bfloat16)
+    binding.attention(to_dev(sent, 0), od, frames, tokens, heads, 0)
+    torch.cuda.synchronize()
+    got = to_np(od)[:tokens]
+    got[:, (5, 50)] /= scale
+    np.testing.assert_allclose(got, po.attention(qkv[:tokens].astype(np.float64), heads), **TOL[0])
