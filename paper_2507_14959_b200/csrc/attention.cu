@@ -1025,7 +1025,7 @@ struct AttnFewSmem {
 };
 
 __global__ void __launch_bounds__(32 * AFEW_WARPS)
-attention_few_kernel(const __grid_constant__ CUtensorMap tm_kv, const bf16* __restrict__ qkv, bf16* __restrict__ out,
+attention_few_kernel(const __grid_constant__ CUtensorMap tm_kv, const bf16* qkv, bf16* out,
                      int tokens, int heads, int* status) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     AttnFewSmem& sm = *reinterpret_cast<AttnFewSmem*>(smem_raw);

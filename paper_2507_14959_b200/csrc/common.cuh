@@ -274,6 +274,9 @@ cudaError_t launch_latency_forward(const Launch& L, const LatArgs& a);
 // Launch with programmatic stream serialization (the kernel may start once every CTA of the one before it on the
 // stream has released its dependents; it awaits that kernel's results itself with dep_wait()), with or
 // without thread-block clusters along x.  The first one after L.ordered was set starts behind its predecessor's end.
+// Such a kernel runs while the operands that the one before it writes still change.  So it reads them, after dep_wait(), with
+// ordinary loads: neither __ldg nor const __restrict__, which promise that nothing changes while the kernel runs and let the
+// compiler take the load ahead of the wait.  (Weights, adapter tables and the routing plan do not change.)
 template <typename... P, typename... A>
 cudaError_t launch_overlapped(const Launch& L, void (*kernel)(P...), dim3 grid, int block, size_t smem, int cluster, const A&... args) {
     cudaLaunchConfig_t cfg = {};

@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(256) layernorm_kernel(const T* __restrict__ x,
 // 768), in one pass relative to each row's first element, which keeps the sum of squares well conditioned.
 // 18912 rows of 768: 9.3 us with a row per warp, 8.3 now; 46492 rows: 17.9 and 14.1.
 constexpr int STATS_ROWS = 4;
-__global__ void __launch_bounds__(256) row_stats_kernel(const bf16* __restrict__ x, float2* __restrict__ stats,
+__global__ void __launch_bounds__(256) row_stats_kernel(const bf16* x, float2* stats,
                                                         int rows, int d, float eps) {
     const int row0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * STATS_ROWS;
     const int lane = threadIdx.x & 31;
@@ -499,7 +499,7 @@ __device__ __forceinline__ float sigmoidf_acc(float v) { return 1.f / (1.f + exp
 constexpr int HB_SLOTS = 16;
 
 // z = LayerNorm(row) of one row by one warp; v[i * 8 + j] = element (lane + 32 i) * 8 + j
-__device__ __forceinline__ void ln_regs(const bf16* __restrict__ xr, const float* __restrict__ g, const float* __restrict__ b,
+__device__ __forceinline__ void ln_regs(const bf16* xr, const float* g, const float* b,
                                         int d, float eps, int lane, float (&v)[32]) {
     const int nch = d >> 3;
     float sum = 0.f;
@@ -853,19 +853,19 @@ __device__ __forceinline__ uint64_t warp_or64(uint64_t v) {
 
 // AW = ceil(n_adapters / 64) mask words per frame
 template <int AW>
-__global__ void __launch_bounds__(SELECT_THREADS) select_kernel(const float* __restrict__ scores, int n_frames,
+__global__ void __launch_bounds__(SELECT_THREADS) select_kernel(const float* scores, int n_frames,
                                                       int n_classes, int n_adapters, float thr,
                                                       int context_copy, int has_prev,
-                                                      uint32_t* __restrict__ prev_labels,
-                                                      const int* __restrict__ prev_off,
-                                                      const int* __restrict__ prev_ids,
-                                                      const int* __restrict__ first,
-                                                      const uint64_t* __restrict__ provider,
+                                                      uint32_t* prev_labels,
+                                                      const int* prev_off,
+                                                      const int* prev_ids,
+                                                      const int* first,
+                                                      const uint64_t* provider,
                                                       uint64_t* scratch,
-                                                      int* __restrict__ next_off,
-                                                      int* __restrict__ next_ids, int ids_capacity,
-                                                      int* __restrict__ status,
-                                                      unsigned long long* __restrict__ metrics) {
+                                                      int* next_off,
+                                                      int* next_ids, int ids_capacity,
+                                                      int* status,
+                                                      unsigned long long* metrics) {
     __shared__ int warp_total[SELECT_THREADS / 32];
     __shared__ int is_last;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = SELECT_THREADS >> 5;
@@ -888,7 +888,7 @@ __global__ void __launch_bounds__(SELECT_THREADS) select_kernel(const float* __r
 #pragma unroll
             for (int i = 0; i < 32; ++i) {              // all loads in flight
                 const int k = (w0 + i) * 32 + lane;
-                sc[i] = k < n_classes ? __ldg(row + k) : -INFINITY;
+                sc[i] = k < n_classes ? row[k] : -INFINITY;
             }
             const bool mine = w0 + lane < NW;
             const uint32_t old = (has_prev && lab && mine) ? lab[w0 + lane] : 0u;
@@ -924,10 +924,10 @@ __global__ void __launch_bounds__(SELECT_THREADS) select_kernel(const float* __r
             }
             for (uint32_t bits = word; bits; bits &= bits - 1) {
                 const int k = (w0 + lane) * 32 + __ffs((int)bits) - 1;
-                const int a = __ldg(first + k);             // -1: nobody provides this label
+                const int a = first[k];             // -1: nobody provides this label
                 bool cov = false;
 #pragma unroll
-                for (int q = 0; q < AW; ++q) cov |= (__ldg(provider + (size_t)k * AW + q) & prev_mask[q]) != 0;
+                for (int q = 0; q < AW; ++q) cov |= (provider[(size_t)k * AW + q] & prev_mask[q]) != 0;
                 if (!cov) covered = false;
                 if ((unsigned)a < (unsigned)n_adapters) {
 #pragma unroll
