@@ -483,12 +483,13 @@ struct pm_handle_s {
         int key_int[4] = {0, 0, 0, 0};
         unsigned long long plan_version = 0;
         cudaStream_t st = nullptr;
+        bool small_batch = true;            // pm_set_small_batch_kernel at the time: chooses kernels linear by linear
         cudaGraphExec_t exec = nullptr;     // null: seen once, not recorded yet
         long long launches = 0;
         unsigned long long last_use = 0;
         bool same_key(const GraphEntry& o) const {
             return std::equal(key_ptr, key_ptr + 5, o.key_ptr) && std::equal(key_int, key_int + 4, o.key_int) &&
-                   plan_version == o.plan_version && st == o.st;
+                   plan_version == o.plan_version && st == o.st && small_batch == o.small_batch;
         }
     };
     std::vector<GraphEntry> graphs;
@@ -513,6 +514,7 @@ int run_graphed(pm_handle_s* h, pm_handle_s::GraphEntry key, F&& enqueue) {
     constexpr size_t MAX_GRAPHS = 8;
     std::string& err = h->err;
     cudaStream_t st = key.st;
+    key.small_batch = h->lat_on;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (!h->graphs_on || h->prof.on || st == nullptr || st == cudaStreamLegacy ||
         cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {

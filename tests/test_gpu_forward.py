@@ -242,6 +242,53 @@ def test_recorded_sequence_follows_changing_sets():
     m.close()
 
 
+@pytest.mark.parametrize("entry", ["forward", "device_sets", "branched"])
+def test_recorded_sequence_follows_the_small_batch_switch(entry):
+    """On a stream of its own a forward is recorded and replayed; the small-batch switch chooses each linear's kernels, so a
+    recording made with it on is not replayed with it off.  Twelve DeiT-small frames: too many for the whole-network
+    kernel, few enough for one kernel per linear."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    w = wl.deit_small_streams()
+    F, K = 12, w.spec.n_classes
+    sets = [list(s)[:1] for s in w.sets()[:F]]
+    if entry == "branched":                             # no adapter may touch the trunk: everything is branches
+        m = binding.model_from_workload(w, dtype=0, max_frames=2 * F)
+    else:
+        m = binding.model_from_workload(w, dtype=0, max_frames=F)
+    off, ids = wl.sets_to_csr(sets)
+    doff, dids = torch.from_numpy(off).cuda(), torch.from_numpy(ids).cuda()
+    fd = frames_to_dev(w.frames[:F], 0)
+    side = torch.cuda.Stream()
+    out = torch.zeros((2, F, K), device="cuda")
+    torch.cuda.synchronize()
+
+    def call():
+        n0 = m.launch_count()
+        with torch.cuda.stream(side):
+            if entry == "forward":
+                m.forward(fd, off, ids, out[0], out[1])
+            elif entry == "device_sets":
+                m.forward_device_sets(fd, doff, dids, out[0], out[1])
+            else:
+                m.forward_branched(fd, off, ids, 0, out[0], out[1])
+        assert m.status(side) == 0
+        return m.launch_count() - n0, out.cpu().numpy().copy()
+    on = [call() for _ in range(3)]
+    m.set_small_batch_kernel(False)
+    off_ = [call() for _ in range(3)]
+    m.set_small_batch_kernel(True)
+    again = call()
+    assert len({c for c, _ in on}) == 1 and len({c for c, _ in off_}) == 1
+    assert on[0][0] < off_[0][0] and again[0] == on[0][0]
+    for _, got in on + [again]:
+        np.testing.assert_array_equal(got, on[0][1])
+    for _, got in off_:
+        np.testing.assert_array_equal(got, off_[0][1])
+    assert np.abs(on[0][1] - off_[0][1]).max() < 1e-2
+    m.close()
+
+
 @pytest.mark.parametrize("dtype", [1, 0])
 def test_paper_variant_query_value_last_blocks(dtype):
     """The paper's own placement of the adapters (Sec. 3.1, Sec. 4): LoRA on the query and value
