@@ -105,3 +105,29 @@ def test_cooccurrence_on_both_sides_of_the_histogram_limit(K, T):
     binding.cooccurrence(torch.from_numpy(bits.view(np.int32)).cuda(), K, co)
     torch.cuda.synchronize()
     np.testing.assert_array_equal(co.cpu().numpy().astype(np.float64), po.cooccurrence(sets, K))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("K,T", [(20, 209), (20, 210), (80, 3239), (80, 3240), (80, 60001), (160, 12881), (320, 51361), (321, 52000)])
+@pytest.mark.parametrize("most", [5, 70])
+def test_cooccurrence_of_frames_with_few_and_many_labels(K, T, most):
+    """Both sides of the line between direct adds and histograms (as many frames as label pairs), blocks with few and with many
+    frames, frames of 0 to 5 and of up to 70 labels, of which the first 64 count.  Counts are integers, compared exactly
+    with a product of the 0/1 label matrix."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    gen = torch.Generator(device="cuda").manual_seed(K + T)
+    rank = torch.rand((T, K), generator=gen, device="cuda").argsort(1).argsort(1)
+    present = rank < torch.randint(0, min(K, most) + 1, (T, 1), generator=gen, device="cuda")
+    nw = (K + 31) // 32
+    padded = torch.zeros((T, 32 * nw), dtype=torch.bool, device="cuda")
+    padded[:, :K] = present
+    words = (padded.view(T, nw, 32).long() << torch.arange(32, device="cuda")).sum(-1)
+    words = torch.where(words >= 2 ** 31, words - 2 ** 32, words).int()
+    co = torch.full((K, K), -1.0, device="cuda")
+    status = torch.full((1,), 7, dtype=torch.int32, device="cuda")
+    binding.cooccurrence(words, K, co, status)
+    counted = present & (present.int().cumsum(1) <= 64)
+    assert int(status.item()) == (binding.PM_ERR_CAPACITY if bool((counted != present).any()) else 0)
+    want = counted.double().T @ counted.double()
+    assert torch.equal(co.double(), want)
