@@ -237,3 +237,36 @@ def test_select_at_the_edges_of_its_passes(n_frames, n_labels, n_ctx):
         want = po.detect_contexts(po.labels_from_scores(scores[f], 0.5), None, ctxs, accs, 0.6, None, False)
         assert sorted(want) == list(i[o[f]:o[f + 1]])
     m.close()
+
+
+@pytest.mark.parametrize("n_frames,n_labels,n_ctx", [(1, 80, 200), (3, 33, 16), (70, 800, 200), (300, 1100, 70)])
+@pytest.mark.parametrize("density", [0.02, 0.3, 1.0])
+def test_select_with_few_and_many_labels_per_frame(n_frames, n_labels, n_ctx, density):
+    """Frames of a few labels, whose words the lanes walk side by side, and of hundreds, which are taken word by word; batches of one
+    and of several frames per thread of the emission.  Two steps (the second with context copy) against the oracle, exactly."""
+    import torch
+    ctxs, accs = wl.random_cover_table(33, n_ctx, n_labels, 12, True)
+    m = small_model(ctxs, accs, n_labels, n_frames)
+    m.set_cover(0.6)
+    g = wl.rng_for("select_density", n_frames, n_labels, density)
+    nw = (n_labels + 31) // 32
+    labels = torch.zeros((n_frames, nw), dtype=torch.int32, device="cuda")
+    lists = [(torch.zeros(n_frames + 1, dtype=torch.int32, device="cuda"),
+              torch.full((n_frames * n_ctx,), -1, dtype=torch.int32, device="cuda")) for _ in range(2)]
+    keep = g.random((n_frames, n_labels)) < density
+    prev = [(None, None)] * n_frames
+    for step in range(2):
+        if step == 1:
+            keep &= g.random((n_frames, n_labels)) < 0.9           # mostly covered by the sets in use
+            keep[::3] = g.random(keep[::3].shape) < density
+        scores = np.where(keep, 0.9, 0.1).astype(np.float32)
+        old, new = lists[(step + 1) % 2], lists[step % 2]
+        m.select(torch.from_numpy(scores).cuda(), 0.5, True, step > 0, labels, old[0], old[1], new[0], new[1])
+        assert m.status() == 0
+        o, i = new[0].cpu().numpy(), new[1].cpu().numpy()
+        for f in range(n_frames):
+            Y = po.labels_from_scores(scores[f], 0.5)
+            want = po.detect_contexts(Y, prev[f][0], ctxs, accs, 0.6, prev[f][1], True)
+            assert sorted(want) == list(i[o[f]:o[f + 1]]), (step, f)
+            prev[f] = (Y, want)
+    m.close()
