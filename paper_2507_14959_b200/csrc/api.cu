@@ -467,6 +467,7 @@ struct pm_handle_s {
     DevBuf scale_dev, rank_dev, hcat, hbias, hcls, hoff;
     AdapterMeta meta;
     bool heads_dirty = true;
+    int most_cls = 0;                // longest class list of an adapter
     // cover tables
     DevBuf first, provider, mask_scratch, metrics;
     bool cover_ready = false;
@@ -580,6 +581,8 @@ int rebuild_heads(pm_handle_s* h) {
     const int d = h->cfg.d, na = h->cfg.max_adapters;
     std::vector<int> hoff(na + 1, 0);
     for (int a = 0; a < na; ++a) hoff[a + 1] = hoff[a] + (h->ranks[a] ? (int)h->cls_ids[a].size() : 0);
+    h->most_cls = 0;
+    for (int a = 0; a < na; ++a) h->most_cls = std::max(h->most_cls, hoff[a + 1] - hoff[a]);
     const int total = hoff[na];
     std::vector<T> hc((size_t)std::max(total, 1) * d);
     std::vector<float> hb(std::max(total, 1));
@@ -714,8 +717,8 @@ int forward_t(pm_handle_s* h, const void* frames, int n_frames, int n_slots, int
     }
     CK(launch_heads<T>(L, X, n_slots, n_frames, n_frames, T_, d, c.ln_eps, h->lnf_g.as<float>(), h->lnf_b.as<float>(),
                        h->Z.as<float>(), h->head_wt.as<T>(), h->head_b.as<float>(), c.n_classes,
-                       h->hcat.as<T>(), h->hbias.as<float>(), h->hcls.as<int>(), h->hoff.as<int>(), R,
-                       scores_out, base_out));
+                       h->hcat.as<T>(), h->hbias.as<float>(), h->hcls.as<int>(), h->hoff.as<int>(), h->most_cls, R,
+                       scores_out, base_out, h->n_sms));
     return PM_OK;
 }
 

@@ -181,14 +181,15 @@ template <typename T>
 cudaError_t launch_fanout_rows(const Launch& L, T* x, const int* src_slot, int first_slot, int n_slots,
                                int tokens, int d);
 // n_slots CLS rows are normalised and feed the adapter heads of their slot; the first n_base_slots
-// also feed the base head; scores_out has n_out_frames rows (several slots may merge into one row)
+// also feed the base head; scores_out has n_out_frames rows (several slots may merge into one row); most_cls: the
+// longest class list of an adapter
 template <typename T>
 cudaError_t launch_heads(const Launch& L, const T* x, int n_slots, int n_out_frames, int n_base_slots,
                          int tokens, int d, float eps,
                          const float* lnf_g, const float* lnf_b, float* z,
                          const T* base_wt, const float* base_b, int n_classes,
-                         const T* hcat, const float* hbias, const int* hcls, const int* hoff,
-                         const RouteDev& R, float* scores_out, float* base_out);
+                         const T* hcat, const float* hbias, const int* hcls, const int* hoff, int most_cls,
+                         const RouteDev& R, float* scores_out, float* base_out, int n_sms);
 // Copies the used parts of a host-built plan (pinned memory) to the device tables: segments of 16-byte units at
 // the same offset in both.
 struct PlanSegments { int n; uint32_t at[8], units[8]; };

@@ -2,6 +2,7 @@
 // segmented heads + sigmoid + merge, Algorithm 2 selection, and the plain CUDA-core kernels of
 // the fp32 debug build (linear with unmerged LoRA terms, attention).
 #include <algorithm>
+#include <algorithm>
 #include <atomic>
 
 #include "common.cuh"
@@ -485,7 +486,7 @@ __device__ __forceinline__ float dot_row(const float* __restrict__ z, const T* _
 __device__ __forceinline__ float sigmoidf_acc(float v) { return 1.f / (1.f + expf(-v)); }
 
 // The heads of the bf16 build, one launch: blocks [0, base_blocks) make 16 slots x 16 NT classes of the base head, the
-// others the adapter heads of one slot each.  Every block normalises the CLS rows it needs itself (a row is d values;
+// others the adapter heads of one slot each (or a part of them).  Every block normalises the CLS rows it needs itself (a row is d values;
 // a kernel of its own for that was a launch in the chain), and all weights are requested before the kernel waits for
 // the last block's output (programmatic dependent launch).
 //   Base head: a [slots x d] x [d x classes] product on mma.sync; the fp32 features enter as three bf16 parts each,
@@ -548,6 +549,7 @@ struct HeadArgs {
     const int *hcls, *hoff, *slot_off, *slot_ids, *perm;
     float* scores;
     int zero_rows;             // 1: a slot's block owns its row of scores and zeroes it; 0: rows are zero already
+    int parts;                 // blocks that share a slot's adapter heads (more than one: zero_rows is 0)
 };
 
 __device__ __forceinline__ void mma_16x8x16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
@@ -646,7 +648,7 @@ __global__ void __launch_bounds__(256, 2) heads_kernel(const HeadArgs args) {
         return;
     }
     // ---------------------------------------------------------------------- adapter heads of one slot
-    const int slot = (int)blockIdx.x - args.base_blocks;
+    const int slot = ((int)blockIdx.x - args.base_blocks) / args.parts, part = ((int)blockIdx.x - args.base_blocks) % args.parts;
     float* out = args.scores + (size_t)args.perm[slot] * args.n_classes;
     const int p0 = args.slot_off[slot], p1 = args.slot_off[slot + 1];
     dep_wait();
@@ -661,7 +663,7 @@ __global__ void __launch_bounds__(256, 2) heads_kernel(const HeadArgs args) {
     for (int p = p0; p < p1; ++p) {
         const int a = args.slot_ids[p];
         const int r0 = args.hoff[a], r1 = args.hoff[a + 1];
-        for (int rb = r0 + warp * 4; rb < r1; rb += 32) {
+        for (int rb = r0 + (part * 8 + warp) * 4; rb < r1; rb += 32 * args.parts) {
             float acc[4];
             uint4 w[4][4];
 #pragma unroll
@@ -770,12 +772,16 @@ cudaError_t launch_heads(const Launch& L, const T* x, int n_slots, int n_out_fra
                          int tokens, int d, float eps,
                          const float* lnf_g, const float* lnf_b, float* z,
                          const T* base_wt, const float* base_b, int n_classes,
-                         const T* hcat, const float* hbias, const int* hcls, const int* hoff,
-                         const RouteDev& R, float* scores_out, float* base_out) {
+                         const T* hcat, const float* hbias, const int* hcls, const int* hoff, int most_cls,
+                         const RouteDev& R, float* scores_out, float* base_out, int n_sms) {
     if (n_slots <= 0) return cudaSuccess;
     ProfScope ps(L, KC_HEADS);
-    // one row of scores per slot: its block zeroes it; several slots per row (branches): zeroed beforehand
-    const bool zero_rows = sizeof(T) == 2 && n_slots == n_out_frames;
+    // few slots with long lists of classes: several blocks per slot (one frame, d = 768, 8 adapters of 400 classes 112 -> 27 us)
+    const int most = R.max_set * most_cls;
+    int parts = most <= 512 ? 1 : std::min(8, most / 256);
+    while (parts > 1 && n_slots * parts > 2 * n_sms) parts >>= 1;
+    // one row of scores and one block per slot: it zeroes the row; else the rows are zeroed beforehand
+    const bool zero_rows = sizeof(T) == 2 && n_slots == n_out_frames && parts == 1;
     if (!zero_rows) {
         cudaError_t e = cudaMemsetAsync(scores_out, 0, (size_t)n_out_frames * n_classes * sizeof(float), L.st);
         if (e != cudaSuccess) return e;
@@ -785,13 +791,13 @@ cudaError_t launch_heads(const Launch& L, const T* x, int n_slots, int n_out_fra
         a.x = x; a.n_slots = n_slots; a.n_base_slots = n_base_slots; a.tokens = tokens; a.d = d; a.n_classes = n_classes; a.eps = eps;
         a.lnf_g = lnf_g; a.lnf_b = lnf_b; a.base_wt = base_wt; a.base_b = base_b; a.base_out = base_out;
         a.hcat = hcat; a.hbias = hbias; a.hcls = hcls; a.hoff = hoff;
-        a.slot_off = R.slot_off; a.slot_ids = R.slot_ids; a.perm = R.perm; a.scores = scores_out; a.zero_rows = zero_rows;
+        a.slot_off = R.slot_off; a.slot_ids = R.slot_ids; a.perm = R.perm; a.scores = scores_out; a.zero_rows = zero_rows; a.parts = parts;
         const int rows = base_out ? (n_base_slots + HB_SLOTS - 1) / HB_SLOTS : 0;
         // few slots: narrow blocks, so that the classes spread over the SMs; many: wide ones, which normalise their rows less often
-        const bool narrow = rows * ((n_classes + 31) / 32) < 148;
+        const bool narrow = rows * ((n_classes + 31) / 32) < n_sms;
         a.base_cols = narrow ? (n_classes + 15) / 16 : (n_classes + 31) / 32;
         a.base_blocks = rows * a.base_cols;
-        const int adapter_blocks = zero_rows || R.max_set > 0 ? n_slots : 0;
+        const int adapter_blocks = zero_rows || R.max_set > 0 ? n_slots * parts : 0;
         const int smem = 3 * HB_SLOTS * (d * 2 + 64);
         static SmemGrant grant1, grant2;
         cudaError_t e = narrow ? grant1.ensure(heads_kernel<1>, smem) : grant2.ensure(heads_kernel<2>, smem);
@@ -820,8 +826,8 @@ cudaError_t launch_heads(const Launch& L, const T* x, int n_slots, int n_out_fra
         return cudaGetLastError();
     }
 }
-template cudaError_t launch_heads<float>(const Launch&, const float*, int, int, int, int, int, float, const float*, const float*, float*, const float*, const float*, int, const float*, const float*, const int*, const int*, const RouteDev&, float*, float*);
-template cudaError_t launch_heads<bf16>(const Launch&, const bf16*, int, int, int, int, int, float, const float*, const float*, float*, const bf16*, const float*, int, const bf16*, const float*, const int*, const int*, const RouteDev&, float*, float*);
+template cudaError_t launch_heads<float>(const Launch&, const float*, int, int, int, int, int, float, const float*, const float*, float*, const float*, const float*, int, const float*, const float*, const int*, const int*, int, const RouteDev&, float*, float*, int);
+template cudaError_t launch_heads<bf16>(const Launch&, const bf16*, int, int, int, int, int, float, const float*, const float*, float*, const bf16*, const float*, int, const bf16*, const float*, const int*, const int*, int, const RouteDev&, float*, float*, int);
 
 // ---------------------------------------------------------------------------------------
 // Algorithm 2 on the device: one warp per frame, any number of blocks

@@ -242,6 +242,49 @@ def test_recorded_sequence_follows_changing_sets():
     m.close()
 
 
+@pytest.mark.parametrize("n_frames", [1, 5, 300])
+def test_adapter_heads_with_long_class_lists(n_frames):
+    """Sets of up to eight adapters that list 300 overlapping classes each: few frames' heads are shared by several blocks, 300
+    frames' are not.  Against the oracle, empty and full sets in one batch."""
+    from paper_2507_14959_b200 import binding
+    d, heads, K, na, per = 128, 2, 420, 9, 300
+    g = np.random.default_rng(n_frames)
+    N = lambda *s: wl.round_bf16((g.standard_normal(s) * 0.05).astype(np.float32))  # noqa: E731
+    bb = {"patch_w": N(768, d), "patch_b": N(d), "cls": N(d), "pos": N(5, d), "ln1_g": 1 + N(1, d), "ln1_b": N(1, d),
+          "qkv_w": N(1, d, 3 * d), "qkv_b": N(1, 3 * d), "proj_w": N(1, d, d), "proj_b": N(1, d), "ln2_g": 1 + N(1, d), "ln2_b": N(1, d),
+          "fc1_w": N(1, d, 256), "fc1_b": N(1, 256), "fc2_w": N(1, 256, d), "fc2_b": N(1, d), "lnf_g": 1 + N(d), "lnf_b": N(d),
+          "head_w": N(d, K), "head_b": N(K)}
+    bb = {k: wl.round_bf16(v) for k, v in bb.items()}
+    m = binding.Model(img=32, d=d, layers=1, heads=heads, mlp=256, n_classes=K, backbone=bb, max_adapters=na, max_rank=4, max_set=8,
+                      max_frames=n_frames)
+    m.set_small_batch_kernel(False)                    # the layer kernels' heads, not the whole-network kernel's
+    adapters = []
+    for a in range(na):
+        ids = np.sort(g.choice(K, per, replace=False)).astype(np.int32)
+        ad = dict(rank=4, scale=2.0, A=[N(d, 4), None, None, None], B=[N(4, 3 * d), None, None, None], class_ids=ids, head_w=N(d, per),
+                  head_b=N(per), acc=np.ones(per, np.float32))
+        m.register_adapter(a, **ad)
+        adapters.append(ad)
+    sets = [sorted(int(a) for a in g.choice(na, size=(8, 0, 3, 1)[f % 4], replace=False)) for f in range(n_frames)]
+    off, ids = wl.sets_to_csr(sets)
+    frames = wl.round_bf16(g.uniform(-1, 1, (n_frames, 3, 32, 32)).astype(np.float32))
+
+    class W:                                            # what run_forward and the oracle need of a workload
+        class spec:
+            n_classes = K
+    s, b = run_forward(m, W, 0, frames=frames, offsets=off, ids=ids)
+    rows = sorted({0, min(1, n_frames - 1), n_frames // 2, n_frames - 1})
+    o2, i2 = wl.sets_to_csr([sets[r] for r in rows])
+    so, bo = po.forward(bb, [wl.Adapter(**ad) for ad in adapters], frames[rows], o2, i2, heads, 16, 1e-6, K)
+    assert np.abs(s[rows] - so).max() < 1e-2 and np.abs(b[rows] - bo).max() < 1e-2
+    for f in range(n_frames):
+        listed = np.zeros(K, bool)
+        for a in sets[f]:
+            listed[adapters[a]["class_ids"]] = True
+        assert np.all(s[f][~listed] == 0) and np.all(s[f][listed] > 0)
+    m.close()
+
+
 @pytest.mark.parametrize("entry", ["forward", "device_sets", "branched"])
 def test_recorded_sequence_follows_the_small_batch_switch(entry):
     """On a stream of its own a forward is recorded and replayed; the small-batch switch chooses each linear's kernels, so a
