@@ -336,7 +336,8 @@ int pm_linear_create(int k_in, int n_out, const float* w, const float* bias,
 int pm_linear_register(pm_linear lin, int adapter_id, int rank, float scale,
                        const float* A, const float* B);
 /* x dev [n_frames*tokens, k_in], residual dev [n_frames*tokens, n_out] or NULL (epilogue 2 only),
- * y dev [n_frames*tokens, n_out]; element type per dtype.  set_offsets / set_ids: host CSR. */
+ * y dev [n_frames*tokens, n_out]; element type per dtype.  set_offsets / set_ids: host CSR.  dtype 0: x, y and a
+ * residual that is added must be 16-byte aligned (else PM_ERR_CUDA). */
 int pm_linear_forward(pm_linear lin, const void* x, int n_frames,
                       const int32_t* set_offsets, const int32_t* set_ids,
                       const void* residual, void* y, void* cuda_stream);

@@ -1294,6 +1294,9 @@ int pm_linear_forward(pm_linear l, const void* x, int n_frames, const int32_t* s
     if (n_frames < 0 || (n_frames > 0 && (!x || !y || !set_offsets))) { err = "NULL argument"; return PM_ERR_ARG; }
     if (l->epilogue == EPI_RESIDUAL && n_frames > 0 && !residual) { err = "epilogue 2 needs a residual"; return PM_ERR_ARG; }
     if (n_frames == 0) return PM_OK;
+    if (l->dtype == 0 && ((uintptr_t)x | (uintptr_t)y | (l->epilogue == EPI_RESIDUAL ? (uintptr_t)residual : 0)) & 15) {
+        err = "x, y and a residual that is added must be 16-byte aligned"; return PM_ERR_CUDA;
+    }
     Launch L; L.st = st; L.launches = &l->launches; L.status = l->status.as<int>();
     int rc = l->router.build(n_frames, set_offsets, set_ids, l->ranks, l->scales, false, L, err);
     if (rc) return rc;
@@ -1302,9 +1305,7 @@ int pm_linear_forward(pm_linear l, const void* x, int n_frames, const int32_t* s
     PatchEpi none;
     if (l->dtype == 0 && small_linear_fits(l->lin.dev, &R, rows, l->epilogue, l->n_sms)) {
         ActMaps sx;
-        if (((uintptr_t)x | (uintptr_t)y | (uintptr_t)residual) & 15 || !act_encode(&sx, x, l->k_in, rows)) {
-            err = "x, y and residual must be 16-byte aligned"; return PM_ERR_CUDA;
-        }
+        if (!act_encode(&sx, x, l->k_in, rows)) { err = "cuTensorMapEncodeTiled failed (x)"; return PM_ERR_CUDA; }
         CK(launch_small_linear(L, l->lin.dev, &R, sx, rows, l->epilogue, (const bf16*)residual, none, (bf16*)y, l->n_sms, 0.f));
     } else if (l->dtype == 0) {
         CUtensorMap tm_x;

@@ -513,3 +513,30 @@ def test_attention_of_large_values_under_large_terms(frames, tokens, heads, expo
     got = to_np(od)[:tokens]
     got[:, (5, 50)] /= scale
     np.testing.assert_allclose(got, po.attention(qkv[:tokens].astype(np.float64), heads), **TOL[0])
+
+
+def test_linear_alignment_of_operands():
+    """x, y and a residual that is added must be 16-byte aligned, on few rows and on many, whatever the kernel; a residual that is
+    not used may lie anywhere."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    for k_in, n_out, frames in ((64, 128, 1), (64, 128, 300), (1536, 768, 1), (768, 768, 60)):
+        rows = frames * 197
+        off, ids = np.zeros(frames + 1, np.int32), np.zeros(0, np.int32)
+        wide = torch.randn((rows * max(k_in, n_out) + 8,), device="cuda").bfloat16()
+        x, res = wide[:rows * k_in].view(rows, k_in), wide[:rows * n_out].view(rows, n_out)
+        odd_x, odd_res = wide[1:1 + rows * k_in].view(rows, k_in), wide[1:1 + rows * n_out].view(rows, n_out)
+        out = torch.zeros((rows * n_out + 8,), device="cuda", dtype=torch.bfloat16)
+        y, odd_y = out[:rows * n_out].view(rows, n_out), out[1:1 + rows * n_out].view(rows, n_out)
+        w = wl.normal((k_in, n_out), 0.02, "align", k_in)
+        for epi in (0, 2):
+            lin = binding.Linear(w, np.zeros(n_out, np.float32), max_adapters=1, max_rank=16, max_set=1, max_frames=frames, tokens=197, epilogue=epi)
+            for a in ((odd_x, res, y), (x, res, odd_y)) + (((x, odd_res, y),) if epi == 2 else ()):
+                with pytest.raises(binding.PolymorphError) as e:
+                    lin.forward(a[0], frames, off, ids, a[2], residual=a[1])
+                assert e.value.code == binding.PM_ERR_CUDA
+            lin.forward(x, frames, off, ids, y, residual=odd_res if epi == 0 else res)
+            assert lin.status() == 0
+            want = x.float() @ torch.from_numpy(w).cuda() + (res.float() if epi == 2 else 0)
+            np.testing.assert_allclose(to_np(y), want.double().cpu().numpy(), **TOL[0])
+            lin.close()
