@@ -102,7 +102,14 @@ struct Launch {
     long long* launches = nullptr;
     int* status = nullptr;      // device status word
     Profiler* prof = nullptr;
-    mutable bool ordered = false;   // a plan upload was enqueued just before: kernels read the plan before they wait
+    // A plan upload was enqueued just before: the next kernel starts behind its end.
+    //
+    // Who may read the routing plan before dep_wait(): the kernels of a forward (shrink, GEMM, few-row linear and heads do).  The
+    // plan's tables are written by plan_upload_kernel or by the plan kernels, and the first kernel behind those starts when they
+    // have ended: in pm_linear_forward because of this flag; in the model's forwards, which upload through a Launch of
+    // their own, because im2col_kernel and the whole-network kernel are launched plainly (a replay's first node likewise).  Every
+    // kernel behind it starts later still.  An overlapped kernel put in their place must read the plan after dep_wait().
+    mutable bool ordered = false;
 };
 
 struct ProfScope {              // brackets the launches made while it is alive

@@ -279,6 +279,7 @@ cudaError_t launch_im2col(const Launch& L, const T* frames, const int* perm, T* 
     const int blocks = (int)((total + 255) / 256 < 148 * 16 ? (total + 255) / 256 : 148 * 16);
     if (blocks == 0) return cudaSuccess;
     ProfScope ps(L, KC_OTHER);
+    // launched plainly: with it the forward's kernels start behind the routing plan, see Launch::ordered
     im2col_kernel<T><<<blocks, 256, 0, L.st>>>(frames, perm, out, n_frames, img, patch, cls, pos, x, d);
     BUMP(L);
     return cudaGetLastError();

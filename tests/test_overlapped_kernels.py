@@ -43,3 +43,17 @@ def test_only_constant_operands_are_loaded_as_invariant():
             continue
         for operand in re.findall(r"__ldg\((.{0,80})", re.sub(r"//.*", "", text)):
             assert CONSTANT.match(operand), (name, operand)
+
+
+def test_what_stands_behind_the_routing_plan_is_launched_plainly():
+    """The kernels of a forward read the routing plan before they wait for the kernel ahead of them; the kernel that follows the
+    plan's writers therefore starts behind their end."""
+    overlapped = overlapped_kernels()
+    for name in ("im2col_kernel", "latency_forward_kernel", "plan_slots_kernel", "plan_tiles_kernel", "fanout_rows_kernel"):
+        assert any(name in text for text in SOURCES.values()) and name not in overlapped, name
+    forward = SOURCES["api.cu"][SOURCES["api.cu"].index("int forward_t("):]
+    first = re.search(r"CK\((launch_\w+|linear)[<(]", forward).group(1)
+    assert first == "launch_im2col"
+    upload = SOURCES["plan_device.cu"]
+    upload = upload[upload.index("cudaError_t launch_plan_upload"):]
+    assert "L.ordered = true;" in upload[:upload.index("\n}\n")]
