@@ -1343,20 +1343,16 @@ size_t latency_smem_bytes(int d, int mlp, int patch_dim, int tokens, int layers)
     return (size_t)lat_layout(d, mlp, patch_dim, tokens, layers, slots * LT_SLOT_BYTES, false).total;
 }
 
-cudaError_t launch_latency_forward(const Launch& L, const LatArgs& a) {
-    if (a.layers * 4 > LT_THREADS) return cudaErrorInvalidValue;
+// Sets `launched` once the kernel is on the stream.  cudaErrorNotSupported: this form does not apply to the geometry or the batch.
+static cudaError_t launch_form(const Launch& L, const LatArgs& a, bool shared, bool& launched) {
+    const int slots = lat_ring_slots(a.d, a.mlp, a.patch_dim, a.tokens, a.layers, shared);
+    if (!slots) return shared ? cudaErrorNotSupported : cudaErrorInvalidValue;
+    const int smem = lat_layout(a.d, a.mlp, a.patch_dim, a.tokens, a.layers, slots * (shared ? LT_SLOT_SHARED : LT_SLOT_BYTES), shared).total;
     static SmemGrant grant[2];
-    int share = 1, slots = 0, smem = 0;
-    for (int shared = 1; shared >= 0; --shared) {
-        slots = lat_ring_slots(a.d, a.mlp, a.patch_dim, a.tokens, a.layers, shared != 0);
-        if (!slots) continue;
-        smem = lat_layout(a.d, a.mlp, a.patch_dim, a.tokens, a.layers, slots * (shared ? LT_SLOT_SHARED : LT_SLOT_BYTES), shared != 0).total;
-        if (cudaError_t e = shared ? grant[1].ensure(latency_forward_kernel<true>, smem) : grant[0].ensure(latency_forward_kernel<false>, smem);
-            e != cudaSuccess) return e;
-        share = shared ? lat_share(a, (size_t)smem) : 1;
-        if (!shared || share > 1) break;
-    }
-    if (!slots) return cudaErrorInvalidValue;
+    if (cudaError_t e = shared ? grant[1].ensure(latency_forward_kernel<true>, smem) : grant[0].ensure(latency_forward_kernel<false>, smem);
+        e != cudaSuccess) return e;
+    const int share = shared ? lat_share(a, (size_t)smem) : 1;
+    if (shared && share == 1) return cudaErrorNotSupported;
     const int ctas = a.n_frames * a.tiles_pf * share;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas);
@@ -1372,7 +1368,6 @@ cudaError_t launch_latency_forward(const Launch& L, const LatArgs& a) {
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = share > 1 ? 2 : 1;
-    ProfScope ps(L, KC_GEMM);
     LatArgs copy = a;
     copy.status = L.status;
     copy.ring_slots = slots;
@@ -1380,6 +1375,20 @@ cudaError_t launch_latency_forward(const Launch& L, const LatArgs& a) {
     cudaError_t e = cudaMemsetAsync(a.bar, 0, sizeof(unsigned int) * a.n_frames * share, L.st);
     if (e != cudaSuccess) return e;
     e = share > 1 ? cudaLaunchKernelEx(&cfg, latency_forward_kernel<true>, copy) : cudaLaunchKernelEx(&cfg, latency_forward_kernel<false>, copy);
+    if (e != cudaSuccess) return e;
+    launched = true;
     BUMP(L);
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_latency_forward(const Launch& L, const LatArgs& a) {
+    if (a.layers * 4 > LT_THREADS) return cudaErrorInvalidValue;
+    // Tiles shared by clusters where that applies, else, or where the launch of the clusters is refused (a profiler, or a
+    // limit on the SMs, may leave room for fewer of them than the device), one CTA per tile.
+    ProfScope ps(L, KC_GEMM);
+    bool launched = false;
+    const cudaError_t e = launch_form(L, a, true, launched);
+    if (launched) return e;
+    if (e != cudaErrorNotSupported) cudaGetLastError();
+    return launch_form(L, a, false, launched);
 }
