@@ -772,7 +772,7 @@ int forward_latency(pm_handle_s* h, const void* frames, int n_frames, const int*
             const size_t kv_rows = (size_t)2 * std::max(1, max_f) * h->tokens;
             CK(h->lat_kv.alloc(kv_rows * 2 * c.d * sizeof(bf16)));
             CK(cudaMemset(h->lat_kv.p, 0, h->lat_kv.bytes));
-            CK(h->lat_bar.alloc(sizeof(unsigned int) * std::max(1, max_f)));
+            CK(h->lat_bar.alloc(sizeof(unsigned int) * std::max(1, max_f) * c.heads));     // a frame's counters: one, or one per head
             const int tpad = (h->tokens + 15) / 16 * 16;
             if (tpad > 256 || !tm_encode_2d(&h->lat_tm_kv, h->lat_kv.p, (uint64_t)2 * c.d, kv_rows, (uint64_t)2 * c.d * 2, 64, tpad, 128)) {
                 err = "cuTensorMapEncodeTiled failed (key/value exchange buffer)"; return PM_ERR_CUDA;
