@@ -388,8 +388,8 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                 for (int c = 0; c < CPW; ++c) fetch_residual<32, EPI>(args, row, n * BN + half * (BN / 2) + c * 32, res + c * 4);
         }
         if constexpr (LNF) {
-            // follow the ring: this thread sums its half of its row of each x block, relative to the mean of its first eight
-            // elements (which keeps the sum of squares well conditioned, whichever of them stand out)
+            // follow the ring: this thread sums its half of its row of each x block, relative to its first element
+            // (which keeps the sum of squares well conditioned)
             float pivot = 0.f;
             uint64_t np = 0, s1 = pk2(0.f, 0.f), s2 = s1;
             int stage = 0;
@@ -410,12 +410,7 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                                      : "r"(row_addr + (((half * 4 + c) ^ (r & 7)) << 4)));
                         const uint32_t w[4] = {q.x, q.y, q.z, q.w};
                         if (kb == 0 && j == 0 && c == 0) {
-                            uint64_t m = pk2(0.f, 0.f);
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) m = add2(m, pk2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xFFFF0000u)));
-                            float lo, hi;
-                            upk2(m, lo, hi);
-                            pivot = 0.125f * (lo + hi);
+                            pivot = __uint_as_float(w[0] << 16);
                             np = pk2(-pivot, -pivot);
                         }
 #pragma unroll
