@@ -198,7 +198,7 @@ class Model:
     def forward(self, frames, set_offsets, set_ids, scores_out, base_out=None, stream=None):
         """frames/scores_out/base_out: torch CUDA tensors; set lists: numpy int32 (host) or torch
         CUDA int32 tensors."""
-        n = frames.size(0)
+        n = len(frames)
         if isinstance(set_offsets, np.ndarray):
             set_offsets = _i32(set_offsets)
         if isinstance(set_ids, np.ndarray):
@@ -209,14 +209,14 @@ class Model:
     def forward_device_sets(self, frames, set_offsets, set_ids, scores_out, base_out=None, stream=None):
         """pm_forward_device_sets: the set lists are torch CUDA int32 tensors (e.g. written by
         select()); the plan is built on the device, nothing synchronises."""
-        self._check(self.lib.pm_forward_device_sets(self.handle, _ptr(frames), frames.size(0),
+        self._check(self.lib.pm_forward_device_sets(self.handle, _ptr(frames), len(frames),
                                                     _ptr(set_offsets), _ptr(set_ids), _ptr(scores_out),
                                                     _ptr(base_out), _stream_ptr(stream)), "pm_forward_device_sets")
 
     def forward_branched(self, frames, set_offsets, set_ids, trunk_layers, scores_out, base_out=None, stream=None):
         """pm_forward_branched: shared trunk of `trunk_layers` blocks, then one branch per active
         adapter (and the base branch if base_out is given).  Arguments as for forward()."""
-        n = frames.size(0)
+        n = len(frames)
         if isinstance(set_offsets, np.ndarray):
             set_offsets = _i32(set_offsets)
         if isinstance(set_ids, np.ndarray):
@@ -227,7 +227,7 @@ class Model:
 
     def select(self, scores, score_thr, context_copy, has_prev, prev_labels, prev_offsets, prev_ids,
                next_offsets, next_ids, stream=None):
-        n = scores.size(0)
+        n = len(scores)
         cap = 0 if next_ids is None else next_ids.numel()
         self._check(self.lib.pm_select(self.handle, _ptr(scores), n, score_thr, int(context_copy),
                                        int(has_prev), _ptr(prev_labels), _ptr(prev_offsets), _ptr(prev_ids),
