@@ -116,10 +116,6 @@ struct LinearObj {
             const int bn = gemm_tile_n(n_out);
             bool ok = tm_encode_2d(&dev.tm_w, wt.p, k_in, n_out, (uint64_t)k_in * 2, 64, bn, 128);
             if (ok && dev.lora.At) {
-                ok = tm_encode_2d(&dev.tm_at, at.p, k_in, (uint64_t)max_adapters * slabs_max * PM_SLAB,
-                                  (uint64_t)k_in * 2, 64, PM_SLAB, 128);
-            }
-            if (ok && dev.lora.At) {
                 ok = tm_encode_2d(&dev.tm_bt, bt.p, PM_SLAB, (uint64_t)max_adapters * slabs_max * n_out,
                                   PM_SLAB * 2, PM_SLAB, bn, 32);
             }
@@ -678,7 +674,7 @@ int forward_t(pm_handle_s* h, const void* frames, int n_frames, int n_slots, int
         }
     };
 
-    CK(launch_im2col<T>(L, (const T*)frames, R.perm, P, n_frames, c.img, c.patch, h->cls.as<float>(), h->pos.as<float>(), X, d));
+    CK(launch_im2col<T>(L, (const T*)frames, R.perm, P, n_frames, c.img, c.patch, h->cls.as<float>(), h->pos.as<float>(), X, d, h->n_sms));
     CK(linear(h->patch, P, &h->tm_patch, n_frames * h->g2, h->g2, false, EPI_PATCH, nullptr, pe, X));
     int n_cur = n_frames;                     // slots the blocks currently run on
     for (int l = 0; l <= c.layers; ++l) {
@@ -834,7 +830,7 @@ int create_t(pm_handle_s* h, const pm_backbone* w) {
     CK(h->QKV.alloc(rows_pad * 3 * d * sizeof(T))); CK(h->ATT.alloc(rows_pad * d * sizeof(T)));
     CK(h->H.alloc(rows_pad * m * sizeof(T)));
     CK(h->PATCH.alloc(rows_pad * h->patch_dim * sizeof(T)));
-    CK(h->Z.alloc((size_t)c.max_frames * d * sizeof(float)));
+    CK(h->Z.alloc(sizeof(T) == 2 ? 0 : (size_t)c.max_frames * d * sizeof(float)));      // the bf16 build's heads normalise their rows themselves
     CK(h->ln_stats.alloc(rows_pad * sizeof(float2)));
     CK(cudaMemset(h->X.p, 0, h->X.bytes)); if (h->U.p) CK(cudaMemset(h->U.p, 0, h->U.bytes));
     CK(cudaMemset(h->QKV.p, 0, h->QKV.bytes)); CK(cudaMemset(h->ATT.p, 0, h->ATT.bytes));

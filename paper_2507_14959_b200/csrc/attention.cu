@@ -200,11 +200,8 @@ __global__ void __launch_bounds__(512) attention_mma_kernel(const bf16* __restri
 // ---------------------------------------------------------------------------------------
 constexpr int AQ = 128;                    // query rows per tile
 constexpr int AKB = 208;                   // keys per score block
-constexpr int ATT_MAX_SHARES = 3;          // softmax warps per lane quarter (they split the key columns)
-#ifndef PM_ATT_SHARES
-#define PM_ATT_SHARES 2
-#endif
-constexpr int ATT_SHARES = PM_ATT_SHARES;  // the multi-block kernel's choice: block = 32 + 128 * ATT_SHARES threads
+constexpr int ATT_SHARES = 2;              // softmax warps per lane quarter of the multi-block kernel (they split the key columns)
+constexpr int ATT_THREADS = 32 + 128 * ATT_SHARES;
 constexpr int AQ_BYTES = AQ * 128;
 constexpr int AKB_BYTES = AKB * 128;
 constexpr int ATT_MAX_BLOCKS = 3;
@@ -511,15 +508,11 @@ __device__ __noinline__ void redo_groups(const AttnArgs& args, const uint32_t* m
         }
 }
 
-// Share k of `shares` takes the 16-key pieces [att_first(shares, k), att_first(shares, k + 1)) of a key
-// block (capped to the block's pieces) and leaves its P at the start of its own score columns.
-__host__ __device__ constexpr int att_first(int shares, int k) {
-    return shares == 1 ? (k == 0 ? 0 : 13) : shares == 2 ? (k == 0 ? 0 : k == 1 ? 7 : 13)
-                                                         : (k == 0 ? 0 : k == 1 ? 5 : k == 2 ? 9 : 13);
-}
+// Share k takes the 16-key pieces [att_first(k), att_first(k + 1)) of a key block (capped to the block's pieces) and
+// leaves its P at the start of its own score columns.
+__host__ __device__ constexpr int att_first(int k) { return k == 0 ? 0 : k == 1 ? 7 : 13; }
 
-template <int SHARES>
-__global__ void __launch_bounds__(32 + 128 * SHARES, 1)
+__global__ void __launch_bounds__(ATT_THREADS, 1)
 attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kv,
                     const __grid_constant__ AttnArgs args) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -548,7 +541,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     auto v_bar = [&](int b) { return bars + 96u + 8u * (uint32_t)b; };       // value block b landed
     uint8_t* bar_ptr = smem_raw + (bars - base);
     float* sums_base = reinterpret_cast<float*>(bar_ptr + 160);  // two tiles in turn: [share][row]
-    constexpr int shares = SHARES;
+    constexpr int shares = ATT_SHARES;
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(bar_ptr + 128);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_ptr + 136);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -646,7 +639,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 // first block are everybody's reference), the others' at the start of their own columns
                 uint32_t p_col = 16;
                 for (int kk = 0; kk < pieces; ++kk) {
-                    if (kk > 0 && (kk == att_first(shares, 1) || kk == att_first(shares, 2))) p_col = (uint32_t)(kk * 16);
+                    if (kk == att_first(1)) p_col = (uint32_t)(kk * 16);
                     umma_bf16_ts(o_tmem, tmem_base + r * (uint32_t)AKB + p_col, dv0 + bo + 128 * kk, idesc_pv, (b > 0 || kk > 0) ? 1u : 0u);
                     p_col += 8;
                 }
@@ -672,7 +665,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         bool ok = true;
         for (int u = u0; u < u1 && ok; ++u) {
             const uint32_t par = (uint32_t)(u - u0) & 1u;
-            float* sums = sums_base + par * ATT_MAX_SHARES * AQ;
+            float* sums = sums_base + par * ATT_SHARES * AQ;
             const int fh = u / args.n_qtiles, qt = u % args.n_qtiles, f = fh / args.heads, h = fh % args.heads;
             const int q_row = qt * AQ + row;
             const bool warp_active = qt * AQ + quarter * 32 < T;      // else: no row of this warp exists
@@ -686,7 +679,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 const uint32_t t_s = t_lane + r * (uint32_t)AKB;
                 // this warp's columns of key block b
                 const int np = min(AKB, args.tpad - b * AKB) / 16;
-                const int p0 = min(att_first(shares, share), np), p1 = min(att_first(shares, share + 1), np);
+                const int p0 = min(att_first(share), np), p1 = min(att_first(share + 1), np);
                 if (warp_active) {
                     if (b == 0) mc = score_reference(t_s, T) * c;
                     if (p1 > p0) {
@@ -695,7 +688,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                         tmem_st_wait();
                     }
                 }
-                if (b == n_blocks - 1 && shares > 1) {
+                if (b == n_blocks - 1) {
                     sums[share * AQ + row] = l;
                     __syncwarp();
                     if (lane == 0) mbar_arrive(sum_bar);
@@ -705,24 +698,22 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 if (lane == 0) mbar_arrive(c_bar(r));
             }
             if (!ok) break;
-            if (shares > 1) {
-                ok = mbar_wait(sum_bar, par, abort_flag, args.status);
-                ok = __all_sync(0xFFFFFFFFu, ok);
-                if (!ok) break;
-                l = 0.f;
+            ok = mbar_wait(sum_bar, par, abort_flag, args.status);
+            ok = __all_sync(0xFFFFFFFFu, ok);
+            if (!ok) break;
+            l = 0.f;
 #pragma unroll
-                for (int k = 0; k < shares; ++k) l += sums[k * AQ + row];
-            }
+            for (int k = 0; k < shares; ++k) l += sums[k * AQ + row];
             if (q_row < T && !(l < ROW_SUM_LIMIT)) redo |= redo_bit(u - u0);
             // O = sum over the key blocks of P V is complete: the finished rows are written out
             ok = mbar_wait(o_bar, par, abort_flag, args.status);
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
             tc_fence_after();
-            // the output columns are split between the first two shares (all 64 to the only one)
-            constexpr int OCOLS = shares == 1 ? 64 : 32;
+            // the output columns are split between the shares
+            constexpr int OCOLS = HD / shares;
             uint32_t v[OCOLS];
-            const bool writes = warp_active && share * OCOLS < 64;
+            const bool writes = warp_active;
             if (writes) {
 #pragma unroll
                 for (int part = 0; part < OCOLS / 32; ++part) tmem_ld32(t_lane + ATT_O_COL + (uint32_t)(share * OCOLS + part * 32), v + part * 32);
@@ -1005,7 +996,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
 
 // ---------------------------------------------------------------------------------------
 // Few (frame, head) pairs of one key block: one CTA per 16 query rows.  With few pairs the kernels above leave most SMs
-// idle and each pair is one long chain (two sweeps over the scores through tensor memory); here the pair's rows
+// idle and each pair is one long chain (a sweep over the scores through tensor memory between two products); here the pair's rows
 // spread over the SMs and four warps split the keys, so a warp has at most four 16-key groups: scores on
 // mma.sync, softmax against the warp's own maximum in registers, P V, and the four partial results are merged
 // through shared memory.  K and V arrive by TMA (128B swizzle, which is what ldmatrix wants), each on a barrier.
@@ -1218,11 +1209,11 @@ cudaError_t launch_attention_tc(const Launch& L, const CUtensorMap& tm_q, const 
         return e;
     }
     // all of tensor memory and most of the shared memory: one CTA per SM
-    const size_t smem = 2 * (size_t)AQ_BYTES + (size_t)a.n_blocks * 2 * AKB_BYTES + 160 + 2 * ATT_MAX_SHARES * AQ * sizeof(float);
+    const size_t smem = 2 * (size_t)AQ_BYTES + (size_t)a.n_blocks * 2 * AKB_BYTES + 160 + 2 * ATT_SHARES * AQ * sizeof(float);
     static SmemGrant grant;
-    if (cudaError_t e = grant.ensure(attention_tc_kernel<ATT_SHARES>, (int)smem); e != cudaSuccess) return e;
+    if (cudaError_t e = grant.ensure(attention_tc_kernel, (int)smem); e != cudaSuccess) return e;
     ProfScope ps(L, KC_ATTENTION);
-    cudaError_t e = launch_overlapped(L, attention_tc_kernel<ATT_SHARES>, n_sms > 0 ? std::min(a.n_units, n_sms) : a.n_units, 32 + 128 * ATT_SHARES,
+    cudaError_t e = launch_overlapped(L, attention_tc_kernel, n_sms > 0 ? std::min(a.n_units, n_sms) : a.n_units, ATT_THREADS,
                                       smem, 1, tm_q, tm_kv, a);
     BUMP(L);
     return e;

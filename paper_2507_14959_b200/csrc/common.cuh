@@ -36,7 +36,7 @@ struct LinearDev {
     float* bias = nullptr;     // [n_out]
     LoraArena lora;
     // tensor maps of the static operands (bf16 build only)
-    CUtensorMap tm_w, tm_at, tm_bt;
+    CUtensorMap tm_w, tm_bt;
     bool has_tm = false;
     // the CTA-pair GEMM's, by index of its tile width: boxes of half a tile's output columns
     CUtensorMap tm_pw[PM_PAIR_WIDTHS], tm_pbt[PM_PAIR_WIDTHS];
@@ -149,7 +149,7 @@ cudaError_t launch_attention_tc(const Launch& L, const CUtensorMap& tm_q, const 
 // patch gather, and the CLS rows of x
 template <typename T>
 cudaError_t launch_im2col(const Launch& L, const T* frames, const int* perm, T* out, int n_frames,
-                          int img, int patch, const float* cls, const float* pos, T* x, int d);
+                          int img, int patch, const float* cls, const float* pos, T* x, int d, int n_sms);
 // fp32 debug / reference-quality linear: t32 = scaled shrink per (row, set position, rank)
 template <typename T>
 cudaError_t launch_naive_linear(const Launch& L, const LinearDev& lin, const RouteDev& R,

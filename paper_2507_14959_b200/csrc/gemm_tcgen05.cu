@@ -822,10 +822,7 @@ bool tm_encode_slab(CUtensorMap* tm, const void* base, int k_in, uint64_t rows, 
     return tm_encode_4d(tm, base, dims, strides, box, 128);
 }
 
-#ifndef PM_GEMM_EPI_WARPS
-#define PM_GEMM_EPI_WARPS 8
-#endif
-constexpr int GEMM_EPI_WARPS = PM_GEMM_EPI_WARPS;      // 4 or 8
+constexpr int GEMM_EPI_WARPS = 8;
 
 template <int BN, int EPI, bool LNF = false>
 static cudaError_t launch_gemm_bn(const Launch& L, const CUtensorMap& tm_x, const CUtensorMap& tm_w,

@@ -273,10 +273,10 @@ __global__ void __launch_bounds__(256) im2col_kernel(const T* __restrict__ frame
 
 template <typename T>
 cudaError_t launch_im2col(const Launch& L, const T* frames, const int* perm, T* out, int n_frames,
-                          int img, int patch, const float* cls, const float* pos, T* x, int d) {
+                          int img, int patch, const float* cls, const float* pos, T* x, int d, int n_sms) {
     const int g = img / patch;
     const size_t total = (size_t)n_frames * g * g * (3 * patch * patch / Vec16<T>::N);
-    const int blocks = (int)((total + 255) / 256 < 148 * 16 ? (total + 255) / 256 : 148 * 16);
+    const int blocks = (int)std::min<size_t>((total + 255) / 256, 16 * (size_t)n_sms);
     if (blocks == 0) return cudaSuccess;
     ProfScope ps(L, KC_OTHER);
     // launched plainly: with it the forward's kernels start behind the routing plan, see Launch::ordered
@@ -284,8 +284,8 @@ cudaError_t launch_im2col(const Launch& L, const T* frames, const int* perm, T* 
     BUMP(L);
     return cudaGetLastError();
 }
-template cudaError_t launch_im2col<float>(const Launch&, const float*, const int*, float*, int, int, int, const float*, const float*, float*, int);
-template cudaError_t launch_im2col<bf16>(const Launch&, const bf16*, const int*, bf16*, int, int, int, const float*, const float*, bf16*, int);
+template cudaError_t launch_im2col<float>(const Launch&, const float*, const int*, float*, int, int, int, const float*, const float*, float*, int, int);
+template cudaError_t launch_im2col<bf16>(const Launch&, const bf16*, const int*, bf16*, int, int, int, const float*, const float*, bf16*, int, int);
 
 // ---------------------------------------------------------------------------------------
 // fp32 debug build: linear with unmerged LoRA terms on CUDA cores
