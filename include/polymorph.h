@@ -261,10 +261,12 @@ int pm_set_graphs(pm_handle h, int on);
 /* Batches of a few frames of a small model (d <= 384 with 64-wide heads, mlp <= 1536, tokens <= 256,
  * max_set * ceil(max_rank / 16) <= 8, bf16 build, and n_frames * ceil(tokens / 16) <= the number of SMs) --
  * the single-stream operating point of Sec. 4 -- run the whole forward (patch embedding, every block with
- * its unmerged LoRA terms of Sec. 3.1, heads, sigmoid, merge) as ONE kernel in which a CTA owns 16 token
- * rows from the first layer to the last.  pm_forward and pm_forward_device_sets use it for such batches
- * (same results within rounding as the layer-by-layer kernels; about 330 against 545 us per DeiT-tiny
- * frame and step on a B200); pm_set_small_batch_kernel(h, 0) sends them through the layer-by-layer kernels
+ * its unmerged LoRA terms of Sec. 3.1, heads, sigmoid, merge) as ONE kernel in which a tile of 16 token rows goes from
+ * the first layer to the last in one CTA or, while the SMs suffice, in a cluster of one CTA per head.  pm_forward and
+ * pm_forward_device_sets use it for such batches (same results within rounding as the layer-by-layer kernels).  On a B200, per
+ * DeiT-tiny forward with one rank-4 adapter on every block: 1 to 3 frames (clusters) 270 against 513 to 525 us, 4 to 11
+ * frames (one CTA per tile) 400 against 525 to 554; with adapters on the last two blocks a frame and step takes 189 us.
+ * pm_set_small_batch_kernel(h, 0) sends such batches through the layer-by-layer kernels
  * instead.  Larger models and batches use a second small-batch form while the switch is on: a linear whose rows
  * are few enough for its output tiles to fit the SMs in one wave runs as one kernel (shrink, LayerNorm
  * statistics, GEMM and LoRA terms together); switched off, every linear takes the kernels of the large batches.
