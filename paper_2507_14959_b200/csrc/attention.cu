@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(512) attention_mma_kernel(const bf16* __restri
 // one (per region: one mbarrier "scores formed", one "probabilities written"), and issues a block's P V product as
 // soon as its probabilities are written.  ATT_SHARES softmax warps per lane quarter split the key columns of a
 // block; they exchange row sums through shared memory.
-// 16 frames of 577 tokens, 12 heads: 77.3 us with a pass for the maxima and a CTA per tile, 44.7 us now.
+// 16 frames of 577 tokens, 12 heads: 77.3 us with a pass for the maxima and a CTA per tile, 45.6 us now.
 // (One key block goes to the pipelined kernel further down.)
 // ---------------------------------------------------------------------------------------
 constexpr int AQ = 128;                    // query rows per tile
@@ -309,7 +309,7 @@ __device__ __forceinline__ float score_probs_sweep(uint32_t t_s, uint32_t t_p, i
 // range is returned.  Software pipeline: while the exponentials of a piece go through the special-function unit, the
 // next piece is loaded and the one before is summed, packed and stored -- with one piece after the other the warps of
 // a scheduler queued for that unit together and idled together.  P of a piece is stored after the next piece has been
-// loaded.  For the kernel with two softmax warps per scheduler (47.9 -> 44.7 us, see there); with four, whose threads
+// loaded.  For the kernel with two softmax warps per scheduler (47.9 -> 44.7 us); with four, whose threads
 // have 96 registers, it spills (86.6 -> 96.9 us).
 __device__ __forceinline__ float score_probs_sweep_ahead(uint32_t t_s, uint32_t t_p, int np, int valid, float c, float mc) {
     uint32_t va[16], vb[16];
@@ -388,7 +388,7 @@ __device__ __forceinline__ float score_probs_sweep_ahead(uint32_t t_s, uint32_t 
 // The rows described above are computed again when the CTA's tiles are done and the operands' shared memory is free, in groups
 // of 16 query rows.  (A call in the sweep's loop costs its registers: 256 frames 87 -> 130 us.)  Until then a thread notes them
 // as one bit per tile of its row; the last bit stands for all further tiles.  256 frames of 197 tokens, 12 heads: 86 us
-// without such rows, 153 with one row in a hundred out of range, 401 with all (row by row in the loop: 87, 1700, 35000).
+// without such rows, 156 with one row in a hundred out of range, 399 with all (row by row in the loop: 87, 1700, 35000).
 __device__ __forceinline__ uint32_t redo_bit(int tile) { return 1u << min(tile, 31); }
 
 // One group by one warp, with the rows' true (running) maxima on mma.sync.  `stage`: REDO_STAGE bytes of shared memory of
@@ -777,7 +777,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 // 32 (w mod 4) .. +31 only) and split the key columns: the first seven 16-key pieces and the rest.
 // The sweeps are chains of dependent operations, so what bounds them is how many warps a scheduler can switch between
 // -- four per scheduler here against two with one warp per quarter -- and how many sweeps a tile needs: one (see
-// score_reference; with a sweep for the row maxima and their exchange in front of it, 256 frames of 197 tokens, 12 heads: 99.6 us, now 86.6).
+// score_reference; with a sweep for the row maxima and their exchange in front of it, 256 frames of 197 tokens, 12 heads: 99.6 us, now 86.4).
 // The halves exchange their row sums through shared memory (mbarriers, bounded waits).
 // Column map of a tile's 256-column slot: scores 0..207; P of the first half over 16..71 (the first 16 columns stay:
 // both halves read their reference there), P of the second half in 208..255 (so that it never lands on scores the
