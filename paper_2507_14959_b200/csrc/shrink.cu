@@ -36,18 +36,24 @@ constexpr int T_F32 = BM * PM_SLAB * 4;                // 8 KB: a slab's partial
 
 // The forms: Full for more than two tiles per SM, Mid for up to two, Wide and Split (a cluster per tile) for up to one.
 //   KPS: K blocks per stage.  EW: epilogue warps.  GROUP: slabs per pass over x.
-//   LIST / C_LIST: slabs whose plan entries / LayerNorm terms fit the prepared list; the rest is read where it is used.
-struct Full { static constexpr int KPS = 1, EW = 4, GROUP = 8, LIST = 32, C_LIST = 12, CTAS = 3; };
-struct Mid { static constexpr int KPS = 1, EW = 8, GROUP = 16, LIST = 64, C_LIST = 32, CTAS = 2; };
-struct Wide { static constexpr int KPS = 2, EW = 8, GROUP = 16, LIST = 64, C_LIST = 64, CTAS = 1; };
-struct Split { static constexpr int KPS = 2, EW = 8, GROUP = 8, LIST = 64, C_LIST = 1, CTAS = 1; };
+//   M_LIST / C_LIST: slabs whose masks and scales / LayerNorm terms fit the prepared list; the rest is read where it is used.
+struct Full { static constexpr int KPS = 1, EW = 4, GROUP = 8, M_LIST = 40, C_LIST = 12, CTAS = 3; };
+struct Mid { static constexpr int KPS = 1, EW = 8, GROUP = 16, M_LIST = 64, C_LIST = 32, CTAS = 2; };
+struct Wide { static constexpr int KPS = 2, EW = 8, GROUP = 16, M_LIST = 64, C_LIST = 64, CTAS = 1; };
+struct Split { static constexpr int KPS = 2, EW = 8, GROUP = 8, M_LIST = 64, C_LIST = 1, CTAS = 1; };
+// Slabs of a pair that are told apart by use: 24 adapters (three frames of eight) of rank 64.  A pair with more takes every slab
+// for both of its tiles.  Lists of 32 (Full) and 64 slabs did that from rank 32 on; 1 to 8 of 128 adapters per 197-token frame,
+// shrink + GEMM, before -> now:  256 frames (Full), rank 32: 768 -> 2304 291 -> 270 us, 3072 -> 768 440 -> 375 us; rank 64:
+// 475 -> 439 and 729 -> 604 us;  128 frames (Mid), rank 64: 260 -> 233 and 462 -> 390 us.
+constexpr int LIST = 96;
 
 template <typename F>
 struct Tail {
-    uint4 mask[F::LIST];
+    uint4 mask[F::M_LIST];
     float c[F::C_LIST][2 * PM_SLAB];                   // LayerNorm folded in: c1 then c2 of the slab
-    float scale[F::LIST];
-    int slab[F::LIST], place[F::LIST];                 // arena slab; place in the tile's list
+    float scale[F::M_LIST];
+    int slab[LIST];                                    // arena slab
+    uint8_t place[LIST];                               // place in the tile's list
     float2 half_stats[F::EW == 8 ? 2 : 1][F::EW == 8 ? BM : 1];     // mean, sum of squared deviations of half a row
     uint64_t bars[2 * MAX_STAGES + 4];
     uint32_t tmem_slot;
@@ -81,7 +87,7 @@ __host__ __device__ constexpr int recv_bytes() { return S > 1 ? (S - 1) * ((F::G
 template <typename F, bool STATS, int S>
 __global__ void __launch_bounds__(32 * (FIRST_EW + F::EW), F::CTAS)
 shrink_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_at, const ShrinkArgs args) {
-    constexpr int KPS = F::KPS, EW = F::EW, GROUP = F::GROUP, LIST = F::LIST;
+    constexpr int KPS = F::KPS, EW = F::EW, GROUP = F::GROUP;
     constexpr int X_BYTES = KPS * X_BLOCK, A_SLAB = KPS * A_BLOCK;
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t base = smem_u32(smem);
@@ -142,7 +148,8 @@ shrink_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ 
             const uint32_t bon = __ballot_sync(0xFFFFFFFFu, on), boff = __ballot_sync(0xFFFFFFFFu, off);
             const uint32_t below = (1u << lane) - 1u;
             const int to = on ? na + __popc(bon & below) : LIST - 1 - nz - __popc(boff & below);
-            if (on || off) { tail.mask[to] = mk; tail.slab[to] = slab; tail.scale[to] = sc; tail.place[to] = i; }
+            if (on || off) { tail.slab[to] = slab; tail.place[to] = (uint8_t)i; }
+            if (on && to < F::M_LIST) { tail.mask[to] = mk; tail.scale[to] = sc; }
             na += __popc(bon);
             nz += __popc(boff);
         }
@@ -352,8 +359,10 @@ shrink_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ 
         const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16);
         // slab i of the list: accumulator -> scale, mask, folded LayerNorm -> bf16 -> t
         auto finish = [&](uint32_t* v, int i) {
-            const uint32_t mk = listed ? reinterpret_cast<const uint32_t*>(&tail.mask[i])[quarter] : __ldg(args.tile_mask + (plan0 + i) * 4 + quarter);
-            const float sc = (mk >> lane) & 1u ? (listed ? tail.scale[i] : __ldg(args.tile_scale + plan0 + i)) : 0.f;
+            const int at = listed ? tail.place[i] : i;
+            const bool held = listed && i < F::M_LIST;
+            const uint32_t mk = held ? reinterpret_cast<const uint32_t*>(&tail.mask[i])[quarter] : __ldg(args.tile_mask + (plan0 + at) * 4 + quarter);
+            const float sc = (mk >> lane) & 1u ? (held ? tail.scale[i] : __ldg(args.tile_scale + plan0 + at)) : 0.f;
             if constexpr (STATS) {
                 if (listed && i < F::C_LIST) {
                     const float* c = tail.c[i];
@@ -373,7 +382,7 @@ shrink_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ 
 #pragma unroll
             for (int j = 0; j < PM_SLAB; j += 2)
                 ow[j >> 1] = pack_bf16(__uint_as_float(v[j]) * sc, __uint_as_float(v[j + 1]) * sc);
-            uint4* dst = reinterpret_cast<uint4*>(args.tbuf + ((plan0 + (listed ? tail.place[i] : i)) * BM + r) * PM_SLAB);
+            uint4* dst = reinterpret_cast<uint4*>(args.tbuf + ((plan0 + at) * BM + r) * PM_SLAB);
             dst[0] = o[0];
             dst[1] = o[1];
         };

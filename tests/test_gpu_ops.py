@@ -367,6 +367,44 @@ def test_lora_linear_several_slab_groups_through_the_shortest_ring(frames, rank,
     lin.close()
 
 
+@pytest.mark.parametrize("frames,tokens,rank,n_ad,largest", [(300, 197, 32, 24, (33, 48)), (300, 197, 64, 24, (65, 96)), (1240, 32, 64, 40, (97, 160))])
+def test_lora_linear_of_long_slab_lists_on_full_grids(frames, tokens, rank, n_ad, largest):
+    """Three shrink CTAs per SM, sets of 0 to 8 adapters: row-tile pairs of up to 48 and 96 slabs, of which a tile's own
+    masks and scales fit the prepared list or do not, and pairs of more slabs than are listed.  Twice, so that a slab
+    left unwritten for a tile that does not use it would show; against float64 sums of the same bf16 inputs, tolerance as
+    for the other linears."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    k_in, n_out, rows = 192, 256, frames * tokens
+    gen = torch.Generator(device="cuda").manual_seed(frames + rank)
+
+    def draw(shape, std):
+        return (torch.randn(shape, generator=gen, device="cuda") * std).bfloat16()
+    x, w, b = draw((rows, k_in), 1.0), draw((k_in, n_out), 0.02), draw((n_out,), 0.02)
+    A = [draw((k_in, rank), 0.02) for _ in range(n_ad)]
+    B = [draw((rank, n_out), 0.02) for _ in range(n_ad)]
+    host = lambda t: t.float().cpu().numpy()  # noqa: E731
+    lin = binding.Linear(host(w), host(b), max_adapters=n_ad, max_rank=rank, max_set=8, max_frames=frames, tokens=tokens, epilogue=0)
+    for a in range(n_ad):
+        lin.register(a, rank, 1.0, host(A[a]), host(B[a]))
+    y = torch.full((rows, n_out), float("nan"), device="cuda", dtype=torch.bfloat16)
+    g = np.random.default_rng(rows + rank)
+    for _ in range(2):
+        sets = [sorted(int(a) for a in g.choice(n_ad, size=int(g.integers(0, 9)), replace=False)) for _ in range(frames)]
+        union = [set().union(*sets[r // tokens:min(r + 255, rows - 1) // tokens + 1]) for r in range(0, rows, 256)]
+        assert largest[0] <= max(len(u) for u in union) * rank // 16 <= largest[1]
+        off, ids = wl.sets_to_csr(sets)
+        lin.forward(x, frames, off, ids, y)
+        assert lin.status() == 0
+        want = x.double() @ w.double() + b.double()
+        for f, s in enumerate(sets):
+            r = slice(f * tokens, (f + 1) * tokens)
+            for a in s:
+                want[r] += (x[r].double() @ A[a].double()) @ B[a].double()
+        np.testing.assert_allclose(to_np(y), want.cpu().numpy(), **TOL[0])
+    lin.close()
+
+
 @pytest.mark.parametrize("frames,what", [(1, "64-wide, K in four"), (2, "128-wide, K in four"), (4, "128-wide, K in two"),
                                          (8, "192-wide, K in two"), (12, "256-wide, K in two"), (33, "shrink with K in two")])
 def test_lora_intermediate_of_a_split_k_is_not_rounded_share_by_share(frames, what):
