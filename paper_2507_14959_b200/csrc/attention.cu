@@ -569,7 +569,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     dep_release();
 
     if (warp == 0) {
-        if (lane == 0 && u0 < u1) {
+        if (u0 < u1 && elect_one()) {
             // ------------------------------------------------------ TMA + MMA issue
             // Steps run over all tiles: key block g % n_blocks of tile u0 + g / n_blocks.  The scores of step g + 1 are formed
             // in the other region while the softmax warps are at step g; products issued by this thread run in issue
@@ -846,7 +846,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     dep_release();
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---------------------------------------------------------------- TMA producer
             bool ok = true;
             dep_wait();                            // everything else follows from what these loads bring
@@ -864,7 +864,7 @@ attention_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---------------------------------------------------------------- MMA issue
             const uint32_t idesc_s = instr_desc(args.tpad), idesc_pv = instr_desc_b_mn(HD);
             bool ok = true;

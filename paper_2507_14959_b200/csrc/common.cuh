@@ -279,6 +279,16 @@ size_t latency_smem_bytes(int d, int mlp, int patch_dim, int tokens, int layers)
 // cooperative launch, which fails with an error instead of starting if it cannot be.
 cudaError_t launch_latency_forward(const Launch& L, const LatArgs& a);
 
+// True in one thread of a converged warp, always the same one.  The loops that issue copies and MMAs run under this and
+// not under `lane == 0`: their instructions take uniform registers, which the compiler fills directly only where it knows
+// that a single thread runs; behind a lane test every operand goes through a converging sequence.  One stage of
+// wait + 4 pair MMAs + commit costs the thread 286 cycles against 585, and 256 x 256 x 64 MMAs need 512.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p) :: "memory");
+    return p != 0;
+}
+
 // Launch with programmatic stream serialization (the kernel may start once every CTA of the one before it on the
 // stream has released its dependents; it awaits that kernel's results itself with dep_wait()), with or
 // without thread-block clusters along x.  The first one after L.ordered was set starts behind its predecessor's end.

@@ -835,7 +835,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
     if (CL) cluster_barrier();                    // every peer runs and has set its barriers up
     // ---- the weight producer: one thread, the whole network's static operands in consumption order
     if (cx.warp == LT_CWARPS) {
-        if (cx.lane == 0) {
+        if (elect_one()) {
             SlabTab none;
             none.n = 0;
             produce_linear<CL>(cx, args.lin + (size_t)args.layers * 4, none, *as, rs, args.slabs_max, d, false);
@@ -850,7 +850,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) latency_forward_kernel(const __
     if (cx.warp == LT_CWARPS + 1) {
         unsigned int* counter = args.bar + (CL ? f * cx.share + cx.rank : f);       // shared tiles: one per frame and head
         uint32_t idx = 0;
-        for (int l = 0; cx.lane == 0 && l < args.layers && !*abort_flag; ++l) {
+        if (elect_one()) for (int l = 0; l < args.layers && !*abort_flag; ++l) {
             // Twice per block -- for the first head, then for the others -- : the consumer warps have stored this
             // CTA's keys and values (ordinary stores, fetched by TMA on the other side: order the two proxies as
             // well as the scopes), so the CTA counts itself in: everything its threads stored up to there is

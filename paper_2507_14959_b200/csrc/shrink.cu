@@ -181,7 +181,7 @@ shrink_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ 
     if (!usable) {
         // fall through to the teardown
     } else if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             // -------------------------------------------------------------- x copies
             int stage = 0;
             uint32_t phase = 0;
@@ -202,7 +202,7 @@ shrink_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ 
             }
         }
     } else if (warp == 2) {
-        if (lane == 0) {
+        if (elect_one()) {
             // -------------------------------------------------------------- adapter copies (not the earlier kernel's results)
             int stage = 0;
             uint32_t phase = 0;
@@ -224,7 +224,7 @@ shrink_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ 
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             // -------------------------------------------------------------- MMA issuer
             const uint64_t da0 = smem_desc(base, 128), db0 = smem_desc_groups(base + X_BYTES, KPS * 1024);
             int stage = 0;

@@ -237,7 +237,7 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     if (!usable) {
         // fall through to the teardown
     } else if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             // -------------------------------------------------------------- x and W copies
             int stage = 0;
             uint32_t phase = 0;
@@ -278,7 +278,7 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
             }
         }
     } else if (warp == 2) {
-        if (lane == 0 && na > 0) {
+        if (na > 0 && elect_one()) {
             // -------------------------------------------------------------- adapter copies
             int stage = 0;
             uint32_t phase = 0;
@@ -308,7 +308,7 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             // -------------------------------------------------------------- MMA issuer
             const uint32_t idesc = instr_desc(BN);
             const uint64_t da0 = smem_desc(base, 128), db0 = smem_desc(base + X_BYTES, 128);

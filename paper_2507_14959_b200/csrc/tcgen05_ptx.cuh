@@ -11,15 +11,6 @@ constexpr long long WAIT_LIMIT_CYCLES = 4000000000ll;     // ~2 s
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
-// True in one thread of a converged warp, always the same one.  The loops that issue copies and MMAs run under this and
-// not under `lane == 0`: their instructions take uniform registers, which the compiler fills directly only where it knows
-// that a single thread runs; behind a lane test every operand goes through a converging sequence.  One stage of
-// wait + 4 pair MMAs + commit costs the thread 286 cycles against 585, and 256 x 256 x 64 MMAs need 512.
-__device__ __forceinline__ bool elect_one() {
-    uint32_t p;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p) :: "memory");
-    return p != 0;
-}
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
