@@ -69,16 +69,16 @@ struct Smem {
 // chunks goes TMEM -> registers -> bias / GELU / residual / patch placement -> bf16 -> shared
 // memory -> TMA store (or straight to global memory).  Returns false once the CTA is aborting.
 // PAIR: the accumulator-free barrier lives in the even CTA of a pair (tempty_addr is a cluster address).
-// RES_SMEM: the residual rows come through shared memory (TMA into res_buf, four 2 KB chunks of this
-// warp, completion on res_bar) instead of per-thread global loads.
+// RES_SMEM: request_residual has asked TMA for the residual rows of this warp's two chunks, into the staging buffers that the
+// results will leave from (completion on res_bar); else per-thread global loads.
 template <int BN, int EPI, int HALVES, bool PAIR, bool LNF, bool RES_SMEM>
 __device__ __forceinline__ bool epilogue_tile(const GemmArgs& args, const CUtensorMap& tm_y, uint32_t staging,
                                               uint32_t& chunk_no, uint32_t tmem_base, int acc, uint32_t acc_phase,
                                               uint32_t tfull_addr, uint32_t tempty_addr, volatile int* abort_flag,
                                               int m, int n, int quarter, int half, int lane,
-                                              const CUtensorMap* tm_res, uint32_t res_buf, uint32_t res_bar,
-                                              uint32_t res_phase) {
+                                              uint32_t res_bar, uint32_t res_phase) {
     constexpr int CPW = BN / 32 / HALVES;         // 32-column chunks per epilogue warp
+    static_assert(!RES_SMEM || CPW == 2, "a staging buffer per chunk");
     const int row = m * BM + quarter * 32 + lane;     // m: 128-row tile index
     const bool row_ok = row < args.rows;
     const int n_chunks = min(BN / 32, (args.n_out - n * BN) / 32);      // even: n_out % 64 == 0
@@ -88,17 +88,7 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs& args, const CUtens
     // their latency hides behind the main loop.  (In-place use, y == residual, is safe: the
     // same thread reads an element here and is the only one to overwrite it below.)
     uint4 rr[(EPI == EPI_RESIDUAL && !RES_SMEM) ? CPW : 1][4];
-    if constexpr (EPI == EPI_RESIDUAL && RES_SMEM) {
-        // one thread asks TMA for this warp's chunks of the residual tile (rows past the end read as
-        // zero); the warp's reads of the previous tile's chunks are ordered before these writes
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) {
-            mbar_expect_tx(res_bar, (uint32_t)(my_chunks * 32 * 64));
-            for (int cc = 0; cc < my_chunks; ++cc)
-                tma_load_2d(res_buf + cc * (32 * 64), tm_res, n * BN + (c0 + cc) * 32, m * BM + quarter * 32, res_bar);
-        }
-    } else if constexpr (EPI == EPI_RESIDUAL) {
+    if constexpr (EPI == EPI_RESIDUAL && !RES_SMEM) {
 #pragma unroll
         for (int cc = 0; cc < CPW; ++cc) {
             if (cc < my_chunks && row_ok) {
@@ -139,7 +129,7 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs& args, const CUtens
             // every TMEM read of this accumulator is done: hand the buffer back early
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) { if (PAIR) mbar_arrive_cluster(tempty_addr); else mbar_arrive(tempty_addr); }
+            if (elect_one()) { if (PAIR) mbar_arrive_cluster(tempty_addr); else mbar_arrive(tempty_addr); }
         }
         // bias (and the folded LayerNorm: rstd (acc - mean g) + b) and GELU, two columns per instruction
         uint64_t fp[16];                                 // columns (2i, 2i+1) of this chunk
@@ -173,8 +163,8 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs& args, const CUtens
             for (int q = 0; q < 4; ++q) {
                 uint4 r4v;
                 if constexpr (RES_SMEM) {
-                    // same 64B swizzle as the store staging: 16-byte chunk q of row `lane`
-                    const uint32_t a = res_buf + cc * (32 * 64) + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4);
+                    // where this thread puts its result below: 16-byte chunk q of row `lane`
+                    const uint32_t a = staging + (chunk_no & 1u) * (32 * 64) + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4);
                     asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
                                  : "=r"(r4v.x), "=r"(r4v.y), "=r"(r4v.z), "=r"(r4v.w) : "r"(a));
                 } else {
@@ -208,14 +198,16 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs& args, const CUtens
             // [32 rows x 64 B] block, 16-byte chunks XOR-swizzled by (row >> 1) & 3 (64B
             // swizzle), then one TMA store; rows past the end are clipped by the tensor map
             const uint32_t buf = staging + (chunk_no & 1u) * (32 * 64);
-            if (lane == 0) bulk_wait_read1();        // the store that last used this buffer has read it
-            __syncwarp();
+            if constexpr (!RES_SMEM) {
+                if (elect_one()) bulk_wait_read1();  // the store that last used this buffer has read it
+                __syncwarp();
+            }
 #pragma unroll
             for (int q = 0; q < 4; ++q)
                 st_shared_v4(buf + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4), o[q]);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
-            if (lane == 0) {
+            if (elect_one()) {
                 tma_store_2d(&tm_y, buf, n0, m * BM + quarter * 32);
                 bulk_commit();
             }
@@ -227,6 +219,19 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs& args, const CUtens
         }
     }
     return true;
+}
+
+// Asks TMA for the residual rows of an epilogue warp's two chunks (rows past the end read as zero), into the warp's staging
+// buffers as soon as the stores of its previous tile have read them: a whole main loop ahead of their use.
+template <int BN>
+__device__ __forceinline__ void request_residual(const CUtensorMap& tm_res, uint32_t staging, uint32_t res_bar, int m, int n, int quarter, int half) {
+    if (elect_one()) {
+        bulk_wait_read0();
+        mbar_expect_tx(res_bar, 2 * 32 * 64);
+        for (int cc = 0; cc < 2; ++cc)
+            tma_load_2d(staging + cc * (32 * 64), &tm_res, n * BN + (half * 2 + cc) * 32, m * BM + quarter * 32, res_bar);
+    }
+    __syncwarp();
 }
 
 template <int BN, int EPI, int EW, bool LNF>
@@ -403,11 +408,11 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
             const int m = tile / args.n_tiles, n = tile % args.n_tiles;
             ok = epilogue_tile<BN, EPI, HALVES, false, LNF, false>(args, tm_y, staging, chunk_no, tmem_base, acc,
                                                               acc_phase, tfull_bar(acc), tempty_bar(acc), abort_flag,
-                                                              m, n, quarter, half, lane, nullptr, 0u, 0u, 0u);
+                                                              m, n, quarter, half, lane, 0u, 0u);
             if (!ok) break;
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
-        if (args.tma_store && lane == 0) bulk_wait_all();
+        if (args.tma_store && elect_one()) bulk_wait_all();
     }
 
     // ---------------------------------------------------------------------- teardown
@@ -437,59 +442,58 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
 //   tempty[a]  (even CTA)   both CTAs' epilogue warps have drained accumulator a
 // Up to six stages per CTA.  No TMA multicast is used.
 // ---------------------------------------------------------------------------------------
-constexpr int P_EW = 8;
-constexpr int P_THREADS = 64 + 32 * P_EW;
 constexpr int P_A_BYTES = BM * BK * 2;                 // 16 KB: this CTA's 128 rows of x
 constexpr int P_T_SLAB_BYTES = BM * PM_SLAB * 2;       // 4 KB
 constexpr int P_MAX_STAGES = 6;
-constexpr int P_RING_BYTES = 192 * 1024;               // stages, then (residual kernels) the residual landing area
-constexpr int P_STAGING_OFFSET = P_RING_BYTES;
-constexpr int P_PLAN_OFFSET = P_STAGING_OFFSET + P_EW * STAGING_BYTES_PER_WARP;
-constexpr int P_BAR_OFFSET = P_PLAN_OFFSET + PLAN_BYTES;
-constexpr int P_SMEM_TOTAL = P_BAR_OFFSET + 256;
-// By tile width and epilogue: a residual epilogue that takes the residual rows through shared memory (RESS) gives part
-// of the ring to an area into which TMA fetches the tile's rows ahead of the accumulator.
-template <int BN, int EPI, bool RESS>
+constexpr int P_MAX_EW = 16;
+constexpr int P_BAR_BYTES = 512;
+// By tile width: an epilogue warp takes 64 columns of one lane quarter (two chunks, a staging buffer for each), so 256 columns
+// take 16 warps.  What the staging leaves is the ring's.
+template <int BN>
 struct PairCfg {
-    static constexpr bool RES = EPI == EPI_RESIDUAL && RESS;
+    static constexpr int HALVES = BN / 64;                                 // epilogue warps per lane quarter
+    static constexpr int EW = 4 * HALVES;
+    static constexpr int THREADS = 64 + 32 * EW;
     static constexpr int B_BYTES = (BN / 2) * BK * 2;                      // this CTA's half of the W^T tile
     static constexpr int STAGE_BYTES = P_A_BYTES + B_BYTES;
     static constexpr int B_SLAB_BYTES = (BN / 2) * PM_SLAB * 2;
-    static constexpr int RES_BYTES_PER_WARP = RES ? (BN / 64) * 32 * 64 : 0;       // [32 rows x 32 bf16] chunks
-    static constexpr int FIT = (P_RING_BYTES - P_EW * RES_BYTES_PER_WARP) / STAGE_BYTES;
+    static constexpr int REST = EW * STAGING_BYTES_PER_WARP + PLAN_BYTES + P_BAR_BYTES;
+    static constexpr int FIT = (227 * 1024 - REST) / STAGE_BYTES;
     static constexpr int STAGES = FIT < P_MAX_STAGES ? FIT : P_MAX_STAGES;
-    static constexpr int RES_OFFSET = STAGES * STAGE_BYTES;
+    static constexpr int STAGING_OFFSET = STAGES * STAGE_BYTES;
+    static constexpr int PLAN_OFFSET = STAGING_OFFSET + EW * STAGING_BYTES_PER_WARP;
+    static constexpr int BAR_OFFSET = PLAN_OFFSET + PLAN_BYTES;
+    static constexpr int TOTAL = BAR_OFFSET + P_BAR_BYTES;
     static_assert(SLABS_PER_STAGE * B_SLAB_BYTES <= B_BYTES, "LoRA stage");
+    static_assert(8 * (2 * P_MAX_STAGES + 4) + 24 + 8 * P_MAX_EW <= P_BAR_BYTES, "barriers");
 };
 
-// RESS (residual epilogue only): residual through shared memory with a four-stage ring (short K, where
-// the epilogue is exposed) instead of per-thread loads with the full six stages (long K).
-template <int BN, int EPI, bool LNF, bool RESS>
-__global__ void __launch_bounds__(P_THREADS, 1)
+template <int BN, int EPI, bool LNF>
+__global__ void __launch_bounds__(PairCfg<BN>::THREADS, 1)
 lora_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                       const __grid_constant__ CUtensorMap tm_t, const __grid_constant__ CUtensorMap tm_bt,
                       const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_res,
                       const GemmArgs args) {
-    using C = PairCfg<BN, EPI, RESS>;
-    constexpr int HALVES = P_EW / 4;
-    constexpr int P_STAGES = C::STAGES;
+    using C = PairCfg<BN>;
+    constexpr int P_STAGES = C::STAGES, P_EW = C::EW;
+    constexpr bool RES = EPI == EPI_RESIDUAL;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = smem_u32(smem_raw);
     const uint32_t rank = cluster_ctarank();          // 0: issues the MMAs, 1: its peer
     uint8_t* smem = smem_raw;
-    const uint32_t bars = base + P_BAR_OFFSET;
+    const uint32_t bars = base + C::BAR_OFFSET;
     auto full_bar = [&](int s) { return bars + 8u * s; };
     auto empty_bar = [&](int s) { return bars + 8u * (P_MAX_STAGES + s); };
     auto tfull_bar = [&](int s) { return bars + 8u * (2 * P_MAX_STAGES + s); };
     auto tempty_bar = [&](int s) { return bars + 8u * (2 * P_MAX_STAGES + 2 + s); };
-    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + P_BAR_OFFSET + 8 * (2 * P_MAX_STAGES + 4));
+    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + C::BAR_OFFSET + 8 * (2 * P_MAX_STAGES + 4));
     // the peer CTA's TMEM base: written only by the peer (any time before the cluster barrier below),
     // never by this CTA, so there is no ordering to get wrong
     volatile uint32_t* peer_slot = tmem_slot + 1;
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + P_BAR_OFFSET + 8 * (2 * P_MAX_STAGES + 4) + 8);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::BAR_OFFSET + 8 * (2 * P_MAX_STAGES + 4) + 8);
     // res_bar[w]: the residual rows of epilogue warp w's chunks have landed (residual kernels)
     auto res_bar = [&](int w) { return bars + 8u * (2 * P_MAX_STAGES + 4) + 24u + 8u * w; };
-    int* plan = reinterpret_cast<int*>(smem + P_PLAN_OFFSET);
+    int* plan = reinterpret_cast<int*>(smem + C::PLAN_OFFSET);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int pair_id = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
@@ -500,7 +504,7 @@ lora_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     const int plan_stride = 1 + args.slab_cap;
     const int plan_tiles = args.tile_nslabs ? PLAN_BYTES / (4 * plan_stride) : 0;
     if (args.tile_nslabs) {
-        for (int i = threadIdx.x / 8; i < plan_tiles; i += P_THREADS / 8) {
+        for (int i = threadIdx.x / 8; i < plan_tiles; i += C::THREADS / 8) {
             const int tile = pair_id + i * n_pairs;
             if (tile >= total_tiles) break;
             const int m = 2 * (tile / args.n_tiles) + (int)rank;
@@ -653,7 +657,7 @@ lora_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         // ------------------------------------------------------------------ epilogue (both CTAs)
         const int quarter = warp & 3;
         const int half = (warp - 2) >> 2;
-        const uint32_t staging = base + P_STAGING_OFFSET + (uint32_t)(warp - 2) * STAGING_BYTES_PER_WARP;
+        const uint32_t staging = base + C::STAGING_OFFSET + (uint32_t)(warp - 2) * STAGING_BYTES_PER_WARP;
         dep_wait();                                   // row statistics, residual; rows that the kernel before still reads
         int acc = 0;
         uint32_t acc_phase = 0, res_phase = 0;
@@ -661,16 +665,16 @@ lora_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         bool ok = true;
         for (int tile = pair_id; tile < total_tiles && ok; tile += n_pairs) {
             const int m = 2 * (tile / args.n_tiles) + (int)rank, n = tile % args.n_tiles;
-            ok = epilogue_tile<BN, EPI, HALVES, true, LNF, C::RES>(
+            if constexpr (RES) request_residual<BN>(tm_res, staging, res_bar(warp - 2), m, n, quarter, half);
+            ok = epilogue_tile<BN, EPI, C::HALVES, true, LNF, RES>(
                 args, tm_y, staging, chunk_no, tmem_base, acc, acc_phase, tfull_bar(acc),
-                mapa_cluster(tempty_bar(acc), 0), abort_flag, m, n, quarter, half, lane, &tm_res,
-                base + C::RES_OFFSET + (uint32_t)(warp - 2) * C::RES_BYTES_PER_WARP,
+                mapa_cluster(tempty_bar(acc), 0), abort_flag, m, n, quarter, half, lane,
                 res_bar(warp - 2), res_phase);
             res_phase ^= 1u;
             if (!ok) break;
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
-        if (args.tma_store && lane == 0) bulk_wait_all();
+        if (args.tma_store && elect_one()) bulk_wait_all();
     }
 
     // ---------------------------------------------------------------------- teardown
@@ -855,7 +859,7 @@ static cudaError_t launch_gemm_epi(const Launch& L, const CUtensorMap& tm_x, con
     }
 }
 
-template <int BN, int EPI, bool LNF = false, bool RESS = false>
+template <int BN, int EPI, bool LNF = false>
 static cudaError_t launch_gemm_pair(const Launch& L, const CUtensorMap& tm_x, const CUtensorMap& tm_w,
                                     const CUtensorMap& tm_t, const CUtensorMap& tm_bt, const CUtensorMap& tm_y,
                                     const GemmArgs& a, int n_sms) {
@@ -866,11 +870,11 @@ static cudaError_t launch_gemm_pair(const Launch& L, const CUtensorMap& tm_x, co
             return cudaErrorInvalidValue;
     }
     static SmemGrant grant;
-    if (cudaError_t e = grant.ensure(lora_gemm_pair_kernel<BN, EPI, LNF, RESS>, P_SMEM_TOTAL); e != cudaSuccess) return e;
+    if (cudaError_t e = grant.ensure(lora_gemm_pair_kernel<BN, EPI, LNF>, PairCfg<BN>::TOTAL); e != cudaSuccess) return e;
     const int total = a.m_tiles * a.n_tiles;
     const int pairs = total < n_sms / 2 ? total : n_sms / 2;
     ProfScope ps(L, KC_GEMM);
-    cudaError_t e = launch_overlapped(L, lora_gemm_pair_kernel<BN, EPI, LNF, RESS>, 2 * pairs, P_THREADS, P_SMEM_TOTAL, 2,
+    cudaError_t e = launch_overlapped(L, lora_gemm_pair_kernel<BN, EPI, LNF>, 2 * pairs, PairCfg<BN>::THREADS, PairCfg<BN>::TOTAL, 2,
                                       tm_x, tm_w, tm_t, tm_bt, tm_y, tm_res, a);
     BUMP(L);
     return e;
@@ -887,9 +891,7 @@ static cudaError_t launch_gemm_pair_epi(const Launch& L, const CUtensorMap& tm_x
     }
     switch (a.epi) {
         case EPI_GELU: return launch_gemm_pair<BN, EPI_GELU>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
-        case EPI_RESIDUAL:
-            if (a.k_in <= 1024) return launch_gemm_pair<BN, EPI_RESIDUAL, false, true>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
-            return launch_gemm_pair<BN, EPI_RESIDUAL>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
+        case EPI_RESIDUAL: return launch_gemm_pair<BN, EPI_RESIDUAL>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
         case EPI_PATCH: return launch_gemm_pair<BN, EPI_PATCH>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
         default: return launch_gemm_pair<BN, EPI_NONE>(L, tm_x, tm_w, tm_t, tm_bt, tm_y, a, n_sms);
     }
