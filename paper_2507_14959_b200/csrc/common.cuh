@@ -15,7 +15,7 @@
 typedef __nv_bfloat16 bf16;
 
 #define PM_TILE_M 128          // rows of one GEMM tile
-#define PM_PAIR_WIDTHS 2       // tile widths of the CTA-pair GEMM: 192, 256
+#define PM_PAIR_WIDTHS 3       // tile widths of the CTA-pair GEMM: 128, 192, 256
 #define PM_SMALL_WIDTHS 4      // tile widths of the few-row linear kernel: 64, 128, 192, 256
 #define PM_SLAB 16             // LoRA ranks are handled in slabs of 16 (one UMMA K step)
 

@@ -13,7 +13,7 @@
 // warps per TMEM lane quarter, each taking half of the tile's columns).
 // Every mbarrier wait is bounded: on expiry the CTA raises an abort flag, records
 // PM_ERR_TIMEOUT in the status word, drains and returns.
-// The CTA-pair variant (lora_gemm_pair_kernel, cta_group::2, 256 x 256 or 256 x 192 tiles) serves most shapes, the single-CTA
+// The CTA-pair variant (lora_gemm_pair_kernel, cta_group::2, 256-row tiles of 128, 192 or 256 columns) serves most shapes, the single-CTA
 // kernel short K and other widths (pick_pair_width).  Both start while the kernel before them on the stream still runs
 // (programmatic dependent launch): 768 -> 768 with shrink on 197 x 256 rows 83.1 -> 79.5 us, on 197 x 37 rows 20.8 -> 19.6 us.
 #include "common.cuh"
@@ -431,7 +431,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
 }
 
 // ---------------------------------------------------------------------------------------
-// The same GEMM on CTA pairs (BN = 192 or 256).  Two CTAs of a cluster share one
+// The same GEMM on CTA pairs (BN = 128, 192 or 256).  Two CTAs of a cluster share one
 // 256 x BN output tile: each stages its own 128 rows of x (and of the t slabs) and HALF of the
 // W^T tile (and of the B slabs), so every byte of W^T crosses the L2 -> SM fabric once per 256
 // rows instead of once per 128, and one tcgen05.mma.cta_group::2 (M = 256) issued by the even
@@ -440,11 +440,11 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
 //   empty[s]   (both CTAs)  the pair MMAs that read stage s are done (multicast commit)
 //   tfull[a]   (both CTAs)  accumulator a is complete (multicast commit)
 //   tempty[a]  (even CTA)   both CTAs' epilogue warps have drained accumulator a
-// Up to six stages per CTA.  No TMA multicast is used.
+// Up to eight stages per CTA.  No TMA multicast is used.
 // ---------------------------------------------------------------------------------------
 constexpr int P_A_BYTES = BM * BK * 2;                 // 16 KB: this CTA's 128 rows of x
 constexpr int P_T_SLAB_BYTES = BM * PM_SLAB * 2;       // 4 KB
-constexpr int P_MAX_STAGES = 6;
+constexpr int P_MAX_STAGES = 8;
 constexpr int P_MAX_EW = 16;
 constexpr int P_BAR_BYTES = 512;
 // By tile width: an epilogue warp takes 64 columns of one lane quarter (two chunks, a staging buffer for each), so 256 columns
@@ -897,7 +897,7 @@ static cudaError_t launch_gemm_pair_epi(const Launch& L, const CUtensorMap& tm_x
     }
 }
 
-constexpr int PAIR_WIDTHS[PM_PAIR_WIDTHS] = {192, 256};
+constexpr int PAIR_WIDTHS[PM_PAIR_WIDTHS] = {128, 192, 256};
 
 bool gemm_encode_pair_maps(LinearDev& lin, int max_adapters, int slabs_max) {
     for (int i = 0; i < PM_PAIR_WIDTHS; ++i) {
@@ -909,18 +909,28 @@ bool gemm_encode_pair_maps(LinearDev& lin, int max_adapters, int slabs_max) {
     return true;
 }
 
-// The tile width of the pair kernel (index into PAIR_WIDTHS), or -1 for the single-CTA kernel.  Measured on 64 and 256
-// frames of 197 tokens, rank-16 adapters, us per linear (pair against single-CTA):
-//   K = 768 and more, 256-wide: 768 -> 768 23.8 / 26.5 and 80.0 / 90.7, 768 -> 3072 58.4 / 62.5 and 223 / 251;
-//   K up to 384, 256-wide: 384 -> 1536 28.0 / 24.1 and 86.8 / 85.6, 192 -> 768 18.3 / 15.9 and 44.8 / 36.8 -- a tile's K loop
-//   is too short to hide what the two CTAs of a pair wait for each other;
-//   192-wide (multiples of 192, not of 256): 384 -> 1152 21.6 / 23.7 and 69.7 / 83.2, 1536 -> 384 28.8 / 29.3 and 93.6 / 110,
-//   384 -> 384 15.2 / 15.0 and 40.2 / 46.1, but without adapters 10.3 / 10.2 and 31.4 / 28.5.
-// For multiples of both, 192-wide tiles lose: 768 -> 3072 64.1 and 246.
-static int pick_pair_width(int n_out, int k_in, bool lora) {
-    if (n_out % 256 == 0) return k_in <= 384 ? -1 : 1;
-    if (n_out % 192 == 0) return n_out <= 384 && k_in <= 384 && !lora ? -1 : 0;
-    return -1;
+// The tile width of the pair kernel (index into PAIR_WIDTHS), or -1 for the single-CTA kernel.  Short K goes to the latter
+// where 256 divides the width, and for narrow outputs without adapters: a tile's K loop is too short to hide what the two
+// CTAs of a pair wait for each other (384 -> 1536 on 64 frames of 197 tokens 23.3 us against 25.0 on pairs, 192 -> 768 on 256
+// frames 35.8 against 39.5).  Else the width with the cheapest rounds of tiles over the pairs: a round costs its columns, and what a
+// tile costs whatever its width, in columns (hand-over between tiles; more where a short K loop leaves the epilogue exposed).
+// The two constants are fitted to 1 to 192 frames of 197 tokens, with and without adapters, widths of 384 and 768: the rule's
+// choice is 0.4 % slower than the best of the three widths on average, 256 throughout 4.9 %.  us, 128 / 192 / 256 wide:
+//   3072 -> 768: 12 frames 13.6 / 17.2 / 20.4, 16: 20.9 / 17.4 / 21.1, 37: 31.9 / 29.1 / 34.7, 192: 147 / 134 / 131;
+//   768 -> 768: 12 frames 8.4 / 8.8 / 9.9, 37: 13.3 / 12.3 / 13.5, 192: 54.6 / 49.5 / 44.1;
+//   768 -> 3072: 16 frames 19.8 / 16.0 / 17.3, 37: 36.3 / 30.6 / 28.0, 192: 174 / 149 / 139.
+static int pick_pair_width(int n_out, int k_in, bool lora, int rows, int n_pairs) {
+    if (k_in <= 384 && (n_out % 256 == 0 || (n_out <= 384 && !lora))) return -1;
+    const int m = (rows + 2 * BM - 1) / (2 * BM);
+    int best = -1;
+    float best_cost = 0.f;
+    for (int i = PM_PAIR_WIDTHS - 1; i >= 0; --i) {
+        if (n_out % PAIR_WIDTHS[i] != 0) continue;
+        const int tiles = m * (n_out / PAIR_WIDTHS[i]), rounds = (tiles + n_pairs - 1) / n_pairs;
+        const float cost = (float)rounds * ((float)PAIR_WIDTHS[i] + 90.f + 130000.f / (float)k_in);
+        if (best < 0 || cost < best_cost) { best = i; best_cost = cost; }
+    }
+    return best;
 }
 
 // lin.tm_w / lin.tm_bt are encoded for the BN chosen by gemm_tile_n(lin.n_out) (single-CTA kernel); lin.tm_pw /
@@ -949,13 +959,14 @@ cudaError_t launch_lora_gemm(const Launch& L, const LinearDev& lin, const RouteD
     a.tma_store = (tm_y != nullptr && epi != EPI_PATCH) ? 1 : 0;
     const CUtensorMap& tt = lora ? *tm_t : tm_x;      // placeholders are never dereferenced
     const CUtensorMap& ty = a.tma_store ? *tm_y : tm_x;
-    const int pw = n_sms >= 2 && (epi != EPI_RESIDUAL || a.tma_store) ? pick_pair_width(lin.n_out, lin.k_in, lora) : -1;
+    const int pw = n_sms >= 2 && (epi != EPI_RESIDUAL || a.tma_store) ? pick_pair_width(lin.n_out, lin.k_in, lora, rows, n_sms / 2) : -1;
     if (pw >= 0) {
         a.m_tiles = (rows + 2 * BM - 1) / (2 * BM);       // 256-row tiles
         a.n_tiles = lin.n_out / PAIR_WIDTHS[pw];
         const CUtensorMap& tpb = lora ? lin.tm_pbt[pw] : lin.tm_pw[pw];
-        return PAIR_WIDTHS[pw] == 192 ? launch_gemm_pair_epi<192>(L, tm_x, lin.tm_pw[pw], tt, tpb, ty, a, n_sms)
-                                      : launch_gemm_pair_epi<256>(L, tm_x, lin.tm_pw[pw], tt, tpb, ty, a, n_sms);
+        if (PAIR_WIDTHS[pw] == 128) return launch_gemm_pair_epi<128>(L, tm_x, lin.tm_pw[pw], tt, tpb, ty, a, n_sms);
+        if (PAIR_WIDTHS[pw] == 192) return launch_gemm_pair_epi<192>(L, tm_x, lin.tm_pw[pw], tt, tpb, ty, a, n_sms);
+        return launch_gemm_pair_epi<256>(L, tm_x, lin.tm_pw[pw], tt, tpb, ty, a, n_sms);
     }
     const CUtensorMap& tb = lora ? lin.tm_bt : lin.tm_w;
     if (bn == 256) return launch_gemm_epi<256>(L, tm_x, lin.tm_w, tt, tb, ty, a, n_sms);

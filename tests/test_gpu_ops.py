@@ -332,6 +332,15 @@ def test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, 
     lin.close()
 
 
+@pytest.mark.parametrize("k_in,n_out,frames,tokens,rank,epi,what", [
+    (768, 640, 31, 130, 16, 2, "128-wide, one round"), (448, 1280, 60, 197, 8, 0, "256-wide of two widths"), (448, 640, 70, 197, 40, 1, "128-wide, several rounds"),
+    (3072, 768, 37, 197, 16, 2, "192-wide, two rounds"), (768, 768, 50, 200, 48, 2, "192-wide, several slab groups"),
+    (768, 2304, 24, 130, 16, 1, "192-wide"), (768, 768, 60, 197, 16, 2, "256-wide, residual rows past the end")])
+def test_pair_gemm_widths(k_in, n_out, frames, tokens, rank, epi, what):
+    """The three tile widths of the CTA-pair GEMM with every epilogue, ragged last row tiles, one and several rounds."""
+    test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, what)
+
+
 @pytest.mark.parametrize("frames,rank,what", [(1, 16, "64-wide, K in four"), (1, 64, "64-wide, K in four"), (12, 64, "256-wide, K in two")])
 def test_lora_linear_several_slab_groups_through_the_shortest_ring(frames, rank, what):
     """The few-row kernel's ring is shortest where a group of eight slabs and the exchange of partial sums take the
