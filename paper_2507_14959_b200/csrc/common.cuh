@@ -326,7 +326,7 @@ bool tm_encode_4d(CUtensorMap* tm, const void* base, const uint64_t* dims4, cons
 // kps blocks, each block 128B-swizzled by itself.  The thread that issues the copies spends about 170 clocks on
 // a pipeline stage's barriers and 44 on each copy whatever its size, so narrow stages take two blocks at once.
 bool tm_encode_kblocks(CUtensorMap* tm, const void* base, int k_in, uint64_t rows, int rows_box, int kps);
-// The same for one LoRA slab (16 arena rows): one copy (coordinates 0, 0, block, row / 8) brings its rows of kps
-// blocks as [2 groups of 8 rows][kps blocks][8 rows][128 bytes], so that slabs stack with a constant distance of
-// kps * 1024 bytes between 8-row groups.
-bool tm_encode_slab(CUtensorMap* tm, const void* base, int k_in, uint64_t rows, int kps);
+// The same in groups of 8 rows: one copy (coordinates 0, 0, block, row / 8) brings its rows of kps blocks as
+// [rows_box / 8 groups][kps blocks][8 rows][128 bytes].  LoRA slabs (16 arena rows) stack with a constant distance of
+// kps * 1024 bytes between 8-row groups, and behind a W tile in the same form they make one operand with it.
+bool tm_encode_groups(CUtensorMap* tm, const void* base, int k_in, uint64_t rows, int rows_box, int kps);

@@ -819,10 +819,10 @@ bool tm_encode_kblocks(CUtensorMap* tm, const void* base, int k_in, uint64_t row
     return tm_encode_3d(tm, base, 64, rows, (uint64_t)(k_in / 64), (uint64_t)k_in * 2, 128, 64, rows_box, kps, 128);
 }
 
-bool tm_encode_slab(CUtensorMap* tm, const void* base, int k_in, uint64_t rows, int kps) {
+bool tm_encode_groups(CUtensorMap* tm, const void* base, int k_in, uint64_t rows, int rows_box, int kps) {
     const uint64_t dims[4] = {64, 8, (uint64_t)(k_in / 64), rows / 8};
     const uint64_t strides[3] = {(uint64_t)k_in * 2, 128, (uint64_t)k_in * 16};
-    const uint32_t box[4] = {64, 8, (uint32_t)kps, 2};
+    const uint32_t box[4] = {64, 8, (uint32_t)kps, (uint32_t)rows_box / 8};
     return tm_encode_4d(tm, base, dims, strides, box, 128);
 }
 

@@ -4,8 +4,8 @@
 // What bounds it is neither bandwidth nor the tensor cores but the chain launch -> first bytes -> K loop -> t ->
 // expand -> epilogue, so every link is shortened:
 //   - the tile is the narrowest that fits the SMs in one wave: many CTAs, each with little to fetch;
-//   - the shrink MMAs ride on the K loop's own x stages (their accumulator sits beside the tile's in tensor
-//     memory) and the epilogue warps take the LayerNorm statistics from the same stages: one pass over x;
+//   - the shrink rides on the K loop's own MMAs (a stage's slab rows lie behind its W rows, the accumulators side by side in
+//     tensor memory: one operand of BN + 16 columns per slab) and the epilogue warps take the LayerNorm statistics from the same stages: one pass over x;
 //   - t stays in tensor memory: rounded in place of its accumulator columns, it is the expand MMAs' A operand there, and
 //     the shared memory is the ring's;
 //   - the copies are issued by two threads (x and W; adapter slabs), since issuing is a serial cost;
@@ -15,8 +15,9 @@
 //     expand included (the expand is linear in t); the partials are exchanged through distributed shared memory
 //     and every CTA sums and stores BN / S columns.  A partial t enters the expand as two bf16 parts (16 significant
 //     bits, two MMAs per slab): rounded to one, shares that cancel would leave their rounding in the sum.
-// One 197-token frame of width 768, rank-16 adapters, back to back, against shrink + pair GEMM: qkv 7.3 (13.4) us,
-// proj 7.3 (14.5), fc1 7.9 (14.6), fc2 10.1 (26.9); eight frames: 13.6 (15.6), 10.9 (16.0), 20.3 (20.9), 18.6 (31.1).
+// One 197-token frame of width 768, rank-16 adapters, replayed back to back: qkv 4.9 us, proj 4.9, fc1 5.6, fc2 8.0; four frames
+// 7.4, 5.6, 9.4 and 12.1; eight frames 12.3, 9.3, 14.4 and 16.8.  (Issued behind a lane test and with the shrink in MMAs of its own:
+// 7.0, 6.9, 7.3, 9.7; 9.7, 7.4, 11.2, 16.0; 13.1, 10.5, 17.4, 19.0.)
 // Warp roles: 0 = x / W copies, 1 = tensor memory + MMA, 2 = adapter copies, 3 = slab list, 4..11 = statistics, t, epilogue.
 #include "common.cuh"
 #include "f32x2.cuh"
@@ -245,7 +246,7 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
             const int pre = min(STG, num_st);
             for (int st = 0; st < pre; ++st) {
                 mbar_expect_tx(full_bar(st), X_BYTES + W_BYTES);
-                tma_load_3d(base + st * stage_bytes + X_BYTES, &tm_w, 0, n * BN, kb0 + st * KPS, full_bar(st));
+                tma_load_4d(base + st * stage_bytes + X_BYTES, &tm_w, 0, 0, kb0 + st * KPS, n * (BN / 8), full_bar(st));
                 if (na == 0) mbar_arrive(full_bar(st));                  // nobody brings slabs
             }
             dep_wait();
@@ -260,7 +261,7 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                         if (g == 0) {
                             mbar_expect_tx(full_bar(stage), X_BYTES + W_BYTES);
                             tma_load_3d(sa, &tm_x, 0, m * BM, kb0 + st * KPS, full_bar(stage));
-                            tma_load_3d(sa + X_BYTES, &tm_w, 0, n * BN, kb0 + st * KPS, full_bar(stage));
+                            tma_load_4d(sa + X_BYTES, &tm_w, 0, 0, kb0 + st * KPS, n * (BN / 8), full_bar(stage));
                             if (na == 0) mbar_arrive(full_bar(stage));
                         } else {                                          // further slabs: another pass over x
                             if (LNF) mbar_arrive_n(empty_bar(stage), EW);
@@ -311,7 +312,7 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
         if (elect_one()) {
             // -------------------------------------------------------------- MMA issuer
             const uint32_t idesc = instr_desc(BN);
-            const uint64_t da0 = smem_desc(base, 128), db0 = smem_desc(base + X_BYTES, 128);
+            const uint64_t da0 = smem_desc(base, 128), db0 = smem_desc_groups(base + X_BYTES, KPS * 1024);
             const uint64_t ds0 = smem_desc_groups(base + X_BYTES + W_BYTES, KPS * 1024);
             int stage = 0;
             uint32_t phase = 0;
@@ -319,6 +320,11 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
             for (int g = 0; g < n_groups && ok; ++g) {
                 const int cnt = min(GROUP, na - g * GROUP);
                 const uint32_t idesc_t = instr_desc(max(cnt, 1) * PM_SLAB);
+                // W tile and slabs are adjacent in a stage and their accumulators in tensor memory: one MMA makes both where
+                // N allows it.  An MMA of 128 rows takes at least 49 cycles however narrow: 64 and 48 columns apart 845
+                // cycles per stage, 112 together 555; 768 -> 2304 on one frame 6.1 -> 4.9 us.
+                const bool joint = BN + max(cnt, 0) * PM_SLAB <= 256;
+                const uint32_t idesc_j = instr_desc(joint ? BN + max(cnt, 0) * PM_SLAB : BN);
                 for (int kb = 0; kb < num_kb; kb += KPS) {
                     ok = mbar_wait(full_bar(stage), phase, abort_flag, args.status);
                     if (!ok) break;
@@ -327,13 +333,13 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
 #pragma unroll
                     for (int j = 0; j < KPS; ++j) {
                         if (j > 0 && kb + j >= num_kb) break;
-                        const uint64_t da = da0 + so + (j * A_BLOCK >> 4), db = db0 + so + (j * B_BLOCK >> 4);
+                        const uint64_t da = da0 + so + (j * A_BLOCK >> 4), db = db0 + so + (j * 1024 >> 4);
                         const uint64_t ds = ds0 + so + (j * 1024 >> 4);
                         if (g == 0) {
 #pragma unroll
-                            for (int k = 0; k < BK / 16; ++k) umma_bf16(tmem_base, da + 2 * k, db + 2 * k, idesc, (kb | j | k) != 0);
+                            for (int k = 0; k < BK / 16; ++k) umma_bf16(tmem_base, da + 2 * k, db + 2 * k, idesc_j, (kb | j | k) != 0);
                         }
-                        if (cnt > 0) {
+                        if (cnt > 0 && (g > 0 || !joint)) {
 #pragma unroll
                             for (int k = 0; k < BK / 16; ++k) umma_bf16(t_tmem, da + 2 * k, ds + 2 * k, idesc_t, (kb | j | k) != 0);
                         }
@@ -630,12 +636,12 @@ Shape pick_shape(const LinearDev& lin, bool lora, int rows, int epi, int n_sms) 
 bool small_linear_encode(LinearDev& lin, int max_adapters, int slabs_max) {
     const uint64_t arena_rows = (uint64_t)max_adapters * slabs_max * PM_SLAB;
     for (int i = 0; i < PM_SMALL_WIDTHS; ++i) {
-        if (!tm_encode_kblocks(&lin.tm_sw[i], lin.Wt, lin.k_in, lin.n_out, WIDTHS[i], kps_of(WIDTHS[i]))) return false;
+        if (!tm_encode_groups(&lin.tm_sw[i], lin.Wt, lin.k_in, lin.n_out, WIDTHS[i], kps_of(WIDTHS[i]))) return false;
         if (lin.lora.At && !tm_encode_2d(&lin.tm_sbt[i], lin.lora.Bt, PM_SLAB, arena_rows / PM_SLAB * lin.n_out, PM_SLAB * 2, PM_SLAB, WIDTHS[i], 32))
             return false;
     }
     for (int k = 0; k < 2; ++k)
-        if (lin.lora.At && !tm_encode_slab(&lin.tm_sat[k], lin.lora.At, lin.k_in, arena_rows, k + 1)) return false;
+        if (lin.lora.At && !tm_encode_groups(&lin.tm_sat[k], lin.lora.At, lin.k_in, arena_rows, PM_SLAB, k + 1)) return false;
     return true;
 }
 
