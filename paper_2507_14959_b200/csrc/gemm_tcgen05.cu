@@ -26,7 +26,6 @@ namespace {
 
 constexpr int BM = PM_TILE_M;
 constexpr int BK = 64;
-constexpr int STAGES = 4;
 constexpr int SLABS_PER_STAGE = 4;
 
 struct GemmArgs {
@@ -47,20 +46,27 @@ struct GemmArgs {
     const float2* ln_stats;
 };
 
-constexpr int STAGING_BYTES_PER_WARP = 2 * 32 * 64;     // two [32 rows x 32 bf16] buffers
+constexpr int STAGING_BYTES = 32 * 64;                  // one chunk: [32 rows x 32 bf16]
+constexpr int STAGING_BYTES_PER_WARP = 2 * STAGING_BYTES;
 constexpr int PLAN_BYTES = 2048;
 constexpr int P_ACC_COLS = 256;                        // pair kernel: tensor-memory columns of one of the two accumulators
 
-// EW = number of epilogue warps (4 or 8); the CTA has 2 + EW warps.
-template <int BN, int EW>
+// The single-CTA kernel: an epilogue warp per 64 columns of a lane quarter, as in the pair kernel below.  The short K loops that
+// run here are no longer than an epilogue: with eight warps 192 -> 768 took 12.2, 16.0 and 27.8 us on 64, 128 and 256 frames
+// of 197 tokens, with sixteen 9.9, 13.1 and 23.7.
+// 256-wide tiles leave room for four stages and one staging buffer per warp.
+template <int BN>
 struct Smem {
+    static constexpr int EW = BN / 16;
+    static constexpr int BUFFERS = BN == 256 ? 1 : 2;
+    static constexpr int STAGES = 4;
     static constexpr int A_BYTES = BM * BK * 2;
     static constexpr int B_BYTES = BN * BK * 2;
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
     static constexpr int T_SLAB_BYTES = BM * PM_SLAB * 2;      // 4096
     static constexpr int B_SLAB_BYTES = BN * PM_SLAB * 2;
     static constexpr int STAGING_OFFSET = STAGES * STAGE_BYTES;
-    static constexpr int PLAN_OFFSET = STAGING_OFFSET + EW * STAGING_BYTES_PER_WARP;
+    static constexpr int PLAN_OFFSET = STAGING_OFFSET + EW * BUFFERS * STAGING_BYTES;
     static constexpr int BAR_OFFSET = PLAN_OFFSET + PLAN_BYTES;
     static constexpr int TOTAL = BAR_OFFSET + 256;             // + barriers (base must be 1024-aligned)
 };
@@ -71,7 +77,7 @@ struct Smem {
 // PAIR: the accumulator-free barrier lives in the even CTA of a pair (tempty_addr is a cluster address).
 // RES_SMEM: request_residual has asked TMA for the residual rows of this warp's two chunks, into the staging buffers that the
 // results will leave from (completion on res_bar); else per-thread global loads.
-template <int BN, int EPI, int HALVES, bool PAIR, bool LNF, bool RES_SMEM>
+template <int BN, int EPI, int HALVES, int BUFFERS, bool PAIR, bool LNF, bool RES_SMEM>
 __device__ __forceinline__ bool epilogue_tile(const GemmArgs& args, const CUtensorMap& tm_y, uint32_t staging,
                                               uint32_t& chunk_no, uint32_t tmem_base, int acc, uint32_t acc_phase,
                                               uint32_t tfull_addr, uint32_t tempty_addr, volatile int* abort_flag,
@@ -164,7 +170,7 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs& args, const CUtens
                 uint4 r4v;
                 if constexpr (RES_SMEM) {
                     // where this thread puts its result below: 16-byte chunk q of row `lane`
-                    const uint32_t a = staging + (chunk_no & 1u) * (32 * 64) + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4);
+                    const uint32_t a = staging + chunk_no % BUFFERS * STAGING_BYTES + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4);
                     asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
                                  : "=r"(r4v.x), "=r"(r4v.y), "=r"(r4v.z), "=r"(r4v.w) : "r"(a));
                 } else {
@@ -197,9 +203,9 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs& args, const CUtens
         if (args.tma_store) {
             // [32 rows x 64 B] block, 16-byte chunks XOR-swizzled by (row >> 1) & 3 (64B
             // swizzle), then one TMA store; rows past the end are clipped by the tensor map
-            const uint32_t buf = staging + (chunk_no & 1u) * (32 * 64);
+            const uint32_t buf = staging + chunk_no % BUFFERS * STAGING_BYTES;
             if constexpr (!RES_SMEM) {
-                if (elect_one()) bulk_wait_read1();  // the store that last used this buffer has read it
+                if (elect_one()) { if constexpr (BUFFERS == 2) bulk_wait_read1(); else bulk_wait_read0(); }      // the store that last used this buffer has read it
                 __syncwarp();
             }
 #pragma unroll
@@ -234,12 +240,13 @@ __device__ __forceinline__ void request_residual(const CUtensorMap& tm_res, uint
     __syncwarp();
 }
 
-template <int BN, int EPI, int EW, bool LNF>
-__global__ void __launch_bounds__(64 + 32 * EW, 1)
+template <int BN, int EPI, bool LNF>
+__global__ void __launch_bounds__(64 + 32 * Smem<BN>::EW, 1)
 lora_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                  const __grid_constant__ CUtensorMap tm_t, const __grid_constant__ CUtensorMap tm_bt,
                  const __grid_constant__ CUtensorMap tm_y, const GemmArgs args) {
-    using S = Smem<BN, EW>;
+    using S = Smem<BN>;
+    constexpr int EW = S::EW, STAGES = S::STAGES;
     constexpr int NTHREADS = 64 + 32 * EW;
     constexpr int HALVES = EW / 4;                // epilogue warps per TMEM lane quarter
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -398,7 +405,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
         // ------------------------------------------------------------------ epilogue (warps 2..)
         const int quarter = warp & 3;                 // TMEM lanes 32*quarter .. +31
         const int half = (warp - 2) >> 2;             // which share of the tile's 32-column chunks
-        const uint32_t staging = base + S::STAGING_OFFSET + (uint32_t)(warp - 2) * STAGING_BYTES_PER_WARP;
+        const uint32_t staging = base + S::STAGING_OFFSET + (uint32_t)(warp - 2) * (S::BUFFERS * STAGING_BYTES);
         dep_wait();                                   // row statistics, residual; rows that the kernel before still reads
         int acc = 0;
         uint32_t acc_phase = 0;
@@ -406,7 +413,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
         bool ok = true;
         for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
             const int m = tile / args.n_tiles, n = tile % args.n_tiles;
-            ok = epilogue_tile<BN, EPI, HALVES, false, LNF, false>(args, tm_y, staging, chunk_no, tmem_base, acc,
+            ok = epilogue_tile<BN, EPI, HALVES, S::BUFFERS, false, LNF, false>(args, tm_y, staging, chunk_no, tmem_base, acc,
                                                               acc_phase, tfull_bar(acc), tempty_bar(acc), abort_flag,
                                                               m, n, quarter, half, lane, 0u, 0u);
             if (!ok) break;
@@ -666,7 +673,7 @@ lora_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         for (int tile = pair_id; tile < total_tiles && ok; tile += n_pairs) {
             const int m = 2 * (tile / args.n_tiles) + (int)rank, n = tile % args.n_tiles;
             if constexpr (RES) request_residual<BN>(tm_res, staging, res_bar(warp - 2), m, n, quarter, half);
-            ok = epilogue_tile<BN, EPI, C::HALVES, true, LNF, RES>(
+            ok = epilogue_tile<BN, EPI, C::HALVES, 2, true, LNF, RES>(
                 args, tm_y, staging, chunk_no, tmem_base, acc, acc_phase, tfull_bar(acc),
                 mapa_cluster(tempty_bar(acc), 0), abort_flag, m, n, quarter, half, lane,
                 res_bar(warp - 2), res_phase);
@@ -826,18 +833,15 @@ bool tm_encode_groups(CUtensorMap* tm, const void* base, int k_in, uint64_t rows
     return tm_encode_4d(tm, base, dims, strides, box, 128);
 }
 
-constexpr int GEMM_EPI_WARPS = 8;
-
 template <int BN, int EPI, bool LNF = false>
 static cudaError_t launch_gemm_bn(const Launch& L, const CUtensorMap& tm_x, const CUtensorMap& tm_w,
                                   const CUtensorMap& tm_t, const CUtensorMap& tm_bt, const CUtensorMap& tm_y,
                                   const GemmArgs& a, int n_sms) {
-    constexpr int EW = GEMM_EPI_WARPS;
     static SmemGrant grant;
-    if (cudaError_t e = grant.ensure(lora_gemm_kernel<BN, EPI, EW, LNF>, Smem<BN, EW>::TOTAL); e != cudaSuccess) return e;
+    if (cudaError_t e = grant.ensure(lora_gemm_kernel<BN, EPI, LNF>, Smem<BN>::TOTAL); e != cudaSuccess) return e;
     const int total = a.m_tiles * a.n_tiles;
     ProfScope ps(L, KC_GEMM);
-    cudaError_t e = launch_overlapped(L, lora_gemm_kernel<BN, EPI, EW, LNF>, total < n_sms ? total : n_sms, 64 + 32 * EW, Smem<BN, EW>::TOTAL, 1, tm_x, tm_w, tm_t, tm_bt, tm_y, a);
+    cudaError_t e = launch_overlapped(L, lora_gemm_kernel<BN, EPI, LNF>, total < n_sms ? total : n_sms, 64 + 32 * Smem<BN>::EW, Smem<BN>::TOTAL, 1, tm_x, tm_w, tm_t, tm_bt, tm_y, a);
     BUMP(L);
     return e;
 }
