@@ -323,8 +323,8 @@ bool tm_encode_3d(CUtensorMap* tm, const void* base, uint64_t d0, uint64_t d1, u
 bool tm_encode_4d(CUtensorMap* tm, const void* base, const uint64_t* dims4, const uint64_t* strides3, const uint32_t* box4,
                   int swizzle);
 // K-major [rows, k_in] operand in blocks of 64 columns: one copy (coordinates 0, row, block) brings rows_box rows of
-// kps blocks, each block 128B-swizzled by itself.  The thread that issues the copies spends about 170 clocks on
-// a pipeline stage's barriers and 44 on each copy whatever its size, so narrow stages take two blocks at once.
+// kps blocks, each block 128B-swizzled by itself.  A pipeline stage costs the threads that issue its copies and
+// MMAs the same whatever its size, so narrow stages take two blocks at once.
 bool tm_encode_kblocks(CUtensorMap* tm, const void* base, int k_in, uint64_t rows, int rows_box, int kps);
 // The same in groups of 8 rows: one copy (coordinates 0, 0, block, row / 8) brings its rows of kps blocks as
 // [rows_box / 8 groups][kps blocks][8 rows][128 bytes].  LoRA slabs (16 arena rows) stack with a constant distance of

@@ -9,8 +9,8 @@
 // GEMM and fetched by TMA like any other operand.  Operands are staged by TMA into 128B- (base)
 // and 32B- (LoRA slab) swizzled shared memory; a single thread issues tcgen05.mma; accumulators
 // live in TMEM (two buffers, so the epilogue of one tile overlaps the main loop of the next).
-// Warp roles: warp 0 = TMA producer, warp 1 = TMEM owner + MMA issuer, warps 2..9 = epilogue (two
-// warps per TMEM lane quarter, each taking half of the tile's columns).
+// Warp roles: warp 0 = TMA producer, warp 1 = TMEM owner + MMA issuer, warps 2.. = epilogue (a warp per
+// 64 columns of a TMEM lane quarter).
 // Every mbarrier wait is bounded: on expiry the CTA raises an abort flag, records
 // PM_ERR_TIMEOUT in the status word, drains and returns.
 // The CTA-pair variant (lora_gemm_pair_kernel, cta_group::2, 256-row tiles of 128, 192 or 256 columns) serves most shapes, the single-CTA
