@@ -121,7 +121,7 @@ shrink_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ 
         mbar_init(tfull_bar, 1);
         mbar_init(tempty_bar, EW);
         mbar_init(stats_bar, EW + 1);
-        mbar_init(recv_bar, S > 1 ? (S - 1) * EW : 1);
+        mbar_init(recv_bar, 1);
         tail.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -162,6 +162,8 @@ shrink_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ 
     const uint32_t tmem_base = tail.tmem_slot;
     const int na = tail.n_active;
     const int per_group = min(na, GROUP);
+    // the first group's slabs i = ks mod S arrive from every other CTA
+    if (S > 1 && threadIdx.x == 0 && na > 0) mbar_expect_tx(recv_bar, (uint32_t)((S - 1) * ((per_group - ks + S - 1) / S) * T_F32));
     const int stage_bytes = X_BYTES + per_group * A_SLAB;
     const int STG = min(MAX_STAGES, args.ring_bytes / stage_bytes);
     // groups of slabs; for the statistics a tile without slabs still makes one pass over x
@@ -408,14 +410,10 @@ shrink_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ 
                     tmem_ld_wait();
                     const int src = ks < j ? ks : ks - 1;
                     const uint32_t dst = mapa_cluster(recv_s, (uint32_t)j) + (uint32_t)((src * PER + i / S) * T_F32 + r * 16);
+                    const uint32_t bar = mapa_cluster(recv_bar, (uint32_t)j);
 #pragma unroll
-                    for (int e = 0; e < 16; e += 4)
-                        asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};"
-                                     ::"r"(dst + (uint32_t)(e / 4 * BM * 16)), "r"(v[e]), "r"(v[e + 1]), "r"(v[e + 2]), "r"(v[e + 3]) : "memory");
+                    for (int e = 0; e < 16; e += 4) st_async_v4(dst + (uint32_t)(e / 4 * BM * 16), v + e, bar);
                 }
-                __syncwarp();
-                if (lane == 0)
-                    for (int jj = 1; jj < S; ++jj) mbar_arrive_cluster(mapa_cluster(recv_bar, (uint32_t)((ks + jj) % S)));
                 ok = mbar_wait_cluster(recv_bar, 0, abort_flag, args.status);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;

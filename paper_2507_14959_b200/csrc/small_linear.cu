@@ -185,10 +185,11 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     if (threadIdx.x == 0) {
         for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(full_bar(s), 2); mbar_init(empty_bar(s), EMPTY_COUNT); }
         mbar_init(tacc_bar, 1); mbar_init(tready_bar, EW); mbar_init(tfull_bar, 1); mbar_init(stats_bar, EW + 1);
-        mbar_init(recv_bar, S > 1 ? (S - 1) * EW : 1);
+        mbar_init(recv_bar, 1);
         tail.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        if (S > 1) mbar_expect_tx(recv_bar, (uint32_t)recv_bytes<BN, S>());
     }
     if (warp == 1) {
         tmem_alloc(smem_u32(&tail.tmem_slot), TMEM_COLS);
@@ -508,21 +509,19 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                 // recv[src][16-byte column group][row]: src = the sender's place among the other CTAs
                 constexpr int CW = HC % 32 == 0 ? 32 : HC % 16 == 0 ? 16 : 8;      // columns at a time
 #pragma unroll
-                for (int jj = 1; jj < S; ++jj) {
-                    const int j = (ks + jj) % S, src = ks < j ? ks : ks - 1;
-                    const uint32_t dst = mapa_cluster(recv_s, (uint32_t)j) + (uint32_t)(((src * (CS / 4) + half * (HC / 4)) * BM + r) * 16);
+                for (int c = 0; c < HC; c += CW) {
+                    uint32_t v[S - 1][CW];
 #pragma unroll
-                    for (int c = 0; c < HC; c += CW) {
-                        uint32_t v[CW];
-                        tmem_ld<CW>(t_row + (uint32_t)(j * CS + half * HC + c), v);
-                        tmem_ld_wait();
+                    for (int jj = 1; jj < S; ++jj) tmem_ld<CW>(t_row + (uint32_t)((ks + jj) % S * CS + half * HC + c), v[jj - 1]);
+                    tmem_ld_wait();
 #pragma unroll
-                        for (int e = 0; e < CW; e += 4)
-                            asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};"
-                                         ::"r"(dst + (uint32_t)((c + e) / 4 * BM * 16)), "r"(v[e]), "r"(v[e + 1]), "r"(v[e + 2]), "r"(v[e + 3]) : "memory");
+                    for (int jj = 1; jj < S; ++jj) {
+                        const int j = (ks + jj) % S, src = ks < j ? ks : ks - 1;
+                        const uint32_t dst = mapa_cluster(recv_s, (uint32_t)j) + (uint32_t)(((src * (CS / 4) + (half * HC + c) / 4) * BM + r) * 16);
+                        const uint32_t bar = mapa_cluster(recv_bar, (uint32_t)j);
+#pragma unroll
+                        for (int e = 0; e < CW; e += 4) st_async_v4(dst + (uint32_t)(e / 4 * BM * 16), v[jj - 1] + e, bar);
                     }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive_cluster(mapa_cluster(recv_bar, (uint32_t)j));
                 }
                 ok = mbar_wait_cluster(recv_bar, 0, abort_flag, args.status);
                 ok = __all_sync(0xFFFFFFFFu, ok);

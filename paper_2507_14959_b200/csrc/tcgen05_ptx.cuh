@@ -231,6 +231,12 @@ __device__ __forceinline__ void cluster_sync_all() {     // every thread of both
 __device__ __forceinline__ void st_cluster_u32(uint32_t cluster_addr, uint32_t v) {
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
 }
+// 16 bytes into a CTA of the cluster, counted on the mbarrier there (its waiter sees them): no release, which would make the
+// sender wait for its earlier stores before every arrival
+__device__ __forceinline__ void st_async_v4(uint32_t cluster_addr, const uint32_t* v, uint32_t bar_cluster_addr) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(cluster_addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(bar_cluster_addr) : "memory");
+}
 // arrive on an mbarrier that may live in the peer CTA (cluster_addr from mapa_cluster)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
