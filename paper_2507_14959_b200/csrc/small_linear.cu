@@ -600,7 +600,7 @@ cudaError_t launch_epi(const Launch& L, const Maps& t, const SmallArgs& a, int e
         case EPI_GELU: return launch<BN, EPI_GELU>(L, t, a, tiles);
         case EPI_RESIDUAL:
             if constexpr (BN <= 128) if (split == 4) return launch<BN, EPI_RESIDUAL, false, 4>(L, t, a, tiles);
-            if constexpr (BN <= 192) if (split == 2) return launch<BN, EPI_RESIDUAL, false, 2>(L, t, a, tiles);
+            if (split == 2) return launch<BN, EPI_RESIDUAL, false, 2>(L, t, a, tiles);
             return launch<BN, EPI_RESIDUAL>(L, t, a, tiles);
         case EPI_PATCH: return launch<BN, EPI_PATCH>(L, t, a, tiles);
         default: return launch<BN, EPI_NONE>(L, t, a, tiles);
@@ -618,7 +618,8 @@ struct Shape { int width = -1, split = 1; };          // width: index into WIDTH
 //   768 -> 768 64-wide 6 frames 5.1 / 6.2, 128-wide 8: 7.5 / 6.7, 16: 10.1 / 8.8;  384 -> 384 64-wide 14: 4.3 / 5.1, 128-wide 16: 6.5 / 4.8;
 //   192 -> 192 192-wide 32: 7.5 / 4.4;  3072 -> 768 in two, 128-wide 6: 10.5 / 11.8, 192-wide 8: 13.2 / 12.7, 256-wide 12: 16.9 / 13.2;
 //   1536 -> 384 in two, 128-wide 10: 7.7 / 7.9, 192-wide 16: 9.8 / 8.8.
-// With adapters the alternative is two kernels: only K in two at 256 columns loses, 12 frames 22.3 / 19.5, 14: 22.4 / 20.6.
+// With adapters the alternative is two kernels, whose t is rounded to bf16 once where the shares' t here keep 16 bits: K in two at 256
+// columns stays here although it is slower (3072 -> 768, 12 frames 22.5 / 19.5, 14: 22.5 / 20.6; 2048 -> 512, 24 frames 18.3 / 21.0).
 Shape pick_shape(const LinearDev& lin, bool lora, int rows, int epi, int n_sms) {
     const long long m = (rows + BM - 1) / BM;
     const bool alone = epi == EPI_RESIDUAL && !lora;
@@ -627,7 +628,7 @@ Shape pick_shape(const LinearDev& lin, bool lora, int rows, int epi, int n_sms) 
             if (split == 4 && WIDTHS[i] > 128) break;
             if (split == 1 && WIDTHS[i] > (alone ? 64 : 192) && !lora) break;
             if (lin.n_out % WIDTHS[i] == 0 && m * (lin.n_out / WIDTHS[i]) * split <= n_sms) {
-                if (split == 2 && WIDTHS[i] > (lora ? 192 : 128)) return Shape();
+                if (split == 2 && WIDTHS[i] > 128 && !lora) return Shape();
                 Shape s;
                 s.width = i; s.split = split;
                 return s;

@@ -444,6 +444,33 @@ def test_lora_intermediate_of_a_split_k_is_not_rounded_share_by_share(frames, wh
     lin.close()
 
 
+@pytest.mark.parametrize("k_in,n_out,frames", [(3072, 768, 1), (3072, 768, 4), (3072, 768, 8), (3072, 768, 12), (3072, 768, 15),
+                                               (2048, 512, 24), (4096, 1024, 8)])
+def test_lora_intermediate_of_a_split_k_is_held_in_more_than_16_bits(k_in, n_out, frames):
+    """W = 0 and no cancellation: the output is t B.  The shares of t carry 16 significant bits, so the error is that of the one
+    rounding of the output to bf16.  Rounding to 8 significant bits errs by at most 2^-8 / m relative to a value of mantissa m in [1, 2),
+    uniformly; over mantissas of equal probability per logarithm E[1/m^2] = 3 / (8 ln 2), and the root mean square is 2^-8 * sqrt(E / 3) =
+    2^-8 * 0.425.  A t rounded to bf16 would add as much again in the sum over its 16 ranks, 2^-8 * 0.60 in all.  The limit lies between."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    tokens, rank, rows = 197, 16, frames * 197
+    gen = torch.Generator(device="cuda").manual_seed(frames)
+    x = torch.randn((rows, k_in), generator=gen, device="cuda").bfloat16()
+    A = (torch.randn((k_in, rank), generator=gen, device="cuda") * 0.02).bfloat16()
+    B = (torch.randn((rank, n_out), generator=gen, device="cuda") * 0.02).bfloat16()
+    lin = binding.Linear(np.zeros((k_in, n_out), np.float32), np.zeros(n_out, np.float32), max_adapters=1, max_rank=rank, max_set=1,
+                         max_frames=frames, tokens=tokens, epilogue=2)
+    lin.register(0, rank, 1.0, A.float().cpu().numpy(), B.float().cpu().numpy())
+    y = torch.full((rows, n_out), float("nan"), device="cuda", dtype=torch.bfloat16)
+    off, ids = wl.sets_to_csr([[0]] * frames)
+    lin.forward(x, frames, off, ids, y, residual=torch.zeros_like(y))
+    assert lin.status() == 0
+    want = (x.double() @ A.double()) @ B.double()
+    error = float((y.double() - want).norm() / want.norm())
+    assert error < 0.5 * 2.0 ** -8, error * 2.0 ** 8
+    lin.close()
+
+
 @pytest.mark.parametrize("frames,tokens,heads", [(1, 1, 1), (2, 16, 3), (1, 17, 2), (3, 49, 1), (1, 208, 12), (49, 33, 1),     # a few pairs
                                                  (50, 33, 1), (60, 1, 1), (20, 197, 3), (17, 208, 4), (13, 129, 12)])           # the pipelined kernel
 def test_attention_of_one_key_block_on_both_sides_of_the_pair_limit(frames, tokens, heads):
