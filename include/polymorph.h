@@ -250,6 +250,16 @@ const char* pm_last_error(pm_handle h);
  *   status  dev int32, trace dev int32 [3] (cleared by the call). */
 int pm_selftest_wait_timeout(long long limit_cycles, int32_t* status, int32_t* trace, void* cuda_stream);
 
+/* Which kernel a bf16 linear of these sizes takes on a GPU of n_sms multiprocessors (no counterpart in the paper: library
+ * diagnostics; nothing is launched and no GPU is needed).  epilogue: 0 to 2 as in pm_linear_create, 3 = patch placement (the
+ * forward's patch projection); adapters != 0: some row uses one (and no row tile lists more than 64 slabs of 16 ranks).
+ *   form[0]  0 = the few-row kernel, one launch; else with adapters a shrink first: 1 = GEMM on CTA pairs, 2 = GEMM of single CTAs
+ *   form[1]  columns of an output tile
+ *   form[2]  CTAs that share K
+ *   form[3]  threads per CTA
+ * Errors: PM_ERR_ARG (k_in and n_out multiples of 64 as in pm_linear_create, rows > 0, form not NULL). */
+int pm_linear_kernel(int k_in, int n_out, int rows, int epilogue, int adapters, int n_sms, int32_t* form);
+
 /* The forward entry points record their launch sequence as a CUDA graph the second time they are
  * called with the same buffers, sizes and stream and the same widest adapter set, and replay it
  * from then on; the adapter sets themselves may change between replays (a new routing plan is

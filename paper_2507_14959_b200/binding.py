@@ -23,7 +23,7 @@ EXPORTS = [
     "pm_create", "pm_register_adapter", "pm_set_cover", "pm_destroy", "pm_forward", "pm_forward_branched", "pm_forward_device_sets", "pm_select",
     "pm_select_static", "pm_metrics_reset", "pm_metrics_read", "pm_status", "pm_last_error", "pm_launch_count", "pm_set_graphs", "pm_set_small_batch_kernel", "pm_profile_enable", "pm_profile_read", "pm_plan_stats", "pm_linear_create", "pm_linear_register",
     "pm_linear_forward", "pm_linear_status", "pm_linear_last_error", "pm_linear_destroy",
-    "pm_layernorm", "pm_attention", "pm_selftest_wait_timeout", "pm_cooccurrence", "pm_build_contexts", "pm_intra_coherence",
+    "pm_layernorm", "pm_attention", "pm_selftest_wait_timeout", "pm_linear_kernel", "pm_cooccurrence", "pm_build_contexts", "pm_intra_coherence",
 ]
 
 
@@ -105,6 +105,7 @@ def load():
     lib.pm_layernorm.argtypes = [vp, vp, vp, vp, ip, ip, C.c_float, ip, vp]
     lib.pm_attention.argtypes = [vp, vp, ip, ip, ip, ip, vp]
     lib.pm_selftest_wait_timeout.argtypes = [C.c_longlong, vp, vp, vp]
+    lib.pm_linear_kernel.argtypes = [ip, ip, ip, ip, ip, ip, C.POINTER(C.c_int32)]
     _lib = lib
     return lib
 
@@ -351,6 +352,15 @@ def selftest_wait_timeout(limit_cycles, status, trace, stream=None):
     rc = load().pm_selftest_wait_timeout(int(limit_cycles), _ptr(status), _ptr(trace), _stream_ptr(stream))
     if rc != PM_OK:
         raise PolymorphError(rc, "pm_selftest_wait_timeout")
+
+
+def linear_kernel(k_in, n_out, rows, epilogue, adapters, n_sms=148):
+    """pm_linear_kernel: (kernel, columns of a tile, CTAs that share K, threads per CTA); kernel is "few rows", "pair" or "single"."""
+    form = (C.c_int32 * 4)()
+    rc = load().pm_linear_kernel(int(k_in), int(n_out), int(rows), int(epilogue), int(bool(adapters)), int(n_sms), form)
+    if rc != PM_OK:
+        raise PolymorphError(rc, "pm_linear_kernel")
+    return ("few rows", "pair", "single")[form[0]], form[1], form[2], form[3]
 
 
 def select_static(scores, n_adapters, score_thr, context_copy, has_prev, prev_labels, prev_offsets, prev_ids,

@@ -1338,6 +1338,14 @@ void pm_linear_destroy(pm_linear l) {
     delete l;
 }
 
+int pm_linear_kernel(int k_in, int n_out, int rows, int epilogue, int adapters, int n_sms, int32_t* form) {
+    if (!form || k_in <= 0 || n_out <= 0 || k_in % 64 || n_out % 64 || rows <= 0 || epilogue < 0 || epilogue > 3 || n_sms < 1) return PM_ERR_ARG;
+    LinearForm f;
+    if (!small_linear_form(k_in, n_out, adapters != 0, rows, epilogue, n_sms, &f)) f = gemm_form(k_in, n_out, adapters != 0, rows, epilogue, n_sms);
+    form[0] = f.kernel; form[1] = f.width; form[2] = f.split; form[3] = f.threads;
+    return PM_OK;
+}
+
 int pm_layernorm(const void* x, const float* gamma, const float* beta, void* y, int rows, int d,
                  float eps, int dtype, void* cuda_stream) {
     if (!x || !gamma || !beta || !y || rows < 0 || d <= 0 || d % 8 || d > 1024 || (dtype != 0 && dtype != 1))

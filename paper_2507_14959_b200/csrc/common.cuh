@@ -178,6 +178,12 @@ cudaError_t launch_lora_gemm(const Launch& L, const LinearDev& lin, const RouteD
 // ---- one kernel per linear for few rows (small_linear.cu)
 bool gemm_encode_pair_maps(LinearDev& lin, int max_adapters, int slabs_max);      // gemm_tcgen05.cu
 bool small_linear_encode(LinearDev& lin, int max_adapters, int slabs_max);
+// Which kernel a linear takes, as small_linear_form and gemm_form answer and the launches follow: its tile's columns, the CTAs that share K
+// and the threads of a CTA.  lora: an adapter is in use.
+enum { LINEAR_FEW_ROWS = 0, LINEAR_PAIR = 1, LINEAR_SINGLE = 2 };
+struct LinearForm { int kernel, width, split, threads; };
+bool small_linear_form(int k_in, int n_out, bool lora, int rows, int epi, int n_sms, LinearForm* form);      // false: not for this kernel
+LinearForm gemm_form(int k_in, int n_out, bool lora, int rows, int epi, int n_sms);
 // whether launch_small_linear serves this call (R: null = no adapters)
 bool small_linear_fits(const LinearDev& lin, const RouteDev* R, int rows, int epi, int n_sms);
 // The whole linear -- shrink, LayerNorm statistics where the LayerNorm is folded in, GEMM, expand, epilogue -- in one launch.

@@ -941,6 +941,15 @@ static int pick_pair_width(int n_out, int k_in, bool lora, int rows, int n_pairs
 // lin.tm_pbt fetch half of a tile's columns for the pair kernel.
 int gemm_tile_n(int n_out) { return (n_out % 256 == 0) ? 256 : 128; }
 
+LinearForm gemm_form(int k_in, int n_out, bool lora, int rows, int epi, int n_sms) {
+    const int pw = n_sms >= 2 ? pick_pair_width(n_out, k_in, lora, rows, n_sms / 2) : -1;
+    if (pw >= 0)
+        return {LINEAR_PAIR, PAIR_WIDTHS[pw], 1, PAIR_WIDTHS[pw] == 128 ? PairCfg<128>::THREADS : PAIR_WIDTHS[pw] == 192 ? PairCfg<192>::THREADS
+                                                                                                  : PairCfg<256>::THREADS};
+    const int bn = gemm_tile_n(n_out);
+    return {LINEAR_SINGLE, bn, 1, 64 + 32 * (bn == 256 ? Smem<256>::EW : Smem<128>::EW)};
+}
+
 cudaError_t launch_lora_gemm(const Launch& L, const LinearDev& lin, const RouteDev* R,
                              const CUtensorMap& tm_x, const CUtensorMap* tm_t, const CUtensorMap* tm_y,
                              int rows, int epi, const bf16* residual, const PatchEpi& pe, bf16* y,

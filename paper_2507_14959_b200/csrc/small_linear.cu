@@ -620,14 +620,14 @@ struct Shape { int width = -1, split = 1; };          // width: index into WIDTH
 //   1536 -> 384 in two, 128-wide 10: 7.7 / 7.9, 192-wide 16: 9.8 / 8.8.
 // With adapters the alternative is two kernels, whose t is rounded to bf16 once where the shares' t here keep 16 bits: K in two at 256
 // columns stays here although it is slower (3072 -> 768, 12 frames 22.5 / 19.5, 14: 22.5 / 20.6; 2048 -> 512, 24 frames 18.3 / 21.0).
-Shape pick_shape(const LinearDev& lin, bool lora, int rows, int epi, int n_sms) {
+Shape pick_shape(int k_in, int n_out, bool lora, int rows, int epi, int n_sms) {
     const long long m = (rows + BM - 1) / BM;
     const bool alone = epi == EPI_RESIDUAL && !lora;
-    for (int split = epi == EPI_RESIDUAL && lin.k_in >= 1536 ? 4 : 1; split >= 1; split >>= 1)
+    for (int split = epi == EPI_RESIDUAL && k_in >= 1536 ? 4 : 1; split >= 1; split >>= 1)
         for (int i = 0; i < PM_SMALL_WIDTHS; ++i) {
             if (split == 4 && WIDTHS[i] > 128) break;
             if (split == 1 && WIDTHS[i] > (alone ? 64 : 192) && !lora) break;
-            if (lin.n_out % WIDTHS[i] == 0 && m * (lin.n_out / WIDTHS[i]) * split <= n_sms) {
+            if (n_out % WIDTHS[i] == 0 && m * (n_out / WIDTHS[i]) * split <= n_sms) {
                 if (split == 2 && WIDTHS[i] > 128 && !lora) return Shape();
                 Shape s;
                 s.width = i; s.split = split;
@@ -659,16 +659,23 @@ static bool has_lora(const LinearDev& lin, const RouteDev* R) {
     return R && R->slab_cap > 0 && R->max_set > 0 && lin.lora.At != nullptr;
 }
 
+bool small_linear_form(int k_in, int n_out, bool lora, int rows, int epi, int n_sms, LinearForm* form) {
+    const Shape s = pick_shape(k_in, n_out, lora, rows, epi, n_sms);
+    if (s.width < 0) return false;
+    *form = {LINEAR_FEW_ROWS, WIDTHS[s.width], s.split, THREADS};
+    return true;
+}
+
 bool small_linear_fits(const LinearDev& lin, const RouteDev* R, int rows, int epi, int n_sms) {
     const bool lora = has_lora(lin, R);
-    return pick_shape(lin, lora, rows, epi, n_sms).width >= 0 && (!lora || R->tile_slab_cap <= LIST);
+    return pick_shape(lin.k_in, lin.n_out, lora, rows, epi, n_sms).width >= 0 && (!lora || R->tile_slab_cap <= LIST);
 }
 
 cudaError_t launch_small_linear(const Launch& L, const LinearDev& lin, const RouteDev* R, const ActMaps& x, int rows,
                                 int epi, const bf16* residual, const PatchEpi& pe, bf16* y, int n_sms, float ln_eps) {
     if (rows <= 0) return cudaSuccess;
     const bool lora = has_lora(lin, R);
-    const Shape shape = pick_shape(lin, lora, rows, epi, n_sms);
+    const Shape shape = pick_shape(lin.k_in, lin.n_out, lora, rows, epi, n_sms);
     const int w = shape.width;
     if (w < 0) return cudaErrorInvalidValue;
     SmallArgs a = {};
