@@ -341,6 +341,40 @@ def test_pair_gemm_widths(k_in, n_out, frames, tokens, rank, epi, what):
     test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, what)
 
 
+@pytest.mark.parametrize("k_in,n_out,frames,tokens,rank,adapters", [(64, 256, 130, 197, 8, 0), (384, 512, 60, 130, 16, 0), (192, 768, 40, 200, 24, 5),
+                                                                    (320, 384, 90, 197, 16, 0), (768, 768, 40, 197, 16, 5), (1536, 640, 30, 130, 16, 0)])
+def test_residual_may_be_the_output_buffer(k_in, n_out, frames, tokens, rank, adapters):
+    """y == residual through the single-CTA and the pair GEMM, ragged last row tiles: bit-equal to separate buffers, and within the
+    tolerance of the other linears of float64 sums."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    assert binding.linear_kernel(k_in, n_out, frames * tokens, 2, adapters)[0] == ("single" if k_in <= 384 else "pair")
+    gen = torch.Generator(device="cuda").manual_seed(k_in + n_out)
+    rows = frames * tokens
+
+    def draw(shape, std):
+        return (torch.randn(shape, generator=gen, device="cuda") * std).bfloat16()
+    x, res, w, b = draw((rows, k_in), 1.0), draw((rows, n_out), 1.0), draw((k_in, n_out), 0.02), draw((n_out,), 0.02)
+    A = [draw((k_in, rank), 0.02) for _ in range(adapters)]
+    B = [draw((rank, n_out), 0.02) for _ in range(adapters)]
+    host = lambda t: t.float().cpu().numpy()  # noqa: E731
+    lin = binding.Linear(host(w), host(b), max_adapters=max(1, adapters), max_rank=rank, max_set=1, max_frames=frames, tokens=tokens, epilogue=2)
+    for a in range(adapters):
+        lin.register(a, rank, 1.0, host(A[a]), host(B[a]))
+    off, ids = wl.sets_to_csr([[f % adapters] if adapters else [] for f in range(frames)])
+    y, z = torch.full((rows, n_out), float("nan"), device="cuda", dtype=torch.bfloat16), res.clone()
+    lin.forward(x, frames, off, ids, y, residual=res)
+    lin.forward(x, frames, off, ids, z, residual=z)
+    assert lin.status() == 0
+    assert torch.equal(y, z)
+    want = x.double() @ w.double() + b.double() + res.double()
+    for f in range(frames if adapters else 0):
+        r = slice(f * tokens, (f + 1) * tokens)
+        want[r] += (x[r].double() @ A[f % adapters].double()) @ B[f % adapters].double()
+    np.testing.assert_allclose(to_np(y), want.cpu().numpy(), **TOL[0])
+    lin.close()
+
+
 @pytest.mark.parametrize("frames,rank,what", [(1, 16, "64-wide, K in four"), (1, 64, "64-wide, K in four"), (12, 64, "256-wide, K in two")])
 def test_lora_linear_several_slab_groups_through_the_shortest_ring(frames, rank, what):
     """The few-row kernel's ring is shortest where a group of eight slabs and the exchange of partial sums take the
