@@ -47,7 +47,6 @@ struct GemmArgs {
 };
 
 constexpr int STAGING_BYTES = 32 * 64;                  // one chunk: [32 rows x 32 bf16]
-constexpr int STAGING_BYTES_PER_WARP = 2 * STAGING_BYTES;
 constexpr int PLAN_BYTES = 2048;
 constexpr int P_ACC_COLS = 256;                        // pair kernel: tensor-memory columns of one of the two accumulators
 
@@ -457,34 +456,39 @@ constexpr int P_T_SLAB_BYTES = BM * PM_SLAB * 2;       // 4 KB
 constexpr int P_MAX_STAGES = 8;
 constexpr int P_MAX_EW = 16;
 constexpr int P_BAR_BYTES = 512;
-// By tile width: an epilogue warp takes 64 columns of one lane quarter (two chunks, a staging buffer for each), so 256 columns
-// take 16 warps.  What the staging leaves is the ring's.
-template <int BN>
+// By tile width: an epilogue warp takes 64 columns of one lane quarter (two chunks), so 256 columns take 16 warps.  With a residual
+// there is a staging buffer for each chunk (request_residual); else 256-wide tiles have one per warp, which leaves the ring its sixth stage.
+// Two per warp and five stages, us, five stages / six, no adapters, frames of 197 tokens: 3072 -> 256, 75 and 256 frames 23.0 / 22.0 and 71.1 / 68.5;
+// 3072 -> 768, 256 frames 165 / 159; 768 -> 2304, 128 frames 67.3 / 66.3, with adapters 81.3 / 77.9.
+template <int BN, int EPI>
 struct PairCfg {
+    static constexpr int BUFFERS = BN < 256 || EPI == EPI_RESIDUAL ? 2 : 1;
+    static constexpr int STAGING_PER_WARP = BUFFERS * STAGING_BYTES;
     static constexpr int HALVES = BN / 64;                                 // epilogue warps per lane quarter
     static constexpr int EW = 4 * HALVES;
     static constexpr int THREADS = 64 + 32 * EW;
     static constexpr int B_BYTES = (BN / 2) * BK * 2;                      // this CTA's half of the W^T tile
     static constexpr int STAGE_BYTES = P_A_BYTES + B_BYTES;
     static constexpr int B_SLAB_BYTES = (BN / 2) * PM_SLAB * 2;
-    static constexpr int REST = EW * STAGING_BYTES_PER_WARP + PLAN_BYTES + P_BAR_BYTES;
+    static constexpr int REST = EW * STAGING_PER_WARP + PLAN_BYTES + P_BAR_BYTES;
     static constexpr int FIT = (227 * 1024 - REST) / STAGE_BYTES;
     static constexpr int STAGES = FIT < P_MAX_STAGES ? FIT : P_MAX_STAGES;
     static constexpr int STAGING_OFFSET = STAGES * STAGE_BYTES;
-    static constexpr int PLAN_OFFSET = STAGING_OFFSET + EW * STAGING_BYTES_PER_WARP;
+    static constexpr int PLAN_OFFSET = STAGING_OFFSET + EW * STAGING_PER_WARP;
     static constexpr int BAR_OFFSET = PLAN_OFFSET + PLAN_BYTES;
     static constexpr int TOTAL = BAR_OFFSET + P_BAR_BYTES;
     static_assert(SLABS_PER_STAGE * B_SLAB_BYTES <= B_BYTES, "LoRA stage");
+    static_assert(STAGES >= (EPI == EPI_RESIDUAL ? 5 : 6), "long K needs the depth");
     static_assert(8 * (2 * P_MAX_STAGES + 4) + 24 + 8 * P_MAX_EW <= P_BAR_BYTES, "barriers");
 };
 
 template <int BN, int EPI, bool LNF>
-__global__ void __launch_bounds__(PairCfg<BN>::THREADS, 1)
+__global__ void __launch_bounds__(PairCfg<BN, EPI>::THREADS, 1)
 lora_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                       const __grid_constant__ CUtensorMap tm_t, const __grid_constant__ CUtensorMap tm_bt,
                       const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_res,
                       const GemmArgs args) {
-    using C = PairCfg<BN>;
+    using C = PairCfg<BN, EPI>;
     constexpr int P_STAGES = C::STAGES, P_EW = C::EW;
     constexpr bool RES = EPI == EPI_RESIDUAL;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -667,7 +671,7 @@ lora_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         // ------------------------------------------------------------------ epilogue (both CTAs)
         const int quarter = warp & 3;
         const int half = (warp - 2) >> 2;
-        const uint32_t staging = base + C::STAGING_OFFSET + (uint32_t)(warp - 2) * STAGING_BYTES_PER_WARP;
+        const uint32_t staging = base + C::STAGING_OFFSET + (uint32_t)(warp - 2) * C::STAGING_PER_WARP;
         dep_wait();                                   // row statistics, residual; rows that the kernel before still reads
         int acc = 0;
         uint32_t acc_phase = 0, res_phase = 0;
@@ -676,7 +680,7 @@ lora_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         for (int tile = pair_id; tile < total_tiles && ok; tile += n_pairs) {
             const int m = 2 * (tile / args.n_tiles) + (int)rank, n = tile % args.n_tiles;
             if constexpr (RES) request_residual<BN>(tm_res, staging, res_bar(warp - 2), m, n, quarter, half);
-            ok = epilogue_tile<BN, EPI, C::HALVES, 2, true, LNF, RES>(
+            ok = epilogue_tile<BN, EPI, C::HALVES, C::BUFFERS, true, LNF, RES>(
                 args, tm_y, staging, chunk_no, tmem_base, acc, acc_phase, tfull_bar(acc),
                 mapa_cluster(tempty_bar(acc), 0), abort_flag, m, n, quarter, half, lane,
                 res_bar(warp - 2), res_phase);
@@ -876,12 +880,13 @@ static cudaError_t launch_gemm_pair(const Launch& L, const CUtensorMap& tm_x, co
         if (!tm_encode_2d(&tm_res, a.residual, a.n_out, a.rows, (uint64_t)a.n_out * 2, 32, 32, 64))
             return cudaErrorInvalidValue;
     }
+    using C = PairCfg<BN, EPI>;
     static SmemGrant grant;
-    if (cudaError_t e = grant.ensure(lora_gemm_pair_kernel<BN, EPI, LNF>, PairCfg<BN>::TOTAL); e != cudaSuccess) return e;
+    if (cudaError_t e = grant.ensure(lora_gemm_pair_kernel<BN, EPI, LNF>, C::TOTAL); e != cudaSuccess) return e;
     const int total = a.m_tiles * a.n_tiles;
     const int pairs = total < n_sms / 2 ? total : n_sms / 2;
     ProfScope ps(L, KC_GEMM);
-    cudaError_t e = launch_overlapped(L, lora_gemm_pair_kernel<BN, EPI, LNF>, 2 * pairs, PairCfg<BN>::THREADS, PairCfg<BN>::TOTAL, 2,
+    cudaError_t e = launch_overlapped(L, lora_gemm_pair_kernel<BN, EPI, LNF>, 2 * pairs, C::THREADS, C::TOTAL, 2,
                                       tm_x, tm_w, tm_t, tm_bt, tm_y, tm_res, a);
     BUMP(L);
     return e;
@@ -947,8 +952,8 @@ int gemm_tile_n(int n_out) { return (n_out % 256 == 0) ? 256 : 128; }
 LinearForm gemm_form(int k_in, int n_out, bool lora, int rows, int epi, int n_sms) {
     const int pw = n_sms >= 2 ? pick_pair_width(n_out, k_in, lora, rows, n_sms / 2) : -1;
     if (pw >= 0)
-        return {LINEAR_PAIR, PAIR_WIDTHS[pw], 1, PAIR_WIDTHS[pw] == 128 ? PairCfg<128>::THREADS : PAIR_WIDTHS[pw] == 192 ? PairCfg<192>::THREADS
-                                                                                                  : PairCfg<256>::THREADS};
+        return {LINEAR_PAIR, PAIR_WIDTHS[pw], 1, PAIR_WIDTHS[pw] == 128 ? PairCfg<128, EPI_NONE>::THREADS : PAIR_WIDTHS[pw] == 192 ? PairCfg<192, EPI_NONE>::THREADS
+                                                                                                  : PairCfg<256, EPI_NONE>::THREADS};
     const int bn = gemm_tile_n(n_out);
     return {LINEAR_SINGLE, bn, 1, 64 + 32 * (bn == 256 ? Smem<256>::EW : Smem<128>::EW)};
 }
