@@ -333,7 +333,7 @@ def test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, 
 
 
 @pytest.mark.parametrize("k_in,n_out,frames,tokens,rank,epi,what", [
-    (768, 640, 31, 130, 16, 2, "128-wide, one round"), (448, 1280, 60, 197, 8, 0, "256-wide of two widths"), (448, 640, 70, 197, 40, 1, "128-wide, several rounds"),
+    (768, 640, 31, 130, 16, 2, "128-wide, one round"), (448, 1280, 60, 197, 8, 0, "256-wide of two widths"), (832, 640, 70, 197, 40, 1, "128-wide, several rounds"), (448, 640, 70, 197, 40, 1, "single, 128-wide"),
     (3072, 768, 37, 197, 16, 2, "192-wide, two rounds"), (768, 768, 50, 200, 48, 2, "192-wide, several slab groups"),
     (768, 2304, 24, 130, 16, 1, "192-wide"), (768, 768, 60, 197, 16, 2, "256-wide, residual rows past the end")])
 def test_pair_gemm_widths(k_in, n_out, frames, tokens, rank, epi, what):

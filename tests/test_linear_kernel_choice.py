@@ -21,3 +21,13 @@ def test_arguments():
 def test_long_k_with_adapters_is_split_while_the_sms_suffice(k_in, n_out, frames, width, split):
     """Each share of t keeps 16 significant bits there, which no other form does."""
     assert binding.linear_kernel(k_in, n_out, frames * TOKENS, RESIDUAL, True)[:3] == ("few rows", width, split)
+
+
+@pytest.mark.parametrize("k_in,n_out,kernel", [(128, 640, "single"), (384, 896, "single"), (448, 1408, "single"), (640, 128, "single"), (768, 640, "pair"), (3072, 128, "pair"),
+                                               (384, 576, "pair"), (448, 1280, "pair"), (384, 1280, "single"), (384, 1152, "pair"), (768, 320, "single")])
+@pytest.mark.parametrize("epilogue,adapters", [(NONE, True), (GELU, False), (RESIDUAL, True), (RESIDUAL, False)])
+def test_widths_that_only_128_divides_take_pairs_for_long_k(k_in, n_out, kernel, epilogue, adapters):
+    got = binding.linear_kernel(k_in, n_out, 300 * TOKENS, epilogue, adapters)
+    assert got[0] == kernel
+    if kernel == "pair" and n_out % 192 and n_out % 256:
+        assert got[1] == 128
