@@ -89,20 +89,22 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs& args, const CUtens
     const int n_chunks = min(BN / 32, (args.n_out - n * BN) / 32);      // even: n_out % 64 == 0
     const int my_chunks = n_chunks / HALVES;
     const int c0 = half * my_chunks;
-    // Without RES_SMEM a thread fetches its residual row a chunk at a time, the first chunk before the accumulator is ready and
-    // the next one as soon as the one before it is added: all of them held over the main loop do not fit the registers that
-    // sixteen warps leave a thread (384 -> 768 on 32, 64 and 256 frames of 197 tokens, no adapters, us with eight warps and the rows held /
-    // sixteen, rows spilled / now: 11.2 / 11.8 / 10.5, 16.5 / 17.5 / 15.7, 55.2 / 57.9 / 54.7).  (In-place use, y == residual, is safe: the same thread reads an element here and is the only
-    // one to overwrite it below, and a chunk's columns are its own.)
+    // Without RES_SMEM a thread fetches its residual rows before the accumulator is ready, so that their latency hides behind the main
+    // loop; where sixteen warps share the registers only the first chunk, and the next one as soon as the one before it is added
+    // (384 -> 768 on 32, 64 and 256 frames of 197 tokens, no adapters, us with eight warps and all rows held / sixteen and all rows, which spilled /
+    // now: 11.2 / 11.8 / 10.5, 16.5 / 17.5 / 15.7, 55.2 / 57.9 / 54.7; 128-wide tiles, eight warps, 384 -> 384 on 20 frames a chunk at a time 5.5, all
+    // rows 5.2).  (In-place use, y == residual, is safe: the same thread reads an element here and is the only one to overwrite it
+    // below, and a chunk's columns are its own.)
     constexpr bool RES_REGS = EPI == EPI_RESIDUAL && !RES_SMEM;
-    uint4 rr[4] = {};
+    constexpr int HELD = RES_REGS && BN <= 128 ? CPW : 1;
+    uint4 rr[HELD][4];
     const uint4* rr_from = nullptr;
     if constexpr (RES_REGS) {
         rr_from = reinterpret_cast<const uint4*>(args.residual + (size_t)row * args.n_out + n * BN + c0 * 32);
-        if (row_ok && my_chunks > 0) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) rr[q] = rr_from[q];
-        }
+        for (int cc = 0; cc < HELD; ++cc)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) rr[cc][q] = row_ok && cc < my_chunks ? rr_from[cc * 4 + q] : make_uint4(0, 0, 0, 0);
     }
     bool ok = PAIR ? mbar_wait_cluster(tfull_addr, acc_phase, abort_flag, args.status)
                    : mbar_wait(tfull_addr, acc_phase, abort_flag, args.status);
@@ -170,17 +172,17 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs& args, const CUtens
                     asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
                                  : "=r"(r4v.x), "=r"(r4v.y), "=r"(r4v.z), "=r"(r4v.w) : "r"(a));
                 } else {
-                    r4v = rr[q];
+                    r4v = rr[cc % HELD][q];
                 }
                 const uint32_t w[4] = {r4v.x, r4v.y, r4v.z, r4v.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
                     fp[q * 4 + e] = add2(fp[q * 4 + e], pk2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xFFFF0000u)));
             }
-            if constexpr (RES_REGS) {
+            if constexpr (RES_REGS && HELD < CPW) {
                 if (row_ok && cc + 1 < my_chunks) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) rr[q] = rr_from[(cc + 1) * 4 + q];
+                    for (int q = 0; q < 4; ++q) rr[0][q] = rr_from[(cc + 1) * 4 + q];
                 }
             }
         } else if constexpr (EPI == EPI_PATCH) {
