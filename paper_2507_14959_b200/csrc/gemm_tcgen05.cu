@@ -938,7 +938,7 @@ bool gemm_encode_pair_maps(LinearDev& lin, int max_adapters, int slabs_max) {
 //   768 -> 3072: 16 frames 19.8 / 16.0 / 17.3, 37: 36.3 / 30.6 / 28.0, 192: 174 / 149 / 139.
 static int pick_pair_width(int n_out, int k_in, bool lora, int rows, int n_pairs) {
     if (k_in <= 384 && (n_out % 256 == 0 || (n_out <= 384 && !lora))) return -1;
-    if (k_in < 768 && n_out % 256 != 0 && n_out % 192 != 0) return -1;
+    if (k_in <= 640 && n_out % 256 != 0 && n_out % 192 != 0) return -1;
     const int m = (rows + 2 * BM - 1) / (2 * BM);
     int best = -1;
     float best_cost = 0.f;
