@@ -184,6 +184,8 @@ enum { LINEAR_FEW_ROWS = 0, LINEAR_PAIR = 1, LINEAR_SINGLE = 2 };
 struct LinearForm { int kernel, width, split, threads; };
 bool small_linear_form(int k_in, int n_out, bool lora, int rows, int epi, int n_sms, LinearForm* form);      // false: not for this kernel
 LinearForm gemm_form(int k_in, int n_out, bool lora, int rows, int epi, int n_sms);
+// whether the GEMM kernels cover rows without adapters in one round of 128-wide tiles
+bool gemm_narrow_round(int k_in, int n_out, int rows, int n_sms);
 // whether launch_small_linear serves this call (R: null = no adapters)
 bool small_linear_fits(const LinearDev& lin, const RouteDev* R, int rows, int epi, int n_sms);
 // The whole linear -- shrink, LayerNorm statistics where the LayerNorm is folded in, GEMM, expand, epilogue -- in one launch.

@@ -964,6 +964,12 @@ LinearForm gemm_form(int k_in, int n_out, bool lora, int rows, int epi, int n_sm
     return {LINEAR_SINGLE, bn, 1, 64 + 32 * (bn == 256 ? Smem<256>::EW : Smem<128>::EW)};
 }
 
+bool gemm_narrow_round(int k_in, int n_out, int rows, int n_sms) {
+    const LinearForm f = gemm_form(k_in, n_out, false, rows, EPI_NONE, n_sms);
+    if (f.kernel == LINEAR_SINGLE) return f.width == 128 && (rows + BM - 1) / BM * ((n_out + 127) / 128) <= n_sms;
+    return n_out % 128 == 0 && (rows + 2 * BM - 1) / (2 * BM) * (n_out / 128) <= n_sms / 2;
+}
+
 cudaError_t launch_lora_gemm(const Launch& L, const LinearDev& lin, const RouteDev* R,
                              const CUtensorMap& tm_x, const CUtensorMap* tm_t, const CUtensorMap* tm_y,
                              int rows, int epi, const bf16* residual, const PatchEpi& pe, bf16* y,

@@ -610,30 +610,34 @@ cudaError_t launch_epi(const Launch& L, const Maps& t, const SmallArgs& a, int e
 struct Shape { int width = -1, split = 1; };          // width: index into WIDTHS, -1 = not for this kernel
 
 // The split of K and the tile width: as many CTAs as fit the SMs in one wave.  K is split where it is long
-// (3072 -> 768 with adapters: 4 ways 10.1 us against 19.0 on 197 rows, 2 ways 18.6 against 25.4 on 1576; at 768
-// inputs splitting costs more than it gives, 8.8 against 7.7 us on 788 rows); the four-way split stops at 128
-// columns, whose partial sums leave the ring room.
-// Where the alternative is the pair GEMM alone (no adapters), wide tiles lose to it.  With a residual, whose rows this kernel
-// fetches and stores by thread, only the narrow ones win, us here / pair GEMM, frames of 197 tokens:
-//   768 -> 768 64-wide 6 frames 5.1 / 6.2, 128-wide 8: 7.5 / 6.7, 16: 10.1 / 8.8;  384 -> 384 64-wide 14: 4.3 / 5.1, 128-wide 16: 6.5 / 4.8;
-//   192 -> 192 192-wide 32: 7.5 / 4.4;  3072 -> 768 in two, 128-wide 6: 10.5 / 11.8, 192-wide 8: 13.2 / 12.7, 256-wide 12: 16.9 / 13.2;
-//   1536 -> 384 in two, 128-wide 10: 7.7 / 7.9, 192-wide 16: 9.8 / 8.8.
+// (3072 -> 768 with adapters: 4 ways 7.1 us against 10.3 on 197 rows, 2 ways 16.9 against 22.7 on 1576; at 768
+// inputs it costs what it gives, 768 -> 768 in two 5.0 against 5.3 us on 197 rows, 5.9 against 5.3 on 394, 9.5 against 5.8 on 788); the
+// four-way split stops at 128 columns, whose partial sums leave the ring room.
+// Without adapters the alternative is a GEMM kernel alone, to which wide tiles lose: unsplit 256-wide ones always.  With a
+// residual, whose rows this kernel fetches and stores by thread, so do all but the narrow ones (64 columns, K in two 128) while the GEMM
+// covers the rows in one round of 128-wide tiles, us here / GEMM, frames of 197 tokens:
+//   768 -> 768 64-wide 6 frames 5.3 / 6.4, 128-wide 8: 7.7 / 6.9, 14: 8.1 / 7.6;  384 -> 384 64-wide 14: 4.5 / 5.2, 128-wide 16: 6.7 / 5.0;
+//   1024 -> 1024 128-wide 10: 8.2 / 8.1;  3072 -> 768 in two, 128-wide 6: 10.7 / 12.0, 192-wide 8: 13.2 / 12.9, 256-wide 12: 16.9 / 13.3;
+//   1536 -> 384 in two, 128-wide 10: 7.8 / 8.0, 192-wide 16: 9.9 / 8.9.
+// Where it would take wider tiles or more rounds, unsplit 128-wide tiles win, or 192-wide ones with K in two; unsplit 192-wide ones still lose:
+//   512 -> 512 128-wide 24: 6.8 / 8.6;  2048 -> 512 24: 11.6, 256-wide in two 14.2 / 15.8;  256 -> 256 (K too short for pairs) 28: 5.4 / 7.1;
+//   3072 -> 576 (pairs are 192-wide) 64-wide 8: 10.7, 192-wide in two 12.5 / 15.7, 12: 13.4 / 15.9;
+//   768 -> 768 192-wide 16: 10.3 / 8.9;  192 -> 192 192-wide 32: 7.6 / 4.4.
 // With adapters the alternative is two kernels, whose t is rounded to bf16 once where the shares' t here keep 16 bits: K in two at 256
 // columns stays here although it is slower (3072 -> 768, 12 frames 22.5 / 19.5, 14: 22.5 / 20.6; 2048 -> 512, 24 frames 18.3 / 21.0).
 Shape pick_shape(int k_in, int n_out, bool lora, int rows, int epi, int n_sms) {
     const long long m = (rows + BM - 1) / BM;
-    const bool alone = epi == EPI_RESIDUAL && !lora;
-    for (int split = epi == EPI_RESIDUAL && k_in >= 1536 ? 4 : 1; split >= 1; split >>= 1)
-        for (int i = 0; i < PM_SMALL_WIDTHS; ++i) {
-            if (split == 4 && WIDTHS[i] > 128) break;
-            if (split == 1 && WIDTHS[i] > (alone ? 64 : 192) && !lora) break;
-            if (n_out % WIDTHS[i] == 0 && m * (n_out / WIDTHS[i]) * split <= n_sms) {
-                if (split == 2 && WIDTHS[i] > 128 && !lora) return Shape();
-                Shape s;
-                s.width = i; s.split = split;
-                return s;
-            }
-        }
+    const bool long_k = epi == EPI_RESIDUAL && k_in >= 1536, alone = epi == EPI_RESIDUAL && !lora;
+    auto fits = [&](int i, int split) { return n_out % WIDTHS[i] == 0 && m * (n_out / WIDTHS[i]) * split <= n_sms; };
+    for (int split = long_k ? 4 : 1; split >= 1; split >>= 1) {
+        const int widest = split == 4 ? 128 : alone ? 64 * split : split == 1 && !lora ? 192 : 256;
+        for (int i = 0; i < PM_SMALL_WIDTHS && WIDTHS[i] <= widest; ++i)
+            if (fits(i, split)) return {i, split};
+    }
+    if (alone && !gemm_narrow_round(k_in, n_out, rows, n_sms)) {
+        if (fits(1, 1)) return {1, 1};
+        if (long_k && fits(2, 2)) return {2, 2};       // (256-wide in two takes as many CTAs as 128-wide unsplit)
+    }
     return Shape();
 }
 

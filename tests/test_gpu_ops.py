@@ -284,6 +284,14 @@ def test_bounded_wait_gives_up_and_reports():
         binding.selftest_wait_timeout(10 ** 12, status, trace)       # limits beyond 1e8 cycles are refused
 
 
+def check_form(k_in, n_out, rows, epi, adapters, form):
+    """The kernel, tile width and split of K that a test names are those of the rule (stated for 148 SMs)."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert binding.linear_kernel(k_in, n_out, rows, epi, adapters)[:3] == form
+
+
 @pytest.mark.parametrize("k_in,n_out,frames,tokens,rank,epi,what", [
     (768, 768, 1, 197, 16, 2, "64-wide tiles"), (320, 576, 2, 130, 24, 0, "64-wide tiles, odd K blocks"),
     (768, 2304, 3, 197, 64, 0, "128-wide tiles, several slab groups"), (192, 1152, 16, 128, 16, 1, "192-wide tiles, whole row tiles"),
@@ -295,7 +303,7 @@ def test_bounded_wait_gives_up_and_reports():
     (1600, 1536, 20, 197, 16, 2, "shrink with K in four, odd K blocks"), (1536, 1536, 40, 197, 48, 2, "shrink with K in two, several slab groups"),
     (320, 768, 70, 130, 64, 1, "shrink of one tile per SM, odd K blocks, slabs beyond the list"),
     (192, 768, 300, 100, 24, 0, "shrink of two tiles per SM"), (192, 256, 300, 197, 40, 1, "shrink of three tiles per SM"), (64, 64, 1, 1, 4, 0, "one row")])
-def test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, what):
+def test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, what, most=6):
     """One case on each side of every line of the few-row kernel's tile rule (on 148 SMs), sets of 0 to 6 of 7
     adapters, against float64 sums of the same bf16 inputs.  Tolerance: as for the other linears (one bf16 rounding of
     the output, one of t)."""
@@ -310,7 +318,7 @@ def test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, 
     A = [draw((k_in, rank), 0.02) for _ in range(n_ad)]
     B = [draw((rank, n_out), 0.02) for _ in range(n_ad)]
     g = np.random.default_rng(rows)
-    sets = [sorted(int(a) for a in g.choice(n_ad, size=int(g.integers(0, 7)), replace=False)) for _ in range(frames)]
+    sets = [sorted(int(a) for a in g.choice(n_ad, size=int(g.integers(0, most + 1)), replace=False)) for _ in range(frames)]
     off, ids = wl.sets_to_csr(sets)
     host = lambda t: t.float().cpu().numpy()  # noqa: E731
     lin = binding.Linear(host(w), host(b), max_adapters=n_ad, max_rank=rank, max_set=6, max_frames=frames, tokens=tokens, epilogue=epi)
@@ -339,6 +347,16 @@ def test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, 
 def test_pair_gemm_widths(k_in, n_out, frames, tokens, rank, epi, what):
     """The three tile widths of the CTA-pair GEMM with every epilogue, ragged last row tiles, one and several rounds."""
     test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, what)
+
+
+@pytest.mark.parametrize("k_in,n_out,frames,form", [
+    (768, 768, 6, ("few rows", 64, 1)), (768, 768, 8, ("pair", 128, 1)), (512, 512, 24, ("few rows", 128, 1)), (512, 512, 28, ("pair", 256, 1)),
+    (3072, 768, 6, ("few rows", 128, 2)), (2048, 512, 12, ("pair", 128, 1)), (2048, 512, 24, ("few rows", 128, 1)), (1600, 576, 9, ("few rows", 64, 1)),
+    (1600, 576, 12, ("few rows", 192, 2)), (3072, 576, 16, ("pair", 192, 1)), (256, 256, 40, ("few rows", 128, 1)), (256, 256, 96, ("single", 256, 1))])
+def test_residual_linear_without_adapters_around_the_few_row_rule(k_in, n_out, frames, form):
+    """A residual and empty sets on both sides of each line of the few-row kernel's rule."""
+    check_form(k_in, n_out, frames * 197, 2, False, form)
+    test_lora_linear_over_the_tile_rule(k_in, n_out, frames, 197, 8, 2, "", most=0)
 
 
 @pytest.mark.parametrize("k_in,n_out,frames,tokens,rank,adapters", [(64, 256, 130, 197, 8, 0), (384, 512, 60, 130, 16, 0), (192, 768, 40, 200, 24, 5),

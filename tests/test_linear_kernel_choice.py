@@ -31,3 +31,15 @@ def test_widths_that_only_128_divides_take_pairs_for_long_k(k_in, n_out, kernel,
     assert got[0] == kernel
     if kernel == "pair" and n_out % 192 and n_out % 256:
         assert got[1] == 128
+
+
+@pytest.mark.parametrize("k_in,n_out,frames,form", [
+    (768, 768, 6, ("few rows", 64, 1)), (768, 768, 8, ("pair", 128, 1)), (768, 768, 14, ("pair", 128, 1)), (768, 768, 16, ("pair", 192, 1)),
+    (1024, 1024, 10, ("pair", 128, 1)), (512, 512, 20, ("pair", 128, 1)), (512, 512, 24, ("few rows", 128, 1)), (512, 512, 28, ("pair", 256, 1)),
+    (1280, 512, 24, ("few rows", 128, 1)), (2048, 512, 10, ("few rows", 128, 2)), (2048, 512, 12, ("pair", 128, 1)), (2048, 512, 24, ("few rows", 128, 1)),
+    (256, 256, 20, ("few rows", 64, 1)), (256, 256, 40, ("few rows", 128, 1)), (256, 256, 96, ("single", 256, 1)), (384, 1024, 10, ("few rows", 128, 1)),
+    (384, 384, 16, ("single", 128, 1)), (192, 192, 32, ("single", 128, 1)), (384, 768, 20, ("single", 256, 1)), (3072, 576, 4, ("few rows", 64, 2)),
+    (3072, 576, 8, ("few rows", 64, 1)), (3072, 576, 12, ("few rows", 192, 2)), (3072, 576, 16, ("pair", 192, 1)), (3072, 768, 6, ("few rows", 128, 2)),
+    (3072, 768, 8, ("pair", 128, 1)), (3072, 768, 12, ("pair", 128, 1)), (768, 320, 8, ("few rows", 64, 1))])
+def test_residuals_without_adapters_leave_the_few_row_kernel_for_narrow_gemm_tiles_only(k_in, n_out, frames, form):
+    assert binding.linear_kernel(k_in, n_out, frames * TOKENS, RESIDUAL, False)[:3] == form
