@@ -926,9 +926,9 @@ bool gemm_encode_pair_maps(LinearDev& lin, int max_adapters, int slabs_max) {
 // The tile width of the pair kernel (index into PAIR_WIDTHS), or -1 for the single-CTA kernel.  Short K goes to the latter
 // where 256 divides the width, and for narrow outputs without adapters: a tile's K loop is too short to hide what the two
 // CTAs of a pair wait for each other (384 -> 1536 on 64 frames of 197 tokens 23.3 us against 25.0 on pairs, 192 -> 768 on 256
-// frames 35.8 against 39.5).  So do widths of which only 128 is a divisor up to K = 640, us single / pair: 128 -> 640 on 32 and 256 frames
+// frames 35.8 against 39.5).  So do widths of which only 128 is a divisor below K = 640, us single / pair: 128 -> 640 on 32 and 256 frames
 // 5.1 / 6.9 and 16.5 / 30.5, 384 -> 640 on 128 frames 14.9 / 19.3, 512 -> 640 with a residual on 256 frames 47.5 / 54.3, 256 -> 128 with adapters
-// on 256 frames 14.2 / 16.6; but 768 -> 640 on 64 and 256 frames 15.1 / 14.8 and 59.1 / 51.3, 3072 -> 640 on 64 frames 57.2 / 43.5.
+// on 256 frames 14.2 / 16.6; but 640 -> 640 with a residual on 48 frames 12.6 / 12.1, 768 -> 640 on 64 and 256 frames 15.1 / 14.8 and 59.1 / 51.3, 3072 -> 640 on 64 frames 57.2 / 43.5.
 // Else the width with the cheapest rounds of tiles over the pairs: a round costs its columns, and what a
 // tile costs whatever its width, in columns (hand-over between tiles; more where a short K loop leaves the epilogue exposed).
 // The two constants are fitted to 1 to 192 frames of 197 tokens, with and without adapters, widths of 384 and 768: the rule's
@@ -938,7 +938,7 @@ bool gemm_encode_pair_maps(LinearDev& lin, int max_adapters, int slabs_max) {
 //   768 -> 3072: 16 frames 19.8 / 16.0 / 17.3, 37: 36.3 / 30.6 / 28.0, 192: 174 / 149 / 139.
 static int pick_pair_width(int n_out, int k_in, bool lora, int rows, int n_pairs) {
     if (k_in <= 384 && (n_out % 256 == 0 || (n_out <= 384 && !lora))) return -1;
-    if (k_in <= 640 && n_out % 256 != 0 && n_out % 192 != 0) return -1;
+    if (k_in < 640 && n_out % 256 != 0 && n_out % 192 != 0) return -1;
     const int m = (rows + 2 * BM - 1) / (2 * BM);
     int best = -1;
     float best_cost = 0.f;

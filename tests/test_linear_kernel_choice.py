@@ -23,7 +23,7 @@ def test_long_k_with_adapters_is_split_while_the_sms_suffice(k_in, n_out, frames
     assert binding.linear_kernel(k_in, n_out, frames * TOKENS, RESIDUAL, True)[:3] == ("few rows", width, split)
 
 
-@pytest.mark.parametrize("k_in,n_out,kernel", [(128, 640, "single"), (384, 896, "single"), (448, 1408, "single"), (640, 128, "single"), (704, 640, "pair"), (768, 640, "pair"), (3072, 128, "pair"),
+@pytest.mark.parametrize("k_in,n_out,kernel", [(128, 640, "single"), (384, 896, "single"), (448, 1408, "single"), (576, 128, "single"), (640, 640, "pair"), (768, 640, "pair"), (3072, 128, "pair"),
                                                (384, 576, "pair"), (448, 1280, "pair"), (384, 1280, "single"), (384, 1152, "pair"), (768, 320, "single")])
 @pytest.mark.parametrize("epilogue,adapters", [(NONE, True), (GELU, False), (RESIDUAL, True), (RESIDUAL, False)])
 def test_widths_that_only_128_divides_take_pairs_for_long_k(k_in, n_out, kernel, epilogue, adapters):
