@@ -522,6 +522,26 @@ def test_deit_small_streams_bf16():
     m.close()
 
 
+@pytest.mark.parametrize("n_frames", [18, 52])
+def test_deit_small_batches_through_128_wide_pair_tiles(n_frames):
+    """128-wide tiles of the CTA-pair GEMM with a folded LayerNorm (qkv on 18 frames) and with patch placement (52 frames), on
+    148 SMs; the first, a middle and the last frame against the oracle."""
+    import torch
+    from paper_2507_14959_b200 import binding
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        sizes = (384, 1152, n_frames * 197, 0, True) if n_frames == 18 else (768, 384, n_frames * 196, 3, False)
+        assert binding.linear_kernel(*sizes)[:3] == ("pair", 128, 1)
+    w = wl.deit_small_streams()
+    off, ids = wl.sets_to_csr(w.sets()[:n_frames])
+    m = binding.model_from_workload(w, dtype=0, max_frames=n_frames)
+    s, b = run_forward(m, w, 0, frames=w.frames[:n_frames], offsets=off, ids=ids)
+    rows = [0, n_frames // 2, n_frames - 1]
+    so, bo = oracle_rows(w, rows)
+    assert np.abs(s[rows] - so).max() < 1e-2
+    assert np.abs(b[rows] - bo).max() < 1e-2
+    m.close()
+
+
 def test_deit_small_fp32_debug_subset():
     from paper_2507_14959_b200 import binding
     w = wl.deit_small_streams()

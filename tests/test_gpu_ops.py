@@ -292,23 +292,26 @@ def check_form(k_in, n_out, rows, epi, adapters, form):
         assert binding.linear_kernel(k_in, n_out, rows, epi, adapters)[:3] == form
 
 
-@pytest.mark.parametrize("k_in,n_out,frames,tokens,rank,epi,what", [
-    (768, 768, 1, 197, 16, 2, "64-wide tiles"), (320, 576, 2, 130, 24, 0, "64-wide tiles, odd K blocks"),
-    (768, 2304, 3, 197, 64, 0, "128-wide tiles, several slab groups"), (192, 1152, 16, 128, 16, 1, "192-wide tiles, whole row tiles"),
-    (768, 3072, 6, 197, 16, 1, "256-wide tiles"), (3072, 768, 1, 197, 16, 2, "64-wide, K in four"),
-    (1600, 768, 3, 200, 16, 2, "128-wide, K in four, odd K blocks"), (3072, 768, 6, 197, 8, 2, "128-wide, K in two"),
-    (3072, 768, 8, 197, 48, 2, "192-wide, K in two, several slab groups"), (3072, 768, 12, 197, 16, 2, "256-wide, K in two"),
-    (3072, 768, 17, 197, 16, 2, "unsplit"), (768, 768, 33, 197, 16, 2, "beyond one wave: shrink and pair GEMM"),
-    (384, 1152, 30, 197, 16, 0, "beyond one wave, narrow"),
-    (1600, 1536, 20, 197, 16, 2, "shrink with K in four, odd K blocks"), (1536, 1536, 40, 197, 48, 2, "shrink with K in two, several slab groups"),
-    (320, 768, 70, 130, 64, 1, "shrink of one tile per SM, odd K blocks, slabs beyond the list"),
-    (192, 768, 300, 100, 24, 0, "shrink of two tiles per SM"), (192, 256, 300, 197, 40, 1, "shrink of three tiles per SM"), (64, 64, 1, 1, 4, 0, "one row")])
-def test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, what, most=6):
-    """One case on each side of every line of the few-row kernel's tile rule (on 148 SMs), sets of 0 to 6 of 7
-    adapters, against float64 sums of the same bf16 inputs.  Tolerance: as for the other linears (one bf16 rounding of
+@pytest.mark.parametrize("k_in,n_out,frames,tokens,rank,epi,form,what", [
+    (768, 768, 1, 197, 16, 2, ("few rows", 64, 1), ""), (320, 576, 2, 130, 24, 0, ("few rows", 64, 1), "odd K blocks"),
+    (768, 2304, 3, 197, 64, 0, ("few rows", 128, 1), "several slab groups"), (192, 1152, 16, 128, 16, 1, ("few rows", 128, 1), "whole row tiles"),
+    (192, 1152, 24, 128, 16, 1, ("few rows", 192, 1), "whole row tiles"), (768, 3072, 6, 197, 16, 1, ("few rows", 256, 1), ""),
+    (3072, 768, 1, 197, 16, 2, ("few rows", 64, 4), ""), (1600, 768, 3, 200, 16, 2, ("few rows", 128, 4), "odd K blocks"),
+    (3072, 768, 6, 197, 8, 2, ("few rows", 128, 2), ""), (3072, 768, 8, 197, 48, 2, ("few rows", 192, 2), "several slab groups"),
+    (3072, 768, 12, 197, 16, 2, ("few rows", 256, 2), ""), (3072, 768, 17, 197, 16, 2, ("few rows", 192, 1), "unsplit"),
+    (768, 768, 33, 197, 16, 2, ("pair", 192, 1), "beyond one wave: shrink and pair GEMM"), (384, 1152, 30, 197, 16, 0, ("pair", 192, 1), "beyond one wave, short K"),
+    (1600, 1536, 20, 197, 16, 2, ("pair", 192, 1), "shrink with K in four, odd K blocks"),
+    (1536, 1536, 40, 197, 48, 2, ("pair", 256, 1), "shrink with K in two, several slab groups"),
+    (320, 768, 70, 130, 64, 1, ("single", 256, 1), "shrink of one tile per SM, odd K blocks, slabs beyond the list"),
+    (192, 768, 300, 100, 24, 0, ("single", 256, 1), "shrink of two tiles per SM"), (192, 256, 300, 197, 40, 1, ("single", 256, 1), "shrink of three tiles per SM"),
+    (64, 64, 1, 1, 4, 0, ("few rows", 64, 1), "one row")])
+def test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, form, what, most=6):
+    """One case on each side of every line of the few-row kernel's tile rule for linears with adapters (on 148 SMs), sets of
+    0 to 6 of 7 adapters, against float64 sums of the same bf16 inputs.  Tolerance: as for the other linears (one bf16 rounding of
     the output, one of t)."""
     import torch
     from paper_2507_14959_b200 import binding
+    check_form(k_in, n_out, frames * tokens, epi, most > 0, form)
     gen = torch.Generator(device="cuda").manual_seed(k_in + n_out + frames)
 
     def draw(shape, std):
@@ -340,13 +343,19 @@ def test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, 
     lin.close()
 
 
-@pytest.mark.parametrize("k_in,n_out,frames,tokens,rank,epi,what", [
-    (768, 640, 31, 130, 16, 2, "128-wide, one round"), (448, 1280, 60, 197, 8, 0, "256-wide of two widths"), (832, 640, 70, 197, 40, 1, "128-wide, several rounds"), (448, 640, 70, 197, 40, 1, "single, 128-wide"),
-    (3072, 768, 37, 197, 16, 2, "192-wide, two rounds"), (768, 768, 50, 200, 48, 2, "192-wide, several slab groups"),
-    (768, 2304, 24, 130, 16, 1, "192-wide"), (768, 768, 60, 197, 16, 2, "256-wide, residual rows past the end")])
-def test_pair_gemm_widths(k_in, n_out, frames, tokens, rank, epi, what):
-    """The three tile widths of the CTA-pair GEMM with every epilogue, ragged last row tiles, one and several rounds."""
-    test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, what)
+@pytest.mark.parametrize("k_in,n_out,frames,tokens,rank,epi,form,rounds", [
+    (768, 640, 31, 130, 16, 2, ("pair", 128, 1), 2), (832, 640, 70, 197, 40, 1, ("pair", 128, 1), 4), (768, 896, 100, 130, 24, 0, ("pair", 128, 1), 5),
+    (3072, 768, 37, 197, 16, 2, ("pair", 192, 1), 2), (768, 576, 40, 200, 48, 2, ("pair", 192, 1), 2), (768, 768, 37, 197, 40, 1, ("pair", 192, 1), 2),
+    (768, 576, 70, 197, 8, 0, ("pair", 192, 1), 3),
+    (448, 1280, 60, 197, 8, 0, ("pair", 256, 1), 4), (768, 768, 50, 200, 48, 2, ("pair", 256, 1), 2), (768, 2304, 24, 130, 16, 1, ("pair", 256, 1), 2),
+    (768, 768, 60, 197, 16, 2, ("pair", 256, 1), 2), (448, 640, 70, 197, 40, 1, ("single", 128, 1), 4)])
+def test_pair_gemm_widths(k_in, n_out, frames, tokens, rank, epi, form, rounds):
+    """The three tile widths of the CTA-pair GEMM, and the single-CTA kernel for a width that only 128 divides, with the plain,
+    the GELU and the residual epilogue, ragged last row tiles, several rounds, up to 21 slabs.  (One round: the residuals
+    without adapters below.  Folded LayerNorm and patch placement: the models' forwards.)"""
+    rows = 256 if form[0] == "pair" else 128
+    assert -(-(-(-frames * tokens // rows) * (n_out // form[1])) // (148 if form[0] == "single" else 74)) == rounds
+    test_lora_linear_over_the_tile_rule(k_in, n_out, frames, tokens, rank, epi, form, "")
 
 
 @pytest.mark.parametrize("k_in,n_out,frames,form", [
@@ -355,8 +364,7 @@ def test_pair_gemm_widths(k_in, n_out, frames, tokens, rank, epi, what):
     (1600, 576, 12, ("few rows", 192, 2)), (3072, 576, 16, ("pair", 192, 1)), (256, 256, 40, ("few rows", 128, 1)), (256, 256, 96, ("single", 256, 1))])
 def test_residual_linear_without_adapters_around_the_few_row_rule(k_in, n_out, frames, form):
     """A residual and empty sets on both sides of each line of the few-row kernel's rule."""
-    check_form(k_in, n_out, frames * 197, 2, False, form)
-    test_lora_linear_over_the_tile_rule(k_in, n_out, frames, 197, 8, 2, "", most=0)
+    test_lora_linear_over_the_tile_rule(k_in, n_out, frames, 197, 8, 2, form, "", most=0)
 
 
 @pytest.mark.parametrize("k_in,n_out,frames,tokens,rank,adapters", [(64, 256, 130, 197, 8, 0), (384, 512, 60, 130, 16, 0), (192, 768, 40, 200, 24, 5),
@@ -393,8 +401,8 @@ def test_residual_may_be_the_output_buffer(k_in, n_out, frames, tokens, rank, ad
     lin.close()
 
 
-@pytest.mark.parametrize("frames,rank,what", [(1, 16, "64-wide, K in four"), (1, 64, "64-wide, K in four"), (12, 64, "256-wide, K in two")])
-def test_lora_linear_several_slab_groups_through_the_shortest_ring(frames, rank, what):
+@pytest.mark.parametrize("frames,rank,form", [(1, 16, ("few rows", 64, 4)), (1, 64, ("few rows", 64, 4)), (12, 64, ("few rows", 256, 2))])
+def test_lora_linear_several_slab_groups_through_the_shortest_ring(frames, rank, form):
     """The few-row kernel's ring is shortest where a group of eight slabs and the exchange of partial sums take the
     rest of the shared memory; further groups of slabs then follow through those stages, x from one thread and the slabs
     from another.  Eight adapters on every frame: one to eight groups per tile.  Several calls in a row, against float64
@@ -402,6 +410,7 @@ def test_lora_linear_several_slab_groups_through_the_shortest_ring(frames, rank,
     import torch
     from paper_2507_14959_b200 import binding
     k_in, n_out, tokens, n_ad, rows = 3072, 768, 197, 16, frames * 197
+    check_form(k_in, n_out, rows, 2, True, form)
     gen = torch.Generator(device="cuda").manual_seed(frames + rank)
 
     def draw(shape, std):
@@ -466,9 +475,9 @@ def test_lora_linear_of_long_slab_lists_on_full_grids(frames, tokens, rank, n_ad
     lin.close()
 
 
-@pytest.mark.parametrize("frames,what", [(1, "64-wide, K in four"), (2, "128-wide, K in four"), (4, "128-wide, K in two"),
-                                         (8, "192-wide, K in two"), (12, "256-wide, K in two"), (33, "shrink with K in two")])
-def test_lora_intermediate_of_a_split_k_is_not_rounded_share_by_share(frames, what):
+@pytest.mark.parametrize("frames,form", [(1, ("few rows", 64, 4)), (2, ("few rows", 128, 4)), (4, ("few rows", 128, 2)), (8, ("few rows", 192, 2)),
+                                         (12, ("few rows", 256, 2)), (33, ("pair", 192, 1))])
+def test_lora_intermediate_of_a_split_k_is_not_rounded_share_by_share(frames, form):
     """t = s x A whose K shares cancel: x is 64 times as large on one part of each half of K and the halves take most of it
     back.  W = 0, so the output is t B.  Root mean square of the error against float64, relative to that of the
     output: one rounding of t and one of the output to bf16, 2^-9 each at most, give below 2^-8; shares rounded
@@ -476,6 +485,7 @@ def test_lora_intermediate_of_a_split_k_is_not_rounded_share_by_share(frames, wh
     import torch
     from paper_2507_14959_b200 import binding
     k_in, n_out, tokens, rank, rows = 3072, 768, 197, 16, frames * 197
+    check_form(k_in, n_out, rows, 2, True, form)        # the last one: shrink with K in two
     gen = torch.Generator(device="cuda").manual_seed(frames)
 
     def draw(shape, std):
@@ -506,6 +516,7 @@ def test_lora_intermediate_of_a_split_k_is_held_in_more_than_16_bits(k_in, n_out
     import torch
     from paper_2507_14959_b200 import binding
     tokens, rank, rows = 197, 16, frames * 197
+    assert binding.linear_kernel(k_in, n_out, rows, 2, True)[2] > 1
     gen = torch.Generator(device="cuda").manual_seed(frames)
     x = torch.randn((rows, k_in), generator=gen, device="cuda").bfloat16()
     A = (torch.randn((k_in, rank), generator=gen, device="cuda") * 0.02).bfloat16()
