@@ -15,7 +15,7 @@
 // PM_ERR_TIMEOUT in the status word, drains and returns.
 // The CTA-pair variant (lora_gemm_pair_kernel, cta_group::2, 256-row tiles of 128, 192 or 256 columns) serves most shapes, the single-CTA
 // kernel short K and other widths (pick_pair_width).  Both start while the kernel before them on the stream still runs
-// (programmatic dependent launch): 768 -> 768 with shrink on 197 x 256 rows 83.1 -> 79.5 us, on 197 x 37 rows 20.8 -> 19.6 us.
+// (programmatic dependent launch): 768 -> 768 with shrink on 197 x 256 rows 77.6 us behind its end, 73.4 so; on 197 x 37 rows 21.2, 15.4.
 #include "common.cuh"
 #include "f32x2.cuh"
 #include "tcgen05_ptx.cuh"
@@ -232,7 +232,8 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs& args, const CUtens
 }
 
 // Asks TMA for the residual rows of an epilogue warp's two chunks (rows past the end read as zero), into the warp's staging
-// buffers as soon as the stores of its previous tile have read them: a whole main loop ahead of their use.
+// buffers as soon as the stores of its previous tile have read them: ahead of their use by what is left of the tile's main loop then
+// (all of it for a CTA's first tile, little where an epilogue takes as long as a main loop).
 template <int BN>
 __device__ __forceinline__ void request_residual(const CUtensorMap& tm_res, uint32_t staging, uint32_t res_bar, int m, int n, int quarter, int half) {
     if (elect_one()) {
@@ -451,7 +452,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
 //   empty[s]   (both CTAs)  the pair MMAs that read stage s are done (multicast commit)
 //   tfull[a]   (both CTAs)  accumulator a is complete (multicast commit)
 //   tempty[a]  (even CTA)   both CTAs' epilogue warps have drained accumulator a
-// Up to eight stages per CTA.  No TMA multicast is used.
+// Eight (128 columns), six, or with a 256-wide residual five stages per CTA.  No TMA multicast is used.
 // ---------------------------------------------------------------------------------------
 constexpr int P_A_BYTES = BM * BK * 2;                 // 16 KB: this CTA's 128 rows of x
 constexpr int P_T_SLAB_BYTES = BM * PM_SLAB * 2;       // 4 KB
@@ -925,17 +926,17 @@ bool gemm_encode_pair_maps(LinearDev& lin, int max_adapters, int slabs_max) {
 
 // The tile width of the pair kernel (index into PAIR_WIDTHS), or -1 for the single-CTA kernel.  Short K goes to the latter
 // where 256 divides the width, and for narrow outputs without adapters: a tile's K loop is too short to hide what the two
-// CTAs of a pair wait for each other (384 -> 1536 on 64 frames of 197 tokens 23.3 us against 25.0 on pairs, 192 -> 768 on 256
-// frames 35.8 against 39.5).  So do widths of which only 128 is a divisor below K = 640, us single / pair: 128 -> 640 on 32 and 256 frames
+// CTAs of a pair wait for each other (GELU, no adapters, 384 -> 1536 on 64 frames of 197 tokens 17.4 us against 20.1 on pairs, 192 -> 768 on
+// 256 frames 23.1 against 29.5).  So do widths of which only 128 is a divisor below K = 640, us single / pair: 128 -> 640 on 32 and 256 frames
 // 5.1 / 6.9 and 16.5 / 30.5, 384 -> 640 on 128 frames 14.9 / 19.3, 512 -> 640 with a residual on 256 frames 47.5 / 54.3, 256 -> 128 with adapters
 // on 256 frames 14.2 / 16.6; but 640 -> 640 with a residual on 48 frames 12.6 / 12.1, 768 -> 640 on 64 and 256 frames 15.1 / 14.8 and 59.1 / 51.3, 3072 -> 640 on 64 frames 57.2 / 43.5.
 // Else the width with the cheapest rounds of tiles over the pairs: a round costs its columns, and what a
 // tile costs whatever its width, in columns (hand-over between tiles; more where a short K loop leaves the epilogue exposed).
-// The two constants are fitted to 1 to 192 frames of 197 tokens, with and without adapters, widths of 384 and 768: the rule's
-// choice is 0.4 % slower than the best of the three widths on average, 256 throughout 4.9 %.  us, 128 / 192 / 256 wide:
-//   3072 -> 768: 12 frames 13.6 / 17.2 / 20.4, 16: 20.9 / 17.4 / 21.1, 37: 31.9 / 29.1 / 34.7, 192: 147 / 134 / 131;
-//   768 -> 768: 12 frames 8.4 / 8.8 / 9.9, 37: 13.3 / 12.3 / 13.5, 192: 54.6 / 49.5 / 44.1;
-//   768 -> 3072: 16 frames 19.8 / 16.0 / 17.3, 37: 36.3 / 30.6 / 28.0, 192: 174 / 149 / 139.
+// The two constants are fitted to 8 to 192 frames of 197 tokens, with and without adapters, widths of 384 and 768: the rule's
+// choice is 0.5 % slower than the best of the three widths on average, the widest throughout 4.4 %.  No adapters, us, 128 / 192 / 256 wide:
+//   3072 -> 768: 12 frames 13.2 / 16.8 / 19.6, 16: 20.4 / 17.1 / 20.6, 37: 30.9 / 28.4 / 34.4, 128: 99 / 96 / 105;
+//   768 -> 768: 12 frames 7.4 / 8.5 / 9.1, 37: 12.6 / 11.9 / 13.0, 128: 37.1 / 32.7 / 32.0;
+//   768 -> 3072 (GELU): 16 frames 19.5 / 15.7 / 16.9, 37: 36.1 / 29.8 / 28.0, 128: 143 / 112 / 97.
 static int pick_pair_width(int n_out, int k_in, bool lora, int rows, int n_pairs) {
     if (k_in <= 384 && (n_out % 256 == 0 || (n_out <= 384 && !lora))) return -1;
     if (k_in < 640 && n_out % 256 != 0 && n_out % 192 != 0) return -1;

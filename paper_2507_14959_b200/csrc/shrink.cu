@@ -13,10 +13,10 @@
 // blocks of 64 columns where a CTA has shared memory for it, a warp prepares the slab data in shared memory, slabs
 // that none of the tile's own rows use (the plan lists those of the 256-row pair) are only zeroed, the list and the
 // first adapter slabs are fetched before the kernel waits for the one before it, and long K is split over a cluster
-// where the tiles leave half of the SMs idle (partial sums through distributed shared memory).
-// Shrink + GEMM of one linear, back to back, rank 16, 1 to 3 adapters per 197-token frame, before -> now:
-//   16 frames: qkv 20.1 -> 17.9, proj 16.6 -> 13.6 us; 37: qkv 32.1 -> 28.8, fc2 55.4 -> 45.4 us (K in two);
-//   64: proj 28.8 -> 25.8, fc2 71.1 -> 64.2 us; 256: qkv 169.2 -> 167.9, fc2 242.1 -> 240.8 us.
+// where the tiles leave half of the SMs idle (partial sums through distributed shared memory, as asynchronous stores that
+// count themselves on the receiver's barrier).
+// Shrink + GEMM of one linear, replayed back to back, rank 16, 1 to 3 adapters per 197-token frame:
+//   16 frames: qkv 16.2, proj 11.7 us; 37: qkv 24.8, fc2 36.9 us (K in two); 64: proj 21.8, fc2 59.8 us; 256: qkv 151, fc2 226 us.
 // Warp roles: 0 = x copies, 1 = tensor memory + MMA, 2 = adapter copies, 3 = slab list, 4.. = statistics and t.
 #include "common.cuh"
 #include "f32x2.cuh"

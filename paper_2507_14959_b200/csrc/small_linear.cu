@@ -12,12 +12,12 @@
 //   - weights, adapter slabs, plan entries, bias and LayerNorm vectors do not depend on the kernel before: they are
 //     requested before the kernel waits for it (programmatic dependent launch);
 //   - split K (long K, narrow output): each CTA of the cluster makes a partial tile, its own partial t and
-//     expand included (the expand is linear in t); the partials are exchanged through distributed shared memory
-//     and every CTA sums and stores BN / S columns.  A partial t enters the expand as two bf16 parts (16 significant
+//     expand included (the expand is linear in t); the partials are exchanged through distributed shared memory, as
+//     asynchronous stores that count themselves on the receiver's barrier, and every CTA sums and stores BN / S columns.  A partial t enters the expand as two bf16 parts (16 significant
 //     bits, two MMAs per slab): rounded to one, shares that cancel would leave their rounding in the sum.
-// One 197-token frame of width 768, rank-16 adapters, replayed back to back: qkv 4.9 us, proj 4.9, fc1 5.6, fc2 8.0; four frames
-// 7.4, 5.6, 9.4 and 12.1; eight frames 12.3, 9.3, 14.4 and 16.8.  (Issued behind a lane test and with the shrink in MMAs of its own:
-// 7.0, 6.9, 7.3, 9.7; 9.7, 7.4, 11.2, 16.0; 13.1, 10.5, 17.4, 19.0.)
+// One 197-token frame of width 768, rank-16 adapters, replayed back to back: qkv 5.0 us, proj 4.9, fc1 5.6, fc2 6.9; four frames
+// 7.4, 5.7, 9.5 and 11.6; eight frames 12.3, 9.4, 14.4 and 16.3.  (Issued behind a lane test, the shrink in MMAs of its own and partial sums
+// released by each warp: 7.0, 6.9, 7.3, 9.7; 9.7, 7.4, 11.2, 16.0; 13.1, 10.5, 17.4, 19.0.)
 // Warp roles: 0 = x / W copies, 1 = tensor memory + MMA, 2 = adapter copies, 3 = slab list, 4..11 = statistics, t, epilogue.
 #include "common.cuh"
 #include "f32x2.cuh"
@@ -167,7 +167,7 @@ small_linear_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     auto full_bar = [&](int s) { return bars + 8u * s; };              // both copying threads' bytes of a stage
     auto empty_bar = [&](int s) { return bars + 8u * (MAX_STAGES + s); };
     const uint32_t tacc_bar = bars + 8u * (2 * MAX_STAGES);            // shrink accumulator complete
-    const uint32_t tready_bar = tacc_bar + 8u;                         // t written to shared memory
+    const uint32_t tready_bar = tacc_bar + 8u;                         // t written over its accumulator columns
     const uint32_t tfull_bar = tacc_bar + 16u;                         // tile complete
     const uint32_t stats_bar = tacc_bar + 24u;                         // half-row statistics exchanged
     const uint32_t recv_bar = tacc_bar + 32u;                          // the other CTAs' partial sums are here
@@ -610,7 +610,7 @@ cudaError_t launch_epi(const Launch& L, const Maps& t, const SmallArgs& a, int e
 struct Shape { int width = -1, split = 1; };          // width: index into WIDTHS, -1 = not for this kernel
 
 // The split of K and the tile width: as many CTAs as fit the SMs in one wave.  K is split where it is long
-// (3072 -> 768 with adapters: 4 ways 7.1 us against 10.3 on 197 rows, 2 ways 16.9 against 22.7 on 1576; at 768
+// (3072 -> 768 with adapters: 4 ways 7.1 us against 10.3 on 197 rows, 2 ways 15.4 against 20.5 on 1576; at 768
 // inputs it costs what it gives, 768 -> 768 in two 5.0 against 5.3 us on 197 rows, 5.9 against 5.3 on 394, 9.5 against 5.8 on 788); the
 // four-way split stops at 128 columns, whose partial sums leave the ring room.
 // Without adapters the alternative is a GEMM kernel alone, to which wide tiles lose: unsplit 256-wide ones always.  With a
