@@ -463,11 +463,13 @@ constexpr int P_BAR_BYTES = 512;
 // there is a staging buffer for each chunk (request_residual); else 256-wide tiles have one per warp, which leaves the ring its sixth stage.
 // Two per warp and five stages, us, five stages / six, no adapters, frames of 197 tokens: 3072 -> 256, 75 and 256 frames 23.0 / 22.0 and 71.1 / 68.5;
 // 3072 -> 768, 256 frames 165 / 159; 768 -> 2304, 128 frames 67.3 / 66.3, with adapters 81.3 / 77.9.
+// Patch placement stores rows by thread straight to memory, where more warps only spread the writes: eight at 256 columns too
+// (768 -> 768 on 96, 128 and 256 frames of 196 patches 45.8, 57.6 and 104.9 us with sixteen, 44.9, 56.6 and 102.8 with eight).
 template <int BN, int EPI>
 struct PairCfg {
     static constexpr int BUFFERS = BN < 256 || EPI == EPI_RESIDUAL ? 2 : 1;
     static constexpr int STAGING_PER_WARP = BUFFERS * STAGING_BYTES;
-    static constexpr int HALVES = BN / 64;                                 // epilogue warps per lane quarter
+    static constexpr int HALVES = BN == 256 && EPI == EPI_PATCH ? 2 : BN / 64;      // epilogue warps per lane quarter
     static constexpr int EW = 4 * HALVES;
     static constexpr int THREADS = 64 + 32 * EW;
     static constexpr int B_BYTES = (BN / 2) * BK * 2;                      // this CTA's half of the W^T tile
@@ -958,9 +960,9 @@ int gemm_tile_n(int n_out) { return (n_out % 256 == 0) ? 256 : 128; }
 
 LinearForm gemm_form(int k_in, int n_out, bool lora, int rows, int epi, int n_sms) {
     const int pw = n_sms >= 2 ? pick_pair_width(n_out, k_in, lora, rows, n_sms / 2) : -1;
-    if (pw >= 0)
-        return {LINEAR_PAIR, PAIR_WIDTHS[pw], 1, PAIR_WIDTHS[pw] == 128 ? PairCfg<128, EPI_NONE>::THREADS : PAIR_WIDTHS[pw] == 192 ? PairCfg<192, EPI_NONE>::THREADS
-                                                                                                  : PairCfg<256, EPI_NONE>::THREADS};
+    if (pw == 0) return {LINEAR_PAIR, 128, 1, PairCfg<128, EPI_NONE>::THREADS};
+    if (pw == 1) return {LINEAR_PAIR, 192, 1, PairCfg<192, EPI_NONE>::THREADS};
+    if (pw == 2) return {LINEAR_PAIR, 256, 1, epi == EPI_PATCH ? PairCfg<256, EPI_PATCH>::THREADS : PairCfg<256, EPI_NONE>::THREADS};
     const int bn = gemm_tile_n(n_out);
     return {LINEAR_SINGLE, bn, 1, 64 + 32 * (bn == 256 ? Smem<256>::EW : Smem<128>::EW)};
 }

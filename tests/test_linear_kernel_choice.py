@@ -43,3 +43,9 @@ def test_widths_that_only_128_divides_take_pairs_for_long_k(k_in, n_out, kernel,
     (3072, 768, 8, ("pair", 128, 1)), (3072, 768, 12, ("pair", 128, 1)), (768, 320, 8, ("few rows", 64, 1))])
 def test_residuals_without_adapters_leave_the_few_row_kernel_for_narrow_gemm_tiles_only(k_in, n_out, frames, form):
     assert binding.linear_kernel(k_in, n_out, frames * TOKENS, RESIDUAL, False)[:3] == form
+
+
+@pytest.mark.parametrize("epilogue,threads", [(NONE, 576), (GELU, 576), (RESIDUAL, 576), (PATCH, 320)])
+def test_epilogue_warps_of_256_wide_pair_tiles(epilogue, threads):
+    """A warp per 64 columns of a lane quarter; patch placement, which stores by thread, keeps eight warps."""
+    assert binding.linear_kernel(768, 768, 256 * 196, epilogue, epilogue != PATCH) == ("pair", 256, 1, threads)
