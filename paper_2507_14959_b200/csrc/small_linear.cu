@@ -625,6 +625,8 @@ struct Shape { int width = -1, split = 1; };          // width: index into WIDTH
 //   768 -> 768 192-wide 16: 10.3 / 8.9;  192 -> 192 192-wide 32: 7.6 / 4.4.
 // With adapters the alternative is two kernels, whose t is rounded to bf16 once where the shares' t here keep 16 bits: K in two at 256
 // columns stays here although it is slower (3072 -> 768, 12 frames 22.5 / 19.5, 14: 22.5 / 20.6; 2048 -> 512, 24 frames 18.3 / 21.0).
+// Unsplit tiles of long K with adapters, which follow where the split no longer fits, are not always the faster side either: 3072 -> 768
+// 192-wide 16 frames 24.2 / 23.4, 28: 30.5 / 29.3; 4096 -> 1024 256-wide 12: 34.8 / 30.0, 24: 39.0 / 41.7; 1536 -> 640 128-wide 12: 12.8 / 14.8.
 Shape pick_shape(int k_in, int n_out, bool lora, int rows, int epi, int n_sms) {
     const long long m = (rows + BM - 1) / BM;
     const bool long_k = epi == EPI_RESIDUAL && k_in >= 1536, alone = epi == EPI_RESIDUAL && !lora;
